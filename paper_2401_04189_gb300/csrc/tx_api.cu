@@ -173,6 +173,8 @@ static void free_ctx(tx_ctx* c) {
         cudaFree(c->d_A64[d]);
         cudaFree(c->f_U[d]);
         cudaFree(c->f_A[d]);
+        cudaFree(c->f_UK[d]);
+        cudaFree(c->f_AK[d]);
         cudaFree(c->f_w[d]);
         cudaFree(c->f_C[d]);
     }
@@ -241,6 +243,10 @@ extern "C" int tx_tucker_setup(tx_ctx** out, const int n[3], const double* x1, c
         SETUP_TRY(dalloc(&c->d_A64[d], (size_t)T * nd * rd));
         SETUP_TRY(dalloc(&c->f_U[d], nd * rd));
         SETUP_TRY(dalloc(&c->f_A[d], (size_t)T * nd * rd));
+        if (d > 0) {
+            SETUP_TRY(dalloc(&c->f_UK[d], rd * pad4((int)nd)));
+            SETUP_TRY(dalloc(&c->f_AK[d], (size_t)T * rd * pad4((int)nd)));
+        }
         SETUP_TRY(dalloc(&c->f_w[d], nd));
         // host float32 copies are made synchronously (the host arrays may be freed on return)
         std::vector<float> fu(nd * rd), fw(nd);
@@ -260,6 +266,7 @@ extern "C" int tx_tucker_setup(tx_ctx** out, const int n[3], const double* x1, c
         cudaMemcpy(c->d_mu, gauss_weights, sizeof(double) * T, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(c->d_err, 0, sizeof(int) * kErrWords) != cudaSuccess)
         SETUP_TRY(fail(TX_ERR_CUDA, "set-up copy failed"));
+    for (int d = 1; d < 3; ++d) SETUP_TRY(simt_kmajor(c->f_U[d], 1, n[d], r[d], c->f_UK[d], s));
     SETUP_TRY(setup_factor_matrices(c, s));
     SETUP_TRY(tx_set_precision(c, precision, stream));
 #undef SETUP_TRY

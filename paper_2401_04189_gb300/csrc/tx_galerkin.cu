@@ -18,10 +18,11 @@ namespace tx {
 namespace {
 
 // B_td[i][k] = sum_a U_d[a][i] w_d[a] A_td[a][k]  (mu_t is already folded into A_t3), and
-// Ut_d[a][k] = U_d[a][k] / w_d[a].  One thread per output element, float64 sums.
+// Ut_d[a][k] = U_d[a][k] / w_d[a] (modes 2 and 3, ldk > 0: stored [k][a] with row stride ldk, as the
+// consumer reads it).  One thread per output element, float64 sums.
 __global__ void k_galerkin_operators(const double* __restrict__ U, const double* __restrict__ w,
-                                     const double* __restrict__ A64, int n, int r, int T, float* __restrict__ B,
-                                     float* __restrict__ Ut) {
+                                     const double* __restrict__ A64, int n, int r, int T, int ldk,
+                                     float* __restrict__ B, float* __restrict__ Ut) {
     const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const long nb = (long)T * r * r;
     if (e < nb) {
@@ -32,7 +33,8 @@ __global__ void k_galerkin_operators(const double* __restrict__ U, const double*
         B[e] = (float)s;
     } else if (e < nb + (long)n * r) {
         const long q = e - nb;
-        Ut[q] = (float)(U[q] / w[q / r]);
+        const long a = q / r, k = q - a * r;
+        Ut[ldk ? k * ldk + a : q] = (float)(U[q] / w[a]);
     }
 }
 
@@ -70,7 +72,7 @@ __global__ void __launch_bounds__(256) k_core_dot(const PairRec* __restrict__ re
 
 size_t galerkin_operator_floats(const tx_ctx* c) {
     size_t f = 0;
-    for (int d = 0; d < 3; ++d) f += (size_t)c->T * c->r[d] * c->r[d] + (size_t)c->n[d] * c->r[d];
+    for (int d = 0; d < 3; ++d) f += pad4(c->T * c->r[d] * c->r[d]) + (size_t)pad4(c->n[d]) * c->r[d];
     return f;
 }
 
@@ -79,13 +81,13 @@ int galerkin_operators(const tx_ctx* c, float* ops, GalerkinOps* g, cudaStream_t
     for (int d = 0; d < 3; ++d) {
         const int n = c->n[d], r = c->r[d];
         float* B = q;
-        float* Ut = B + (size_t)c->T * r * r;
-        q = Ut + (size_t)n * r;
+        float* Ut = B + pad4(c->T * r * r);
+        q = Ut + (size_t)pad4(n) * r;
         g->B[d] = B;
         g->Ut[d] = Ut;
         const long total = (long)c->T * r * r + (long)n * r;
         k_galerkin_operators<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(c->d_U[d], c->d_w[d], c->d_A64[d], n, r,
-                                                                            c->T, B, Ut);
+                                                                            c->T, d ? pad4(n) : 0, B, Ut);
         TX_LAUNCHED();
     }
     return TX_OK;

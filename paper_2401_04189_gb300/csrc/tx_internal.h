@@ -95,6 +95,8 @@ struct tx_ctx {
     // float32 copies
     float* f_U[3];       // [n_d][r_d]
     float* f_A[3];       // [T][n_d][r_d]; mu_t folded into mode 3
+    float* f_UK[3];      // modes 2 and 3 of f_U with the grid index fastest: [r_d][pad4(n_d)], zero-padded
+    float* f_AK[3];      // modes 2 and 3 of f_A the same way: [T][r_d][pad4(n_d)]
     float* f_w[3];       // [n_d]
     float* f_C[3];       // [T][n_d][n_d] convolution matrices, mu_t folded into mode 3 (per-pair path; lazy)
     bool c_valid;        // f_C matches the current quadrature
@@ -176,7 +178,11 @@ long pair_count(int mode, int n_occ, int n_tgt);
 // forward projection: ws_S2[p][x][g][b] = sum_{y,z} U2[y][b] U3[z][g] rho_p[x][y][z]
 int simt_project_s2(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f,
                     int flags, float* S2, cudaStream_t s);
-// expansion consumer: modes 2 and 3 for every term, Hadamard epilogue, energy partials
+inline int pad4(int v) { return (v + 3) & ~3; }
+// dst[t][k][i] = src[t][i][k], i < n, row stride pad4(n) (zero-padded): the layout the consumer reads
+int simt_kmajor(const float* src, int nt, int n, int r, float* dst, cudaStream_t s);
+// expansion consumer: modes 2 and 3 for every term, Hadamard epilogue, energy partials.
+// M2 [nterms][r2][pad4(n2)] and M3 [nterms][r3][pad4(n3)] (per pair with strides m2_ps, m3_ps)
 int simt_expand_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f,
                         const float* Z, int nterms, const float* M2, const float* M3, int flags,
                         double* epart, cudaStream_t s, long m2_ps = 0, long m3_ps = 0);

@@ -62,11 +62,11 @@ int simt_mode1_project(const tx_ctx* c, const float* S2, float* G, int np, cudaS
 int simt_mode1_expand(const tx_ctx* c, const float* G, const float* M1, int nt, float* Z, int np, cudaStream_t s) {
     const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
     GemmArgs q{};
-    q.M = n1; q.N = rr; q.K = r1;
-    q.A = M1; q.a_m = r1; q.a_k = 1; q.a_b1 = (long)n1 * r1;
+    q.M = nt * n1; q.N = rr; q.K = r1;
+    q.A = M1; q.a_m = r1; q.a_k = 1;
     q.B = G; q.b_k = 1; q.b_n = r1; q.b_b2 = (long)rr * r1;
-    q.C = Z; q.c_m = rr; q.c_n = 1; q.c_b1 = (long)n1 * rr; q.c_b2 = (long)nt * n1 * rr;
-    q.nb1 = nt; q.nb2 = np; q.alpha = 1.f;
+    q.C = Z; q.c_m = rr; q.c_n = 1; q.c_b2 = (long)nt * n1 * rr;
+    q.nb1 = 1; q.nb2 = np; q.alpha = 1.f;
     return simt_gemm(q, s);
 }
 
@@ -126,7 +126,7 @@ extern "C" int tx_exchange_apply_static(tx_ctx* c, const float* psi_occ, int n_o
         TX_TRY(simt_project_s2(c, recs, (int)p0, np, f, 0, S2, s));
         TX_TRY(simt_mode1_project(c, S2, G, np, s));
         TX_TRY(simt_mode1_expand(c, G, c->f_A[0], c->T, Z, np, s));
-        TX_TRY(simt_expand_consume(c, recs, (int)p0, np, f, Z, c->T, c->f_A[1], c->f_A[2], EPI_OUT, nullptr, s));
+        TX_TRY(simt_expand_consume(c, recs, (int)p0, np, f, Z, c->T, c->f_AK[1], c->f_AK[2], EPI_OUT, nullptr, s));
     }
     return TX_OK;
 }

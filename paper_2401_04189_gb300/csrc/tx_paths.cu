@@ -56,11 +56,11 @@ int gemm_mode1_expand(const tx_ctx* c, const float* G, const float* M1, int nt, 
                       long m1_ps = 0) {
     const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
     GemmArgs g{};
-    g.M = n1; g.N = rr; g.K = r1;
-    g.A = M1; g.a_m = r1; g.a_k = 1; g.a_b1 = (long)n1 * r1; g.a_b2 = m1_ps;
-    g.B = G; g.b_k = 1; g.b_n = r1; g.b_b1 = 0; g.b_b2 = (long)rr * r1;
-    g.C = Z; g.c_m = rr; g.c_n = 1; g.c_b1 = (long)n1 * rr; g.c_b2 = (long)nt * n1 * rr;
-    g.nb1 = nt; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
+    g.M = nt * n1; g.N = rr; g.K = r1;         // the terms' rows (t, x) follow one another in M1 and in Z
+    g.A = M1; g.a_m = r1; g.a_k = 1; g.a_b2 = m1_ps;
+    g.B = G; g.b_k = 1; g.b_n = r1; g.b_b2 = (long)rr * r1;
+    g.C = Z; g.c_m = rr; g.c_n = 1; g.c_b2 = (long)nt * n1 * rr;
+    g.nb1 = 1; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
     return simt_gemm(g, s);
 }
 
@@ -85,13 +85,13 @@ int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec
             if (cs.kind == CALL_APPLY) flags = EPI_OUT | (cs.e_dev ? EPI_ENERGY : 0);
             if (cs.kind == CALL_ENERGY) flags = EPI_ENERGY;
             if (cs.kind == CALL_GRAD) flags = EPI_OUT | EPI_MULW | (cs.e_dev ? EPI_ENERGY : 0);
-            TX_TRY(simt_expand_consume(c, recs, p0, np, f, Z, c->T, c->f_A[1], c->f_A[2], flags, epart, s));
+            TX_TRY(simt_expand_consume(c, recs, p0, np, f, Z, c->T, c->f_AK[1], c->f_AK[2], flags, epart, s));
             if (cs.kind == CALL_GRAD) {
                 // second term: - sum_j psi_j * L^T(w rho_kj)
                 TX_TRY(simt_adjoint_r(c, recs, p0, np, f, PROD_MULW, Z, s));
                 TX_TRY(gemm_mode1_adjoint(c, Z, G, np, s));
                 TX_TRY(gemm_mode1_expand(c, G, c->f_U[0], 1, Z, np, s));
-                TX_TRY(simt_expand_consume(c, recs, p0, np, f, Z, 1, c->f_U[1], c->f_U[2], EPI_OUT, epart, s));
+                TX_TRY(simt_expand_consume(c, recs, p0, np, f, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, epart, s));
             }
             return TX_OK;
         }
@@ -104,7 +104,7 @@ int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec
                 TX_TRY(simt_project_s2(c, recs, p0, np, f, 0, S2, s));
                 TX_TRY(gemm_mode1_project(c, S2, c->f_U[0], G, np, s));
                 TX_TRY(gemm_mode1_expand(c, G, c->f_A[0], c->T, Z, np, s));
-                TX_TRY(simt_expand_consume(c, recs, p0, np, f, Z, c->T, c->f_A[1], c->f_A[2], EPI_OUT, epart, s));
+                TX_TRY(simt_expand_consume(c, recs, p0, np, f, Z, c->T, c->f_AK[1], c->f_AK[2], EPI_OUT, epart, s));
             }
             // zeta_kj = L^T(cot_k psi_j): grad_tgt_k -= psi_j zeta, grad_occ_j -= psi_tgt_k zeta
             FieldArgs f2{};
@@ -114,7 +114,7 @@ int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec
             TX_TRY(simt_adjoint_r(c, recs2, p0, np, f2, 0, Z, s));
             TX_TRY(gemm_mode1_adjoint(c, Z, G, np, s));
             TX_TRY(gemm_mode1_expand(c, G, c->f_U[0], 1, Z, np, s));
-            TX_TRY(simt_expand_consume(c, recs2, p0, np, f2, Z, 1, c->f_U[1], c->f_U[2], EPI_OUT, epart, s));
+            TX_TRY(simt_expand_consume(c, recs2, p0, np, f2, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, epart, s));
             return TX_OK;
         }
     }

@@ -192,8 +192,8 @@ size_t sthosvd_floats_per_pair(const tx_ctx* c) {
            n3 * r2 * r1 +                       // T2
            r3 * r2 * r1 +                       // G
            nmax * nmax +                        // Gram matrix
-           n1 * r1 + n2 * r2 + n3 * r3 +        // U_d
-           T * (n1 * r1 + n2 * r2 + n3 * r3) +  // A_td per pair
+           n1 * r1 + n2 * r2 + n3 * r3 + 8 +    // U_d (8: the operators after them start on 16 bytes)
+           pad4((int)(T * n1 * r1)) + T * (pad4((int)n2) * r2 + pad4((int)n3) * r3) +  // A_td per pair
            T * n1 * r3 * r2;                    // Z
 }
 
@@ -217,10 +217,12 @@ int sthosvd_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, int p0, in
     float* U1 = S + (size_t)np * nmax * nmax;
     float* U2 = U1 + (size_t)np * n1 * r1;
     float* U3 = U2 + (size_t)np * n2 * r2;
-    float* A1 = U3 + (size_t)np * n3 * r3;
-    float* A2 = A1 + (size_t)np * T * n1 * r1;
-    float* A3 = A2 + (size_t)np * T * n2 * r2;
-    float* Z = A3 + (size_t)np * T * n3 * r3;
+    // modes 2 and 3 with the grid index fastest (the consumer's layout), 16-byte aligned
+    const long a1_ps = pad4(T * n1 * r1), a2_ps = (long)T * pad4(n2) * r2, a3_ps = (long)T * pad4(n3) * r3;
+    float* A1 = (float*)(((uintptr_t)(U3 + (size_t)np * n3 * r3) + 15) & ~(uintptr_t)15);
+    float* A2 = A1 + (size_t)np * a1_ps;
+    float* A3 = A2 + (size_t)np * a2_ps;
+    float* Z = A3 + (size_t)np * a3_ps;
     const bool subset = cs.mode == PAIRS_SUBSET;
     FieldArgs f{};
     f.SA = subset ? cs.occ : cs.tgt;
@@ -282,14 +284,18 @@ int sthosvd_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, int p0, in
         g.M = n; g.N = r; g.K = n;
         g.A = c->f_C[d]; g.a_m = n; g.a_k = 1; g.a_b1 = (long)n * n; g.a_b2 = 0;
         g.B = Us[d]; g.b_k = r; g.b_n = 1; g.b_b1 = 0; g.b_b2 = (long)n * r;
-        g.C = As[d]; g.c_m = r; g.c_n = 1; g.c_b1 = (long)n * r; g.c_b2 = (long)T * n * r;
+        g.C = As[d];
+        if (d == 0) {
+            g.c_m = r; g.c_n = 1; g.c_b1 = (long)n * r; g.c_b2 = a1_ps;
+        } else {
+            g.c_m = 1; g.c_n = pad4(n); g.c_b1 = (long)pad4(n) * r; g.c_b2 = d == 1 ? a2_ps : a3_ps;
+        }
         g.nb1 = T; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
         TX_TRY(simt_gemm(g, s));
     }
     // ---- expansion with the per-pair operators, Hadamard epilogue
-    TX_TRY(simt_expand_mode1_pp(c, G, A1, (long)T * n1 * r1, T, Z, np, s));
-    return simt_expand_consume(c, recs, p0, np, f, Z, T, A2, A3, EPI_OUT, epart, s, (long)T * n2 * r2,
-                               (long)T * n3 * r3);
+    TX_TRY(simt_expand_mode1_pp(c, G, A1, a1_ps, T, Z, np, s));
+    return simt_expand_consume(c, recs, p0, np, f, Z, T, A2, A3, EPI_OUT, epart, s, a2_ps, a3_ps);
 }
 
 }  // namespace tx

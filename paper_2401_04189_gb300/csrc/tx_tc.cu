@@ -255,11 +255,11 @@ static int f32_mode1_project(const tx_ctx* c, const float* S2, float* G, int np,
 static int f32_mode1_expand(const tx_ctx* c, const float* G, float* Z, int np, cudaStream_t s) {
     const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2], T = c->T;
     GemmArgs g{};
-    g.M = n1; g.N = rr; g.K = r1;
-    g.A = c->f_A[0]; g.a_m = r1; g.a_k = 1; g.a_b1 = (long)n1 * r1;
+    g.M = T * n1; g.N = rr; g.K = r1;
+    g.A = c->f_A[0]; g.a_m = r1; g.a_k = 1;
     g.B = G; g.b_k = 1; g.b_n = r1; g.b_b2 = (long)rr * r1;
-    g.C = Z; g.c_m = rr; g.c_n = 1; g.c_b1 = (long)n1 * rr; g.c_b2 = (long)T * n1 * rr;
-    g.nb1 = T; g.nb2 = np; g.alpha = 1.f;
+    g.C = Z; g.c_m = rr; g.c_n = 1; g.c_b2 = (long)T * n1 * rr;
+    g.nb1 = 1; g.nb2 = np; g.alpha = 1.f;
     return simt_gemm(g, s);
 }
 
@@ -399,7 +399,7 @@ static int tc_adjoint(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, con
     }
     TX_TRY(simt_adjoint_mode1(c, R, H, np, s));                  // H = sum_{t,x} R A_t1
     TX_TRY(simt_expand_mode1(c, H, c->f_U[0], 1, Z, np, s));     // Z = U1 H
-    return simt_expand_consume(c, recs, b.p0, np, fo, Z, 1, c->f_U[1], c->f_U[2], EPI_OUT, b.epart, s);
+    return simt_expand_consume(c, recs, b.p0, np, fo, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, b.epart, s);
 }
 
 size_t tc_adjoint_bytes_per_pair(const tx_ctx* c) {
