@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256) k_core_dot(const PairRec* __restrict__ re
 
 size_t galerkin_operator_floats(const tx_ctx* c) {
     size_t f = 0;
-    for (int d = 0; d < 3; ++d) f += pad4(c->T * c->r[d] * c->r[d]) + (size_t)pad4(c->n[d]) * c->r[d];
+    for (int d = 0; d < 3; ++d) f += pad4(c->T * c->r[d] * c->r[d]) + (size_t)std::max(simt_ld2(c->n[d]), simt_ld3(c->n[d])) * c->r[d];
     return f;
 }
 
@@ -82,12 +82,12 @@ int galerkin_operators(const tx_ctx* c, float* ops, GalerkinOps* g, cudaStream_t
         const int n = c->n[d], r = c->r[d];
         float* B = q;
         float* Ut = B + pad4(c->T * r * r);
-        q = Ut + (size_t)pad4(n) * r;
+        q = Ut + (size_t)std::max(simt_ld2(n), simt_ld3(n)) * r;
         g->B[d] = B;
         g->Ut[d] = Ut;
         const long total = (long)c->T * r * r + (long)n * r;
         k_galerkin_operators<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(c->d_U[d], c->d_w[d], c->d_A64[d], n, r,
-                                                                            c->T, d ? pad4(n) : 0, B, Ut);
+                                                                            c->T, d == 0 ? 0 : d == 1 ? simt_ld2(n) : simt_ld3(n), B, Ut);
         TX_LAUNCHED();
     }
     return TX_OK;
@@ -95,30 +95,30 @@ int galerkin_operators(const tx_ctx* c, float* ops, GalerkinOps* g, cudaStream_t
 
 // H[p] = sum_t G[p] x1 B_t1 x2 B_t2 x3 B_t3, three batched GEMM passes over all terms.  Each pass
 // contracts the fastest index of its input and writes the new index slowest, so the layout
-// turns [g][b][a] -> [a'][g][b] -> [b'][a'][g] -> [g'][b'][a'] (back to G's own order).
+// turns [b][g][a] -> [a'][b][g] -> [g'][a'][b] -> [b'][g'][a'] (back to G's own order).
 int galerkin_core(const tx_ctx* c, const GalerkinOps& o, const float* G, float* X1, float* X2, float* H, int np,
                   cudaStream_t s) {
     const int r1 = c->r[0], r2 = c->r[1], r3 = c->r[2], T = c->T;
     const long m = (long)r1 * r2 * r3;
     GemmArgs g{};
     g.nb1 = T; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
-    // mode 1: X1[p][t][a'][(g,b)] = sum_a B_t1[a'][a] G[p][(g,b)][a]
+    // mode 1: X1[p][t][a'][(b,g)] = sum_a B_t1[a'][a] G[p][(b,g)][a]
     g.M = r1; g.N = r3 * r2; g.K = r1;
     g.A = o.B[0]; g.a_m = r1; g.a_k = 1; g.a_b1 = (long)r1 * r1; g.a_b2 = 0;
     g.B = G; g.b_k = 1; g.b_n = r1; g.b_b1 = 0; g.b_b2 = m;
     g.C = X1; g.c_m = (long)r3 * r2; g.c_n = 1; g.c_b1 = m; g.c_b2 = T * m;
     TX_TRY(simt_gemm(g, s));
-    // mode 2: X2[p][t][b'][(a',g)] = sum_b B_t2[b'][b] X1[p][t][(a',g)][b]
-    g.M = r2; g.N = r1 * r3; g.K = r2;
-    g.A = o.B[1]; g.a_m = r2; g.a_k = 1; g.a_b1 = (long)r2 * r2; g.a_b2 = 0;
-    g.B = X1; g.b_k = 1; g.b_n = r2; g.b_b1 = m; g.b_b2 = T * m;
-    g.C = X2; g.c_m = (long)r1 * r3; g.c_n = 1; g.c_b1 = m; g.c_b2 = T * m;
-    TX_TRY(simt_gemm(g, s));
-    // mode 3: X1[p][t][g'][(b',a')] = sum_g B_t3[g'][g] X2[p][t][(b',a')][g]   (mu_t inside B_t3)
-    g.M = r3; g.N = r2 * r1; g.K = r3;
+    // mode 3: X2[p][t][g'][(a',b)] = sum_g B_t3[g'][g] X1[p][t][(a',b)][g]   (mu_t inside B_t3)
+    g.M = r3; g.N = r1 * r2; g.K = r3;
     g.A = o.B[2]; g.a_m = r3; g.a_k = 1; g.a_b1 = (long)r3 * r3; g.a_b2 = 0;
-    g.B = X2; g.b_k = 1; g.b_n = r3; g.b_b1 = m; g.b_b2 = T * m;
-    g.C = X1; g.c_m = (long)r2 * r1; g.c_n = 1; g.c_b1 = m; g.c_b2 = T * m;
+    g.B = X1; g.b_k = 1; g.b_n = r3; g.b_b1 = m; g.b_b2 = T * m;
+    g.C = X2; g.c_m = (long)r1 * r2; g.c_n = 1; g.c_b1 = m; g.c_b2 = T * m;
+    TX_TRY(simt_gemm(g, s));
+    // mode 2: X1[p][t][b'][(g',a')] = sum_b B_t2[b'][b] X2[p][t][(g',a')][b]
+    g.M = r2; g.N = r3 * r1; g.K = r2;
+    g.A = o.B[1]; g.a_m = r2; g.a_k = 1; g.a_b1 = (long)r2 * r2; g.a_b2 = 0;
+    g.B = X2; g.b_k = 1; g.b_n = r2; g.b_b1 = m; g.b_b2 = T * m;
+    g.C = X1; g.c_m = (long)r3 * r1; g.c_n = 1; g.c_b1 = m; g.c_b2 = T * m;
     TX_TRY(simt_gemm(g, s));
     const long total = np * m;
     const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 16);

@@ -95,8 +95,8 @@ struct tx_ctx {
     // float32 copies
     float* f_U[3];       // [n_d][r_d]
     float* f_A[3];       // [T][n_d][r_d]; mu_t folded into mode 3
-    float* f_UK[3];      // modes 2 and 3 of f_U with the grid index fastest: [r_d][pad4(n_d)], zero-padded
-    float* f_AK[3];      // modes 2 and 3 of f_A the same way: [T][r_d][pad4(n_d)]
+    float* f_UK[3];      // modes 2 and 3 of f_U with the grid index fastest: [r_d][simt_ld(n_d)], zero-padded
+    float* f_AK[3];      // modes 2 and 3 of f_A the same way: [T][r_d][simt_ld(n_d)]
     float* f_w[3];       // [n_d]
     float* f_C[3];       // [T][n_d][n_d] convolution matrices, mu_t folded into mode 3 (per-pair path; lazy)
     bool c_valid;        // f_C matches the current quadrature
@@ -175,19 +175,24 @@ struct FieldArgs {          // orbital-space arrays of one call
 int build_pairs(PairRec* d_recs, int mode, int role, int n_occ, int n_tgt, int k0, cudaStream_t s);
 long pair_count(int mode, int n_occ, int n_tgt);
 
-// forward projection: ws_S2[p][x][g][b] = sum_{y,z} U2[y][b] U3[z][g] rho_p[x][y][z]
+// forward projection: ws_S2[p][x][(b,g)] = sum_{y,z} U2[y][b] U3[z][g] rho_p[x][y][z] ((g,b) order without bg)
 int simt_project_s2(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f,
-                    int flags, float* S2, cudaStream_t s);
+                    int flags, float* S2, cudaStream_t s, bool bg = true);
 inline int pad4(int v) { return (v + 3) & ~3; }
-// dst[t][k][i] = src[t][i][k], i < n, row stride pad4(n) (zero-padded): the layout the consumer reads
-int simt_kmajor(const float* src, int nt, int n, int r, float* dst, cudaStream_t s);
+// row strides of the operators that the float32 consumer reads, [r2][simt_ld2(n2)] and
+// [r3][simt_ld3(n3)] with the grid index fastest (rows padded to its thread tiles)
+int simt_ld2(int n2);
+int simt_ld3(int n3);
+// dst[t][k][i] = src[t][i][k], i < n, row stride ld (zero-padded)
+int simt_kmajor(const float* src, int nt, int n, int r, int ld, float* dst, cudaStream_t s);
 // expansion consumer: modes 2 and 3 for every term, Hadamard epilogue, energy partials.
-// M2 [nterms][r2][pad4(n2)] and M3 [nterms][r3][pad4(n3)] (per pair with strides m2_ps, m3_ps)
+// Z [np][nterms][n1][(b,g)] (z_bg) or [(g,b)]; M2 [nterms][r2][simt_ld2] and M3 [nterms][r3][simt_ld3]
+// (per pair with strides m2_ps, m3_ps)
 int simt_expand_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f,
                         const float* Z, int nterms, const float* M2, const float* M3, int flags,
-                        double* epart, cudaStream_t s, long m2_ps = 0, long m3_ps = 0);
+                        double* epart, cudaStream_t s, bool z_bg = true, long m2_ps = 0, long m3_ps = 0);
 int simt_expand_consume_blocks(const tx_ctx* c);
-// adjoint stage: R[p][t][x][g][b] = sum_{y,z} A_t2[y][b] A_t3[z][g] (prod)[x][y][z]
+// adjoint stage: R[p][t][x][b][g] = sum_{y,z} A_t2[y][b] A_t3[z][g] (prod)[x][y][z]
 int simt_adjoint_r(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f,
                    int flags, float* R, cudaStream_t s);
 // energy reductions

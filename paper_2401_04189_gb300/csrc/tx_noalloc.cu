@@ -46,7 +46,7 @@ int static_scratch(int dev, void** out) {
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// G[p][(g,b)][a] = sum_x S2[p][x][(g,b)] U1[x][a]  (mode 1 of the projection)
+// G[p][(b,g)][a] = sum_x S2[p][x][(b,g)] U1[x][a]  (mode 1 of the projection)
 int simt_mode1_project(const tx_ctx* c, const float* S2, float* G, int np, cudaStream_t s) {
     const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
     GemmArgs q{};
@@ -58,7 +58,7 @@ int simt_mode1_project(const tx_ctx* c, const float* S2, float* G, int np, cudaS
     return simt_gemm(q, s);
 }
 
-// Z[p][t][x][(g,b)] = sum_a M1_t[x][a] G[p][(g,b)][a]  (mode 1 of the expansion, every term)
+// Z[p][t][x][(b,g)] = sum_a M1_t[x][a] G[p][(b,g)][a]  (mode 1 of the expansion, every term)
 int simt_mode1_expand(const tx_ctx* c, const float* G, const float* M1, int nt, float* Z, int np, cudaStream_t s) {
     const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
     GemmArgs q{};

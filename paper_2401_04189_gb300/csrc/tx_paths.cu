@@ -26,7 +26,7 @@ SimtLayout simt_layout(const tx_ctx* c) {
     return L;
 }
 
-// G[p][(g,b)][a] = sum_x S2[p][x][(g,b)] M1[x][a]   (mode 1 of the projection; M1 = U1)
+// G[p][(b,g)][a] = sum_x S2[p][x][(b,g)] M1[x][a]   (mode 1 of the projection; M1 = U1)
 int gemm_mode1_project(const tx_ctx* c, const float* S2, const float* M1, float* G, int np, cudaStream_t s) {
     const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
     GemmArgs g{};
@@ -38,7 +38,7 @@ int gemm_mode1_project(const tx_ctx* c, const float* S2, const float* M1, float*
     return simt_gemm(g, s);
 }
 
-// H[p][(g,b)][a] = sum_{t,x} R[p][t][x][(g,b)] A_t1[x][a]   (mode 1 of the adjoint, summed over t)
+// H[p][(b,g)][a] = sum_{t,x} R[p][t][x][(b,g)] A_t1[x][a]   (mode 1 of the adjoint, summed over t)
 int gemm_mode1_adjoint(const tx_ctx* c, const float* R, float* H, int np, cudaStream_t s) {
     const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2], T = c->T;
     GemmArgs g{};
@@ -50,7 +50,7 @@ int gemm_mode1_adjoint(const tx_ctx* c, const float* R, float* H, int np, cudaSt
     return simt_gemm(g, s);
 }
 
-// Z[p][t][x][(g,b)] = sum_a M1_t[x][a] G[p][(g,b)][a]   (mode 1 of the expansion, every term;
+// Z[p][t][x][(b,g)] = sum_a M1_t[x][a] G[p][(b,g)][a]   (mode 1 of the expansion, every term;
 // M1 per pair when m1_ps > 0)
 int gemm_mode1_expand(const tx_ctx* c, const float* G, const float* M1, int nt, float* Z, int np, cudaStream_t s,
                       long m1_ps = 0) {
@@ -138,7 +138,7 @@ int galerkin_batch(tx_ctx* c, const CallSpec& cs, const GalerkinOps& o, const Pa
     TX_TRY(gemm_mode1_project(c, S2, c->f_U[0], G, np, s));
     TX_TRY(galerkin_core(c, o, G, X1, X2, H, np, s));
     if (cs.kind == CALL_ENERGY) return galerkin_core_dot(c, recs, p0, G, H, np, epart, s);
-    float* Z = S2;   // [np][1][n1][r3 r2]: the size of S2
+    float* Z = S2;   // [np][1][n1][r2 r3]: the size of S2
     TX_TRY(gemm_mode1_expand(c, H, o.Ut[0], 1, Z, np, s));
     return simt_expand_consume(c, recs, p0, np, f, Z, 1, o.Ut[1], o.Ut[2], EPI_OUT, epart, s);
 }
@@ -188,7 +188,8 @@ int run_call(tx_ctx* c, const CallSpec& cs, cudaStream_t s) {
     per_pair += sizeof(double) * epp;
     size_t avail = c->ws_limit > recs_bytes + prefix + 4096 ? c->ws_limit - recs_bytes - prefix - 4096 : 0;
     long Pb = std::max<long>(1, std::min<long>(P, (long)(avail / per_pair)));
-    Pb = std::min<long>(Pb, 65535 / std::max(1, c->T));   // grid.z of the per-term GEMMs is T * pairs
+    // grid.z of the batched GEMMs is T * pairs (per-pair bases: also r1 or r2 times the pairs)
+    Pb = std::min<long>(Pb, 65535 / std::max(std::max(1, c->T), pp ? std::max(c->r[0], c->r[1]) : 1));
     const long nb = (P + Pb - 1) / Pb;
     const size_t batch_bytes = align_up((size_t)Pb * per_pair, 256) + 4096;
     TX_TRY(ensure_workspace(c, recs_bytes + prefix + batch_bytes));

@@ -34,7 +34,7 @@ int simt_expand_mode1_pp(const tx_ctx* c, const float* G, const float* M1, long 
 // two-sided (Galerkin) projection (tx_galerkin.cu): B_td = U_d^T D_d A_td and D_d^-1 U_d
 struct GalerkinOps {
     const float* B[3];           // [T][r_d][r_d], mu_t folded into mode 3
-    const float* Ut[3];          // mode 1 [n_1][r_1]; modes 2, 3 [r_d][pad4(n_d)]
+    const float* Ut[3];          // mode 1 [n_1][r_1]; modes 2, 3 [r_d][simt_ld(n_d)]
 };
 size_t galerkin_operator_floats(const tx_ctx* c);
 int galerkin_operators(const tx_ctx* c, float* ops, GalerkinOps* g, cudaStream_t s);

@@ -130,7 +130,7 @@ int setup_factor_matrices_fe(tx_ctx* c, int order, int points, cudaStream_t s, b
                                                                          with_c ? c->f_C[dd] : nullptr);
         count_launch();
         if (cudaGetLastError() != cudaSuccess) st = fail(TX_ERR_CUDA, "k_conv_factor_fe launch");
-        if (st == TX_OK && dd > 0) st = simt_kmajor(c->f_A[dd], c->T, n, r, c->f_AK[dd], s);
+        if (st == TX_OK && dd > 0) st = simt_kmajor(c->f_A[dd], c->T, n, r, dd == 1 ? simt_ld2(n) : simt_ld3(n), c->f_AK[dd], s);
     }
     cudaStreamSynchronize(s);
     cudaFree(d);
@@ -145,7 +145,7 @@ int setup_factor_matrices(tx_ctx* c, cudaStream_t s, bool with_c) {
                                                         d == 2 ? 1 : 0, c->d_A64[d], c->f_A[d],
                                                         with_c ? c->f_C[d] : nullptr);
         TX_LAUNCHED();
-        if (d > 0) TX_TRY(simt_kmajor(c->f_A[d], c->T, n, r, c->f_AK[d], s));
+        if (d > 0) TX_TRY(simt_kmajor(c->f_A[d], c->T, n, r, d == 1 ? simt_ld2(n) : simt_ld3(n), c->f_AK[d], s));
     }
     return TX_OK;
 }

@@ -134,7 +134,7 @@ __device__ __forceinline__ int gemm_index(int t, int i) {
 }
 
 template <int BM, int BN>
-__global__ void __launch_bounds__(256) k_gemm(GemmArgs g, int modeA, int modeB, int vecC) {
+__global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3) k_gemm(GemmArgs g, int modeA, int modeB, int vecC) {
     constexpr int TM = BM / 16, TN = BN / 16;
     __shared__ __align__(16) float As[2][GK * (BM + 4)];
     __shared__ __align__(16) float Bs[2][GK * (BN + 4)];
@@ -260,54 +260,63 @@ __global__ void k_build_pairs(PairRec* recs, int mode, int role, int n_occ, int 
 }
 
 // ====================================================================================
-// The two inner loops every float32 mode product is built from.  A thread owns 4 neighbouring
-// rows (one 16-byte fragment, two packed pairs) and RG columns tz, tz + 8, ... of a panel:
-// acc[c] += A[k][row .. row + 3] * B[k][tz + 8 c], both operands K-major in shared memory.
-// The 8 column lanes x 4 row groups of a warp read one 64-byte and one 32-byte segment per
-// fragment (broadcast), so the float32 pipes, not shared memory, bound it from RG = 4 on.
-// ====================================================================================
-constexpr int kMaxRG = 8;          // columns per thread; a panel is at most 64 columns wide
-
-template <int RG>
-__device__ __forceinline__ void panel(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, int K,
-                                      uint64_t (&acc)[kMaxRG][2]) {
-#pragma unroll 4
-    for (int k = 0; k < K; ++k) {
-        const ulonglong2 a = *(const ulonglong2*)(A + k * lda);
-#pragma unroll
-        for (int c = 0; c < RG; ++c) {
-            const uint64_t b = dup2(B[k * ldb + 8 * c]);
-            fma2(acc[c][0], a.x, b);
-            fma2(acc[c][1], a.y, b);
-        }
-    }
-}
-
-// B must be readable up to column 8 * rg - 1 (its row stride is at least that)
-__device__ __forceinline__ void panel_any(int rg, const float* A, int lda, const float* B, int ldb, int K,
-                                          uint64_t (&acc)[kMaxRG][2]) {
-    switch (rg) {
-        case 1: panel<1>(A, lda, B, ldb, K, acc); break;
-        case 2: panel<2>(A, lda, B, ldb, K, acc); break;
-        case 3: panel<3>(A, lda, B, ldb, K, acc); break;
-        case 4: panel<4>(A, lda, B, ldb, K, acc); break;
-        case 5: panel<5>(A, lda, B, ldb, K, acc); break;
-        case 6: panel<6>(A, lda, B, ldb, K, acc); break;
-        case 7: panel<7>(A, lda, B, ldb, K, acc); break;
-        default: panel<8>(A, lda, B, ldb, K, acc); break;
-    }
-}
-
-// ====================================================================================
-// modes 3 and 2 of a projection: out[p][t][x][g][b] = sum_{y,z} M2_t[y][b] M3_t[z][g] q_p[x][y][z]
+// modes 3 and 2 of a projection: out[p][t][x][(b,g)] = sum_{y,z} M2_t[y][b] M3_t[z][g] q_p[x][y][z]
 // with q_p the product of two orbitals (times the quadrature weights where asked).  One term with
 // M3 = U3, M2 = U2 is the projection onto the core; the Gaussian terms' A_t3, A_t2 give the
 // adjoint's first two modes.  One CTA per (x, pair): the plane's product is staged z-major in
-// slices of PZ columns, mode 3 leaves S1[y][g] in shared memory and mode 2 reads it there.
-// With rows of 4 y x RG g per thread instead of one output per thread, the Pt-shaped projection
-// (96^3, rank 40) takes 8.7 us per pair instead of 16.3.
+// slices of PZ columns (the next slice's orbitals are already in registers), mode 3 (8 y x up to
+// 8 g per thread) leaves S1[y][g] in shared memory and mode 2 (4 b x up to 8 g) reads it there.
+// Bound by shared-memory reads and the float32 pipes about equally.  Pt-shaped projection (96^3,
+// rank 40): 6.6 us per pair; 8.7 with 4 rows per thread and no prefetch, 16.3 with one output per thread.
 // ====================================================================================
-constexpr int PZ = 32;             // z columns per slice
+constexpr int kRows = 8;           // rows per thread of the tall thread tiles
+constexpr int PZ = 16;             // z columns per slice
+
+// acc[c] += A[k][8 rows] * B[k][CL c], both K-major in shared memory
+template <int CL, int RG, int NA>
+__device__ __forceinline__ void panel8(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, int K,
+                                       uint64_t (&acc)[NA][4]) {
+#pragma unroll 2
+    for (int k = 0; k < K; ++k) {
+        const ulonglong2 a = *(const ulonglong2*)(A + k * lda), a2 = *(const ulonglong2*)(A + k * lda + 4);
+#pragma unroll
+        for (int c = 0; c < RG; ++c) {
+            const uint64_t b = dup2(B[k * ldb + CL * c]);
+            fma2(acc[c][0], a.x, b);
+            fma2(acc[c][1], a.y, b);
+            fma2(acc[c][2], a2.x, b);
+            fma2(acc[c][3], a2.y, b);
+        }
+    }
+}
+// the same for rg column groups, rg <= NA (a runtime value: every warp takes the same branch)
+template <int CL, int NA>
+__device__ __forceinline__ void panel8_any(int rg, const float* A, int lda, const float* B, int ldb, int K,
+                                           uint64_t (&acc)[NA][4]) {
+    if (rg == 1) panel8<CL, 1>(A, lda, B, ldb, K, acc);
+    else if (rg == 2) panel8<CL, 2>(A, lda, B, ldb, K, acc);
+    else if (rg == 3) panel8<CL, 3>(A, lda, B, ldb, K, acc);
+    else if (NA == 4 || rg == 4) panel8<CL, 4>(A, lda, B, ldb, K, acc);
+    else if (NA == 5 || rg == 5) panel8<CL, NA < 5 ? 4 : 5>(A, lda, B, ldb, K, acc);
+    else if (rg == 6) panel8<CL, NA < 6 ? 4 : 6>(A, lda, B, ldb, K, acc);
+    else panel8<CL, NA < 8 ? 4 : 8>(A, lda, B, ldb, K, acc);
+}
+
+// s[c] += sum_k M[k][4 b] * S[k][col[c]]
+template <int CB>
+__device__ __forceinline__ void panel4(const float* __restrict__ M, int ldm, const float* __restrict__ S, int lds,
+                                       const int (&col)[8], int K, uint64_t (&s)[8][2]) {
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+        const ulonglong2 m = *(const ulonglong2*)(M + k * ldm);
+#pragma unroll
+        for (int c = 0; c < CB; ++c) {
+            const uint64_t q = dup2(S[k * lds + col[c]]);
+            fma2(s[c][0], m.x, q);
+            fma2(s[c][1], m.y, q);
+        }
+    }
+}
 
 struct ChainArgs {
     Dims d;
@@ -322,17 +331,18 @@ struct ChainArgs {
     const float* w3;
     int flags;
     float* out;
-    int ty, gw, bw;                // y rows per tile (a multiple of 4), g (<= 64) and b (<= 256) columns per pass
+    int ty, gw, bw, mh;            // y rows per tile (a multiple of 8), g (<= 64) and b (<= 256) columns per pass, M2 rows held
     int ldy, ldg, ldb, vec;        // shared-memory row strides; vec: 16-byte orbital rows
+    int bg;                        // 1: out[b][g] (the float32 consumer's order), 0: out[g][b]
 };
 
-__global__ void __launch_bounds__(512) k_chain(const ChainArgs a) {
+__global__ void __launch_bounds__(384) k_chain(const ChainArgs a) {
     extern __shared__ __align__(16) float sm[];
     const Dims d = a.d;
     float* qs = sm;                            // [PZ][ldy]   the pair product, z-major
-    float* m3s = qs + PZ * a.ldy;              // [PZ][ldg]
+    float* m2s = qs + PZ * a.ldy;              // [mh][ldb]
+    float* m3s = m2s + a.mh * a.ldb;           // [PZ][ldg]
     float* s1 = m3s + PZ * a.ldg;              // [ty][ldg]
-    float* m2s = s1 + a.ty * a.ldg;            // [PZ][ldb]
     const int x = blockIdx.x, pl = blockIdx.y, tid = threadIdx.x, nth = blockDim.x;
     const PairRec rec = a.recs[a.p0 + pl];
     const long N3 = (long)d.n1 * d.n2 * d.n3;
@@ -340,9 +350,32 @@ __global__ void __launch_bounds__(512) k_chain(const ChainArgs a) {
     const float* pb = a.SB + rec.ib * N3 + (long)x * d.n2 * d.n3;
     const bool mulw = (a.flags & PROD_MULW) != 0;
     const float wx = mulw ? a.w1[x] : 1.f;
-    const int tz = tid & 7, row0 = 4 * (tid >> 3);
+    const int tz = tid & 7, row0 = kRows * (tid >> 3);
     const int nbq = a.bw / 4, ngt = nth / nbq;                    // mode 2: 4 b per thread
-    const int bq = tid % nbq, gq = tid / nbq;
+    // the index that out has fastest runs along the lanes
+    const int bq = a.bg ? tid / ngt : tid % nbq, gq = a.bg ? tid % ngt : tid / nbq;
+    const bool act2 = a.bg ? bq < nbq : gq < ngt;
+    const long og = a.bg ? 1 : d.r2, ob = a.bg ? d.r3 : 1;
+    // 16-byte pieces of a slice: 32 lanes are 16 rows x 2 neighbouring pieces (whole sectors; with
+    // ldy = 4 (mod 8) the transposed stores hit 32 different banks)
+    const int ngr = (min(a.ty, d.n2) + 15) / 16, npc = ngr * (PZ / 8) * 32;
+    float4 fa[4], fb[4];                       // at most 4 pieces per thread (the launch has a thread per 4)
+    auto piece = [&](int i, int z0, int yn, int& yy, int& z) -> bool {
+        const int e = i * nth + tid, grp = e >> 5, l = e & 31;
+        yy = (grp % ngr) * 16 + (l & 15);
+        z = 4 * (2 * (grp / ngr) + (l >> 4));
+        return e < npc && yy < yn && z0 + z < d.n3;
+    };
+    auto fetch = [&](int y0, int yn, int z0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            int yy, z;
+            if (!piece(i, z0, yn, yy, z)) continue;
+            const long o = (long)(y0 + yy) * d.n3 + z0 + z;
+            fa[i] = *(const float4*)(pa + o);
+            fb[i] = *(const float4*)(pb + o);
+        }
+    };
     for (int t = 0; t < a.nt; ++t) {
         const float* M3 = a.M3 + (long)t * d.n3 * d.r3;
         const float* M2 = a.M2 + (long)t * d.n2 * d.r2;
@@ -351,23 +384,19 @@ __global__ void __launch_bounds__(512) k_chain(const ChainArgs a) {
             const int gn = min(a.gw, d.r3 - g0), rg = (gn + 7) / 8;
             for (int y0 = 0; y0 < d.n2; y0 += a.ty) {
                 const int yn = min(a.ty, d.n2 - y0);
-                uint64_t acc[kMaxRG][2];
+                uint64_t acc[8][4];
 #pragma unroll
-                for (int c = 0; c < kMaxRG; ++c) acc[c][0] = acc[c][1] = 0ull;
+                for (int c = 0; c < 8; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0ull;
+                if (a.vec) fetch(y0, yn, 0);
                 for (int z0 = 0; z0 < d.n3; z0 += PZ) {
                     const int zn = min(PZ, d.n3 - z0);
-                    __syncthreads();           // the previous slice (and S1) has been read
+                    __syncthreads();           // the previous slice (and S1, M2) has been read
                     if (a.vec) {
-                        // 2 neighbouring 16-byte pieces x 16 rows per warp: whole sectors, and with
-                        // ldy = 4 (mod 8) the transposed stores hit 32 different banks
-                        const int ngr = (yn + 15) / 16;
-                        for (int e = tid; e < ngr * (PZ / 8) * 32; e += nth) {
-                            const int grp = e >> 5, l = e & 31;
-                            const int yy = (grp % ngr) * 16 + (l & 15), z = 4 * (2 * (grp / ngr) + (l >> 4));
-                            if (yy >= yn || z >= zn) continue;
-                            const long o = (long)(y0 + yy) * d.n3 + z0 + z;
-                            const float4 u = *(const float4*)(pa + o), v = *(const float4*)(pb + o);
-                            float q[4] = {u.x * v.x, u.y * v.y, u.z * v.z, u.w * v.w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            int yy, z;
+                            if (!piece(i, z0, yn, yy, z)) continue;
+                            float q[4] = {fa[i].x * fb[i].x, fa[i].y * fb[i].y, fa[i].z * fb[i].z, fa[i].w * fb[i].w};
                             if (mulw) {
                                 const float wxy = wx * a.w2[y0 + yy];
 #pragma unroll
@@ -389,63 +418,76 @@ __global__ void __launch_bounds__(512) k_chain(const ChainArgs a) {
                         const int z = e / gn, g = e - z * gn;
                         m3s[z * a.ldg + g] = M3[(long)(z0 + z) * d.r3 + g0 + g];
                     }
+                    if (z0 == 0 && a.mh >= a.ty && d.r2 <= a.bw)      // the whole M2 tile, under mode 3
+                        for (int e = tid; e < yn * d.r2; e += nth) {
+                            const int yy = e / d.r2, bb = e - yy * d.r2;
+                            cp_async4(m2s + yy * a.ldb + bb, M2 + (long)(y0 + yy) * d.r2 + bb);
+                        }
                     __syncthreads();
-                    if (row0 < a.ty) panel_any(rg, qs + row0, a.ldy, m3s + tz, a.ldg, zn, acc);
+                    if (a.vec && z0 + PZ < d.n3) fetch(y0, yn, z0 + PZ);
+                    if (row0 < a.ty) panel8_any<8>(rg, qs + row0, a.ldy, m3s + tz, a.ldg, zn, acc);
                 }
                 if (row0 < a.ty) {
 #pragma unroll
-                    for (int c = 0; c < kMaxRG; ++c)
+                    for (int c = 0; c < 8; ++c)
                         if (c < rg) {
-                            const float2 u = unpack2(acc[c][0]), v = unpack2(acc[c][1]);
-                            float* p = s1 + row0 * a.ldg + tz + 8 * c;
-                            p[0] = u.x; p[a.ldg] = u.y; p[2 * a.ldg] = v.x; p[3 * a.ldg] = v.y;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const float2 u = unpack2(acc[c][i]);
+                                float* p = s1 + (row0 + 2 * i) * a.ldg + tz + 8 * c;
+                                p[0] = u.x;
+                                p[a.ldg] = u.y;
+                            }
                         }
                 }
+                cp_async_wait_all();
                 // mode 2: S2[g][b] = sum_y S1[y][g] M2[y][b], this y tile's share added to the earlier ones'
+                const int npass = (gn + 8 * ngt - 1) / (8 * ngt), cb = (gn + ngt * npass - 1) / (ngt * npass);
                 for (int b0 = 0; b0 < d.r2; b0 += a.bw)
-                    for (int gc = 0; gc < gn; gc += 4 * ngt) {
+                    for (int gc = 0; gc < gn; gc += cb * ngt) {
                         const int bn = min(a.bw, d.r2 - b0);
-                        uint64_t s[4][2];
+                        uint64_t s[8][2];
+                        int col[8];
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) s[c][0] = s[c][1] = 0ull;
-                        for (int yb = 0; yb < yn; yb += PZ) {
-                            const int ync = min(PZ, yn - yb);
-                            __syncthreads();       // S1 written; the previous M2 slice has been read
-                            for (int e = tid; e < ync * bn; e += nth) {
-                                const int yy = e / bn, bb = e - yy * bn;
-                                m2s[yy * a.ldb + bb] = M2[(long)(y0 + yb + yy) * d.r2 + b0 + bb];
+                        for (int c = 0; c < 8; ++c) {
+                            s[c][0] = s[c][1] = 0ull;
+                            col[c] = min(gc + gq + c * ngt, a.ldg - 1);      // past gn: a padding column, never stored
+                        }
+                        for (int yb = 0; yb < yn; yb += a.mh) {
+                            const int ync = min(a.mh, yn - yb);
+                            __syncthreads();       // S1 (and the M2 tile) written; the previous M2 slice has been read
+                            if (a.mh < a.ty || d.r2 > a.bw) {
+                                for (int e = tid; e < ync * bn; e += nth) {
+                                    const int yy = e / bn, bb = e - yy * bn;
+                                    m2s[yy * a.ldb + bb] = M2[(long)(y0 + yb + yy) * d.r2 + b0 + bb];
+                                }
+                                __syncthreads();
                             }
-                            __syncthreads();
-                            if (gq < ngt) {
+                            if (act2) {
                                 const float* sp = s1 + yb * a.ldg;
                                 const float* mp = m2s + 4 * bq;
-                                // columns past gn repeat the last padding column (never stored)
-                                const int cl = a.ldg - 1, c0 = gc + gq;
-                                const int o0 = min(c0, cl), o1 = min(c0 + ngt, cl), o2 = min(c0 + 2 * ngt, cl),
-                                          o3 = min(c0 + 3 * ngt, cl);
-#pragma unroll 4
-                                for (int k = 0; k < ync; ++k) {
-                                    const ulonglong2 m = *(const ulonglong2*)(mp + k * a.ldb);
-                                    const float* q = sp + k * a.ldg;
-                                    const uint64_t b0_ = dup2(q[o0]), b1_ = dup2(q[o1]), b2_ = dup2(q[o2]), b3_ = dup2(q[o3]);
-                                    fma2(s[0][0], m.x, b0_); fma2(s[0][1], m.y, b0_);
-                                    fma2(s[1][0], m.x, b1_); fma2(s[1][1], m.y, b1_);
-                                    fma2(s[2][0], m.x, b2_); fma2(s[2][1], m.y, b2_);
-                                    fma2(s[3][0], m.x, b3_); fma2(s[3][1], m.y, b3_);
+                                switch (cb) {
+                                    case 1: panel4<1>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
+                                    case 2: panel4<2>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
+                                    case 3: panel4<3>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
+                                    case 4: panel4<4>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
+                                    case 5: panel4<5>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
+                                    case 6: panel4<6>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
+                                    default: panel4<8>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
                                 }
                             }
                         }
-                        if (gq < ngt) {
+                        if (act2) {
 #pragma unroll
-                            for (int c = 0; c < 4; ++c) {
+                            for (int c = 0; c < 8; ++c) {
                                 const int g = gc + gq + c * ngt;
-                                if (g >= gn) continue;
+                                if (c >= cb || g >= gn) continue;
                                 const float2 u = unpack2(s[c][0]), v = unpack2(s[c][1]);
                                 const float q[4] = {u.x, u.y, v.x, v.y};
-                                float* o = out + (long)(g0 + g) * d.r2 + b0 + 4 * bq;
+                                float* o = out + (g0 + g) * og + (b0 + 4 * bq) * ob;
 #pragma unroll
                                 for (int k = 0; k < 4; ++k)
-                                    if (4 * bq + k < bn) o[k] = y0 ? o[k] + q[k] : q[k];
+                                    if (4 * bq + k < bn) o[k * ob] = y0 ? o[k * ob] + q[k] : q[k];
                             }
                         }
                     }
@@ -469,18 +511,23 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // expansion consumer: for each term t, Y_t = Z_t x2 M2_t (a tile of rows (x, y)), then
 // phi += Y_t x3 M3_t; epilogue Hadamard-accumulate and energy sums.
 //
-// A CTA owns `rows` rows: px planes x ty y-rows, 2 threads per row; a thread owns 4 rows and
-// 4 * RN4 + 2 * H columns of phi (8 column lanes, 16-byte pieces 32 columns apart), kept in
+// A CTA owns `rows` rows: px planes x ty y-rows.  A thread owns 8 neighbouring rows and
+// RN = 4 RN4 + 2 H columns of phi (CL column lanes, 16-byte pieces 4 CL columns apart), kept in
 // registers over every term.  Per term mode 2 leaves Y in shared memory (K-major) and mode 3 reads
-// it back: 4 * RN multiply-adds per 1 + RN4 16-byte fragments.  The next operator tiles arrive
+// it back: 8 RN multiply-adds per 2 + RN4 16-byte fragments.  The next operator tiles arrive
 // by cp.async under the arithmetic: M3 under mode 2, the next term's M2 and Z under mode 3.
-// Ranks above 64 run in parts of K (the Y tile, M2 and Z slices stay at most 64 deep).
-// Bound by the float32 pipes.  Pt-shaped pair (96^3, rank 40, 40 terms): 114 us (35 TF/s) instead of 461.
+// Ranks above a part (gc, bc) run in parts of K.
+// Bound by the float32 pipes and, next, by the shared-memory reads: with 4 rows per thread the
+// reads took 57% of their peak at 46% of the multiply-adds', so the thread tile is as tall as the
+// registers allow (8 x 12 up to 96 columns; 16 column lanes above).  Pt-shaped pair (96^3, rank
+// 40, 40 terms): 94 us (43 TF/s); 114 with 4 rows per
+// thread, 461 with one output per thread.
 // ====================================================================================
 struct SimtPlan {
-    int rn4, h;                // columns: 32 * rn4 + 16 * h
-    int ty, ny, px, nx, rows;  // y rows per plane (a multiple of 4), y tiles, planes per CTA, x slabs, rows per CTA
+    int cl, rn2;               // column lanes, columns per thread / 2
+    int ty, ny, px, nx, rows;  // y rows per plane (a multiple of 8), y tiles, planes per CTA, x slabs, rows per CTA
     int gc, bc;                // K parts of mode 3 and mode 2
+    int threads;
     size_t smem;
 };
 
@@ -488,10 +535,10 @@ struct ConsumeF32Args {
     Dims d;
     const PairRec* recs;
     int p0, nt;
-    const float* Z;            // [np][nt][n1][r3][r2]
+    const float* Z;            // [np][nt][n1][r2][r3], or [r3][r2] slices (z_mode)
     const float* M2;           // [nt][r2][ld2], y fastest
-    const float* M3;           // [nt][r3][ld3], z fastest
-    int ld2, ld3;
+    const float* M3;           // [nt][r3][NC], z fastest
+    int ld2;
     long m2_ps, m3_ps;
     FieldArgs f;
     const float* w1;
@@ -500,108 +547,126 @@ struct ConsumeF32Args {
     int flags;
     double* epart;
     int ty, px, ny, gc, bc, rows, vec;
+    int m2_flat, z_mode;       // M2 part / Z part as one contiguous run (z_mode 2), Z rows of g (1) or of b (0)
 };
 
-// threads per CTA: 2 per row, and registers for phi
-__host__ __device__ constexpr int consume_max_threads(int units) { return units <= 6 ? 512 : (units <= 10 ? 384 : 256); }
+// Registers: 8 RN for phi, 8 per mode-2 column; the K part of mode 3 (gc) is at most CL * kMaxPart
+// columns so that both fit the 168 registers that leave 12 warps per SM (255 above 12 columns).
+__host__ __device__ constexpr int consume_max_rg(int cl, int rn) { return cl == 16 ? 4 : (rn > 8 ? 5 : 8); }
+__host__ __device__ constexpr int consume_max_threads(int cl, int rn) { return rn <= 12 ? 384 : 256; }
 
-template <int RN4, int H>
-__global__ void __launch_bounds__(consume_max_threads(2 * RN4 + H)) k_consume(const ConsumeF32Args a) {
-    constexpr int NC = 32 * RN4 + 16 * H;              // columns of phi
+template <int CL, int RN4, int H>
+__global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_consume(const ConsumeF32Args a) {
+    constexpr int NC = CL * (4 * RN4 + 2 * H);         // columns of phi
+    constexpr int MRG = consume_max_rg(CL, 4 * RN4 + 2 * H);
+    constexpr int NP = 2 * RN4 + H;                    // packed column pairs per thread
     extern __shared__ __align__(16) float sm[];
     __shared__ double red[16];
     const Dims d = a.d;
-    const int ldy = a.rows + 4, ldz = a.gc | 1, rgw = 8 * ((a.gc + 7) / 8);
+    const int ldy = a.rows + 4, ldz = a.z_mode ? a.gc : (a.gc | 1), rgw = CL * ((a.gc + CL - 1) / CL);
     float* m2s = sm;                                   // [bc][ty]
     float* m3s = m2s + a.bc * a.ty;                    // [gc][NC]
-    float* ys = m3s + a.gc * NC;                       // [gc][ldy]
+    float* ys = m3s + a.gc * NC;                       // [rgw][ldy]
     float* zs = ys + rgw * ldy;                        // [px][bc][ldz]
     const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
     const int iy = blockIdx.x % a.ny, x0 = (blockIdx.x / a.ny) * a.px, pl = blockIdx.y;
     const int y0 = iy * a.ty;
     const PairRec rec = a.recs[a.p0 + pl];
-    const int tz = tid & 7, row0 = 4 * (tid >> 3);
+    const int tz = tid % CL, row0 = kRows * (tid / CL);
     const int pr = min(row0 / a.ty, a.px - 1);         // plane of this thread's rows
-    const int yr = min(row0 - pr * a.ty, a.ty - 4);    // rows past the last plane repeat valid ones (not stored)
+    const int yr = min(row0 - pr * a.ty, a.ty - kRows);    // rows past the last plane repeat valid ones (not stored)
     const long zslice = (long)d.r3 * d.r2;
     const int ng = (d.r3 + a.gc - 1) / a.gc, nb = (d.r2 + a.bc - 1) / a.bc;
 
-    uint64_t acc[4][2 * RN4 + H];
+    uint64_t acc[kRows][NP];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < kRows; ++i)
 #pragma unroll
-        for (int c = 0; c < 2 * RN4 + H; ++c) acc[i][c] = 0ull;
+        for (int c = 0; c < NP; ++c) acc[i][c] = 0ull;
 
     // M2 and Z of part (t, g part, b part)
     auto load2 = [&](int t, int gp, int bp) {
         const int g0 = gp * a.gc, gn = min(a.gc, d.r3 - g0), b0 = bp * a.bc, bn = min(a.bc, d.r2 - b0);
         const float* m2 = a.M2 + pl * a.m2_ps + ((long)t * d.r2 + b0) * a.ld2 + y0;
-        const int nq = min(a.ty, a.ld2 - y0) / 4;      // ld2 is n2 rounded up to 4
-        for (int e = tid; e < bn * nq; e += nth) {
-            const int k = e / nq, q = e - k * nq;
-            cp_async16(m2s + k * a.ty + 4 * q, m2 + (long)k * a.ld2 + 4 * q);
+        if (a.m2_flat) {
+            for (int e = 4 * tid; e < bn * a.ty; e += 4 * nth) cp_async16(m2s + e, m2 + e);
+        } else {
+            const int w = min(a.ty, a.ld2 - y0);       // ld2 is n2 rounded up to 8
+            for (int k = warp; k < bn; k += nw)
+                for (int q = 4 * lane; q < w; q += 128) cp_async16(m2s + k * a.ty + q, m2 + (long)k * a.ld2 + q);
         }
-        // Z comes with b fastest and is wanted with g fastest: the odd row stride spreads the
-        // transposed 4-byte stores over the banks
         for (int p = 0; p < a.px; ++p) {
             if (x0 + p >= d.n1) break;
-            const float* zt = a.Z + (((long)pl * a.nt + t) * d.n1 + x0 + p) * zslice + (long)g0 * d.r2 + b0;
+            const float* zt = a.Z + (((long)pl * a.nt + t) * d.n1 + x0 + p) * zslice;
             float* zd = zs + p * a.bc * ldz;
-            for (int g = warp; g < gn; g += nw)
-                for (int b = lane; b < bn; b += 32) cp_async4(zd + b * ldz + g, zt + (long)g * d.r2 + b);
+            if (a.z_mode == 2) {
+                zt += (long)b0 * d.r3;
+                for (int e = 4 * tid; e < bn * d.r3; e += 4 * nth) cp_async16(zd + e, zt + e);
+            } else if (a.z_mode == 1) {
+                zt += (long)b0 * d.r3 + g0;
+                for (int b = warp; b < bn; b += nw)
+                    for (int g = lane; g < gn; g += 32) cp_async4(zd + b * ldz + g, zt + (long)b * d.r3 + g);
+            } else {                                   // the odd row stride spreads the transposed stores over the banks
+                zt += (long)g0 * d.r2 + b0;
+                for (int g = warp; g < gn; g += nw)
+                    for (int b = lane; b < bn; b += 32) cp_async4(zd + b * ldz + g, zt + (long)g * d.r2 + b);
+            }
         }
         cp_async_commit();
     };
     auto load3 = [&](int t, int gp) {
-        const int g0 = gp * a.gc, gn = min(a.gc, d.r3 - g0), nq = a.ld3 / 4;
-        const float* m3 = a.M3 + pl * a.m3_ps + ((long)t * d.r3 + g0) * a.ld3;
-        for (int e = tid; e < gn * nq; e += nth) {
-            const int k = e / nq, q = e - k * nq;
-            cp_async16(m3s + k * NC + 4 * q, m3 + (long)k * a.ld3 + 4 * q);
-        }
+        const int g0 = gp * a.gc, gn = min(a.gc, d.r3 - g0);
+        const float* m3 = a.M3 + pl * a.m3_ps + ((long)t * d.r3 + g0) * NC;
+        for (int e = 4 * tid; e < gn * NC; e += 4 * nth) cp_async16(m3s + e, m3 + e);
         cp_async_commit();
     };
 
     load2(0, 0, 0);
     for (int t = 0; t < a.nt; ++t)
         for (int gp = 0; gp < ng; ++gp) {
-            const int gn = min(a.gc, d.r3 - gp * a.gc), rg = (gn + 7) / 8;
-            uint64_t y[kMaxRG][2];
+            const int gn = min(a.gc, d.r3 - gp * a.gc), rg = (gn + CL - 1) / CL;
+            uint64_t y[MRG][4];
 #pragma unroll
-            for (int c = 0; c < kMaxRG; ++c) y[c][0] = y[c][1] = 0ull;
+            for (int c = 0; c < MRG; ++c) y[c][0] = y[c][1] = y[c][2] = y[c][3] = 0ull;
             for (int bp = 0; bp < nb; ++bp) {
                 cp_async_wait_all();
                 __syncthreads();               // M2 and Z have landed; the previous mode 3 is done
                 if (bp == 0) load3(t, gp);
-                panel_any(rg, m2s + yr, a.ty, zs + pr * a.bc * ldz + tz, ldz, min(a.bc, d.r2 - bp * a.bc), y);
+                panel8_any<CL>(rg, m2s + yr, a.ty, zs + pr * a.bc * ldz + tz, ldz, min(a.bc, d.r2 - bp * a.bc), y);
                 if (bp + 1 < nb) {
                     __syncthreads();
                     load2(t, gp, bp + 1);
                 }
             }
 #pragma unroll
-            for (int c = 0; c < kMaxRG; ++c)
-                if (c < rg) *(ulonglong2*)(ys + (tz + 8 * c) * ldy + row0) = make_ulonglong2(y[c][0], y[c][1]);
+            for (int c = 0; c < MRG; ++c)
+                if (c < rg) {
+                    float* p = ys + (tz + CL * c) * ldy + row0;
+                    *(ulonglong2*)p = make_ulonglong2(y[c][0], y[c][1]);
+                    *(ulonglong2*)(p + 4) = make_ulonglong2(y[c][2], y[c][3]);
+                }
             cp_async_wait_all();
             __syncthreads();                   // Y and M3 are there, M2 and Z free
             if (gp + 1 < ng) load2(t, gp + 1, 0);
             else if (t + 1 < a.nt) load2(t + 1, 0, 0);
-#pragma unroll 4
+#pragma unroll 2
             for (int g = 0; g < gn; ++g) {
-                const float4 yv = *(const float4*)(ys + g * ldy + row0);
-                uint64_t b[2 * RN4 + H];
+                const float4 ya = *(const float4*)(ys + g * ldy + row0), yb = *(const float4*)(ys + g * ldy + row0 + 4);
+                uint64_t b[NP];
 #pragma unroll
                 for (int c = 0; c < RN4; ++c) {
-                    const ulonglong2 q = *(const ulonglong2*)(m3s + g * NC + 4 * tz + 32 * c);
+                    const ulonglong2 q = *(const ulonglong2*)(m3s + g * NC + 4 * tz + 4 * CL * c);
                     b[2 * c] = q.x;
                     b[2 * c + 1] = q.y;
                 }
-                if constexpr (H) b[2 * RN4] = *(const uint64_t*)(m3s + g * NC + 32 * RN4 + 2 * tz);
-                const uint64_t y4[4] = {dup2(yv.x), dup2(yv.y), dup2(yv.z), dup2(yv.w)};
+                if constexpr (H) b[2 * RN4] = *(const uint64_t*)(m3s + g * NC + 4 * CL * RN4 + 2 * tz);
+                const float yv[kRows] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < kRows; ++i) {
+                    const uint64_t yi = dup2(yv[i]);
 #pragma unroll
-                    for (int c = 0; c < 2 * RN4 + H; ++c) fma2(acc[i][c], y4[i], b[c]);
+                    for (int c = 0; c < NP; ++c) fma2(acc[i][c], yi, b[c]);
+                }
             }
         }
     // epilogue
@@ -616,14 +681,14 @@ __global__ void __launch_bounds__(consume_max_threads(2 * RN4 + H)) k_consume(co
     float* out1 = a.f.OUT1 + rec.o1 * N3;
     const float wx = x < d.n1 ? a.w1[x] : 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kRows; ++i) {
         const int y = y0 + yr + i;
         if (!rows_ok || y >= d.n2) continue;
         const float wxy = wx * a.w2[y];
         const long base = ((long)x * d.n2 + y) * d.n3;
 #pragma unroll
-        for (int c = 0; c < 2 * RN4 + H; ++c) {
-            const int z = c < 2 * RN4 ? 32 * (c / 2) + 4 * tz + 2 * (c & 1) : 32 * RN4 + 2 * tz;
+        for (int c = 0; c < NP; ++c) {
+            const int z = c < 2 * RN4 ? 4 * CL * (c / 2) + 4 * tz + 2 * (c & 1) : 4 * CL * RN4 + 2 * tz;
             const float2 ph = unpack2(acc[i][c]);
             const float phi[2] = {ph.x, ph.y};
             if (a.vec && z < d.n3) {           // even n3: the pair z, z + 1 is inside and 8-byte aligned
@@ -800,16 +865,16 @@ constexpr size_t kSmemLimit = 232448;      // 227 KB per CTA
 
 // modes 3 and 2 of a projection for nt terms of (M3 [nt][n3][r3], M2 [nt][n2][r2])
 int launch_chain(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, int nt, const float* M2,
-                 const float* M3, int flags, float* out, const char* name, cudaStream_t s) {
+                 const float* M3, int flags, float* out, bool bg, const char* name, cudaStream_t s) {
     ChainArgs a{};
     a.d = dims_of(c);
     a.recs = recs; a.p0 = p0; a.nt = nt;
     a.SA = f.SA; a.SB = f.SB; a.M2 = M2; a.M3 = M3;
     a.w1 = c->f_w[0]; a.w2 = c->f_w[1]; a.w3 = c->f_w[2];
-    a.flags = flags; a.out = out;
-    // y tiles of at most 128 rows of equal height, 2 threads per row (at least 128 threads)
-    const int ny = (a.d.n2 + 127) / 128, tyv = (a.d.n2 + ny - 1) / ny;
-    a.ty = (tyv + 3) & ~3;
+    a.flags = flags; a.out = out; a.bg = bg ? 1 : 0;
+    // y tiles of at most 256 rows of equal height, one thread per row
+    const int ny = (a.d.n2 + 255) / 256, tyv = (a.d.n2 + ny - 1) / ny;
+    a.ty = (tyv + 7) & ~7;
     const int ngp = (a.d.r3 + 63) / 64;
     a.gw = (a.d.r3 + ngp - 1) / ngp;
     a.ldy = ((a.ty + 7) & ~7) + 4;
@@ -817,10 +882,10 @@ int launch_chain(const tx_ctx* c, const PairRec* recs, int p0, int np, const Fie
     a.bw = std::min(256, pad4(a.d.r2));
     a.ldb = a.bw + 4;
     a.vec = a.d.n3 % 4 == 0 && (((uintptr_t)f.SA | (uintptr_t)f.SB) & 15u) == 0;
-    // qs and m3s rows are 16-byte multiples where float4 reads them (qs, m2s); s1 and m3s are read as scalars
-    const size_t words = (size_t)PZ * a.ldy + (size_t)PZ * a.ldg + (size_t)a.ty * a.ldg;
-    const size_t smem = sizeof(float) * (words + (size_t)PZ * a.ldb);
-    const int threads = std::max(128, ((2 * a.ty + 31) / 32) * 32);
+    a.mh = (size_t)a.ty * a.ldb * sizeof(float) <= 64 * 1024 ? a.ty : 32;
+    const size_t smem = sizeof(float) * ((size_t)PZ * a.ldy + (size_t)a.mh * a.ldb + (size_t)(PZ + a.ty) * a.ldg);
+    // at least 64 threads; at least one per 4 b; at most 4 pieces of a slice per thread
+    const int threads = std::max(std::max(64, (a.bw / 4 + 31) & ~31), (a.ty + 31) & ~31);
     TX_TRY(smem_attr((const void*)k_chain, smem));
     const int ps = prof_begin(name, s);
     k_chain<<<dim3(a.d.n1, np), threads, smem, s>>>(a);
@@ -829,35 +894,40 @@ int launch_chain(const tx_ctx* c, const PairRec* recs, int p0, int np, const Fie
     return TX_OK;
 }
 
-// The split of one pair's (x, y) rows over CTAs.  Phi's columns per thread fix the registers and so
-// the threads (512 up to 96 columns, 384 up to 160, 256 above); among the row tiles that fit, the
-// one with the least padding, preferring those that let two CTAs share an SM.
+// The split of one pair's (x, y) rows over CTAs.  Up to 96 columns of phi take 8 column lanes of at
+// most 12 columns; above, 16 lanes (of at most 12 columns up to 192).  Among the row tiles that fit
+// the threads and shared memory, the one with the least padding, preferring 64 rows or more and
+// shared memory that lets several CTAs share an SM (one CTA's barriers hide behind another's
+// arithmetic).
 bool simt_plan(const Dims& d, SimtPlan* out) {
     if (d.n3 > 256) return false;
-    const int units = (d.n3 + 15) / 16;
     SimtPlan p{};
-    p.rn4 = units / 2;
-    p.h = units & 1;
-    const int ncol = 16 * units, max_rows = consume_max_threads(units) / 2;
-    const int ngp = (d.r3 + 63) / 64, nbp = (d.r2 + 63) / 64;
+    p.cl = d.n3 <= 96 ? 8 : 16;
+    p.rn2 = (d.n3 + 2 * p.cl - 1) / (2 * p.cl);
+    const int rn = 2 * p.rn2, ncol = p.cl * rn, wrows = kRows * (32 / p.cl);    // rows per warp
+    const int max_rows = consume_max_threads(p.cl, rn) / p.cl * kRows;
+    const int gmax = p.cl * consume_max_rg(p.cl, rn);
+    const int ngp = (d.r3 + gmax - 1) / gmax, nbp = (d.r2 + 63) / 64;
     p.gc = (d.r3 + ngp - 1) / ngp;
     p.bc = (d.r2 + nbp - 1) / nbp;
-    const int rgw = 8 * ((p.gc + 7) / 8), ldz = p.gc | 1;
+    const int rgw = p.cl * ((p.gc + p.cl - 1) / p.cl), ldz = p.gc | 1;
     double best = -1.0;
-    for (int ny = (d.n2 + max_rows - 1) / max_rows; ny <= (d.n2 + 15) / 16; ++ny) {
+    for (int ny = (d.n2 + max_rows - 1) / max_rows; ny <= (d.n2 + 7) / 8; ++ny) {
         p.ny = ny;
-        p.ty = (((d.n2 + ny - 1) / ny) + 3) & ~3;
-        for (p.px = 1; p.px <= d.n1 && ((p.px * p.ty + 15) & ~15) <= max_rows; ++p.px) {
+        p.ty = (((d.n2 + ny - 1) / ny) + 7) & ~7;
+        for (p.px = 1; p.px <= d.n1; ++p.px) {
+            p.rows = (p.px * p.ty + wrows - 1) / wrows * wrows;
+            if (p.rows > max_rows) break;
             p.nx = (d.n1 + p.px - 1) / p.px;
-            p.rows = (p.px * p.ty + 15) & ~15;
-            // 8 more floats: the last column group of a panel may read past a Z row
+            p.threads = p.rows / kRows * p.cl;
+            // the last column group of a panel may read up to CL floats past a Z row
             p.smem = sizeof(float) * ((size_t)p.bc * p.ty + (size_t)p.gc * ncol + (size_t)rgw * (p.rows + 4) +
-                                      (size_t)p.px * p.bc * ldz + 8);
+                                      (size_t)p.px * p.bc * ldz + 16);
             if (p.smem > kSmemLimit) continue;
             double score = (double)d.n1 * d.n2 / ((double)p.ny * p.nx * p.rows);
-            if (p.rows < 96) score *= p.rows < 64 ? 0.8 : 0.9;
-            if (p.smem > kSmemLimit / 2) score *= 0.85;
-            if (p.rows > 192) score *= 0.95;
+            if (p.rows < 64) score *= p.rows < 32 ? 0.6 : 0.85;
+            if (p.smem > kSmemLimit / 2) score *= 0.8;
+            else if (p.smem > kSmemLimit / 3) score *= 0.93;
             if (score > best + 1e-9) {
                 best = score;
                 *out = p;
@@ -867,11 +937,11 @@ bool simt_plan(const Dims& d, SimtPlan* out) {
     return best > 0.0;
 }
 
-template <int RN4, int H>
+template <int CL, int RN4, int H>
 int launch_consume(const ConsumeF32Args& a, const SimtPlan& p, int np, cudaStream_t s) {
-    TX_TRY(smem_attr((const void*)k_consume<RN4, H>, p.smem));
+    TX_TRY(smem_attr((const void*)k_consume<CL, RN4, H>, p.smem));
     const int ps = prof_begin("consume", s);
-    k_consume<RN4, H><<<dim3(p.nx * p.ny, np), 2 * p.rows, p.smem, s>>>(a);
+    k_consume<CL, RN4, H><<<dim3(p.nx * p.ny, np), p.threads, p.smem, s>>>(a);
     prof_end(ps, s);
     TX_LAUNCHED();
     return TX_OK;
@@ -879,11 +949,11 @@ int launch_consume(const ConsumeF32Args& a, const SimtPlan& p, int np, cudaStrea
 }  // namespace
 
 int simt_project_s2(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, int flags,
-                    float* S2, cudaStream_t s) {
+                    float* S2, cudaStream_t s, bool bg) {
     const Dims d = dims_of(c);
     if (sizeof(float) * ((size_t)d.n3 * d.r3 + (size_t)d.n2 * d.r3 + 8 * (size_t)d.n3) > kSmemLimit)
         return fail(TX_ERR_CUDA, "float32 projection: (n2 + n3) * r3 too large");
-    return launch_chain(c, recs, p0, np, f, 1, c->f_U[1], c->f_U[2], flags, S2, "project", s);
+    return launch_chain(c, recs, p0, np, f, 1, c->f_U[1], c->f_U[2], flags, S2, bg, "project", s);
 }
 
 int simt_expand_consume_blocks(const tx_ctx* c) {
@@ -891,16 +961,23 @@ int simt_expand_consume_blocks(const tx_ctx* c) {
     return simt_plan(dims_of(c), &p) ? p.nx * p.ny : 1;
 }
 
-int simt_kmajor(const float* src, int nt, int n, int r, float* dst, cudaStream_t s) {
-    const long cnt = (long)nt * r * pad4(n);
-    k_kmajor<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(src, nt, n, r, pad4(n), dst);
+int simt_ld2(int n2) { return (n2 + 7) & ~7; }
+int simt_ld3(int n3) {
+    if (n3 > 256) return pad4(n3);             // no float32 consumer: never read
+    const int cl = n3 <= 96 ? 8 : 16;
+    return (n3 + 2 * cl - 1) / (2 * cl) * (2 * cl);
+}
+
+int simt_kmajor(const float* src, int nt, int n, int r, int ld, float* dst, cudaStream_t s) {
+    const long cnt = (long)nt * r * ld;
+    k_kmajor<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(src, nt, n, r, ld, dst);
     TX_LAUNCHED();
     return TX_OK;
 }
 
 int simt_expand_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, const float* Z,
                         int nterms, const float* M2, const float* M3, int flags, double* epart, cudaStream_t s,
-                        long m2_ps, long m3_ps) {
+                        bool z_bg, long m2_ps, long m3_ps) {
     const Dims d = dims_of(c);
     if (d.n3 > 256) return fail(TX_ERR_UNSUPPORTED_SHAPE, "float32 path supports n3 <= 256");
     SimtPlan p{};
@@ -911,31 +988,36 @@ int simt_expand_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, co
     a.d = d;
     a.recs = recs; a.p0 = p0; a.nt = nterms;
     a.Z = Z; a.M2 = M2; a.M3 = M3;
-    a.ld2 = pad4(d.n2); a.ld3 = pad4(d.n3);
+    a.ld2 = simt_ld2(d.n2);
     a.m2_ps = m2_ps; a.m3_ps = m3_ps;
     a.f = f;
     a.w1 = c->f_w[0]; a.w2 = c->f_w[1]; a.w3 = c->f_w[2];
     a.flags = flags; a.epart = epart;
     a.ty = p.ty; a.px = p.px; a.ny = p.ny; a.gc = p.gc; a.bc = p.bc; a.rows = p.rows;
+    a.m2_flat = p.ny == 1;
+    // a part of Z is one 16-byte aligned run where g is its fastest index and the part holds every g
+    const long rr = (long)d.r2 * d.r3;
+    a.z_mode = !z_bg ? 0
+               : (p.gc == d.r3 && rr % 4 == 0 && (p.bc == d.r2 || ((long)p.bc * d.r3) % 4 == 0) &&
+                  ((uintptr_t)Z & 15u) == 0) ? 2 : 1;
     // pairs of z as one access: even rows, and arrays (callers' blocks and slices) that start on 8 bytes
     a.vec = d.n3 % 2 == 0 && (((uintptr_t)f.MUL0 | (uintptr_t)f.MUL1 | (uintptr_t)f.OUT0 | (uintptr_t)f.OUT1) & 7u) == 0;
-    switch (2 * p.rn4 + p.h) {
-        case 1: return launch_consume<0, 1>(a, p, np, s);
-        case 2: return launch_consume<1, 0>(a, p, np, s);
-        case 3: return launch_consume<1, 1>(a, p, np, s);
-        case 4: return launch_consume<2, 0>(a, p, np, s);
-        case 5: return launch_consume<2, 1>(a, p, np, s);
-        case 6: return launch_consume<3, 0>(a, p, np, s);
-        case 7: return launch_consume<3, 1>(a, p, np, s);
-        case 8: return launch_consume<4, 0>(a, p, np, s);
-        case 9: return launch_consume<4, 1>(a, p, np, s);
-        case 10: return launch_consume<5, 0>(a, p, np, s);
-        case 11: return launch_consume<5, 1>(a, p, np, s);
-        case 12: return launch_consume<6, 0>(a, p, np, s);
-        case 13: return launch_consume<6, 1>(a, p, np, s);
-        case 14: return launch_consume<7, 0>(a, p, np, s);
-        case 15: return launch_consume<7, 1>(a, p, np, s);
-        default: return launch_consume<8, 0>(a, p, np, s);
+    if (p.cl == 8) {
+        switch (p.rn2) {
+            case 1: return launch_consume<8, 0, 1>(a, p, np, s);
+            case 2: return launch_consume<8, 1, 0>(a, p, np, s);
+            case 3: return launch_consume<8, 1, 1>(a, p, np, s);
+            case 4: return launch_consume<8, 2, 0>(a, p, np, s);
+            case 5: return launch_consume<8, 2, 1>(a, p, np, s);
+            default: return launch_consume<8, 3, 0>(a, p, np, s);
+        }
+    }
+    switch (p.rn2) {
+        case 4: return launch_consume<16, 2, 0>(a, p, np, s);
+        case 5: return launch_consume<16, 2, 1>(a, p, np, s);
+        case 6: return launch_consume<16, 3, 0>(a, p, np, s);
+        case 7: return launch_consume<16, 3, 1>(a, p, np, s);
+        default: return launch_consume<16, 4, 0>(a, p, np, s);
     }
 }
 
@@ -944,7 +1026,7 @@ int simt_adjoint_r(const tx_ctx* c, const PairRec* recs, int p0, int np, const F
     const Dims d = dims_of(c);
     if (sizeof(float) * ((size_t)d.n2 * d.n3 + (size_t)d.n2 * d.r3) > 220 * 1024)
         return fail(TX_ERR_UNSUPPORTED_SHAPE, "float32 adjoint needs n2*(n3+r3) <= 56K");
-    return launch_chain(c, recs, p0, np, f, c->T, c->f_A[1], c->f_A[2], flags, R, "adjoint", s);
+    return launch_chain(c, recs, p0, np, f, c->T, c->f_A[1], c->f_A[2], flags, R, true, "adjoint", s);
 }
 
 int reduce_energy_batch(const double* epart, long count, double* dst, cudaStream_t s) {

@@ -4,7 +4,7 @@
 //   mode 1: S1 = Gram of the mode-1 unfolding of rho    (k_gram), U1 = its r1 leading
 //           eigenvectors (k_jacobi_eig), T1 = rho x1 U1^T                        [a][y][z]
 //   mode 2: S2 from T1, U2, T2 = T1 x2 U2^T, stored                              [z][b][a]
-//   mode 3: S3 from T2, U3, G = T2 x3 U3^T, stored                               [g][b][a]
+//   mode 3: S3 from T2, U3, G = T2 x3 U3^T, stored                               [b][g][a]
 //   A_td,ij = C_td U_d,ij for every term                (simt_gemm, mu_t inside C_t3)
 //   Z = G x1 A_t1,ij for every term, then modes 2 and 3, the sum over t and the Hadamard
 //   epilogue with the per-pair operators                (the float32 path's kernels)
@@ -193,7 +193,7 @@ size_t sthosvd_floats_per_pair(const tx_ctx* c) {
            r3 * r2 * r1 +                       // G
            nmax * nmax +                        // Gram matrix
            n1 * r1 + n2 * r2 + n3 * r3 + 8 +    // U_d (8: the operators after them start on 16 bytes)
-           pad4((int)(T * n1 * r1)) + T * (pad4((int)n2) * r2 + pad4((int)n3) * r3) +  // A_td per pair
+           pad4((int)(T * n1 * r1)) + T * (simt_ld2((int)n2) * r2 + simt_ld3((int)n3) * r3) +  // A_td per pair
            T * n1 * r3 * r2;                    // Z
 }
 
@@ -218,7 +218,8 @@ int sthosvd_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, int p0, in
     float* U2 = U1 + (size_t)np * n1 * r1;
     float* U3 = U2 + (size_t)np * n2 * r2;
     // modes 2 and 3 with the grid index fastest (the consumer's layout), 16-byte aligned
-    const long a1_ps = pad4(T * n1 * r1), a2_ps = (long)T * pad4(n2) * r2, a3_ps = (long)T * pad4(n3) * r3;
+    const long a1_ps = pad4(T * n1 * r1), a2_ps = (long)T * simt_ld2(n2) * r2,
+               a3_ps = (long)T * simt_ld3(n3) * r3;
     float* A1 = (float*)(((uintptr_t)(U3 + (size_t)np * n3 * r3) + 15) & ~(uintptr_t)15);
     float* A2 = A1 + (size_t)np * a1_ps;
     float* A3 = A2 + (size_t)np * a2_ps;
@@ -264,15 +265,15 @@ int sthosvd_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, int p0, in
         g.nb1 = r1; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
         TX_TRY(simt_gemm(g, s));
     }
-    // ---- mode 3: Gram of T2 [z][(b,a)]; G[g][(b,a)] = sum_z U3[z][g] T2[z][(b,a)]
+    // ---- mode 3: Gram of T2 [z][(b,a)]; G[b][g][a] = sum_z U3[z][g] T2[z][(b,a)], one GEMM per b
     TX_TRY(gram_eig(T2, 1, n3, r2 * r1, (long)n3 * r2 * r1, U3, r3));
     {
         GemmArgs g{};
-        g.M = r3; g.N = r2 * r1; g.K = n3;
+        g.M = r3; g.N = r1; g.K = n3;
         g.A = U3; g.a_m = 1; g.a_k = r3; g.a_b1 = 0; g.a_b2 = (long)n3 * r3;
-        g.B = T2; g.b_k = (long)r2 * r1; g.b_n = 1; g.b_b1 = 0; g.b_b2 = (long)n3 * r2 * r1;
-        g.C = G; g.c_m = (long)r2 * r1; g.c_n = 1; g.c_b1 = 0; g.c_b2 = (long)r3 * r2 * r1;
-        g.nb1 = 1; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
+        g.B = T2; g.b_k = (long)r2 * r1; g.b_n = 1; g.b_b1 = r1; g.b_b2 = (long)n3 * r2 * r1;
+        g.C = G; g.c_m = r1; g.c_n = 1; g.c_b1 = (long)r3 * r1; g.c_b2 = (long)r3 * r2 * r1;
+        g.nb1 = r2; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
         TX_TRY(simt_gemm(g, s));
     }
     // ---- A_td,ij = C_td U_d,ij for every term (mu_t inside C_t3)
@@ -288,14 +289,14 @@ int sthosvd_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, int p0, in
         if (d == 0) {
             g.c_m = r; g.c_n = 1; g.c_b1 = (long)n * r; g.c_b2 = a1_ps;
         } else {
-            g.c_m = 1; g.c_n = pad4(n); g.c_b1 = (long)pad4(n) * r; g.c_b2 = d == 1 ? a2_ps : a3_ps;
+            g.c_m = 1; g.c_n = d == 1 ? simt_ld2(n) : simt_ld3(n); g.c_b1 = g.c_n * r; g.c_b2 = d == 1 ? a2_ps : a3_ps;
         }
         g.nb1 = T; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
         TX_TRY(simt_gemm(g, s));
     }
     // ---- expansion with the per-pair operators, Hadamard epilogue
     TX_TRY(simt_expand_mode1_pp(c, G, A1, a1_ps, T, Z, np, s));
-    return simt_expand_consume(c, recs, p0, np, f, Z, T, A2, A3, EPI_OUT, epart, s, a2_ps, a3_ps);
+    return simt_expand_consume(c, recs, p0, np, f, Z, T, A2, A3, EPI_OUT, epart, s, true, a2_ps, a3_ps);
 }
 
 }  // namespace tx

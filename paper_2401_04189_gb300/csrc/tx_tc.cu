@@ -290,7 +290,7 @@ static int tc_forward(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, con
         FieldArgs fa{};
         fa.SA = SA;
         fa.SB = SB;
-        TX_TRY(simt_project_s2(c, recs, b.p0, np, fa, 0, S2f, s));
+        TX_TRY(simt_project_s2(c, recs, b.p0, np, fa, 0, S2f, s, false));
         TX_TRY(f32_mode1_project(c, S2f, Gf, np, s));
         TX_TRY(f32_mode1_expand(c, Gf, Zf, np, s));
         const long rows = (long)np * T * n1 * r3;
@@ -399,7 +399,7 @@ static int tc_adjoint(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, con
     }
     TX_TRY(simt_adjoint_mode1(c, R, H, np, s));                  // H = sum_{t,x} R A_t1
     TX_TRY(simt_expand_mode1(c, H, c->f_U[0], 1, Z, np, s));     // Z = U1 H
-    return simt_expand_consume(c, recs, b.p0, np, fo, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, b.epart, s);
+    return simt_expand_consume(c, recs, b.p0, np, fo, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, b.epart, s, false);
 }
 
 size_t tc_adjoint_bytes_per_pair(const tx_ctx* c) {
