@@ -174,10 +174,10 @@ static void free_ctx(tx_ctx* c) {
         cudaFree(c->f_U[d]);
         cudaFree(c->f_A[d]);
         cudaFree(c->f_UK[d]);
-        cudaFree(c->f_AK[d]);
         cudaFree(c->f_w[d]);
         cudaFree(c->f_C[d]);
     }
+    free_terms(c);
     cudaFree(c->d_theta);
     cudaFree(c->d_mu);
     cudaFree(c->ws);
@@ -245,7 +245,6 @@ extern "C" int tx_tucker_setup(tx_ctx** out, const int n[3], const double* x1, c
         SETUP_TRY(dalloc(&c->f_A[d], (size_t)T * nd * rd));
         if (d > 0) {
             SETUP_TRY(dalloc(&c->f_UK[d], rd * (d == 1 ? simt_ld2((int)nd) : simt_ld3((int)nd))));
-            SETUP_TRY(dalloc(&c->f_AK[d], (size_t)T * rd * (d == 1 ? simt_ld2((int)nd) : simt_ld3((int)nd))));
         }
         SETUP_TRY(dalloc(&c->f_w[d], nd));
         // host float32 copies are made synchronously (the host arrays may be freed on return)
@@ -267,6 +266,7 @@ extern "C" int tx_tucker_setup(tx_ctx** out, const int n[3], const double* x1, c
         cudaMemset(c->d_err, 0, sizeof(int) * kErrWords) != cudaSuccess)
         SETUP_TRY(fail(TX_ERR_CUDA, "set-up copy failed"));
     for (int d = 1; d < 3; ++d) SETUP_TRY(simt_kmajor(c->f_U[d], 1, n[d], r[d], d == 1 ? simt_ld2(n[d]) : simt_ld3(n[d]), c->f_UK[d], s));
+    SETUP_TRY(plan_terms(c, xs, gauss_exponents, gauss_weights));
     SETUP_TRY(setup_factor_matrices(c, s));
     SETUP_TRY(tx_set_precision(c, precision, stream));
 #undef SETUP_TRY

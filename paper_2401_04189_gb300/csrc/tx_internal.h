@@ -71,13 +71,36 @@ enum : int {
     EPI_MULW = 1,        // multiply the field by the quadrature weight w(x) before the Hadamard product
     EPI_ENERGY = 2,      // accumulate ew * sum_x w * SA * SB * field into the energy partials
     EPI_OUT = 4,         // perform the Hadamard-accumulate into out0 / out1
-    PROD_MULW = 8        // multiply the pair density by w(x) (adjoint producer)
+    PROD_MULW = 8,       // multiply the pair density by w(x) (adjoint producer)
+    EPI_STORE = 16,      // write the field itself, pair by pair, to OUT0 (no Hadamard product)
+    PROD_PLAIN = 32      // the producer's field is SA[p], not a product of two orbitals
 };
 
 // ------------------------------------------------------------------------------------
 // the context
 // ------------------------------------------------------------------------------------
 struct TcOperands;   // tensor-core operand copies (tx_tc.cu)
+
+// The Gaussian sum split into sharp and smooth terms (tx_setup.cu).  A smooth term's potential is
+// band-limited on the scale of a coarse grid of r_d Chebyshev nodes per mode, so it is evaluated there and
+// all smooth terms together are interpolated to the fine grid as ONE more term:
+//   phi = sum_{t sharp} mu_t G x_d A_td + (sum_{t smooth} mu_t G x_d Q_td) x_d I_d,
+//   Q_td[k][g] = sum_b C_t(xi_k, x_b) U_d[b][g],   I_d[a][k] = L_k(x_a)
+// nf = sharp terms + 1 (the interpolation, last), nc = smooth terms.  Without a split (nc = 0)
+// nf = T and F is the context's f_A.
+struct TermSplit {
+    int nf, nc;
+    double* d_theta;     // exponents, sharp then smooth
+    double* d_mu;
+    double* d_xi[3];     // [r_d] coarse nodes
+    double* F64[3];      // [nf][n_d][r_d] fine operators (mu_t folded into mode 3); null without a split
+    float* F[3];         // the same in float32
+    float* FK[3];        // modes 2 and 3 with the grid index fastest: [nf][r_d][simt_ld(n_d)]
+    double* Q64[3];      // [nc][r_d][r_d] coarse operators (mu_t folded into mode 3)
+    float* Q[3];
+    float* QK[3];        // modes 2 and 3 for the consumer: [nc][r_d][simt_ld(r_d)]
+    float* QKs[3];       // the same for cores stored [g][b]: modes 2 and 3 in each other's place
+};
 
 }  // namespace tx
 
@@ -96,7 +119,7 @@ struct tx_ctx {
     float* f_U[3];       // [n_d][r_d]
     float* f_A[3];       // [T][n_d][r_d]; mu_t folded into mode 3
     float* f_UK[3];      // modes 2 and 3 of f_U with the grid index fastest: [r_d][simt_ld(n_d)], zero-padded
-    float* f_AK[3];      // modes 2 and 3 of f_A the same way: [T][r_d][simt_ld(n_d)]
+    tx::TermSplit ts;    // the terms as the float32 kernels sum them
     float* f_w[3];       // [n_d]
     float* f_C[3];       // [T][n_d][n_d] convolution matrices, mu_t folded into mode 3 (per-pair path; lazy)
     bool c_valid;        // f_C matches the current quadrature
@@ -163,8 +186,24 @@ struct GemmArgs {
     int nb1, nb2;
     float alpha;
     int accumulate;
+    // split != 0: C is the hi part of a split operand (1: TF32 in float, 2: bf16) and the lo part lies
+    // c_lo elements behind it; column n = (g, b), b < nb, goes to element g * ld_b + b of the row, and
+    // nb <= b < ld_b is zero-filled
+    int split, nb, ld_b;
+    long c_lo;
 };
 int simt_gemm(const GemmArgs& g, cudaStream_t s);
+
+// grid and core sizes (and quadrature weights) that a float32 kernel works on
+struct Shape {
+    int n1, n2, n3, r1, r2, r3;
+    const float* w1;
+    const float* w2;
+    const float* w3;
+};
+Shape fine_shape(const tx_ctx* c);
+// the coarse grid of the smooth terms: r_d nodes, ranks r_d (weights unused); swapped: modes 2 and 3 exchanged
+Shape coarse_shape(const tx_ctx* c, bool swapped = false);
 
 struct FieldArgs {          // orbital-space arrays of one call
     const float* SA; const float* SB;          // producer sources
@@ -188,13 +227,15 @@ int simt_kmajor(const float* src, int nt, int n, int r, int ld, float* dst, cuda
 // expansion consumer: modes 2 and 3 for every term, Hadamard epilogue, energy partials.
 // Z [np][nterms][n1][(b,g)] (z_bg) or [(g,b)]; M2 [nterms][r2][simt_ld2] and M3 [nterms][r3][simt_ld3]
 // (per pair with strides m2_ps, m3_ps)
-int simt_expand_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f,
+// With EPI_STORE phi itself goes to f.OUT0 [np][n1][n2][n3] instead.
+int simt_expand_consume(const Shape& sh, const PairRec* recs, int p0, int np, const FieldArgs& f,
                         const float* Z, int nterms, const float* M2, const float* M3, int flags,
                         double* epart, cudaStream_t s, bool z_bg = true, long m2_ps = 0, long m3_ps = 0);
-int simt_expand_consume_blocks(const tx_ctx* c);
+int simt_expand_consume_blocks(const Shape& sh);
 // adjoint stage: R[p][t][x][b][g] = sum_{y,z} A_t2[y][b] A_t3[z][g] (prod)[x][y][z]
-int simt_adjoint_r(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f,
-                   int flags, float* R, cudaStream_t s);
+// for nt terms (M2 [nt][n2][r2], M3 [nt][n3][r3]); with PROD_PLAIN q_p is the field SA[p] itself
+int simt_adjoint_r(const Shape& sh, const PairRec* recs, int p0, int np, const FieldArgs& f, int nt, const float* M2,
+                   const float* M3, int flags, float* R, cudaStream_t s);
 // energy reductions
 int reduce_energy_batch(const double* epart, long count, double* dst, cudaStream_t s);
 int finalize_energy(const double* batches, int nb, double scale, double* e_dev, cudaStream_t s);
@@ -203,6 +244,9 @@ int finalize_energy(const double* batches, int nb, double scale, double* e_dev, 
 int weighted_dot(const tx_ctx* c, const float* A, const float* B, int count, double* partial, int nblocks, double scale,
                  double* e_dev, cudaStream_t s);
 
+// decides the term split of a new context and allocates its operators (host float64 inputs)
+int plan_terms(tx_ctx* c, const double* const x[3], const double* theta, const double* mu);
+void free_terms(tx_ctx* c);
 // setup -- tx_setup.cu (with_c: also write the float32 convolution matrices f_C)
 int setup_factor_matrices(tx_ctx* c, cudaStream_t s, bool with_c = false);
 // the same with finite-element quadrature (Lagrange elements of `order`, `points` Gauss points)

@@ -58,18 +58,6 @@ int simt_mode1_project(const tx_ctx* c, const float* S2, float* G, int np, cudaS
     return simt_gemm(q, s);
 }
 
-// Z[p][t][x][(b,g)] = sum_a M1_t[x][a] G[p][(b,g)][a]  (mode 1 of the expansion, every term)
-int simt_mode1_expand(const tx_ctx* c, const float* G, const float* M1, int nt, float* Z, int np, cudaStream_t s) {
-    const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
-    GemmArgs q{};
-    q.M = nt * n1; q.N = rr; q.K = r1;
-    q.A = M1; q.a_m = r1; q.a_k = 1;
-    q.B = G; q.b_k = 1; q.b_n = r1; q.b_b2 = (long)rr * r1;
-    q.C = Z; q.c_m = rr; q.c_n = 1; q.c_b2 = (long)nt * n1 * rr;
-    q.nb1 = 1; q.nb2 = np; q.alpha = 1.f;
-    return simt_gemm(q, s);
-}
-
 }  // namespace
 }  // namespace tx
 
@@ -125,8 +113,9 @@ extern "C" int tx_exchange_apply_static(tx_ctx* c, const float* psi_occ, int n_o
         const int np = (int)std::min<long>(Pb, P - p0);
         TX_TRY(simt_project_s2(c, recs, (int)p0, np, f, 0, S2, s));
         TX_TRY(simt_mode1_project(c, S2, G, np, s));
-        TX_TRY(simt_mode1_expand(c, G, c->f_A[0], c->T, Z, np, s));
-        TX_TRY(simt_expand_consume(c, recs, (int)p0, np, f, Z, c->T, c->f_AK[1], c->f_AK[2], EPI_OUT, nullptr, s));
+        TX_TRY(simt_expand_all(c, G, S2, Z, np, s));
+        TX_TRY(simt_expand_consume(fine_shape(c), recs, (int)p0, np, f, Z, c->ts.nf, c->ts.FK[1], c->ts.FK[2], EPI_OUT,
+                                   nullptr, s));
     }
     return TX_OK;
 }

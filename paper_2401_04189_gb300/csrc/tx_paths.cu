@@ -22,7 +22,8 @@ SimtLayout simt_layout(const tx_ctx* c) {
     SimtLayout L;
     L.s2 = n1 * r3 * r2;
     L.g = r3 * r2 * r1;
-    L.z = (size_t)c->T * n1 * r3 * r2;
+    // Z of the fine terms, or (earlier in the batch) of the coarse ones
+    L.z = std::max((size_t)c->ts.nf * n1, (size_t)c->ts.nc * r1) * r3 * r2;
     return L;
 }
 
@@ -38,35 +39,91 @@ int gemm_mode1_project(const tx_ctx* c, const float* S2, const float* M1, float*
     return simt_gemm(g, s);
 }
 
-// H[p][(b,g)][a] = sum_{t,x} R[p][t][x][(b,g)] A_t1[x][a]   (mode 1 of the adjoint, summed over t)
-int gemm_mode1_adjoint(const tx_ctx* c, const float* R, float* H, int np, cudaStream_t s) {
-    const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2], T = c->T;
+// H[p][(b,g)][a] (+)= sum_{t,x} R[p][t][x][(b,g)] M1_t[x][a] over the first nt of R's nr terms on a grid
+// of n1 nodes (mode 1 of the adjoint, summed over t)
+int gemm_mode1_adjoint(const tx_ctx* c, const float* R, const float* M1, int n1, int nt, int nr, float* H, bool add,
+                       int np, cudaStream_t s) {
+    const int r1 = c->r[0], rr = c->r[1] * c->r[2];
     GemmArgs g{};
-    g.M = rr; g.N = r1; g.K = T * n1;
-    g.A = R; g.a_m = 1; g.a_k = rr; g.a_b1 = 0; g.a_b2 = (long)T * n1 * rr;
-    g.B = c->f_A[0]; g.b_k = r1; g.b_n = 1; g.b_b1 = 0; g.b_b2 = 0;
+    g.M = rr; g.N = r1; g.K = nt * n1;
+    g.A = R; g.a_m = 1; g.a_k = rr; g.a_b1 = 0; g.a_b2 = (long)nr * n1 * rr;
+    g.B = M1; g.b_k = r1; g.b_n = 1; g.b_b1 = 0; g.b_b2 = 0;
     g.C = H; g.c_m = r1; g.c_n = 1; g.c_b1 = 0; g.c_b2 = (long)rr * r1;
+    g.nb1 = 1; g.nb2 = np; g.alpha = 1.f; g.accumulate = add ? 1 : 0;
+    return simt_gemm(g, s);
+}
+
+// Z[p][t][x][(b,g)] = sum_a M1_t[x][a] G[p][(b,g)][a] for nt terms on a grid of n1 nodes, written as terms
+// t0, t0 + 1, ... of nz (mode 1 of the expansion; M1 per pair when m1_ps > 0).  With core_a_first the
+// core is [a][(b,g)] instead.
+int gemm_mode1_expand(const tx_ctx* c, const float* G, const float* M1, int n1, int nt, int t0, int nz, float* Z, int np,
+                      cudaStream_t s, long m1_ps = 0, bool core_a_first = false) {
+    const int r1 = c->r[0], rr = c->r[1] * c->r[2];
+    GemmArgs g{};
+    g.M = nt * n1; g.N = rr; g.K = r1;         // the terms' rows (t, x) follow one another in M1 and in Z
+    g.A = M1; g.a_m = r1; g.a_k = 1; g.a_b2 = m1_ps;
+    g.B = G; g.b_k = core_a_first ? rr : 1; g.b_n = core_a_first ? 1 : r1; g.b_b2 = (long)rr * r1;
+    g.C = Z + (size_t)t0 * n1 * rr; g.c_m = rr; g.c_n = 1; g.c_b2 = (long)nz * n1 * rr;
     g.nb1 = 1; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
     return simt_gemm(g, s);
 }
 
-// Z[p][t][x][(b,g)] = sum_a M1_t[x][a] G[p][(b,g)][a]   (mode 1 of the expansion, every term;
-// M1 per pair when m1_ps > 0)
-int gemm_mode1_expand(const tx_ctx* c, const float* G, const float* M1, int nt, float* Z, int np, cudaStream_t s,
-                      long m1_ps = 0) {
-    const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
+}  // namespace
+
+int simt_expand_all(const tx_ctx* c, const float* G, float* H, float* Z, int np, cudaStream_t s) {
+    const TermSplit& ts = c->ts;
+    const int n1 = c->n[0];
+    if (!ts.nc) return gemm_mode1_expand(c, G, ts.F[0], n1, ts.nf, 0, ts.nf, Z, np, s);
+    // the smooth terms on the coarse grid: H[p][a][b][g] = sum_t mu_t G x_d Q_td
+    TX_TRY(gemm_mode1_expand(c, G, ts.Q[0], c->r[0], ts.nc, 0, ts.nc, Z, np, s));
+    FieldArgs fc{};
+    fc.OUT0 = H;
+    TX_TRY(simt_expand_consume(coarse_shape(c), nullptr, 0, np, fc, Z, ts.nc, ts.QK[1], ts.QK[2], EPI_STORE, nullptr, s));
+    // the sharp terms from G, the interpolation (the last fine term) from H
+    if (ts.nf > 1) TX_TRY(gemm_mode1_expand(c, G, ts.F[0], n1, ts.nf - 1, 0, ts.nf, Z, np, s));
+    return gemm_mode1_expand(c, H, ts.F[0] + (size_t)(ts.nf - 1) * n1 * c->r[0], n1, 1, ts.nf - 1, ts.nf, Z, np, s, 0, true);
+}
+
+namespace {
+
+// The adjoint's sums over the terms: H[p][(b,g)][a] from R[p][t][x][(b,g)] of every fine term (nf * n1 rows
+// per pair).  The smooth terms' transposes run behind one fine-grid term, q x_d I_d^T on the coarse
+// grid (Y, r1 r2 r3 floats per pair), then Q_td^T there (R is overwritten).  The order (b,g) may as
+// well be (g,b): `swapped` exchanges modes 2 and 3 of the coarse grid.
+int adjoint_sums(const tx_ctx* c, float* R, float* Y, float* H, bool swapped, int np, cudaStream_t s) {
+    const TermSplit& ts = c->ts;
+    const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2], ns = ts.nf - 1;
+    if (ns) TX_TRY(gemm_mode1_adjoint(c, R, ts.F[0], n1, ns, ts.nf, H, false, np, s));
+    // Y[p][k][(b,g)] = sum_x I_1[x][k] R[p][ns][x][(b,g)]
     GemmArgs g{};
-    g.M = nt * n1; g.N = rr; g.K = r1;         // the terms' rows (t, x) follow one another in M1 and in Z
-    g.A = M1; g.a_m = r1; g.a_k = 1; g.a_b2 = m1_ps;
-    g.B = G; g.b_k = 1; g.b_n = r1; g.b_b2 = (long)rr * r1;
-    g.C = Z; g.c_m = rr; g.c_n = 1; g.c_b2 = (long)nt * n1 * rr;
-    g.nb1 = 1; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
-    return simt_gemm(g, s);
+    g.M = r1; g.N = rr; g.K = n1;
+    g.A = ts.F[0] + (size_t)ns * n1 * r1; g.a_m = 1; g.a_k = r1;
+    g.B = R + (size_t)ns * n1 * rr; g.b_k = rr; g.b_n = 1; g.b_b2 = (long)ts.nf * n1 * rr;
+    g.C = Y; g.c_m = rr; g.c_n = 1; g.c_b2 = (long)r1 * rr;
+    g.nb1 = 1; g.nb2 = np; g.alpha = 1.f;
+    TX_TRY(simt_gemm(g, s));
+    FieldArgs fy{};
+    fy.SA = Y;
+    fy.SB = Y;
+    TX_TRY(simt_adjoint_r(coarse_shape(c, swapped), nullptr, 0, np, fy, ts.nc, ts.Q[swapped ? 2 : 1], ts.Q[swapped ? 1 : 2],
+                          PROD_PLAIN, R, s));
+    return gemm_mode1_adjoint(c, R, ts.Q[0], r1, ts.nc, ts.nc, H, ns > 0, np, s);
+}
+
+// H[p][(b,g)][a] = sum_t mu_t q_p x_d A_td^T (the adjoint onto the core) for the products q_p that recs and
+// f name; Y holds r1 r2 r3 floats per pair, R the Z share
+int simt_adjoint_core(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, int flags, float* Y,
+                      float* R, float* H, cudaStream_t s) {
+    const TermSplit& ts = c->ts;
+    TX_TRY(simt_adjoint_r(fine_shape(c), recs, p0, np, f, ts.nf, ts.F[1], ts.F[2], flags, R, s));
+    if (!ts.nc) return gemm_mode1_adjoint(c, R, ts.F[0], c->n[0], ts.nf, ts.nf, H, false, np, s);
+    return adjoint_sums(c, R, Y, H, false, np, s);
 }
 
 int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec* recs2, int p0, int np,
                float* S2, float* G, float* Z, double* epart, cudaStream_t s) {
     const bool subset = cs.mode == PAIRS_SUBSET;
+    const Shape sh = fine_shape(c);
     FieldArgs f{};
     switch (cs.kind) {
         case CALL_APPLY:
@@ -80,18 +137,17 @@ int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec
             f.OUT1 = cs.out0;
             TX_TRY(simt_project_s2(c, recs, p0, np, f, 0, S2, s));
             TX_TRY(gemm_mode1_project(c, S2, c->f_U[0], G, np, s));
-            TX_TRY(gemm_mode1_expand(c, G, c->f_A[0], c->T, Z, np, s));
+            TX_TRY(simt_expand_all(c, G, S2, Z, np, s));
             int flags = 0;
             if (cs.kind == CALL_APPLY) flags = EPI_OUT | (cs.e_dev ? EPI_ENERGY : 0);
             if (cs.kind == CALL_ENERGY) flags = EPI_ENERGY;
             if (cs.kind == CALL_GRAD) flags = EPI_OUT | EPI_MULW | (cs.e_dev ? EPI_ENERGY : 0);
-            TX_TRY(simt_expand_consume(c, recs, p0, np, f, Z, c->T, c->f_AK[1], c->f_AK[2], flags, epart, s));
+            TX_TRY(simt_expand_consume(sh, recs, p0, np, f, Z, c->ts.nf, c->ts.FK[1], c->ts.FK[2], flags, epart, s));
             if (cs.kind == CALL_GRAD) {
                 // second term: - sum_j psi_j * L^T(w rho_kj)
-                TX_TRY(simt_adjoint_r(c, recs, p0, np, f, PROD_MULW, Z, s));
-                TX_TRY(gemm_mode1_adjoint(c, Z, G, np, s));
-                TX_TRY(gemm_mode1_expand(c, G, c->f_U[0], 1, Z, np, s));
-                TX_TRY(simt_expand_consume(c, recs, p0, np, f, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, epart, s));
+                TX_TRY(simt_adjoint_core(c, recs, p0, np, f, PROD_MULW, S2, Z, G, s));
+                TX_TRY(gemm_mode1_expand(c, G, c->f_U[0], sh.n1, 1, 0, 1, Z, np, s));
+                TX_TRY(simt_expand_consume(sh, recs, p0, np, f, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, epart, s));
             }
             return TX_OK;
         }
@@ -103,18 +159,17 @@ int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec
                 f.MUL1 = nullptr; f.OUT1 = nullptr;
                 TX_TRY(simt_project_s2(c, recs, p0, np, f, 0, S2, s));
                 TX_TRY(gemm_mode1_project(c, S2, c->f_U[0], G, np, s));
-                TX_TRY(gemm_mode1_expand(c, G, c->f_A[0], c->T, Z, np, s));
-                TX_TRY(simt_expand_consume(c, recs, p0, np, f, Z, c->T, c->f_AK[1], c->f_AK[2], EPI_OUT, epart, s));
+                TX_TRY(simt_expand_all(c, G, S2, Z, np, s));
+                TX_TRY(simt_expand_consume(sh, recs, p0, np, f, Z, c->ts.nf, c->ts.FK[1], c->ts.FK[2], EPI_OUT, epart, s));
             }
             // zeta_kj = L^T(cot_k psi_j): grad_tgt_k -= psi_j zeta, grad_occ_j -= psi_tgt_k zeta
             FieldArgs f2{};
             f2.SA = cs.cot; f2.SB = cs.occ;
             f2.MUL0 = cs.occ; f2.OUT0 = cs.out1;
             f2.MUL1 = cs.tgt; f2.OUT1 = cs.out0;
-            TX_TRY(simt_adjoint_r(c, recs2, p0, np, f2, 0, Z, s));
-            TX_TRY(gemm_mode1_adjoint(c, Z, G, np, s));
-            TX_TRY(gemm_mode1_expand(c, G, c->f_U[0], 1, Z, np, s));
-            TX_TRY(simt_expand_consume(c, recs2, p0, np, f2, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, epart, s));
+            TX_TRY(simt_adjoint_core(c, recs2, p0, np, f2, 0, S2, Z, G, s));
+            TX_TRY(gemm_mode1_expand(c, G, c->f_U[0], sh.n1, 1, 0, 1, Z, np, s));
+            TX_TRY(simt_expand_consume(sh, recs2, p0, np, f2, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, epart, s));
             return TX_OK;
         }
     }
@@ -139,21 +194,28 @@ int galerkin_batch(tx_ctx* c, const CallSpec& cs, const GalerkinOps& o, const Pa
     TX_TRY(galerkin_core(c, o, G, X1, X2, H, np, s));
     if (cs.kind == CALL_ENERGY) return galerkin_core_dot(c, recs, p0, G, H, np, epart, s);
     float* Z = S2;   // [np][1][n1][r2 r3]: the size of S2
-    TX_TRY(gemm_mode1_expand(c, H, o.Ut[0], 1, Z, np, s));
-    return simt_expand_consume(c, recs, p0, np, f, Z, 1, o.Ut[1], o.Ut[2], EPI_OUT, epart, s);
+    TX_TRY(gemm_mode1_expand(c, H, o.Ut[0], c->n[0], 1, 0, 1, Z, np, s));
+    return simt_expand_consume(fine_shape(c), recs, p0, np, f, Z, 1, o.Ut[1], o.Ut[2], EPI_OUT, epart, s);
 }
 
 }  // namespace
 
 int simt_adjoint_mode1(const tx_ctx* c, const float* R, float* H, int np, cudaStream_t s) {
-    return gemm_mode1_adjoint(c, R, H, np, s);
+    return gemm_mode1_adjoint(c, R, c->f_A[0], c->n[0], c->T, c->T, H, false, np, s);
+}
+int simt_adjoint_split(const tx_ctx* c, float* R, float* Y, float* H, int np, cudaStream_t s) {
+    return adjoint_sums(c, R, Y, H, true, np, s);
+}
+int simt_expand_mode1_grid(const tx_ctx* c, const float* G, const float* M1, int n1, int nt, float* Z, int np,
+                           cudaStream_t s) {
+    return gemm_mode1_expand(c, G, M1, n1, nt, 0, nt, Z, np, s);
 }
 int simt_expand_mode1(const tx_ctx* c, const float* G, const float* M1, int nt, float* Z, int np, cudaStream_t s) {
-    return gemm_mode1_expand(c, G, M1, nt, Z, np, s);
+    return gemm_mode1_expand(c, G, M1, c->n[0], nt, 0, nt, Z, np, s);
 }
 int simt_expand_mode1_pp(const tx_ctx* c, const float* G, const float* M1, long m1_pair_stride, int nt, float* Z,
                          int np, cudaStream_t s) {
-    return gemm_mode1_expand(c, G, M1, nt, Z, np, s, m1_pair_stride);
+    return gemm_mode1_expand(c, G, M1, c->n[0], nt, 0, nt, Z, np, s, m1_pair_stride);
 }
 
 int run_call(tx_ctx* c, const CallSpec& cs, cudaStream_t s) {
@@ -174,16 +236,16 @@ int run_call(tx_ctx* c, const CallSpec& cs, cudaStream_t s) {
     if (pp) {
         TX_TRY(sthosvd_check(c));
         per_pair = sizeof(float) * sthosvd_floats_per_pair(c);
-        epp = simt_expand_consume_blocks(c);
+        epp = simt_expand_consume_blocks(fine_shape(c));
     } else if (gk) {
         per_pair = sizeof(float) * (L.s2 + 2 * L.g + 2 * (size_t)c->T * L.g);
-        epp = cs.kind == CALL_ENERGY ? 1 : simt_expand_consume_blocks(c);
+        epp = cs.kind == CALL_ENERGY ? 1 : simt_expand_consume_blocks(fine_shape(c));
     } else if (tc) {
         per_pair = tc_batch_bytes_per_pair(c, cs.kind);
         epp = tc_epart_per_pair(c);
     } else {
         per_pair = sizeof(float) * (L.s2 + L.g + L.z);
-        epp = simt_expand_consume_blocks(c);
+        epp = simt_expand_consume_blocks(fine_shape(c));
     }
     per_pair += sizeof(double) * epp;
     size_t avail = c->ws_limit > recs_bytes + prefix + 4096 ? c->ws_limit - recs_bytes - prefix - 4096 : 0;

@@ -45,6 +45,10 @@ int galerkin_core(const tx_ctx* c, const GalerkinOps& o, const float* G, float* 
 int galerkin_core_dot(const tx_ctx* c, const PairRec* recs, int p0, const float* G, const float* H, int np,
                       double* epart, cudaStream_t s);
 
+// Z[p][t][x][(b,g)] for every fine term of the split (nf of them) from the cores G[p][(b,g)][a]; H holds
+// r1 r2 r3 floats per pair of scratch (untouched without a split)
+int simt_expand_all(const tx_ctx* c, const float* G, float* H, float* Z, int np, cudaStream_t s);
+
 int run_call(tx_ctx* c, const CallSpec& cs, cudaStream_t s);
 int ensure_workspace(tx_ctx* c, size_t bytes);
 int ensure_ebatch(tx_ctx* c, int nb);
@@ -61,6 +65,12 @@ size_t tc_batch_bytes_per_pair(const tx_ctx* c, int kind);
 // float32 building blocks shared with the tensor-core adjoint (tx_paths.cu):
 // H[p][(g,b)][a] = sum_{t,x} R[p][t][x][(g,b)] A_t1[x][a]
 int simt_adjoint_mode1(const tx_ctx* c, const float* R, float* H, int np, cudaStream_t s);
+// the same from the fine terms' R[p][t][x][(g,b)], the smooth terms through the coarse grid (Y: r1 r2 r3
+// floats per pair of scratch; R is overwritten and holds at least nc r1 r2 r3 floats per pair)
+int simt_adjoint_split(const tx_ctx* c, float* R, float* Y, float* H, int np, cudaStream_t s);
+// Z[p][t][x][(g,b)] = sum_a M1_t[x][a] G[p][(g,b)][a] on a grid of n1 nodes
+int simt_expand_mode1_grid(const tx_ctx* c, const float* G, const float* M1, int n1, int nt, float* Z, int np,
+                           cudaStream_t s);
 // Z[p][t][x][(g,b)] = sum_a M1_t[x][a] G[p][(g,b)][a]  (nt terms of M1 = [nt][n1][r1])
 int simt_expand_mode1(const tx_ctx* c, const float* G, const float* M1, int nt, float* Z, int np, cudaStream_t s);
 long tc_epart_per_pair(const tx_ctx* c);

@@ -7,22 +7,27 @@
 // mu_t is folded into the mode-3 factor in float64 before any rounding.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
+#include <cstring>
+#include <string>
+#include <vector>
 
 #include "tx_internal.h"
 
 namespace tx {
 namespace {
 
-__global__ void k_conv_factor(const double* __restrict__ x, const double* __restrict__ w,
+// rows a of C_td at the target points xt (the grid itself, or the coarse nodes of the smooth terms)
+__global__ void k_conv_factor(const double* __restrict__ xt, const double* __restrict__ x, const double* __restrict__ w,
                               const double* __restrict__ U, const double* __restrict__ theta,
                               const double* __restrict__ mu, int n, int r, int fold_mu,
                               double* __restrict__ A64, float* __restrict__ A32, float* __restrict__ C32) {
     extern __shared__ double kv[];   // [n]: row a of C_td
-    const int a = blockIdx.x, t = blockIdx.y;
+    const int a = blockIdx.x, t = blockIdx.y, na = gridDim.x;
     const double th = theta[t];
     for (int b = threadIdx.x; b < n; b += blockDim.x) {
-        const double dx = x[a] - x[b];
+        const double dx = xt[a] - x[b];
         kv[b] = w[b] * exp(-th * dx * dx);
     }
     __syncthreads();
@@ -33,7 +38,7 @@ __global__ void k_conv_factor(const double* __restrict__ x, const double* __rest
         double s = 0.0;
         for (int b = 0; b < n; ++b) s = fma(kv[b], U[(long)b * r + k], s);
         s *= scale;
-        const long o = ((long)t * n + a) * r + k;
+        const long o = ((long)t * na + a) * r + k;
         A64[o] = s;
         A32[o] = (float)s;
     }
@@ -43,13 +48,13 @@ __global__ void k_conv_factor(const double* __restrict__ x, const double* __rest
 // elements of order p (element e holds nodes p e .. p e + p) and each convolution integral is
 // evaluated with q Gauss-Legendre points per element:
 //   C_td[a][b] = sum_{e contains b} sum_q J_e w_q N_b(x_q) exp(-theta_t (x_a - x_q)^2)
-__global__ void k_conv_factor_fe(const double* __restrict__ x, const double* __restrict__ U,
+__global__ void k_conv_factor_fe(const double* __restrict__ xt, const double* __restrict__ x, const double* __restrict__ U,
                                  const double* __restrict__ theta, const double* __restrict__ mu, int n, int r,
                                  int fold_mu, int p, int q, const double* __restrict__ gx, const double* __restrict__ gw,
                                  double* __restrict__ A64, float* __restrict__ A32, float* __restrict__ C32) {
     extern __shared__ double kv[];   // [n]: row a of C_td
-    const int a = blockIdx.x, t = blockIdx.y;
-    const double th = theta[t], xa = x[a];
+    const int a = blockIdx.x, t = blockIdx.y, na = gridDim.x;
+    const double th = theta[t], xa = xt[a];
     const int nel = (n - 1) / p;
     for (int b = threadIdx.x; b < n; b += blockDim.x) {
         double v = 0.0;
@@ -79,7 +84,7 @@ __global__ void k_conv_factor_fe(const double* __restrict__ x, const double* __r
         double s = 0.0;
         for (int b = 0; b < n; ++b) s = fma(kv[b], U[(long)b * r + k], s);
         s *= scale;
-        const long o = ((long)t * n + a) * r + k;
+        const long o = ((long)t * na + a) * r + k;
         A64[o] = s;
         A32[o] = (float)s;
     }
@@ -110,6 +115,47 @@ static void gauss_legendre(int q, double* xg, double* wg) {
     }
 }
 
+// A_td for nt terms at the target points xt (na of them), by the context's quadrature rule: FE
+// elements where gx (Gauss points) is given, the nodal rule otherwise
+static int conv_factors(const tx_ctx* c, int d, const double* xt, int na, const double* theta, const double* mu, int nt,
+                        int order, int points, const double* gx, double* A64, float* A32, float* C32, cudaStream_t s) {
+    const int n = c->n[d], r = c->r[d];
+    const size_t smem = sizeof(double) * n;
+    if (gx)
+        k_conv_factor_fe<<<dim3(na, nt), 128, smem, s>>>(xt, c->d_x[d], c->d_U[d], theta, mu, n, r, d == 2 ? 1 : 0, order,
+                                                         points, gx, gx + points, A64, A32, C32);
+    else
+        k_conv_factor<<<dim3(na, nt), 128, smem, s>>>(xt, c->d_x[d], c->d_w[d], c->d_U[d], theta, mu, n, r, d == 2 ? 1 : 0,
+                                                      A64, A32, C32);
+    TX_LAUNCHED();
+    return TX_OK;
+}
+
+static int ld_of(int d, int n) { return d == 1 ? simt_ld2(n) : simt_ld3(n); }
+
+// every operator of the context for one quadrature rule
+static int all_factors(tx_ctx* c, int order, int points, const double* gx, cudaStream_t s, bool with_c) {
+    const TermSplit& ts = c->ts;
+    for (int d = 0; d < 3; ++d) {
+        const int n = c->n[d], r = c->r[d];
+        TX_TRY(conv_factors(c, d, c->d_x[d], n, c->d_theta, c->d_mu, c->T, order, points, gx, c->d_A64[d], c->f_A[d],
+                            with_c ? c->f_C[d] : nullptr, s));
+        if (ts.nc) {
+            const int ns = ts.nf - 1;
+            if (ns) TX_TRY(conv_factors(c, d, c->d_x[d], n, ts.d_theta, ts.d_mu, ns, order, points, gx, ts.F64[d], ts.F[d],
+                                        nullptr, s));
+            TX_TRY(conv_factors(c, d, ts.d_xi[d], r, ts.d_theta + ns, ts.d_mu + ns, ts.nc, order, points, gx, ts.Q64[d],
+                                ts.Q[d], nullptr, s));
+            if (d > 0) {
+                TX_TRY(simt_kmajor(ts.Q[d], ts.nc, r, r, ld_of(d, r), ts.QK[d], s));
+                TX_TRY(simt_kmajor(ts.Q[d], ts.nc, r, r, ld_of(3 - d, r), ts.QKs[d], s));
+            }
+        }
+        if (d > 0) TX_TRY(simt_kmajor(ts.F[d], ts.nf, n, r, ld_of(d, n), ts.FK[d], s));
+    }
+    return TX_OK;
+}
+
 int setup_factor_matrices_fe(tx_ctx* c, int order, int points, cudaStream_t s, bool with_c) {
     double hx[64], hw[64];
     gauss_legendre(points, hx, hw);
@@ -122,32 +168,141 @@ int setup_factor_matrices_fe(tx_ctx* c, int order, int points, cudaStream_t s, b
     if (cudaMemcpy(d, hx, sizeof(double) * points, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d + points, hw, sizeof(double) * points, cudaMemcpyHostToDevice) != cudaSuccess)
         st = fail(TX_ERR_CUDA, "quadrature points copy");
-    for (int dd = 0; dd < 3 && st == TX_OK; ++dd) {
-        const int n = c->n[dd], r = c->r[dd];
-        k_conv_factor_fe<<<dim3(n, c->T), 128, sizeof(double) * n, s>>>(c->d_x[dd], c->d_U[dd], c->d_theta, c->d_mu, n, r,
-                                                                         dd == 2 ? 1 : 0, order, points, d, d + points,
-                                                                         c->d_A64[dd], c->f_A[dd],
-                                                                         with_c ? c->f_C[dd] : nullptr);
-        count_launch();
-        if (cudaGetLastError() != cudaSuccess) st = fail(TX_ERR_CUDA, "k_conv_factor_fe launch");
-        if (st == TX_OK && dd > 0) st = simt_kmajor(c->f_A[dd], c->T, n, r, dd == 1 ? simt_ld2(n) : simt_ld3(n), c->f_AK[dd], s);
-    }
+    if (st == TX_OK) st = all_factors(c, order, points, d, s, with_c);
     cudaStreamSynchronize(s);
     cudaFree(d);
     return st;
 }
 
-int setup_factor_matrices(tx_ctx* c, cudaStream_t s, bool with_c) {
+int setup_factor_matrices(tx_ctx* c, cudaStream_t s, bool with_c) { return all_factors(c, 0, 0, nullptr, s, with_c); }
+
+// ======================================================================================
+// the split of the Gaussian sum
+// ======================================================================================
+// Bound on the error of interpolating exp(-theta (x - c)^2), any real c, on an interval of half-length h
+// at N + 1 Chebyshev nodes: 4 M rho^-N / (rho - 1) with M the largest modulus on the Bernstein ellipse of
+// parameter rho = e^eta (Trefethen, Approximation Theory and Approximation Practice, Thm 8.2).  On the
+// ellipse |Im z| <= h sinh(eta), so M = exp(theta h^2 sinh(eta)^2); the exponent
+// theta h^2 sinh(eta)^2 - N eta is least at sinh(2 eta) = N / (theta h^2).
+static double chebyshev_bound(double theta, double h, int N) {
+    const double a = theta * h * h;
+    const double eta = 0.5 * std::asinh((double)N / a), sh = std::sinh(eta);
+    return 4.0 * std::exp(a * sh * sh - (double)N * eta) / (std::exp(eta) - 1.0);
+}
+
+// A term is smooth where every mode's r_d Chebyshev nodes interpolate its kernel to 1e-9 of its maximum:
+// 60 times below the float32 rounding of the operators, so the split changes results by rounding only.
+constexpr double kSmoothTol = 1e-9;
+
+int plan_terms(tx_ctx* c, const double* const x[3], const double* theta, const double* mu) {
+    TermSplit& ts = c->ts;
+    std::memset(&ts, 0, sizeof(ts));
+    double lo[3], hi[3];
     for (int d = 0; d < 3; ++d) {
-        const int n = c->n[d], r = c->r[d];
-        const size_t smem = sizeof(double) * n;
-        k_conv_factor<<<dim3(n, c->T), 128, smem, s>>>(c->d_x[d], c->d_w[d], c->d_U[d], c->d_theta, c->d_mu, n, r,
-                                                        d == 2 ? 1 : 0, c->d_A64[d], c->f_A[d],
-                                                        with_c ? c->f_C[d] : nullptr);
-        TX_LAUNCHED();
-        if (d > 0) TX_TRY(simt_kmajor(c->f_A[d], c->T, n, r, d == 1 ? simt_ld2(n) : simt_ld3(n), c->f_AK[d], s));
+        lo[d] = *std::min_element(x[d], x[d] + c->n[d]);
+        hi[d] = *std::max_element(x[d], x[d] + c->n[d]);
+    }
+    std::vector<double> th, m, th_c, m_c;
+    for (int t = 0; t < c->T; ++t) {
+        bool smooth = true;
+        for (int d = 0; d < 3 && smooth; ++d)
+            smooth = chebyshev_bound(theta[t], 0.5 * (hi[d] - lo[d]), c->r[d] - 1) <= kSmoothTol;
+        (smooth ? th_c : th).push_back(theta[t]);
+        (smooth ? m_c : m).push_back(mu[t]);
+    }
+    // worth it where the smooth terms' fine-grid work is more than their coarse work plus the
+    // interpolation (one fine term); a tenth of a fine term stands for the extra launches
+    auto mode_flops = [&](const int n[3]) {
+        const double r1 = c->r[0], r2 = c->r[1], r3 = c->r[2];
+        return n[0] * r1 * r2 * r3 + (double)n[0] * n[1] * r2 * r3 + (double)n[0] * n[1] * n[2] * r3;
+    };
+    const double fine = mode_flops(c->n), coarse = mode_flops(c->r), nc = (double)th_c.size();
+    // (coarse grids up to 160 nodes per mode: every float32 kernel takes them)
+    const bool on = nc * fine > 1.1 * fine + nc * coarse && std::max(c->r[1], c->r[2]) <= 160;
+    ts.nc = on ? (int)th_c.size() : 0;
+    ts.nf = on ? (int)th.size() + 1 : c->T;
+    auto dalloc = [&](auto** p, size_t count) -> int {
+        if (cudaMalloc((void**)p, sizeof(**p) * std::max<size_t>(count, 1)) == cudaSuccess) return TX_OK;
+        cudaGetLastError();
+        *p = nullptr;
+        return fail(TX_ERR_OOM, "operators of the term split");
+    };
+    for (int d = 0; d < 3; ++d) {
+        const size_t n = c->n[d], r = c->r[d];
+        if (d > 0) TX_TRY(dalloc(&ts.FK[d], (size_t)ts.nf * r * ld_of(d, (int)n)));
+        if (!on) {
+            ts.F[d] = c->f_A[d];
+            continue;
+        }
+        TX_TRY(dalloc(&ts.F64[d], (size_t)ts.nf * n * r));
+        TX_TRY(dalloc(&ts.F[d], (size_t)ts.nf * n * r));
+        TX_TRY(dalloc(&ts.Q64[d], (size_t)ts.nc * r * r));
+        TX_TRY(dalloc(&ts.Q[d], (size_t)ts.nc * r * r));
+        if (d > 0) TX_TRY(dalloc(&ts.QK[d], (size_t)ts.nc * r * ld_of(d, (int)r)));
+        if (d > 0) TX_TRY(dalloc(&ts.QKs[d], (size_t)ts.nc * r * ld_of(3 - d, (int)r)));
+        TX_TRY(dalloc(&ts.d_xi[d], r));
+        // Chebyshev nodes and the barycentric Lagrange values at the grid nodes
+        const double pi = 3.14159265358979323846;
+        std::vector<double> xi(r), bw(r), I(n * r);
+        std::vector<float> If(n * r);
+        for (size_t k = 0; k < r; ++k) {
+            xi[k] = 0.5 * (lo[d] + hi[d]) - 0.5 * (hi[d] - lo[d]) * std::cos(pi * (k + 0.5) / r);
+            bw[k] = (k % 2 ? -1.0 : 1.0) * std::sin(pi * (k + 0.5) / r);
+        }
+        for (size_t a = 0; a < n; ++a) {
+            double den = 0.0;
+            size_t hit = r;
+            for (size_t k = 0; k < r; ++k) {
+                if (x[d][a] == xi[k]) hit = k;
+                else den += bw[k] / (x[d][a] - xi[k]);
+            }
+            for (size_t k = 0; k < r; ++k) {
+                I[a * r + k] = hit < r ? (k == hit ? 1.0 : 0.0) : bw[k] / (x[d][a] - xi[k]) / den;
+                If[a * r + k] = (float)I[a * r + k];
+            }
+        }
+        const size_t o = (size_t)(ts.nf - 1) * n * r;
+        if (cudaMemcpy(ts.d_xi[d], xi.data(), sizeof(double) * r, cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemcpy(ts.F64[d] + o, I.data(), sizeof(double) * n * r, cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemcpy(ts.F[d] + o, If.data(), sizeof(float) * n * r, cudaMemcpyHostToDevice) != cudaSuccess)
+            return fail(TX_ERR_CUDA, "term split copy");
+    }
+    if (on) {
+        th.insert(th.end(), th_c.begin(), th_c.end());
+        m.insert(m.end(), m_c.begin(), m_c.end());
+        TX_TRY(dalloc(&ts.d_theta, th.size()));
+        TX_TRY(dalloc(&ts.d_mu, m.size()));
+        if (cudaMemcpy(ts.d_theta, th.data(), sizeof(double) * th.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemcpy(ts.d_mu, m.data(), sizeof(double) * m.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+            return fail(TX_ERR_CUDA, "term split copy");
     }
     return TX_OK;
+}
+
+void free_terms(tx_ctx* c) {
+    TermSplit& ts = c->ts;
+    for (int d = 0; d < 3; ++d) {
+        cudaFree(ts.d_xi[d]);
+        cudaFree(ts.F64[d]);
+        if (ts.F[d] != c->f_A[d]) cudaFree(ts.F[d]);
+        cudaFree(ts.FK[d]);
+        cudaFree(ts.Q64[d]);
+        cudaFree(ts.Q[d]);
+        cudaFree(ts.QK[d]);
+        cudaFree(ts.QKs[d]);
+    }
+    cudaFree(ts.d_theta);
+    cudaFree(ts.d_mu);
+    std::memset(&ts, 0, sizeof(ts));
+}
+
+Shape fine_shape(const tx_ctx* c) {
+    return Shape{c->n[0], c->n[1], c->n[2], c->r[0], c->r[1], c->r[2], c->f_w[0], c->f_w[1], c->f_w[2]};
+}
+Shape coarse_shape(const tx_ctx* c, bool swapped) {
+    if (swapped)
+        return Shape{c->r[0], c->r[2], c->r[1], c->r[0], c->r[2], c->r[1], c->f_w[0], c->f_w[1], c->f_w[2]};
+    return Shape{c->r[0], c->r[1], c->r[2], c->r[0], c->r[1], c->r[2], c->f_w[0], c->f_w[1], c->f_w[2]};
 }
 
 }  // namespace tx

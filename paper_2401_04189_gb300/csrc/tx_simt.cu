@@ -14,6 +14,7 @@
 #include <string>
 
 #include "tx_internal.h"
+#include "tx_tc_common.cuh"
 
 namespace tx {
 
@@ -198,6 +199,38 @@ __global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3) k_gemm(GemmArgs 
         }
         // the other buffer was last read one slice ago, before this slice's barrier
     }
+    if (g.split) {
+        // hi + lo parts straight from the accumulators: the float32 product never reaches memory
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            const int n = n0 + gemm_index<TN>(tn, j);
+            if (n >= g.N) continue;
+            const int gg = n / g.nb;
+            const int npad = n - gg * g.nb == g.nb - 1 ? g.ld_b - g.nb : 0;    // zeros after the last b
+            const long col = b1 * g.c_b1 + b2 * g.c_b2 + (long)gg * g.ld_b + (n - gg * g.nb);
+#pragma unroll
+            for (int i = 0; i < TM; ++i) {
+                const int m = m0 + gemm_index<TM>(tm, i);
+                if (m >= g.M) continue;
+                const float2 q = unpack2(acc[i][j / 2]);
+                const float v = g.alpha * ((j & 1) ? q.y : q.x);
+                const long o = col + m * g.c_m;
+                if (g.split == 1) {
+                    const float h = tc::tf32_hi(v);
+                    g.C[o] = h;
+                    g.C[o + g.c_lo] = tc::tf32_hi(v - h);
+                    for (int k = 1; k <= npad; ++k) g.C[o + k] = g.C[o + k + g.c_lo] = 0.f;
+                } else {
+                    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+                    __nv_bfloat16* C16 = (__nv_bfloat16*)g.C;
+                    C16[o] = h;
+                    C16[o + g.c_lo] = __float2bfloat16_rn(v - __bfloat162float(h));
+                    for (int k = 1; k <= npad; ++k) C16[o + k] = C16[o + k + g.c_lo] = __float2bfloat16_rn(0.f);
+                }
+            }
+        }
+        return;
+    }
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         const int m = m0 + gemm_index<TM>(tm, i);
@@ -228,9 +261,7 @@ struct Dims {
     int n1, n2, n3, r1, r2, r3;
 };
 
-Dims dims_of(const tx_ctx* c) {
-    return Dims{c->n[0], c->n[1], c->n[2], c->r[0], c->r[1], c->r[2]};
-}
+Dims dims_of(const Shape& h) { return Dims{h.n1, h.n2, h.n3, h.r1, h.r2, h.r3}; }
 
 // ====================================================================================
 // pair tables
@@ -344,10 +375,11 @@ __global__ void __launch_bounds__(384) k_chain(const ChainArgs a) {
     float* m3s = m2s + a.mh * a.ldb;           // [PZ][ldg]
     float* s1 = m3s + PZ * a.ldg;              // [ty][ldg]
     const int x = blockIdx.x, pl = blockIdx.y, tid = threadIdx.x, nth = blockDim.x;
-    const PairRec rec = a.recs[a.p0 + pl];
+    const bool plain = (a.flags & PROD_PLAIN) != 0;
+    const PairRec rec = plain ? PairRec{} : a.recs[a.p0 + pl];
     const long N3 = (long)d.n1 * d.n2 * d.n3;
-    const float* pa = a.SA + rec.ia * N3 + (long)x * d.n2 * d.n3;
-    const float* pb = a.SB + rec.ib * N3 + (long)x * d.n2 * d.n3;
+    const float* pa = a.SA + (plain ? pl : rec.ia) * N3 + (long)x * d.n2 * d.n3;
+    const float* pb = plain ? pa : a.SB + rec.ib * N3 + (long)x * d.n2 * d.n3;
     const bool mulw = (a.flags & PROD_MULW) != 0;
     const float wx = mulw ? a.w1[x] : 1.f;
     const int tz = tid & 7, row0 = kRows * (tid >> 3);
@@ -373,7 +405,7 @@ __global__ void __launch_bounds__(384) k_chain(const ChainArgs a) {
             if (!piece(i, z0, yn, yy, z)) continue;
             const long o = (long)(y0 + yy) * d.n3 + z0 + z;
             fa[i] = *(const float4*)(pa + o);
-            fb[i] = *(const float4*)(pb + o);
+            fb[i] = plain ? make_float4(1.f, 1.f, 1.f, 1.f) : *(const float4*)(pb + o);
         }
     };
     for (int t = 0; t < a.nt; ++t) {
@@ -409,7 +441,7 @@ __global__ void __launch_bounds__(384) k_chain(const ChainArgs a) {
                         for (int e = tid; e < yn * zn; e += nth) {
                             const int yy = e / zn, z = e - yy * zn;
                             const long o = (long)(y0 + yy) * d.n3 + z0 + z;
-                            float q = pa[o] * pb[o];
+                            float q = plain ? pa[o] : pa[o] * pb[o];
                             if (mulw) q *= wx * a.w2[y0 + yy] * a.w3[z0 + z];
                             qs[z * a.ldy + yy] = q;
                         }
@@ -571,7 +603,7 @@ __global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_co
     const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
     const int iy = blockIdx.x % a.ny, x0 = (blockIdx.x / a.ny) * a.px, pl = blockIdx.y;
     const int y0 = iy * a.ty;
-    const PairRec rec = a.recs[a.p0 + pl];
+    const PairRec rec = (a.flags & EPI_STORE) ? PairRec{} : a.recs[a.p0 + pl];
     const int tz = tid % CL, row0 = kRows * (tid / CL);
     const int pr = min(row0 / a.ty, a.px - 1);         // plane of this thread's rows
     const int yr = min(row0 - pr * a.ty, a.ty - kRows);    // rows past the last plane repeat valid ones (not stored)
@@ -691,6 +723,12 @@ __global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_co
             const int z = c < 2 * RN4 ? 4 * CL * (c / 2) + 4 * tz + 2 * (c & 1) : 4 * CL * RN4 + 2 * tz;
             const float2 ph = unpack2(acc[i][c]);
             const float phi[2] = {ph.x, ph.y};
+            if (a.flags & EPI_STORE) {
+                float* dst = a.f.OUT0 + pl * N3 + base + z;
+                if (z < d.n3) dst[0] = phi[0];
+                if (z + 1 < d.n3) dst[1] = phi[1];
+                continue;
+            }
             if (a.vec && z < d.n3) {           // even n3: the pair z, z + 1 is inside and 8-byte aligned
                 float f[2] = {phi[0], phi[1]};
                 if (a.flags & EPI_MULW) {
@@ -864,13 +902,13 @@ namespace {
 constexpr size_t kSmemLimit = 232448;      // 227 KB per CTA
 
 // modes 3 and 2 of a projection for nt terms of (M3 [nt][n3][r3], M2 [nt][n2][r2])
-int launch_chain(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, int nt, const float* M2,
+int launch_chain(const Shape& sh, const PairRec* recs, int p0, int np, const FieldArgs& f, int nt, const float* M2,
                  const float* M3, int flags, float* out, bool bg, const char* name, cudaStream_t s) {
     ChainArgs a{};
-    a.d = dims_of(c);
+    a.d = dims_of(sh);
     a.recs = recs; a.p0 = p0; a.nt = nt;
     a.SA = f.SA; a.SB = f.SB; a.M2 = M2; a.M3 = M3;
-    a.w1 = c->f_w[0]; a.w2 = c->f_w[1]; a.w3 = c->f_w[2];
+    a.w1 = sh.w1; a.w2 = sh.w2; a.w3 = sh.w3;
     a.flags = flags; a.out = out; a.bg = bg ? 1 : 0;
     // y tiles of at most 256 rows of equal height, one thread per row
     const int ny = (a.d.n2 + 255) / 256, tyv = (a.d.n2 + ny - 1) / ny;
@@ -950,15 +988,16 @@ int launch_consume(const ConsumeF32Args& a, const SimtPlan& p, int np, cudaStrea
 
 int simt_project_s2(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, int flags,
                     float* S2, cudaStream_t s, bool bg) {
-    const Dims d = dims_of(c);
+    const Shape sh = fine_shape(c);
+    const Dims d = dims_of(sh);
     if (sizeof(float) * ((size_t)d.n3 * d.r3 + (size_t)d.n2 * d.r3 + 8 * (size_t)d.n3) > kSmemLimit)
         return fail(TX_ERR_CUDA, "float32 projection: (n2 + n3) * r3 too large");
-    return launch_chain(c, recs, p0, np, f, 1, c->f_U[1], c->f_U[2], flags, S2, bg, "project", s);
+    return launch_chain(sh, recs, p0, np, f, 1, c->f_U[1], c->f_U[2], flags, S2, bg, "project", s);
 }
 
-int simt_expand_consume_blocks(const tx_ctx* c) {
+int simt_expand_consume_blocks(const Shape& sh) {
     SimtPlan p{};
-    return simt_plan(dims_of(c), &p) ? p.nx * p.ny : 1;
+    return simt_plan(dims_of(sh), &p) ? p.nx * p.ny : 1;
 }
 
 int simt_ld2(int n2) { return (n2 + 7) & ~7; }
@@ -975,10 +1014,10 @@ int simt_kmajor(const float* src, int nt, int n, int r, int ld, float* dst, cuda
     return TX_OK;
 }
 
-int simt_expand_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, const float* Z,
+int simt_expand_consume(const Shape& sh, const PairRec* recs, int p0, int np, const FieldArgs& f, const float* Z,
                         int nterms, const float* M2, const float* M3, int flags, double* epart, cudaStream_t s,
                         bool z_bg, long m2_ps, long m3_ps) {
-    const Dims d = dims_of(c);
+    const Dims d = dims_of(sh);
     if (d.n3 > 256) return fail(TX_ERR_UNSUPPORTED_SHAPE, "float32 path supports n3 <= 256");
     SimtPlan p{};
     if (!simt_plan(d, &p) || sizeof(float) * ((size_t)d.r3 * (d.r2 + 1) + 32 * (size_t)(d.r3 + 1) +
@@ -991,7 +1030,7 @@ int simt_expand_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, co
     a.ld2 = simt_ld2(d.n2);
     a.m2_ps = m2_ps; a.m3_ps = m3_ps;
     a.f = f;
-    a.w1 = c->f_w[0]; a.w2 = c->f_w[1]; a.w3 = c->f_w[2];
+    a.w1 = sh.w1; a.w2 = sh.w2; a.w3 = sh.w3;
     a.flags = flags; a.epart = epart;
     a.ty = p.ty; a.px = p.px; a.ny = p.ny; a.gc = p.gc; a.bc = p.bc; a.rows = p.rows;
     a.m2_flat = p.ny == 1;
@@ -1021,12 +1060,12 @@ int simt_expand_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, co
     }
 }
 
-int simt_adjoint_r(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, int flags, float* R,
-                   cudaStream_t s) {
-    const Dims d = dims_of(c);
+int simt_adjoint_r(const Shape& sh, const PairRec* recs, int p0, int np, const FieldArgs& f, int nt, const float* M2,
+                   const float* M3, int flags, float* R, cudaStream_t s) {
+    const Dims d = dims_of(sh);
     if (sizeof(float) * ((size_t)d.n2 * d.n3 + (size_t)d.n2 * d.r3) > 220 * 1024)
         return fail(TX_ERR_UNSUPPORTED_SHAPE, "float32 adjoint needs n2*(n3+r3) <= 56K");
-    return launch_chain(c, recs, p0, np, f, c->T, c->f_A[1], c->f_A[2], flags, R, true, "adjoint", s);
+    return launch_chain(sh, recs, p0, np, f, nt, M2, M3, flags, R, true, "adjoint", s);
 }
 
 int reduce_energy_batch(const double* epart, long count, double* dst, cudaStream_t s) {

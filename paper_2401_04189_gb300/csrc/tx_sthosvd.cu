@@ -296,7 +296,7 @@ int sthosvd_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, int p0, in
     }
     // ---- expansion with the per-pair operators, Hadamard epilogue
     TX_TRY(simt_expand_mode1_pp(c, G, A1, a1_ps, T, Z, np, s));
-    return simt_expand_consume(c, recs, p0, np, f, Z, T, A2, A3, EPI_OUT, epart, s, true, a2_ps, a3_ps);
+    return simt_expand_consume(fine_shape(c), recs, p0, np, f, Z, T, A2, A3, EPI_OUT, epart, s, true, a2_ps, a3_ps);
 }
 
 }  // namespace tx

@@ -68,32 +68,19 @@ __global__ void __launch_bounds__(32, 1) k_wait_selftest(int* err, int hold_tmem
     if (hold_tmem) tc::tmem_dealloc(tbase, 32);
 }
 
-// Z of the split precisions: the float32 first-mode product Zf[p][t][x][g][b] (b < r2) rounded
-// into the expansion's operand layout Z[p][t][(x, g)][ld_b] as hi + lo parts (lo after the
-// batch's hi part), with the b padding zero
-__global__ void k_split_z(const float* __restrict__ Zf, long rows, int r2, int ld_b, int tf32, void* Z, size_t lo_elems) {
-    const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (i >= rows * ld_b) return;
-    const long row = i / ld_b;
-    const int b = (int)(i - row * ld_b);
-    const float v = b < r2 ? Zf[row * r2 + b] : 0.f;
-    if (tf32) {
-        const float h = tc::tf32_hi(v);
-        ((float*)Z)[i] = h;
-        ((float*)Z)[i + lo_elems] = tc::tf32_hi(v - h);
-    } else {
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        ((__nv_bfloat16*)Z)[i] = h;
-        ((__nv_bfloat16*)Z)[i + lo_elems] = __float2bfloat16_rn(v - __bfloat162float(h));
-    }
-}
-
 }  // namespace
 
 int tc_wait_selftest(tx_ctx* c, int hold_tmem, cudaStream_t s) {
     k_wait_selftest<<<1, 32, 0, s>>>(c->d_err, hold_tmem ? 1 : 0);
     TX_LAUNCHED();
     return TX_OK;
+}
+
+// Gaussian terms the tensor-core operands hold: the split precisions sum the smooth terms on the
+// coarse grid in float32 and run only the sharp ones and the interpolation on the tensor cores.  The
+// single-pass precisions keep every term: their results are fixed by the rounding of each term's operands.
+int tc_terms(const tx_ctx* c) {
+    return (c->prec == TX_PREC_TF32X3 || c->prec == TX_PREC_BF16X3) ? c->ts.nf : c->T;
 }
 
 TcScratch tc_scratch(const tx_ctx* c) {
@@ -107,7 +94,7 @@ TcScratch tc_scratch(const tx_ctx* c) {
     s.s1 = r3 * n1 * s.ld_y;
     s.s2 = r3 * s.ld_b * s.ld_x;
     s.g = r3 * s.ld_b * s.ld_a;
-    s.z = (size_t)c->T * n1 * r3 * s.ld_b;
+    s.z = (size_t)tc_terms(c) * n1 * r3 * s.ld_b;
     return s;
 }
 
@@ -146,11 +133,13 @@ int tc_prepare(tx_ctx* c, cudaStream_t s) {
     op->tf32 = c->prec == TX_PREC_TF32 || c->prec == TX_PREC_TF32X3;
     op->split = c->prec == TX_PREC_TF32X3 || c->prec == TX_PREC_BF16X3;
     op->esize = op->tf32 ? 4 : 2;
-    const int n1 = c->n[0], n2 = c->n[1], n3 = c->n[2], r1 = c->r[0], r2 = c->r[1], r3 = c->r[2], T = c->T;
+    const int n1 = c->n[0], n2 = c->n[1], n3 = c->n[2], r1 = c->r[0], r2 = c->r[1], r3 = c->r[2], T = tc_terms(c);
+    double* const* A64 = op->split && c->ts.nc ? c->ts.F64 : c->d_A64;
     // every static operand row is K padded with zeros to a whole number of 32-byte sectors
     const int eb = op->esize;
     const size_t e_u3 = (size_t)r3 * ldk(n3, eb), e_u2 = (size_t)r2 * ldk(n2, eb), e_u1 = (size_t)r1 * ldk(n1, eb);
-    const size_t e_a1 = (size_t)T * n1 * ldk(r1, eb), e_a2 = (size_t)T * n2 * ldk(r2, eb);
+    // (the split forms run mode 1 of the expansion in float32)
+    const size_t e_a1 = op->split ? 0 : (size_t)T * n1 * ldk(r1, eb), e_a2 = (size_t)T * n2 * ldk(r2, eb);
     const size_t e_a3 = (size_t)T * n3 * ldk(r3, eb), e_a3f = (size_t)T * n3 * pad8(r3);
     const size_t e_a3t = (size_t)T * r3 * ldk(n3, eb), e_a2t = (size_t)T * r2 * ldk(n2, eb);
     auto al = [](size_t e) { return (e + 127) & ~(size_t)127; };   // 256-byte aligned pieces
@@ -194,19 +183,19 @@ int tc_prepare(tx_ctx* c, cudaStream_t s) {
     TX_TRY(conv(c->d_U[1], r2, n2, 1, r2, ldk(n2, eb), op->st.U2T));
     TX_TRY(conv(c->d_U[0], r1, n1, 1, r1, ldk(n1, eb), op->st.U1T));
     // A_td: [T][n_d][r_d] -> rows (t, x), K = r_d
-    TX_TRY(conv(c->d_A64[0], (long)T * n1, r1, r1, 1, ldk(r1, eb), op->st.A1s));
-    TX_TRY(conv(c->d_A64[1], (long)T * n2, r2, r2, 1, ldk(r2, eb), op->st.A2));
-    TX_TRY(conv(c->d_A64[2], (long)T * n3, r3, r3, 1, ldk(r3, eb), op->st.A3));
+    if (!op->split) TX_TRY(conv(A64[0], (long)T * n1, r1, r1, 1, ldk(r1, eb), op->st.A1s));
+    TX_TRY(conv(A64[1], (long)T * n2, r2, r2, 1, ldk(r2, eb), op->st.A2));
+    TX_TRY(conv(A64[2], (long)T * n3, r3, r3, 1, ldk(r3, eb), op->st.A3));
     // the adjoint's transposed operators, one term at a time: rows gamma (beta), K = z (y)
     for (int t = 0; t < T; ++t) {
-        TX_TRY(conv(c->d_A64[2] + (size_t)t * n3 * r3, r3, n3, 1, r3, ldk(n3, eb),
+        TX_TRY(conv(A64[2] + (size_t)t * n3 * r3, r3, n3, 1, r3, ldk(n3, eb),
                     (char*)op->st.A3T + (size_t)t * r3 * ldk(n3, eb) * op->esize));
-        TX_TRY(conv(c->d_A64[1] + (size_t)t * n2 * r2, r2, n2, 1, r2, ldk(n2, eb),
+        TX_TRY(conv(A64[1] + (size_t)t * n2 * r2, r2, n2, 1, r2, ldk(n2, eb),
                     (char*)op->st.A2T + (size_t)t * r2 * ldk(n2, eb) * op->esize));
     }
     if (a3f_extra) {
         const long n = (long)T * n3 * r3;
-        k_static_operand<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(c->d_A64[2], (long)T * n3, r3, r3, 1, pad8(r3), 1, 0,
+        k_static_operand<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(A64[2], (long)T * n3, r3, r3, 1, pad8(r3), 1, 0,
                                                                     op->st.A3f, 0);
         TX_LAUNCHED();
     }
@@ -214,13 +203,14 @@ int tc_prepare(tx_ctx* c, cudaStream_t s) {
     return TX_OK;
 }
 
-// float32 scratch of the split precisions' projection and first expansion mode (elements per pair)
+// float32 scratch of the split precisions (elements per pair): the projection's modes and the coarse
+// grid's first expansion mode
 struct SplitF32 {
     size_t s2, g, z;
 };
 static SplitF32 split_f32(const tx_ctx* c) {
     const size_t n1 = c->n[0], r1 = c->r[0], r2 = c->r[1], r3 = c->r[2];
-    return SplitF32{n1 * r3 * r2, r3 * r2 * r1, (size_t)c->T * n1 * r3 * r2};
+    return SplitF32{n1 * r3 * r2, r3 * r2 * r1, (size_t)c->ts.nc * r1 * r3 * r2};
 }
 
 size_t tc_adjoint_bytes_per_pair(const tx_ctx* c);
@@ -251,15 +241,21 @@ static int f32_mode1_project(const tx_ctx* c, const float* S2, float* G, int np,
     return simt_gemm(g, s);
 }
 
-// Zf[p][t][x][(g,b)] = sum_a A_t1[x][a] G[p][(g,b)][a]  (float32, mode 1 of the expansion, every term)
-static int f32_mode1_expand(const tx_ctx* c, const float* G, float* Z, int np, cudaStream_t s) {
-    const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2], T = c->T;
+// Z[p][t][(x,g)][b] (hi, and lo z elements behind) for nt fine terms from t0 on: mode 1 of the expansion in
+// float32, sum_a M1_t[x][a] G[p][(g,b)][a] (a_first: cores [a][(g,b)]), split as it leaves the
+// accumulators (the b padding is written as zeros).
+static int f32_mode1_expand(const tx_ctx* c, const float* G, bool a_first, int t0, int nt, void* Z, size_t lo, int np,
+                            cudaStream_t s) {
+    const TcOperands* op = c->tc;
+    const TcScratch sc = tc_scratch(c);
+    const int n1 = c->n[0], r1 = c->r[0], r2 = c->r[1], r3 = c->r[2], rr = r2 * r3;
     GemmArgs g{};
-    g.M = T * n1; g.N = rr; g.K = r1;
-    g.A = c->f_A[0]; g.a_m = r1; g.a_k = 1;
-    g.B = G; g.b_k = 1; g.b_n = r1; g.b_b2 = (long)rr * r1;
-    g.C = Z; g.c_m = rr; g.c_n = 1; g.c_b2 = (long)T * n1 * rr;
+    g.M = nt * n1; g.N = rr; g.K = r1;
+    g.A = c->ts.F[0] + (size_t)t0 * n1 * r1; g.a_m = r1; g.a_k = 1;
+    g.B = G; g.b_k = a_first ? rr : 1; g.b_n = a_first ? 1 : r1; g.b_b2 = (long)rr * r1;
+    g.C = (float*)((char*)Z + (size_t)t0 * n1 * r3 * sc.ld_b * op->esize); g.c_m = (long)r3 * sc.ld_b; g.c_b2 = (long)sc.z;
     g.nb1 = 1; g.nb2 = np; g.alpha = 1.f;
+    g.split = op->tf32 ? 1 : 2; g.nb = r2; g.ld_b = sc.ld_b; g.c_lo = (long)lo;
     return simt_gemm(g, s);
 }
 
@@ -277,27 +273,37 @@ static int tc_forward(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, con
     const int eb = op->esize;
     const int n1 = c->n[0], n2 = c->n[1], r1 = c->r[0], r2 = c->r[1], r3 = c->r[2], T = c->T;
     if (op->split) {
-        // Split precisions: the projection onto the core and the first expansion mode run in
-        // float32 on the CUDA cores (13% of the flops on the Pt-shaped block), so that the core
-        // and Z carry full float32 precision into the hi + lo split; modes 2 and 3 and the sum
-        // over terms run on the tensor cores (tc_consume).
+        // Split precisions: the projection onto the core, the smooth terms on the coarse grid and the
+        // first expansion mode run in float32 on the CUDA cores, so that the core and Z carry full
+        // float32 precision into the hi + lo split; modes 2 and 3 and the sum over the fine terms run
+        // on the tensor cores (tc_consume).
+        const TermSplit& ts = c->ts;
         const SplitF32 f = split_f32(c);
         float* S2f = (float*)b.scratch;
         float* Gf = S2f + (size_t)np * f.s2;
-        float* Zf = Gf + (size_t)np * f.g;
-        char* Z = (char*)(Zf + (size_t)np * f.z);
+        float* Zc = Gf + (size_t)np * f.g;
+        char* Z = (char*)(Zc + (size_t)np * f.z);
         Z = (char*)(((uintptr_t)Z + 255) & ~(uintptr_t)255);
         FieldArgs fa{};
         fa.SA = SA;
         fa.SB = SB;
         TX_TRY(simt_project_s2(c, recs, b.p0, np, fa, 0, S2f, s, false));
         TX_TRY(f32_mode1_project(c, S2f, Gf, np, s));
-        TX_TRY(f32_mode1_expand(c, Gf, Zf, np, s));
-        const long rows = (long)np * T * n1 * r3;
-        const long nz = rows * sc.ld_b;
-        k_split_z<<<(unsigned)((nz + 255) / 256), 256, 0, s>>>(Zf, rows, r2, sc.ld_b, op->tf32 ? 1 : 0, Z,
-                                                              (size_t)np * sc.z);
-        TX_LAUNCHED();
+        const size_t lo = (size_t)np * sc.z;
+        if (ts.nc) {
+            // H[p][a][(g,b)] = sum over the smooth terms of G x_d Q_td; the cores are [g][b], so modes 2
+            // and 3 take each other's place
+            float* H = S2f;
+            TX_TRY(simt_expand_mode1_grid(c, Gf, ts.Q[0], c->r[0], ts.nc, Zc, np, s));
+            FieldArgs fc{};
+            fc.OUT0 = H;
+            TX_TRY(simt_expand_consume(coarse_shape(c, true), nullptr, 0, np, fc, Zc, ts.nc, ts.QKs[2], ts.QKs[1], EPI_STORE,
+                                       nullptr, s));
+            if (ts.nf > 1) TX_TRY(f32_mode1_expand(c, Gf, false, 0, ts.nf - 1, Z, lo, np, s));
+            TX_TRY(f32_mode1_expand(c, H, true, ts.nf - 1, 1, Z, lo, np, s));
+        } else {
+            TX_TRY(f32_mode1_expand(c, Gf, false, 0, ts.nf, Z, lo, np, s));
+        }
         return tc_consume(c, recs, b.p0, np, Z, SA, SB, MUL0, MUL1, OUT0, OUT1, cnt, flags, b.epart, s, subset);
     }
     char* S1 = b.scratch;
@@ -355,7 +361,8 @@ struct AdjF32 {
 };
 static AdjF32 adj_f32(const tx_ctx* c) {
     const size_t n1 = c->n[0], r1 = c->r[0], rr = (size_t)c->r[1] * c->r[2];
-    return AdjF32{(size_t)c->T * n1 * rr, rr * r1, n1 * rr};
+    const size_t coarse = c->tc->split ? (size_t)c->ts.nc * r1 * rr : 0;
+    return AdjF32{std::max((size_t)tc_terms(c) * n1 * rr, coarse), rr * r1, n1 * rr};
 }
 
 // The adjoint of one pair batch (derived; the paper has no gradient): with L = sum_t mu_t
@@ -371,15 +378,13 @@ static int tc_adjoint(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, con
     const TcScratch sc = tc_scratch(c);
     const int np = b.np;
     const int eb = op->esize, mult = op->split ? 2 : 1;
-    const int n1 = c->n[0], n2 = c->n[1], n3 = c->n[2], r2 = c->r[1], r3 = c->r[2], T = c->T;
+    const int n1 = c->n[0], n2 = c->n[1], n3 = c->n[2], r2 = c->r[1], r3 = c->r[2], T = tc_terms(c);
     const long rr = (long)r2 * r3;
     const AdjF32 f = adj_f32(c);
     char* S1 = b.scratch;
     float* R = (float*)(((uintptr_t)(S1 + (size_t)np * sc.s1 * eb * mult) + 255) & ~(uintptr_t)255);
     float* H = R + (size_t)np * f.r;
     float* Z = H + (size_t)np * f.h;
-    const int out_type = op->tf32 ? (op->split ? TC_OUT_F32_SPLIT : TC_OUT_F32) : (op->split ? TC_OUT_BF16_SPLIT : TC_OUT_BF16);
-    (void)out_type;
     for (int t = 0; t < T; ++t) {
         // S1[p][g][x][y] = sum_z y_p[x][y][z] (mu_t A_t3)[z][g]
         const char* a3t = (const char*)op->st.A3T + (size_t)t * r3 * ldk(n3, eb) * eb;
@@ -393,13 +398,18 @@ static int tc_adjoint(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, con
         TcGemmArgs g{};
         g.M = r3 * n1; g.N = r2; g.K = n2; g.nb1 = np; g.nb2 = 1;
         g.a_z1 = 1;
-        g.C = R + (size_t)t * n1 * rr; g.rdiv = n1; g.c_mh = r2; g.c_m = rr; g.c_n = 1; g.c_b1 = (long)f.r;
+        g.C = R + (size_t)t * n1 * rr; g.rdiv = n1; g.c_mh = r2; g.c_m = rr; g.c_n = 1; g.c_b1 = (long)T * n1 * rr;
         g.c_type = TC_OUT_F32; g.alpha = 1.f; g.err = c->d_err;
         TX_TRY(tc_gemm_launch(A, B, g, op->tf32, op->split, "tc_adj2", s));
     }
-    TX_TRY(simt_adjoint_mode1(c, R, H, np, s));                  // H = sum_{t,x} R A_t1
+    if (op->split && c->ts.nc) {
+        // sharp terms from R, the smooth ones through the coarse grid (Z is free until the expansion)
+        TX_TRY(simt_adjoint_split(c, R, Z, H, np, s));
+    } else {
+        TX_TRY(simt_adjoint_mode1(c, R, H, np, s));              // H = sum_{t,x} R A_t1
+    }
     TX_TRY(simt_expand_mode1(c, H, c->f_U[0], 1, Z, np, s));     // Z = U1 H
-    return simt_expand_consume(c, recs, b.p0, np, fo, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, b.epart, s, false);
+    return simt_expand_consume(fine_shape(c), recs, b.p0, np, fo, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, b.epart, s, false);
 }
 
 size_t tc_adjoint_bytes_per_pair(const tx_ctx* c) {

@@ -2787,7 +2787,7 @@ int tc_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const void*
     const TcOperands* op = c->tc;
     ConsumePlan p;
     if (!choose_plan(c, op->tf32, op->split, &p)) return fail(TX_ERR_UNSUPPORTED_SHAPE, "no expansion tile plan");
-    const int n1 = c->n[0], n2 = c->n[1], n3 = c->n[2], r2 = c->r[1], r3 = c->r[2], T = c->T;
+    const int n1 = c->n[0], n2 = c->n[1], n3 = c->n[2], r2 = c->r[1], r3 = c->r[2], T = tc_terms(c);
     const TcScratch sc = tc_scratch(c);
     const int m = op->split ? 2 : 1;
     tcc::ConsumeArgs a{};

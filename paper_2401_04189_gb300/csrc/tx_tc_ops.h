@@ -47,6 +47,7 @@ struct TcScratch {
     int ld_y, ld_x, ld_a, ld_b;
 };
 TcScratch tc_scratch(const tx_ctx* c);
+int tc_terms(const tx_ctx* c);   // Gaussian terms of the tensor-core operands
 
 // S1 = (SA * SB (* w)) x3 B^T with B the operand U3^T (forward projection, Bhi NULL) or a term's
 // mu_t A_t3^T (the adjoint's first mode)
