@@ -23,56 +23,151 @@
 namespace tx {
 namespace {
 
-constexpr int kGramTile = 16;     // 16 x 16 (i, j) outputs per CTA
-constexpr int kGramChunk = 32;    // grid points per shared-memory chunk
+constexpr int kGramChunk = 64;    // grid points per shared-memory chunk
+constexpr int kGramLd = kGramChunk + 4;
 
-// partial[s][i][j] = sum over slice s of the grid of w(x) A_i(x) B_j(x): float32 within a chunk
-// of 32 points, float64 across chunks
-__global__ void __launch_bounds__(256) k_wgram(const float* __restrict__ A, int na, const float* __restrict__ B, int nb,
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool ok) {
+    const int bytes = ok ? 16 : 0;       // 0: the 16 bytes are zero-filled and src is not read
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(bytes)
+                 : "memory");
+}
+
+// partial[s][i][j] = sum over slice s of the grid of w(x) A_i(x) B_j(x): float32 within a chunk of 64
+// points (two sums of 32), and across chunks a compensated float32 sum (Kahan; a pair of floats
+// carries 48 bits), as this GPU adds float64 at 1/64 of the float32 rate.  BI x BJ outputs per CTA
+// of 128 threads (8 x 16), (BI / 8) x (BJ / 16) each.  The orbitals keep their own layout in shared
+// memory (rows along the grid, stride 68: the 16-byte reads of 16 rows hit different banks) and the
+// packed multiply-adds run along the grid, so nothing is transposed or duplicated; two buffers, filled
+// by cp.async.  64 x 64 orbitals of 96^3: 245 us; 317 with 4 x 4 outputs per thread and chunks of
+// 32, 1554 with one output per thread and a float64 add per chunk (the orbitals take 67 us of HBM time).
+template <int BI, int BJ>
+__global__ void __launch_bounds__(128) k_wgram(const float* __restrict__ A, int na, const float* __restrict__ B, int nb,
                                                const float* __restrict__ w1, const float* __restrict__ w2,
-                                               const float* __restrict__ w3, int n1, int n2, int n3, long slice,
+                                               const float* __restrict__ w3, int n1, int n2, int n3, long slice, int vec,
                                                double* __restrict__ partial) {
-    __shared__ float As[kGramTile][kGramChunk + 1], Bs[kGramTile][kGramChunk + 1], ws[kGramChunk];
+    constexpr int TI = BI / 8, TJ = BJ / 16;
+    extern __shared__ __align__(16) float sm[];
+    constexpr int kBuf = (BI + BJ) * kGramLd + kGramChunk;      // A rows, B rows, weights
     const long N3 = (long)n1 * n2 * n3, N23 = (long)n2 * n3;
-    const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
-    const int i0 = blockIdx.x * kGramTile, j0 = blockIdx.y * kGramTile;
+    const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
+    const int i0 = blockIdx.x * BI, j0 = blockIdx.y * BJ;
     const long x0 = (long)blockIdx.z * slice, x1 = min(N3, x0 + slice);
-    double acc = 0.0;
-    for (long xc = x0; xc < x1; xc += kGramChunk) {
-        for (int e = threadIdx.x; e < kGramTile * kGramChunk; e += 256) {
-            const int r = e / kGramChunk, k = e - r * kGramChunk;
-            const long x = xc + k;
-            const bool in = x < x1;
-            As[r][k] = (in && i0 + r < na) ? A[(long)(i0 + r) * N3 + x] : 0.f;
-            Bs[r][k] = (in && j0 + r < nb) ? B[(long)(j0 + r) * N3 + x] : 0.f;
+    auto load = [&](long xc, int buf) {
+        float* As = sm + buf * kBuf;
+        float* Bs = As + BI * kGramLd;
+        if (vec) {
+            for (int e = tid; e < BI * (kGramChunk / 4); e += 128) {
+                const int r = e / (kGramChunk / 4), q = 4 * (e % (kGramChunk / 4));
+                const bool ok = i0 + r < na && xc + q < x1;
+                cp_async16(As + r * kGramLd + q, ok ? A + (long)(i0 + r) * N3 + xc + q : A, ok);
+            }
+            for (int e = tid; e < BJ * (kGramChunk / 4); e += 128) {
+                const int r = e / (kGramChunk / 4), q = 4 * (e % (kGramChunk / 4));
+                const bool ok = j0 + r < nb && xc + q < x1;
+                cp_async16(Bs + r * kGramLd + q, ok ? B + (long)(j0 + r) * N3 + xc + q : B, ok);
+            }
+        } else {
+            for (int e = tid; e < BI * kGramChunk; e += 128) {
+                const int r = e / kGramChunk, q = e % kGramChunk;
+                As[r * kGramLd + q] = (i0 + r < na && xc + q < x1) ? A[(long)(i0 + r) * N3 + xc + q] : 0.f;
+            }
+            for (int e = tid; e < BJ * kGramChunk; e += 128) {
+                const int r = e / kGramChunk, q = e % kGramChunk;
+                Bs[r * kGramLd + q] = (j0 + r < nb && xc + q < x1) ? B[(long)(j0 + r) * N3 + xc + q] : 0.f;
+            }
         }
-        if (threadIdx.x < kGramChunk) {
-            const long x = xc + threadIdx.x;
+        if (tid < kGramChunk) {
+            const long x = xc + tid;
             float wv = 0.f;
             if (x < x1) {
                 const int a = (int)(x / N23), yz = (int)(x - a * N23), b = yz / n3, c = yz - b * n3;
                 wv = w1[a] * w2[b] * w3[c];
             }
-            ws[threadIdx.x] = wv;
+            Bs[BJ * kGramLd + tid] = wv;
         }
-        __syncthreads();
-        float f = 0.f;
-#pragma unroll 8
-        for (int k = 0; k < kGramChunk; ++k) f += ws[k] * As[ti][k] * Bs[tj][k];
-        acc += (double)f;
-        __syncthreads();
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float sum[TI][TJ], comp[TI][TJ];
+#pragma unroll
+    for (int i = 0; i < TI; ++i)
+#pragma unroll
+        for (int j = 0; j < TJ; ++j) sum[i][j] = comp[i][j] = 0.f;
+    if (x0 < x1) load(x0, 0);
+    int buf = 0;
+    for (long xc = x0; xc < x1; xc += kGramChunk, buf ^= 1) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();                 // this chunk has landed; the other buffer has been read
+        if (xc + kGramChunk < x1) load(xc + kGramChunk, buf ^ 1);
+        const float* As = sm + buf * kBuf;
+        const float* Bs = As + BI * kGramLd;
+        const float* ws = Bs + BJ * kGramLd;
+        uint64_t acc[TI][TJ];
+#pragma unroll
+        for (int i = 0; i < TI; ++i)
+#pragma unroll
+            for (int j = 0; j < TJ; ++j) acc[i][j] = 0ull;
+#pragma unroll 4
+        for (int k = 0; k < kGramChunk; k += 4) {
+            const ulonglong2 w = *(const ulonglong2*)(ws + k);
+            ulonglong2 a[TI], b[TJ];
+#pragma unroll
+            for (int j = 0; j < TJ; ++j) {
+                const ulonglong2 v = *(const ulonglong2*)(Bs + (tj + 16 * j) * kGramLd + k);
+                b[j] = make_ulonglong2(mul2(v.x, w.x), mul2(v.y, w.y));
+            }
+#pragma unroll
+            for (int i = 0; i < TI; ++i) a[i] = *(const ulonglong2*)(As + (ti + 8 * i) * kGramLd + k);
+#pragma unroll
+            for (int i = 0; i < TI; ++i)
+#pragma unroll
+                for (int j = 0; j < TJ; ++j) {
+                    fma2(acc[i][j], a[i].x, b[j].x);
+                    fma2(acc[i][j], a[i].y, b[j].y);
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < TI; ++i)
+#pragma unroll
+            for (int j = 0; j < TJ; ++j) {
+                const float f = __uint_as_float((uint32_t)acc[i][j]) + __uint_as_float((uint32_t)(acc[i][j] >> 32));
+                const float y = f - comp[i][j], t = sum[i][j] + y;
+                const float r = (t - sum[i][j]) - y;
+                comp[i][j] = fabsf(r) < INFINITY ? r : 0.f;      // an infinite sum stays infinite
+                sum[i][j] = t;
+            }
     }
-    const int i = i0 + ti, j = j0 + tj;
-    if (i < na && j < nb) partial[((long)blockIdx.z * na + i) * nb + j] = acc;
+#pragma unroll
+    for (int i = 0; i < TI; ++i)
+#pragma unroll
+        for (int j = 0; j < TJ; ++j) {
+            const int r = i0 + ti + 8 * i, c = j0 + tj + 16 * j;
+            if (r < na && c < nb) partial[((long)blockIdx.z * na + r) * nb + c] = (double)sum[i][j] - (double)comp[i][j];
+        }
 }
 
-// G[i][j] = sum_s partial[s][i][j] (fixed order), and optionally its transpose in float32 scaled
-__global__ void k_gram_reduce(const double* __restrict__ partial, int ns, int na, int nb, double* __restrict__ G,
-                              float* __restrict__ GTf, float scale) {
-    const long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (idx >= (long)na * nb) return;
+// G[i][j] = sum_s partial[s][i][j] (fixed order: 8 interleaved sums, then their sum), and
+// optionally its transpose in float32 scaled.  32 outputs x 8 slice groups per CTA.
+__global__ void __launch_bounds__(256) k_gram_reduce(const double* __restrict__ partial, int ns, int na, int nb,
+                                                     double* __restrict__ G, float* __restrict__ GTf, float scale) {
+    __shared__ double red[8][33];
+    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const long cnt = (long)na * nb, idx = blockIdx.x * 32L + lane;
     double s = 0.0;
-    for (int k = 0; k < ns; ++k) s += partial[(long)k * na * nb + idx];
+    if (idx < cnt)
+        for (int k = grp; k < ns; k += 8) s += partial[(long)k * cnt + idx];
+    red[grp][lane] = s;
+    __syncthreads();
+    if (grp || idx >= cnt) return;
+    for (int g = 1; g < 8; ++g) s += red[g][lane];
     if (G) G[idx] = s;
     if (GTf) {
         const int i = (int)(idx / nb), j = (int)(idx - (long)i * nb);
@@ -137,70 +232,69 @@ __global__ void __launch_bounds__(1024) k_ace_factor(const double* __restrict__ 
     if (threadIdx.x == 0) flag[0] = 0;
 }
 
-constexpr int kMixK = 32;     // output orbitals per CTA
-constexpr int kMixI = 32;     // input orbitals per shared-memory tile
-
-// out[k][x] = alpha * sum_i C[k][i] X[i][x]  (C float32 [nk][ni], X float32 [ni][N3])
-__global__ void __launch_bounds__(256) k_mix(const float* __restrict__ C, int nk, int ni, const float* __restrict__ X,
-                                             long N3, float alpha, float* __restrict__ out) {
-    __shared__ float Cs[kMixK][kMixI];
-    const long x = blockIdx.x * 256L + threadIdx.x;
-    const int k0 = blockIdx.y * kMixK;
-    float acc[kMixK];
-#pragma unroll
-    for (int k = 0; k < kMixK; ++k) acc[k] = 0.f;
-    for (int i0 = 0; i0 < ni; i0 += kMixI) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < kMixK * kMixI; e += 256) {
-            const int k = e / kMixI, i = e - k * kMixI;
-            Cs[k][i] = (k0 + k < nk && i0 + i < ni) ? C[(long)(k0 + k) * ni + i0 + i] : 0.f;
-        }
-        __syncthreads();
-        if (x < N3) {
-            const int iend = min(kMixI, ni - i0);
-            for (int i = 0; i < iend; ++i) {
-                const float v = X[(long)(i0 + i) * N3 + x];
-#pragma unroll
-                for (int k = 0; k < kMixK; ++k) acc[k] += Cs[k][i] * v;
-            }
-        }
-    }
-    if (x < N3)
-#pragma unroll
-        for (int k = 0; k < kMixK; ++k)
-            if (k0 + k < nk) out[(long)(k0 + k) * N3 + x] = alpha * acc[k];
-}
-
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+
+// output tile of the Gram kernel along one side: the block size padded least
+int gram_tile(int n) { return n <= 16 ? 16 : (n <= 32 ? 32 : 64); }
+
+// grid slices of the Gram kernel: as many CTAs as the GPU holds at once, of at least 1024 points (and
+// whole chunks) each
+int gram_slices(long N3, int na, int nb) {
+    const int bi = gram_tile(na), bj = gram_tile(nb);
+    const long tiles = (long)((na + bi - 1) / bi) * ((nb + bj - 1) / bj);
+    const long per_sm = bi * bj >= 64 * 64 ? 2 : 4;
+    const long want = std::max<long>(1, (per_sm * 152 + tiles - 1) / tiles);
+    return (int)std::min<long>(want, std::max<long>(1, N3 / 1024));
+}
 
 // weighted Gram matrix of A (na orbitals) and B (nb orbitals) into G (float64 [na][nb]) and/or
 // the scaled float32 transpose GTf [nb][na]; partials in `scratch`
 int wgram(const tx_ctx* c, const float* A, int na, const float* B, int nb, double* partial, int ns, double* G,
           float* GTf, float scale, cudaStream_t s) {
     const long N3 = (long)c->n[0] * c->n[1] * c->n[2];
-    const long slice = (N3 + ns - 1) / ns;
-    dim3 grid((unsigned)((na + kGramTile - 1) / kGramTile), (unsigned)((nb + kGramTile - 1) / kGramTile), (unsigned)ns);
-    k_wgram<<<grid, 256, 0, s>>>(A, na, B, nb, c->f_w[0], c->f_w[1], c->f_w[2], c->n[0], c->n[1], c->n[2], slice,
-                                 partial);
+    const long slice = ((N3 + ns - 1) / ns + kGramChunk - 1) / kGramChunk * kGramChunk;
+    const int bi = gram_tile(na), bj = gram_tile(nb);
+    const dim3 grid((unsigned)((na + bi - 1) / bi), (unsigned)((nb + bj - 1) / bj), (unsigned)ns);
+    const int vec = c->n[2] % 4 == 0 && (((uintptr_t)A | (uintptr_t)B) & 15u) == 0;
+    const size_t smem = sizeof(float) * 2 * ((bi + bj) * kGramLd + kGramChunk);
+#define TX_GRAM(BI_, BJ_)                                                                                              \
+    if (bi == BI_ && bj == BJ_) {                                                                                      \
+        if (smem > 48 * 1024)                                                                                          \
+            TX_TRY_CUDA(cudaFuncSetAttribute(k_wgram<BI_, BJ_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+        k_wgram<BI_, BJ_><<<grid, 128, smem, s>>>(A, na, B, nb, c->f_w[0], c->f_w[1], c->f_w[2], c->n[0], c->n[1],      \
+                                                  c->n[2], slice, vec, partial);                                       \
+    }
+    TX_GRAM(16, 16);
+    TX_GRAM(16, 32);
+    TX_GRAM(16, 64);
+    TX_GRAM(32, 16);
+    TX_GRAM(32, 32);
+    TX_GRAM(32, 64);
+    TX_GRAM(64, 16);
+    TX_GRAM(64, 32);
+    TX_GRAM(64, 64);
+#undef TX_GRAM
     TX_LAUNCHED();
     const long cnt = (long)na * nb;
-    k_gram_reduce<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(partial, ns, na, nb, G, GTf, scale);
+    k_gram_reduce<<<(unsigned)((cnt + 31) / 32), 256, 0, s>>>(partial, ns, na, nb, G, GTf, scale);
     TX_LAUNCHED();
     return TX_OK;
 }
 
+// out[k][x] = alpha * sum_i C[k][i] X[i][x]  (C float32 [nk][ni], X float32 [ni][N3])
 int mix(const float* C, int nk, int ni, const float* X, long N3, float alpha, float* out, cudaStream_t s) {
-    dim3 grid((unsigned)((N3 + 255) / 256), (unsigned)((nk + kMixK - 1) / kMixK));
-    k_mix<<<grid, 256, 0, s>>>(C, nk, ni, X, N3, alpha, out);
-    TX_LAUNCHED();
+    // the GEMM's column index is an int: blocks of grid points on very large grids
+    const long block = 1L << 30;
+    for (long x = 0; x < N3; x += block) {
+        GemmArgs g{};
+        g.M = nk; g.N = (int)std::min(block, N3 - x); g.K = ni;
+        g.A = C; g.a_m = ni; g.a_k = 1;
+        g.B = X + x; g.b_k = N3; g.b_n = 1;
+        g.C = out + x; g.c_m = N3; g.c_n = 1;
+        g.nb1 = g.nb2 = 1; g.alpha = alpha;
+        TX_TRY(simt_gemm(g, s));
+    }
     return TX_OK;
-}
-
-// grid slices of the Gram kernel: enough CTAs to fill the GPU a few times over
-int gram_slices(long N3, int na, int nb) {
-    const long tiles = (long)((na + kGramTile - 1) / kGramTile) * ((nb + kGramTile - 1) / kGramTile);
-    const long want = std::max<long>(1, (4L * 152 + tiles - 1) / tiles);
-    return (int)std::min<long>(want, std::max<long>(1, N3 / 4096));
 }
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
