@@ -170,6 +170,7 @@ static void free_ctx(tx_ctx* c) {
         cudaFree(c->d_x[d]);
         cudaFree(c->d_w[d]);
         cudaFree(c->d_U[d]);
+        cudaFree(c->d_UW[d]);
         cudaFree(c->d_A64[d]);
         cudaFree(c->f_U[d]);
         cudaFree(c->f_A[d]);
@@ -240,6 +241,7 @@ extern "C" int tx_tucker_setup(tx_ctx** out, const int n[3], const double* x1, c
         SETUP_TRY(dalloc(&c->d_x[d], nd));
         SETUP_TRY(dalloc(&c->d_w[d], nd));
         SETUP_TRY(dalloc(&c->d_U[d], nd * rd));
+        SETUP_TRY(dalloc(&c->d_UW[d], nd * rd));
         SETUP_TRY(dalloc(&c->d_A64[d], (size_t)T * nd * rd));
         SETUP_TRY(dalloc(&c->f_U[d], nd * rd));
         SETUP_TRY(dalloc(&c->f_A[d], (size_t)T * nd * rd));
@@ -249,11 +251,16 @@ extern "C" int tx_tucker_setup(tx_ctx** out, const int n[3], const double* x1, c
         SETUP_TRY(dalloc(&c->f_w[d], nd));
         // host float32 copies are made synchronously (the host arrays may be freed on return)
         std::vector<float> fu(nd * rd), fw(nd);
-        for (size_t i = 0; i < nd * rd; ++i) fu[i] = (float)Us[d][i];
+        std::vector<double> uw(nd * rd);
+        for (size_t i = 0; i < nd * rd; ++i) {
+            fu[i] = (float)Us[d][i];
+            uw[i] = Us[d][i] * ws[d][i / rd];
+        }
         for (size_t i = 0; i < nd; ++i) fw[i] = (float)ws[d][i];
         if (cudaMemcpy(c->d_x[d], xs[d], sizeof(double) * nd, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(c->d_w[d], ws[d], sizeof(double) * nd, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(c->d_U[d], Us[d], sizeof(double) * nd * rd, cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemcpy(c->d_UW[d], uw.data(), sizeof(double) * nd * rd, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(c->f_U[d], fu.data(), sizeof(float) * nd * rd, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(c->f_w[d], fw.data(), sizeof(float) * nd, cudaMemcpyHostToDevice) != cudaSuccess)
             SETUP_TRY(fail(TX_ERR_CUDA, "set-up copy failed"));

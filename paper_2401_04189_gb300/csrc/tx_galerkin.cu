@@ -17,48 +17,52 @@
 namespace tx {
 namespace {
 
+struct OperatorArgs {
+    const double* UW[3];       // U_d[a][i] w_d[a]
+    const double* U[3];
+    const double* w[3];
+    const double* A64[3];
+    float* B[3];
+    float* Ut[3];
+    int n[3], r[3], ldb[3], ldu[3];
+    int T;
+};
+
 // B_td[i][k] = sum_a U_d[a][i] w_d[a] A_td[a][k]  (mu_t is already folded into A_t3), and
-// Ut_d[a][k] = U_d[a][k] / w_d[a] (modes 2 and 3, ldk > 0: stored [k][a] with row stride ldk, as the
-// consumer reads it).  One thread per output element, float64 sums.
-__global__ void k_galerkin_operators(const double* __restrict__ U, const double* __restrict__ w,
-                                     const double* __restrict__ A64, int n, int r, int T, int ldk,
-                                     float* __restrict__ B, float* __restrict__ Ut) {
+// Ut_d[a][k] = U_d[a][k] / w_d[a].  Modes 2 and 3 (ldb, ldu > 0) are stored [k][i] and [k][a] with those
+// row strides, as the consumer reads them.  blockIdx.y is the mode; one thread per output element,
+// float64 sums: bound by float64 multiply-adds, one per point (w_d is folded into U_d at set-up).
+__global__ void k_galerkin_operators(const OperatorArgs o) {
+    const int d = blockIdx.y, n = o.n[d], r = o.r[d];
     const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long nb = (long)T * r * r;
+    const long nb = (long)o.T * r * r;
     if (e < nb) {
         const int t = (int)(e / ((long)r * r)), i = (int)((e / r) % r), k = (int)(e % r);
-        const double* At = A64 + (long)t * n * r;
+        const double* At = o.A64[d] + (long)t * n * r;
+        const double* UW = o.UW[d];
         double s = 0.0;
-        for (int a = 0; a < n; ++a) s = fma(U[(long)a * r + i] * w[a], At[(long)a * r + k], s);
-        B[e] = (float)s;
+        for (int a = 0; a < n; ++a) s = fma(UW[(long)a * r + i], At[(long)a * r + k], s);
+        o.B[d][o.ldb[d] ? ((long)t * r + k) * o.ldb[d] + i : e] = (float)s;
     } else if (e < nb + (long)n * r) {
         const long q = e - nb;
         const long a = q / r, k = q - a * r;
-        Ut[ldk ? k * ldk + a : q] = (float)(U[q] / w[a]);
+        o.Ut[d][o.ldu[d] ? k * o.ldu[d] + a : q] = (float)(o.U[d][q] / o.w[d][a]);
     }
 }
 
-// H[p][e] = sum_t X[p][t][e]
-__global__ void k_sum_terms(const float* __restrict__ X, int T, long m, int np, float* __restrict__ H) {
-    const long total = (long)np * m;
-    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (long)gridDim.x * blockDim.x) {
-        const long p = q / m, e = q % m;
-        const float* x = X + (long)p * T * m + e;
-        float s = 0.f;
-        for (int t = 0; t < T; ++t) s += x[(long)t * m];
-        H[q] = s;
-    }
-}
-
-// epart[p] = ew_p * sum_e G[p][e] H[p][e]   (float64 sum; one block per pair)
+// epart[p] = ew_p * <G_p, H_p> with G [(b,g)][a] and H [a][(b,g)]  (float64 sum; one block per pair)
 __global__ void __launch_bounds__(256) k_core_dot(const PairRec* __restrict__ recs, int p0, const float* __restrict__ G,
-                                                  const float* __restrict__ H, long m, double* __restrict__ epart) {
+                                                  const float* __restrict__ H, int r1, long rr, double* __restrict__ epart) {
     __shared__ double red[256];
     const int p = blockIdx.x;
+    const long m = r1 * rr;
     const float* g = G + (long)p * m;
     const float* h = H + (long)p * m;
     double s = 0.0;
-    for (long e = threadIdx.x; e < m; e += blockDim.x) s += (double)g[e] * (double)h[e];
+    for (long e = threadIdx.x; e < m; e += blockDim.x) {
+        const long q = e / r1, a = e - q * r1;
+        s += (double)g[e] * (double)h[a * rr + q];
+    }
     red[threadIdx.x] = s;
     __syncthreads();
     for (int k = 128; k > 0; k >>= 1) {
@@ -68,69 +72,53 @@ __global__ void __launch_bounds__(256) k_core_dot(const PairRec* __restrict__ re
     if (threadIdx.x == 0) epart[p] = red[0] * (double)recs[p0 + p].ew;
 }
 
+int ldb_of(const tx_ctx* c, int d) { return d == 0 ? 0 : d == 1 ? simt_ld2(c->r[1]) : simt_ld3(c->r[2]); }
+int ldu_of(const tx_ctx* c, int d) { return d == 0 ? 0 : d == 1 ? simt_ld2(c->n[1]) : simt_ld3(c->n[2]); }
+size_t b_floats(const tx_ctx* c, int d) { return (size_t)pad4(c->T * c->r[d] * (d ? ldb_of(c, d) : c->r[d])); }
+size_t ut_floats(const tx_ctx* c, int d) { return (size_t)pad4(c->r[d] * (d ? ldu_of(c, d) : c->n[d])); }
+
 }  // namespace
 
 size_t galerkin_operator_floats(const tx_ctx* c) {
     size_t f = 0;
-    for (int d = 0; d < 3; ++d) f += pad4(c->T * c->r[d] * c->r[d]) + (size_t)std::max(simt_ld2(c->n[d]), simt_ld3(c->n[d])) * c->r[d];
+    for (int d = 0; d < 3; ++d) f += b_floats(c, d) + ut_floats(c, d);
     return f;
 }
 
 int galerkin_operators(const tx_ctx* c, float* ops, GalerkinOps* g, cudaStream_t s) {
+    OperatorArgs o{};
     float* q = ops;
+    long most = 0;
     for (int d = 0; d < 3; ++d) {
-        const int n = c->n[d], r = c->r[d];
-        float* B = q;
-        float* Ut = B + pad4(c->T * r * r);
-        q = Ut + (size_t)std::max(simt_ld2(n), simt_ld3(n)) * r;
-        g->B[d] = B;
-        g->Ut[d] = Ut;
-        const long total = (long)c->T * r * r + (long)n * r;
-        k_galerkin_operators<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(c->d_U[d], c->d_w[d], c->d_A64[d], n, r,
-                                                                            c->T, d == 0 ? 0 : d == 1 ? simt_ld2(n) : simt_ld3(n), B, Ut);
-        TX_LAUNCHED();
+        o.B[d] = q;
+        o.Ut[d] = q + b_floats(c, d);
+        q = o.Ut[d] + ut_floats(c, d);
+        g->B[d] = o.B[d];
+        g->Ut[d] = o.Ut[d];
+        o.UW[d] = c->d_UW[d]; o.U[d] = c->d_U[d]; o.w[d] = c->d_w[d]; o.A64[d] = c->d_A64[d];
+        o.n[d] = c->n[d]; o.r[d] = c->r[d]; o.ldb[d] = ldb_of(c, d); o.ldu[d] = ldu_of(c, d);
+        most = std::max(most, (long)c->T * c->r[d] * c->r[d] + (long)c->n[d] * c->r[d]);
     }
-    return TX_OK;
-}
-
-// H[p] = sum_t G[p] x1 B_t1 x2 B_t2 x3 B_t3, three batched GEMM passes over all terms.  Each pass
-// contracts the fastest index of its input and writes the new index slowest, so the layout
-// turns [b][g][a] -> [a'][b][g] -> [g'][a'][b] -> [b'][g'][a'] (back to G's own order).
-int galerkin_core(const tx_ctx* c, const GalerkinOps& o, const float* G, float* X1, float* X2, float* H, int np,
-                  cudaStream_t s) {
-    const int r1 = c->r[0], r2 = c->r[1], r3 = c->r[2], T = c->T;
-    const long m = (long)r1 * r2 * r3;
-    GemmArgs g{};
-    g.nb1 = T; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
-    // mode 1: X1[p][t][a'][(b,g)] = sum_a B_t1[a'][a] G[p][(b,g)][a]
-    g.M = r1; g.N = r3 * r2; g.K = r1;
-    g.A = o.B[0]; g.a_m = r1; g.a_k = 1; g.a_b1 = (long)r1 * r1; g.a_b2 = 0;
-    g.B = G; g.b_k = 1; g.b_n = r1; g.b_b1 = 0; g.b_b2 = m;
-    g.C = X1; g.c_m = (long)r3 * r2; g.c_n = 1; g.c_b1 = m; g.c_b2 = T * m;
-    TX_TRY(simt_gemm(g, s));
-    // mode 3: X2[p][t][g'][(a',b)] = sum_g B_t3[g'][g] X1[p][t][(a',b)][g]   (mu_t inside B_t3)
-    g.M = r3; g.N = r1 * r2; g.K = r3;
-    g.A = o.B[2]; g.a_m = r3; g.a_k = 1; g.a_b1 = (long)r3 * r3; g.a_b2 = 0;
-    g.B = X1; g.b_k = 1; g.b_n = r3; g.b_b1 = m; g.b_b2 = T * m;
-    g.C = X2; g.c_m = (long)r1 * r2; g.c_n = 1; g.c_b1 = m; g.c_b2 = T * m;
-    TX_TRY(simt_gemm(g, s));
-    // mode 2: X1[p][t][b'][(g',a')] = sum_b B_t2[b'][b] X2[p][t][(g',a')][b]
-    g.M = r2; g.N = r3 * r1; g.K = r2;
-    g.A = o.B[1]; g.a_m = r2; g.a_k = 1; g.a_b1 = (long)r2 * r2; g.a_b2 = 0;
-    g.B = X2; g.b_k = 1; g.b_n = r2; g.b_b1 = m; g.b_b2 = T * m;
-    g.C = X1; g.c_m = (long)r3 * r1; g.c_n = 1; g.c_b1 = m; g.c_b2 = T * m;
-    TX_TRY(simt_gemm(g, s));
-    const long total = np * m;
-    const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 16);
-    k_sum_terms<<<blocks, 256, 0, s>>>(X1, T, m, np, H);
+    o.T = c->T;
+    k_galerkin_operators<<<dim3((unsigned)((most + 255) / 256), 3), 256, 0, s>>>(o);
     TX_LAUNCHED();
     return TX_OK;
 }
 
+// H[p][a'][b'][g'] = sum_t G[p] x1 B_t1 x2 B_t2 x3 B_t3: the expansion onto a grid of r_d points whose
+// operators are B_td.  Mode 1 of every term is one GEMM; the consumer runs modes 2 and 3 and the sum
+// over t in registers (X1 holds [np][T][r1][(b,g)]).  Differentiation-shaped block (rank 32, 35 terms, 136
+// pairs): 845 us; 1456 as three GEMM passes over every term and a sum.
+int galerkin_core(const tx_ctx* c, const GalerkinOps& o, const float* G, float* X1, float* H, int np, cudaStream_t s) {
+    TX_TRY(simt_expand_mode1_grid(c, G, o.B[0], c->r[0], c->T, X1, np, s));
+    FieldArgs f{};
+    f.OUT0 = H;
+    return simt_expand_consume(coarse_shape(c), nullptr, 0, np, f, X1, c->T, o.B[1], o.B[2], EPI_STORE, nullptr, s);
+}
+
 int galerkin_core_dot(const tx_ctx* c, const PairRec* recs, int p0, const float* G, const float* H, int np,
                       double* epart, cudaStream_t s) {
-    const long m = (long)c->r[0] * c->r[1] * c->r[2];
-    k_core_dot<<<np, 256, 0, s>>>(recs, p0, G, H, m, epart);
+    k_core_dot<<<np, 256, 0, s>>>(recs, p0, G, H, c->r[0], (long)c->r[1] * c->r[2], epart);
     TX_LAUNCHED();
     return TX_OK;
 }

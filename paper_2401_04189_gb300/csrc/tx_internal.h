@@ -112,6 +112,7 @@ struct tx_ctx {
     double* d_x[3];
     double* d_w[3];
     double* d_U[3];
+    double* d_UW[3];     // U_d[a][i] w_d[a] (two-sided projection)
     double* d_theta;
     double* d_mu;
     double* d_A64[3];    // [T][n_d][r_d]; mu_t folded into mode 3

@@ -180,7 +180,7 @@ int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec
 // convolution, then either the core-space energy or one reconstruction with D^-1 U and the
 // Hadamard epilogue.
 int galerkin_batch(tx_ctx* c, const CallSpec& cs, const GalerkinOps& o, const PairRec* recs, int p0, int np,
-                   float* S2, float* G, float* H, float* X1, float* X2, double* epart, cudaStream_t s) {
+                   float* S2, float* G, float* H, float* X1, double* epart, cudaStream_t s) {
     const bool subset = cs.mode == PAIRS_SUBSET;
     FieldArgs f{};
     f.SA = subset ? cs.occ : cs.tgt;
@@ -191,10 +191,10 @@ int galerkin_batch(tx_ctx* c, const CallSpec& cs, const GalerkinOps& o, const Pa
     f.OUT1 = cs.out0;
     TX_TRY(simt_project_s2(c, recs, p0, np, f, 0, S2, s));
     TX_TRY(gemm_mode1_project(c, S2, c->f_U[0], G, np, s));
-    TX_TRY(galerkin_core(c, o, G, X1, X2, H, np, s));
+    TX_TRY(galerkin_core(c, o, G, X1, H, np, s));
     if (cs.kind == CALL_ENERGY) return galerkin_core_dot(c, recs, p0, G, H, np, epart, s);
     float* Z = S2;   // [np][1][n1][r2 r3]: the size of S2
-    TX_TRY(gemm_mode1_expand(c, H, o.Ut[0], c->n[0], 1, 0, 1, Z, np, s));
+    TX_TRY(gemm_mode1_expand(c, H, o.Ut[0], c->n[0], 1, 0, 1, Z, np, s, 0, true));
     return simt_expand_consume(fine_shape(c), recs, p0, np, f, Z, 1, o.Ut[1], o.Ut[2], EPI_OUT, epart, s);
 }
 
@@ -238,7 +238,7 @@ int run_call(tx_ctx* c, const CallSpec& cs, cudaStream_t s) {
         per_pair = sizeof(float) * sthosvd_floats_per_pair(c);
         epp = simt_expand_consume_blocks(fine_shape(c));
     } else if (gk) {
-        per_pair = sizeof(float) * (L.s2 + 2 * L.g + 2 * (size_t)c->T * L.g);
+        per_pair = sizeof(float) * (L.s2 + 2 * L.g + (size_t)c->T * L.g);
         epp = cs.kind == CALL_ENERGY ? 1 : simt_expand_consume_blocks(fine_shape(c));
     } else if (tc) {
         per_pair = tc_batch_bytes_per_pair(c, cs.kind);
@@ -289,8 +289,7 @@ int run_call(tx_ctx* c, const CallSpec& cs, cudaStream_t s) {
             float* G = S2 + (size_t)Pb * L.s2;
             float* H = G + (size_t)Pb * L.g;
             float* X1 = H + (size_t)Pb * L.g;
-            float* X2 = X1 + (size_t)Pb * c->T * L.g;
-            TX_TRY(galerkin_batch(c, cs, gops, recs, p0, np, S2, G, H, X1, X2, epart, s));
+            TX_TRY(galerkin_batch(c, cs, gops, recs, p0, np, S2, G, H, X1, epart, s));
         } else if (tc) {
             BatchBuffers bb{recs, recs2, p0, np, scratch, epart};
             TX_TRY(tc_run_batch(c, cs, bb, s));

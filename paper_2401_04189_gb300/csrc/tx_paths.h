@@ -31,16 +31,16 @@ int sthosvd_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, int p0, in
 int simt_expand_mode1_pp(const tx_ctx* c, const float* G, const float* M1, long m1_pair_stride, int nt, float* Z,
                          int np, cudaStream_t s);
 
-// two-sided (Galerkin) projection (tx_galerkin.cu): B_td = U_d^T D_d A_td and D_d^-1 U_d
+// two-sided (Galerkin) projection (tx_galerkin.cu): B_td = U_d^T D_d A_td and D_d^-1 U_d, modes 2 and 3
+// with the left index fastest
 struct GalerkinOps {
-    const float* B[3];           // [T][r_d][r_d], mu_t folded into mode 3
+    const float* B[3];           // mode 1 [T][r_1][r_1]; modes 2, 3 [T][r_d][simt_ld(r_d)], mu_t folded into mode 3
     const float* Ut[3];          // mode 1 [n_1][r_1]; modes 2, 3 [r_d][simt_ld(n_d)]
 };
 size_t galerkin_operator_floats(const tx_ctx* c);
 int galerkin_operators(const tx_ctx* c, float* ops, GalerkinOps* g, cudaStream_t s);
-// H[p] = sum_t G[p] x_d B_td (X1, X2: [np][T][r1 r2 r3] scratch)
-int galerkin_core(const tx_ctx* c, const GalerkinOps& o, const float* G, float* X1, float* X2, float* H, int np,
-                  cudaStream_t s);
+// H[p][a][(b,g)] = sum_t G[p] x_d B_td from G[p][(b,g)][a] (X1: [np][T][r1 r2 r3] scratch)
+int galerkin_core(const tx_ctx* c, const GalerkinOps& o, const float* G, float* X1, float* H, int np, cudaStream_t s);
 // epart[p] = ew_p <G_p, H_p>
 int galerkin_core_dot(const tx_ctx* c, const PairRec* recs, int p0, const float* G, const float* H, int np,
                       double* epart, cudaStream_t s);

@@ -32,6 +32,11 @@ __device__ __forceinline__ uint64_t dup2(float v) {
 __device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 __device__ __forceinline__ float2 unpack2(uint64_t v) {
     float2 r;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
@@ -584,7 +589,7 @@ struct ConsumeF32Args {
 
 // Registers: 8 RN for phi, 8 per mode-2 column; the K part of mode 3 (gc) is at most CL * kMaxPart
 // columns so that both fit the 168 registers that leave 12 warps per SM (255 above 12 columns).
-__host__ __device__ constexpr int consume_max_rg(int cl, int rn) { return cl == 16 ? 4 : (rn > 8 ? 5 : 8); }
+__host__ __device__ constexpr int consume_max_rg(int cl, int rn) { return cl == 16 ? 4 : (rn > 8 ? 5 : (rn == 6 ? 6 : 8)); }
 __host__ __device__ constexpr int consume_max_threads(int cl, int rn) { return rn <= 12 ? 384 : 256; }
 
 template <int CL, int RN4, int H>
@@ -610,11 +615,17 @@ __global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_co
     const long zslice = (long)d.r3 * d.r2;
     const int ng = (d.r3 + a.gc - 1) / a.gc, nb = (d.r2 + a.bc - 1) / a.bc;
 
-    uint64_t acc[kRows][NP];
+    // Where the registers allow (grids of at most 48 columns, the coarse grids among them), each term is
+    // summed by itself and then added to the total: two short float32 sums round less than one long one.
+    constexpr bool FOLD = 4 * RN4 + 2 * H <= 6;
+    uint64_t acc[kRows][NP], total[FOLD ? kRows : 1][FOLD ? NP : 1];
 #pragma unroll
     for (int i = 0; i < kRows; ++i)
 #pragma unroll
-        for (int c = 0; c < NP; ++c) acc[i][c] = 0ull;
+        for (int c = 0; c < NP; ++c) {
+            acc[i][c] = 0ull;
+            if constexpr (FOLD) total[i][c] = 0ull;
+        }
 
     // M2 and Z of part (t, g part, b part)
     auto load2 = [&](int t, int gp, int bp) {
@@ -700,6 +711,15 @@ __global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_co
                     for (int c = 0; c < NP; ++c) fma2(acc[i][c], yi, b[c]);
                 }
             }
+            if constexpr (FOLD)
+                if (gp + 1 == ng)
+#pragma unroll
+                    for (int i = 0; i < kRows; ++i)
+#pragma unroll
+                        for (int c = 0; c < NP; ++c) {
+                            total[i][c] = add2(total[i][c], acc[i][c]);
+                            acc[i][c] = 0ull;
+                        }
         }
     // epilogue
     const long N3 = (long)d.n1 * d.n2 * d.n3;
@@ -721,7 +741,9 @@ __global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_co
 #pragma unroll
         for (int c = 0; c < NP; ++c) {
             const int z = c < 2 * RN4 ? 4 * CL * (c / 2) + 4 * tz + 2 * (c & 1) : 4 * CL * RN4 + 2 * tz;
-            const float2 ph = unpack2(acc[i][c]);
+            float2 ph;
+            if constexpr (FOLD) ph = unpack2(total[i][c]);
+            else ph = unpack2(acc[i][c]);
             const float phi[2] = {ph.x, ph.y};
             if (a.flags & EPI_STORE) {
                 float* dst = a.f.OUT0 + pl * N3 + base + z;
@@ -1020,8 +1042,8 @@ int simt_expand_consume(const Shape& sh, const PairRec* recs, int p0, int np, co
     const Dims d = dims_of(sh);
     if (d.n3 > 256) return fail(TX_ERR_UNSUPPORTED_SHAPE, "float32 path supports n3 <= 256");
     SimtPlan p{};
-    if (!simt_plan(d, &p) || sizeof(float) * ((size_t)d.r3 * (d.r2 + 1) + 32 * (size_t)(d.r3 + 1) +
-                                              (size_t)d.n3 * (d.r3 | 1)) > kSmemLimit)
+    if (!simt_plan(d, &p) || (!(flags & EPI_STORE) && sizeof(float) * ((size_t)d.r3 * (d.r2 + 1) + 32 * (size_t)(d.r3 + 1) +
+                                              (size_t)d.n3 * (d.r3 | 1)) > kSmemLimit))
         return fail(TX_ERR_CUDA, "float32 expansion: (r2 + n3) * r3 too large");
     ConsumeF32Args a{};
     a.d = d;
