@@ -86,13 +86,16 @@ int simt_expand_all(const tx_ctx* c, const float* G, float* H, float* Z, int np,
 
 namespace {
 
-// The adjoint's sums over the terms: H[p][(b,g)][a] from R[p][t][x][(b,g)] of every fine term (nf * n1 rows
-// per pair).  The smooth terms' transposes run behind one fine-grid term, q x_d I_d^T on the coarse
-// grid (Y, r1 r2 r3 floats per pair), then Q_td^T there (R is overwritten).  The order (b,g) may as
-// well be (g,b): `swapped` exchanges modes 2 and 3 of the coarse grid.
-int adjoint_sums(const tx_ctx* c, float* R, float* Y, float* H, bool swapped, int np, cudaStream_t s) {
+}  // namespace
+
+int simt_adjoint_core(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, int flags, float* Y,
+                      float* R, float* H, cudaStream_t s) {
     const TermSplit& ts = c->ts;
     const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2], ns = ts.nf - 1;
+    TX_TRY(simt_adjoint_r(fine_shape(c), recs, p0, np, f, ts.nf, ts.F[1], ts.F[2], flags, R, s));
+    if (!ts.nc) return gemm_mode1_adjoint(c, R, ts.F[0], n1, ts.nf, ts.nf, H, false, np, s);
+    // the smooth terms' transposes run behind one fine-grid term: Y = q x_d I_d^T on the coarse grid, then
+    // Q_td^T there
     if (ns) TX_TRY(gemm_mode1_adjoint(c, R, ts.F[0], n1, ns, ts.nf, H, false, np, s));
     // Y[p][k][(b,g)] = sum_x I_1[x][k] R[p][ns][x][(b,g)]
     GemmArgs g{};
@@ -105,19 +108,17 @@ int adjoint_sums(const tx_ctx* c, float* R, float* Y, float* H, bool swapped, in
     FieldArgs fy{};
     fy.SA = Y;
     fy.SB = Y;
-    TX_TRY(simt_adjoint_r(coarse_shape(c, swapped), nullptr, 0, np, fy, ts.nc, ts.Q[swapped ? 2 : 1], ts.Q[swapped ? 1 : 2],
-                          PROD_PLAIN, R, s));
+    TX_TRY(simt_adjoint_r(coarse_shape(c), nullptr, 0, np, fy, ts.nc, ts.Q[1], ts.Q[2], PROD_PLAIN, R, s));
     return gemm_mode1_adjoint(c, R, ts.Q[0], r1, ts.nc, ts.nc, H, ns > 0, np, s);
 }
 
-// H[p][(b,g)][a] = sum_t mu_t q_p x_d A_td^T (the adjoint onto the core) for the products q_p that recs and
-// f name; Y holds r1 r2 r3 floats per pair, R the Z share
-int simt_adjoint_core(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, int flags, float* Y,
-                      float* R, float* H, cudaStream_t s) {
-    const TermSplit& ts = c->ts;
-    TX_TRY(simt_adjoint_r(fine_shape(c), recs, p0, np, f, ts.nf, ts.F[1], ts.F[2], flags, R, s));
-    if (!ts.nc) return gemm_mode1_adjoint(c, R, ts.F[0], c->n[0], ts.nf, ts.nf, H, false, np, s);
-    return adjoint_sums(c, R, Y, H, false, np, s);
+namespace {
+
+// planes the float32 precision's gradients accept
+int simt_adjoint_limit(const Shape& sh) {
+    if (sizeof(float) * ((size_t)sh.n2 * sh.n3 + (size_t)sh.n2 * sh.r3) > 220 * 1024)
+        return fail(TX_ERR_UNSUPPORTED_SHAPE, "float32 adjoint needs n2*(n3+r3) <= 56K");
+    return TX_OK;
 }
 
 int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec* recs2, int p0, int np,
@@ -135,6 +136,7 @@ int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec
             f.MUL1 = cs.occ;
             f.OUT0 = cs.out0;
             f.OUT1 = cs.out0;
+            if (cs.kind == CALL_GRAD) TX_TRY(simt_adjoint_limit(sh));
             TX_TRY(simt_project_s2(c, recs, p0, np, f, 0, S2, s));
             TX_TRY(gemm_mode1_project(c, S2, c->f_U[0], G, np, s));
             TX_TRY(simt_expand_all(c, G, S2, Z, np, s));
@@ -152,6 +154,7 @@ int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec
             return TX_OK;
         }
         case CALL_VJP: {
+            TX_TRY(simt_adjoint_limit(sh));
             if (cs.out0) {
                 // grad_occ_j -= cot_k * phi_kj
                 f.SA = cs.tgt; f.SB = cs.occ;
@@ -202,9 +205,6 @@ int galerkin_batch(tx_ctx* c, const CallSpec& cs, const GalerkinOps& o, const Pa
 
 int simt_adjoint_mode1(const tx_ctx* c, const float* R, float* H, int np, cudaStream_t s) {
     return gemm_mode1_adjoint(c, R, c->f_A[0], c->n[0], c->T, c->T, H, false, np, s);
-}
-int simt_adjoint_split(const tx_ctx* c, float* R, float* Y, float* H, int np, cudaStream_t s) {
-    return adjoint_sums(c, R, Y, H, true, np, s);
 }
 int simt_expand_mode1_grid(const tx_ctx* c, const float* G, const float* M1, int n1, int nt, float* Z, int np,
                            cudaStream_t s) {

@@ -65,9 +65,10 @@ size_t tc_batch_bytes_per_pair(const tx_ctx* c, int kind);
 // float32 building blocks shared with the tensor-core adjoint (tx_paths.cu):
 // H[p][(g,b)][a] = sum_{t,x} R[p][t][x][(g,b)] A_t1[x][a]
 int simt_adjoint_mode1(const tx_ctx* c, const float* R, float* H, int np, cudaStream_t s);
-// the same from the fine terms' R[p][t][x][(g,b)], the smooth terms through the coarse grid (Y: r1 r2 r3
-// floats per pair of scratch; R is overwritten and holds at least nc r1 r2 r3 floats per pair)
-int simt_adjoint_split(const tx_ctx* c, float* R, float* Y, float* H, int np, cudaStream_t s);
+// H[p][(b,g)][a] = sum_t mu_t q_p x_d A_td^T (the adjoint onto the core) for the products q_p that recs and
+// f name; Y holds r1 r2 r3 floats per pair of scratch, R max(nf n1, nc r1) r2 r3
+int simt_adjoint_core(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, int flags, float* Y,
+                      float* R, float* H, cudaStream_t s);
 // Z[p][t][x][(g,b)] = sum_a M1_t[x][a] G[p][(g,b)][a] on a grid of n1 nodes
 int simt_expand_mode1_grid(const tx_ctx* c, const float* G, const float* M1, int n1, int nt, float* Z, int np,
                            cudaStream_t s);

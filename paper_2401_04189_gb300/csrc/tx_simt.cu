@@ -368,24 +368,27 @@ struct ChainArgs {
     int flags;
     float* out;
     int ty, gw, bw, mh;            // y rows per tile (a multiple of 8), g (<= 64) and b (<= 256) columns per pass, M2 rows held
-    int ldy, ldg, ldb, vec;        // shared-memory row strides; vec: 16-byte orbital rows
+    int zq;                        // z columns of the product held: PZ (a slice), or n3 (the whole plane, over every term)
+    int ldy, ldg, lds, ldb, vec;   // row strides of the product, M3, S1 and M2; vec: 16-byte orbital rows
+    int flat3, flat2;              // M3 / M2 tiles are contiguous runs of whole 16-byte pieces
     int bg;                        // 1: out[b][g] (the float32 consumer's order), 0: out[g][b]
 };
 
 __global__ void __launch_bounds__(384) k_chain(const ChainArgs a) {
     extern __shared__ __align__(16) float sm[];
     const Dims d = a.d;
-    float* qs = sm;                            // [PZ][ldy]   the pair product, z-major
-    float* m2s = qs + PZ * a.ldy;              // [mh][ldb]
-    float* m3s = m2s + a.mh * a.ldb;           // [PZ][ldg]
-    float* s1 = m3s + PZ * a.ldg;              // [ty][ldg]
+    float* qs = sm;                            // [zq][ldy]   the pair product, z-major
+    float* m2s = qs + a.zq * a.ldy;            // [mh][ldb]
+    float* m3s = m2s + a.mh * a.ldb;           // [zq][ldg]
+    float* s1 = m3s + ((a.zq * a.ldg + 3) & ~3);   // [ty][lds]
     const int x = blockIdx.x, pl = blockIdx.y, tid = threadIdx.x, nth = blockDim.x;
     const bool plain = (a.flags & PROD_PLAIN) != 0;
     const PairRec rec = plain ? PairRec{} : a.recs[a.p0 + pl];
     const long N3 = (long)d.n1 * d.n2 * d.n3;
     const float* pa = a.SA + (plain ? pl : rec.ia) * N3 + (long)x * d.n2 * d.n3;
     const float* pb = plain ? pa : a.SB + rec.ib * N3 + (long)x * d.n2 * d.n3;
-    const bool mulw = (a.flags & PROD_MULW) != 0;
+    const bool mulw = (a.flags & PROD_MULW) != 0, whole = a.zq > PZ, m2_tile = a.mh >= a.ty && d.r2 <= a.bw;
+    const bool pre3 = whole && m2_tile && a.gw >= d.r3;           // the next term's M3 is loaded one stage ahead
     const float wx = mulw ? a.w1[x] : 1.f;
     const int tz = tid & 7, row0 = kRows * (tid >> 3);
     const int nbq = a.bw / 4, ngt = nth / nbq;                    // mode 2: 4 b per thread
@@ -393,75 +396,105 @@ __global__ void __launch_bounds__(384) k_chain(const ChainArgs a) {
     const int bq = a.bg ? tid / ngt : tid % nbq, gq = a.bg ? tid % ngt : tid / nbq;
     const bool act2 = a.bg ? bq < nbq : gq < ngt;
     const long og = a.bg ? 1 : d.r2, ob = a.bg ? d.r3 : 1;
-    // 16-byte pieces of a slice: 32 lanes are 16 rows x 2 neighbouring pieces (whole sectors; with
-    // ldy = 4 (mod 8) the transposed stores hit 32 different banks)
+    // this thread's (at most 4) 16-byte pieces of a slice, the same in every slice: 32 lanes are 16 rows
+    // x 2 neighbouring pieces (whole sectors; with ldy = 4 (mod 8) the transposed stores hit 32 banks)
     const int ngr = (min(a.ty, d.n2) + 15) / 16, npc = ngr * (PZ / 8) * 32;
-    float4 fa[4], fb[4];                       // at most 4 pieces per thread (the launch has a thread per 4)
-    auto piece = [&](int i, int z0, int yn, int& yy, int& z) -> bool {
+    int py[4], pz[4];                          // row in the tile and first column in the slice; py < 0: none
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
         const int e = i * nth + tid, grp = e >> 5, l = e & 31;
-        yy = (grp % ngr) * 16 + (l & 15);
-        z = 4 * (2 * (grp / ngr) + (l >> 4));
-        return e < npc && yy < yn && z0 + z < d.n3;
-    };
+        py[i] = e < npc ? (grp % ngr) * 16 + (l & 15) : -1;
+        pz[i] = 4 * (2 * (grp / ngr) + (l >> 4));
+    }
+    float4 fa[4], fb[4];
     auto fetch = [&](int y0, int yn, int z0) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            int yy, z;
-            if (!piece(i, z0, yn, yy, z)) continue;
-            const long o = (long)(y0 + yy) * d.n3 + z0 + z;
+            if (py[i] < 0 || py[i] >= yn || z0 + pz[i] >= d.n3) continue;
+            const long o = (long)(y0 + py[i]) * d.n3 + z0 + pz[i];
             fa[i] = *(const float4*)(pa + o);
             fb[i] = plain ? make_float4(1.f, 1.f, 1.f, 1.f) : *(const float4*)(pb + o);
         }
     };
-    for (int t = 0; t < a.nt; ++t) {
-        const float* M3 = a.M3 + (long)t * d.n3 * d.r3;
-        const float* M2 = a.M2 + (long)t * d.n2 * d.r2;
-        float* out = a.out + (((long)pl * a.nt + t) * d.n1 + x) * d.r3 * d.r2;
-        for (int g0 = 0; g0 < d.r3; g0 += a.gw) {
-            const int gn = min(a.gw, d.r3 - g0), rg = (gn + 7) / 8;
-            for (int y0 = 0; y0 < d.n2; y0 += a.ty) {
-                const int yn = min(a.ty, d.n2 - y0);
+    // the slice z0 .. of the product into q rows [0, PZ)
+    auto stage = [&](float* q0, int y0, int yn, int z0, int zn) {
+        if (a.vec) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (py[i] < 0 || py[i] >= yn || z0 + pz[i] >= d.n3) continue;
+                float q[4] = {fa[i].x * fb[i].x, fa[i].y * fb[i].y, fa[i].z * fb[i].z, fa[i].w * fb[i].w};
+                if (mulw) {
+                    const float wxy = wx * a.w2[y0 + py[i]];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) q[k] *= wxy * a.w3[z0 + pz[i] + k];
+                }
+                float* dst = q0 + pz[i] * a.ldy + py[i];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) dst[k * a.ldy] = q[k];
+            }
+        } else {
+            for (int e = tid; e < yn * zn; e += nth) {
+                const int yy = e / zn, z = e - yy * zn;
+                const long o = (long)(y0 + yy) * d.n3 + z0 + z;
+                float q = plain ? pa[o] : pa[o] * pb[o];
+                if (mulw) q *= wx * a.w2[y0 + yy] * a.w3[z0 + z];
+                q0[z * a.ldy + yy] = q;
+            }
+        }
+    };
+    // M3 rows z0 .. z0 + zn - 1 (columns g0 .. of a pass) of term t
+    auto load3 = [&](int t, int z0, int zn, int g0, int gn) {
+        const float* M3 = a.M3 + ((long)t * d.n3 + z0) * d.r3;
+        if (a.flat3) {
+            for (int e = 4 * tid; e < zn * d.r3; e += 4 * nth) cp_async16(m3s + e, M3 + e);
+        } else {
+            for (int e = tid; e < zn * gn; e += nth) {
+                const int z = e / gn, g = e - z * gn;
+                cp_async4(m3s + z * a.ldg + g, M3 + (long)z * d.r3 + g0 + g);
+            }
+        }
+    };
+    // rows y0 + yb .. of M2 (columns b0 ..) of term t
+    auto load2 = [&](int t, int y0, int yn, int b0, int bn) {
+        const float* M2 = a.M2 + ((long)t * d.n2 + y0) * d.r2;
+        if (a.flat2) {
+            for (int e = 4 * tid; e < yn * d.r2; e += 4 * nth) cp_async16(m2s + e, M2 + e);
+        } else {
+            for (int e = tid; e < yn * bn; e += nth) {
+                const int yy = e / bn, bb = e - yy * bn;
+                cp_async4(m2s + yy * a.ldb + bb, M2 + (long)yy * d.r2 + b0 + bb);
+            }
+        }
+    };
+    for (int y0 = 0; y0 < d.n2; y0 += a.ty) {
+        const int yn = min(a.ty, d.n2 - y0);
+        if (whole) {                           // the tile's product once, for every term
+            if (a.vec) fetch(y0, yn, 0);
+            __syncthreads();                   // the previous tile's last readers
+            for (int z0 = 0; z0 < d.n3; z0 += PZ) {
+                stage(qs + z0 * a.ldy, y0, yn, z0, min(PZ, d.n3 - z0));
+                if (a.vec && z0 + PZ < d.n3) fetch(y0, yn, z0 + PZ);
+            }
+        }
+        for (int t = 0; t < a.nt; ++t) {
+            float* out = a.out + (((long)pl * a.nt + t) * d.n1 + x) * d.r3 * d.r2;
+            for (int g0 = 0; g0 < d.r3; g0 += a.gw) {
+                const int gn = min(a.gw, d.r3 - g0), rg = (gn + 7) / 8;
                 uint64_t acc[8][4];
 #pragma unroll
                 for (int c = 0; c < 8; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0ull;
-                if (a.vec) fetch(y0, yn, 0);
-                for (int z0 = 0; z0 < d.n3; z0 += PZ) {
-                    const int zn = min(PZ, d.n3 - z0);
-                    __syncthreads();           // the previous slice (and S1, M2) has been read
-                    if (a.vec) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            int yy, z;
-                            if (!piece(i, z0, yn, yy, z)) continue;
-                            float q[4] = {fa[i].x * fb[i].x, fa[i].y * fb[i].y, fa[i].z * fb[i].z, fa[i].w * fb[i].w};
-                            if (mulw) {
-                                const float wxy = wx * a.w2[y0 + yy];
-#pragma unroll
-                                for (int k = 0; k < 4; ++k) q[k] *= wxy * a.w3[z0 + z + k];
-                            }
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) qs[(z + k) * a.ldy + yy] = q[k];
-                        }
-                    } else {
-                        for (int e = tid; e < yn * zn; e += nth) {
-                            const int yy = e / zn, z = e - yy * zn;
-                            const long o = (long)(y0 + yy) * d.n3 + z0 + z;
-                            float q = plain ? pa[o] : pa[o] * pb[o];
-                            if (mulw) q *= wx * a.w2[y0 + yy] * a.w3[z0 + z];
-                            qs[z * a.ldy + yy] = q;
-                        }
+                if (a.vec && !whole) fetch(y0, yn, 0);
+                for (int z0 = 0; z0 < d.n3; z0 += a.zq) {
+                    const int zn = min(a.zq, d.n3 - z0);
+                    if (!pre3 || t == 0) {
+                        __syncthreads();       // the previous slice (and S1, M2) has been read
+                        if (!whole) stage(qs, y0, yn, z0, zn);
+                        load3(t, z0, zn, g0, gn);
                     }
-                    for (int e = tid; e < zn * gn; e += nth) {
-                        const int z = e / gn, g = e - z * gn;
-                        m3s[z * a.ldg + g] = M3[(long)(z0 + z) * d.r3 + g0 + g];
-                    }
-                    if (z0 == 0 && a.mh >= a.ty && d.r2 <= a.bw)      // the whole M2 tile, under mode 3
-                        for (int e = tid; e < yn * d.r2; e += nth) {
-                            const int yy = e / d.r2, bb = e - yy * d.r2;
-                            cp_async4(m2s + yy * a.ldb + bb, M2 + (long)(y0 + yy) * d.r2 + bb);
-                        }
+                    cp_async_wait_all();
                     __syncthreads();
-                    if (a.vec && z0 + PZ < d.n3) fetch(y0, yn, z0 + PZ);
+                    if (z0 == 0 && m2_tile) load2(t, y0, yn, 0, d.r2);      // lands under mode 3
+                    if (a.vec && !whole && z0 + PZ < d.n3) fetch(y0, yn, z0 + PZ);
                     if (row0 < a.ty) panel8_any<8>(rg, qs + row0, a.ldy, m3s + tz, a.ldg, zn, acc);
                 }
                 if (row0 < a.ty) {
@@ -471,13 +504,12 @@ __global__ void __launch_bounds__(384) k_chain(const ChainArgs a) {
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
                                 const float2 u = unpack2(acc[c][i]);
-                                float* p = s1 + (row0 + 2 * i) * a.ldg + tz + 8 * c;
+                                float* p = s1 + (row0 + 2 * i) * a.lds + tz + 8 * c;
                                 p[0] = u.x;
-                                p[a.ldg] = u.y;
+                                p[a.lds] = u.y;
                             }
                         }
                 }
-                cp_async_wait_all();
                 // mode 2: S2[g][b] = sum_y S1[y][g] M2[y][b], this y tile's share added to the earlier ones'
                 const int npass = (gn + 8 * ngt - 1) / (8 * ngt), cb = (gn + ngt * npass - 1) / (ngt * npass);
                 for (int b0 = 0; b0 < d.r2; b0 += a.bw)
@@ -488,29 +520,29 @@ __global__ void __launch_bounds__(384) k_chain(const ChainArgs a) {
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {
                             s[c][0] = s[c][1] = 0ull;
-                            col[c] = min(gc + gq + c * ngt, a.ldg - 1);      // past gn: a padding column, never stored
+                            col[c] = min(gc + gq + c * ngt, a.lds - 1);      // past gn: a padding column, never stored
                         }
                         for (int yb = 0; yb < yn; yb += a.mh) {
                             const int ync = min(a.mh, yn - yb);
+                            cp_async_wait_all();
                             __syncthreads();       // S1 (and the M2 tile) written; the previous M2 slice has been read
-                            if (a.mh < a.ty || d.r2 > a.bw) {
-                                for (int e = tid; e < ync * bn; e += nth) {
-                                    const int yy = e / bn, bb = e - yy * bn;
-                                    m2s[yy * a.ldb + bb] = M2[(long)(y0 + yb + yy) * d.r2 + b0 + bb];
-                                }
+                            if (pre3 && gc == 0 && t + 1 < a.nt) load3(t + 1, 0, d.n3, 0, d.r3);    // lands under mode 2
+                            if (!m2_tile) {
+                                load2(t, y0 + yb, ync, b0, bn);
+                                cp_async_wait_all();
                                 __syncthreads();
                             }
                             if (act2) {
-                                const float* sp = s1 + yb * a.ldg;
+                                const float* sp = s1 + yb * a.lds;
                                 const float* mp = m2s + 4 * bq;
                                 switch (cb) {
-                                    case 1: panel4<1>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
-                                    case 2: panel4<2>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
-                                    case 3: panel4<3>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
-                                    case 4: panel4<4>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
-                                    case 5: panel4<5>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
-                                    case 6: panel4<6>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
-                                    default: panel4<8>(mp, a.ldb, sp, a.ldg, col, ync, s); break;
+                                    case 1: panel4<1>(mp, a.ldb, sp, a.lds, col, ync, s); break;
+                                    case 2: panel4<2>(mp, a.ldb, sp, a.lds, col, ync, s); break;
+                                    case 3: panel4<3>(mp, a.ldb, sp, a.lds, col, ync, s); break;
+                                    case 4: panel4<4>(mp, a.ldb, sp, a.lds, col, ync, s); break;
+                                    case 5: panel4<5>(mp, a.ldb, sp, a.lds, col, ync, s); break;
+                                    case 6: panel4<6>(mp, a.ldb, sp, a.lds, col, ync, s); break;
+                                    default: panel4<8>(mp, a.ldb, sp, a.lds, col, ync, s); break;
                                 }
                             }
                         }
@@ -938,12 +970,23 @@ int launch_chain(const Shape& sh, const PairRec* recs, int p0, int np, const Fie
     const int ngp = (a.d.r3 + 63) / 64;
     a.gw = (a.d.r3 + ngp - 1) / ngp;
     a.ldy = ((a.ty + 7) & ~7) + 4;
-    a.ldg = 8 * ((a.gw + 7) / 8) + 2;
+    a.ldg = a.gw;                              // read as scalars by neighbouring lanes: no padding needed
+    a.lds = 8 * ((a.gw + 7) / 8) + 2;
     a.bw = std::min(256, pad4(a.d.r2));
-    a.ldb = a.bw + 4;
+    a.flat2 = a.d.r2 % 4 == 0 && a.d.r2 <= a.bw && ((uintptr_t)M2 & 15u) == 0;
+    a.ldb = a.flat2 ? a.d.r2 : a.bw + 4;
+    // a slice starts at a multiple of 16 rows of r3 floats; a term at a multiple of n3 r3; the slice's own length counts too
+    a.flat3 = ngp == 1 && ((long)a.d.n3 * a.d.r3) % 4 == 0 && ((uintptr_t)M3 & 15u) == 0;
     a.vec = a.d.n3 % 4 == 0 && (((uintptr_t)f.SA | (uintptr_t)f.SB) & 15u) == 0;
     a.mh = (size_t)a.ty * a.ldb * sizeof(float) <= 64 * 1024 ? a.ty : 32;
-    const size_t smem = sizeof(float) * ((size_t)PZ * a.ldy + (size_t)a.mh * a.ldb + (size_t)(PZ + a.ty) * a.ldg);
+    // 8 more floats behind M3: the last column group of a panel may read past its last row
+    auto bytes = [&](int zq) {
+        return sizeof(float) * ((size_t)zq * a.ldy + (size_t)a.mh * a.ldb + (((size_t)zq * a.ldg + 3) & ~(size_t)3) +
+                                (size_t)a.ty * a.lds + 8);
+    };
+    // several terms: hold the whole plane's product where two CTAs still share an SM
+    a.zq = nt > 1 && a.d.n3 > PZ && bytes(a.d.n3) <= kSmemLimit / 2 ? a.d.n3 : PZ;
+    const size_t smem = bytes(a.zq);
     // at least 64 threads; at least one per 4 b; at most 4 pieces of a slice per thread
     const int threads = std::max(std::max(64, (a.bw / 4 + 31) & ~31), (a.ty + 31) & ~31);
     TX_TRY(smem_attr((const void*)k_chain, smem));
@@ -1084,9 +1127,6 @@ int simt_expand_consume(const Shape& sh, const PairRec* recs, int p0, int np, co
 
 int simt_adjoint_r(const Shape& sh, const PairRec* recs, int p0, int np, const FieldArgs& f, int nt, const float* M2,
                    const float* M3, int flags, float* R, cudaStream_t s) {
-    const Dims d = dims_of(sh);
-    if (sizeof(float) * ((size_t)d.n2 * d.n3 + (size_t)d.n2 * d.r3) > 220 * 1024)
-        return fail(TX_ERR_UNSUPPORTED_SHAPE, "float32 adjoint needs n2*(n3+r3) <= 56K");
     return launch_chain(sh, recs, p0, np, f, nt, M2, M3, flags, R, true, "adjoint", s);
 }
 

@@ -138,10 +138,10 @@ int tc_prepare(tx_ctx* c, cudaStream_t s) {
     // every static operand row is K padded with zeros to a whole number of 32-byte sectors
     const int eb = op->esize;
     const size_t e_u3 = (size_t)r3 * ldk(n3, eb), e_u2 = (size_t)r2 * ldk(n2, eb), e_u1 = (size_t)r1 * ldk(n1, eb);
-    // (the split forms run mode 1 of the expansion in float32)
+    // (the split forms run mode 1 of the expansion and the adjoint in float32)
     const size_t e_a1 = op->split ? 0 : (size_t)T * n1 * ldk(r1, eb), e_a2 = (size_t)T * n2 * ldk(r2, eb);
     const size_t e_a3 = (size_t)T * n3 * ldk(r3, eb), e_a3f = (size_t)T * n3 * pad8(r3);
-    const size_t e_a3t = (size_t)T * r3 * ldk(n3, eb), e_a2t = (size_t)T * r2 * ldk(n2, eb);
+    const size_t e_a3t = op->split ? 0 : (size_t)T * r3 * ldk(n3, eb), e_a2t = op->split ? 0 : (size_t)T * r2 * ldk(n2, eb);
     auto al = [](size_t e) { return (e + 127) & ~(size_t)127; };   // 256-byte aligned pieces
     const size_t tot = al(e_u3) + al(e_u2) + al(e_u1) + al(e_a1) + al(e_a2) + al(e_a3) + al(e_a3t) + al(e_a2t);
     // bf16 single pass: the stage-3 B operand also in float32 (TF32), after everything else
@@ -187,7 +187,7 @@ int tc_prepare(tx_ctx* c, cudaStream_t s) {
     TX_TRY(conv(A64[1], (long)T * n2, r2, r2, 1, ldk(r2, eb), op->st.A2));
     TX_TRY(conv(A64[2], (long)T * n3, r3, r3, 1, ldk(r3, eb), op->st.A3));
     // the adjoint's transposed operators, one term at a time: rows gamma (beta), K = z (y)
-    for (int t = 0; t < T; ++t) {
+    for (int t = 0; t < T && !op->split; ++t) {
         TX_TRY(conv(A64[2] + (size_t)t * n3 * r3, r3, n3, 1, r3, ldk(n3, eb),
                     (char*)op->st.A3T + (size_t)t * r3 * ldk(n3, eb) * op->esize));
         TX_TRY(conv(A64[1] + (size_t)t * n2 * r2, r2, n2, 1, r2, ldk(n2, eb),
@@ -365,58 +365,63 @@ static AdjF32 adj_f32(const tx_ctx* c) {
     return AdjF32{std::max((size_t)tc_terms(c) * n1 * rr, coarse), rr * r1, n1 * rr};
 }
 
+// S1 of the tensor-core adjoint (single-pass precisions)
+static size_t adj_s1_bytes(const tx_ctx* c) { return c->tc->split ? 0 : tc_scratch(c).s1 * c->tc->esize; }
+
 // The adjoint of one pair batch (derived; the paper has no gradient): with L = sum_t mu_t
 // (x)_d A_td U_d^T, zeta_p = L^T y_p = (x)_d U_d [sum_t mu_t y_p x1 A_t1^T x2 A_t2^T x3 A_t3^T] for the
 // pair products y_p = SA[ia] * SB[ib] (* w), then fo.OUT0[o0] -= fo.MUL0[m0] * zeta and
 // fo.OUT1[o1] -= fo.MUL1[m1] * zeta.  Modes 3 and 2 of every term (2 n^3 r + 2 n^2 r^2 flops per
-// term, the adjoint's dominant work) run on the tensor cores; the sum over terms and x of mode 1
-// and the single-term expansion with U run in float32 on the CUDA cores (as the split forms'
-// projection does, so that the split forms keep float32 accuracy there).
+// term, the adjoint's dominant work) run on the tensor cores in the single-pass precisions; the sum
+// over terms and x of mode 1 and the single-term expansion with U run in float32 on the CUDA cores.
+// The split precisions run the whole adjoint there (simt_adjoint_core): with the smooth terms on the
+// coarse grid the remaining terms' modes 3 and 2 take 9.9 us per pair at the differentiation shape (64^3,
+// rank 32) against 30 for three passes per term on the tensor cores, whose products went through
+// memory term by term.
 static int tc_adjoint(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, const float* SA, int nA, const float* SB,
                       int nB, int pflags, const FieldArgs& fo, cudaStream_t s) {
     const TcOperands* op = c->tc;
     const TcScratch sc = tc_scratch(c);
     const int np = b.np;
-    const int eb = op->esize, mult = op->split ? 2 : 1;
-    const int n1 = c->n[0], n2 = c->n[1], n3 = c->n[2], r2 = c->r[1], r3 = c->r[2], T = tc_terms(c);
+    const int eb = op->esize;
+    const int n1 = c->n[0], n2 = c->n[1], n3 = c->n[2], r2 = c->r[1], r3 = c->r[2], T = c->T;
     const long rr = (long)r2 * r3;
     const AdjF32 f = adj_f32(c);
     char* S1 = b.scratch;
-    float* R = (float*)(((uintptr_t)(S1 + (size_t)np * sc.s1 * eb * mult) + 255) & ~(uintptr_t)255);
+    float* R = (float*)(((uintptr_t)(S1 + (size_t)np * adj_s1_bytes(c)) + 255) & ~(uintptr_t)255);
     float* H = R + (size_t)np * f.r;
     float* Z = H + (size_t)np * f.h;
+    if (op->split) {
+        FieldArgs fa = fo;
+        fa.SA = SA;
+        fa.SB = SB;
+        TX_TRY(simt_adjoint_core(c, recs, b.p0, np, fa, pflags, Z, R, H, s));
+        TX_TRY(simt_expand_mode1(c, H, c->f_U[0], 1, Z, np, s));     // Z = U1 H
+        return simt_expand_consume(fine_shape(c), recs, b.p0, np, fo, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, b.epart, s);
+    }
     for (int t = 0; t < T; ++t) {
         // S1[p][g][x][y] = sum_z y_p[x][y][z] (mu_t A_t3)[z][g]
         const char* a3t = (const char*)op->st.A3T + (size_t)t * r3 * ldk(n3, eb) * eb;
         TX_TRY(tc_project_mode3(c, recs, b.p0, np, SA, nA, SB, nB, pflags, S1, s, a3t));
         // R[p][t][x][g][b] = sum_y S1[p][(g,x)][y] A_t2[y][b]   (float32)
         const char* a2t = (const char*)op->st.A2T + (size_t)t * r2 * ldk(n2, eb) * eb;
-        TcOperand A{S1, op->split ? S1 + (size_t)np * sc.s1 * eb : nullptr, (uint64_t)n2, (uint64_t)r3 * n1, (uint64_t)np,
-                    (uint64_t)sc.ld_y, sc.s1};
-        TcOperand B{a2t, op->split ? a2t + op->st.off_lo : nullptr, (uint64_t)ldk(n2, eb), (uint64_t)r2, 1,
-                    (uint64_t)ldk(n2, eb), 0};
+        TcOperand A{S1, nullptr, (uint64_t)n2, (uint64_t)r3 * n1, (uint64_t)np, (uint64_t)sc.ld_y, sc.s1};
+        TcOperand B{a2t, nullptr, (uint64_t)ldk(n2, eb), (uint64_t)r2, 1, (uint64_t)ldk(n2, eb), 0};
         TcGemmArgs g{};
         g.M = r3 * n1; g.N = r2; g.K = n2; g.nb1 = np; g.nb2 = 1;
         g.a_z1 = 1;
         g.C = R + (size_t)t * n1 * rr; g.rdiv = n1; g.c_mh = r2; g.c_m = rr; g.c_n = 1; g.c_b1 = (long)T * n1 * rr;
         g.c_type = TC_OUT_F32; g.alpha = 1.f; g.err = c->d_err;
-        TX_TRY(tc_gemm_launch(A, B, g, op->tf32, op->split, "tc_adj2", s));
+        TX_TRY(tc_gemm_launch(A, B, g, op->tf32, false, "tc_adj2", s));
     }
-    if (op->split && c->ts.nc) {
-        // sharp terms from R, the smooth ones through the coarse grid (Z is free until the expansion)
-        TX_TRY(simt_adjoint_split(c, R, Z, H, np, s));
-    } else {
-        TX_TRY(simt_adjoint_mode1(c, R, H, np, s));              // H = sum_{t,x} R A_t1
-    }
+    TX_TRY(simt_adjoint_mode1(c, R, H, np, s));                  // H = sum_{t,x} R A_t1
     TX_TRY(simt_expand_mode1(c, H, c->f_U[0], 1, Z, np, s));     // Z = U1 H
     return simt_expand_consume(fine_shape(c), recs, b.p0, np, fo, Z, 1, c->f_UK[1], c->f_UK[2], EPI_OUT, b.epart, s, false);
 }
 
 size_t tc_adjoint_bytes_per_pair(const tx_ctx* c) {
-    const TcScratch sc = tc_scratch(c);
-    const TcOperands* op = c->tc;
     const AdjF32 f = adj_f32(c);
-    return sc.s1 * op->esize * (op->split ? 2 : 1) + (f.r + f.h + f.z) * sizeof(float) + 1024;
+    return adj_s1_bytes(c) + (f.r + f.h + f.z) * sizeof(float) + 1024;
 }
 
 int tc_run_batch(tx_ctx* c, const CallSpec& cs, const BatchBuffers& b, cudaStream_t s) {
