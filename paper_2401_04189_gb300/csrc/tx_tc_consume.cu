@@ -9,11 +9,9 @@
 // Z_t = G x1 A_t1 comes from the first-mode GEMM.  Three kernels:
 //  - k_consume (the split precisions, below): stage 2 puts y on the TMEM lanes and g on the
 //    columns, so each converter lane already holds one row (x, y) of the K-major stage-3
-//    operand: it splits the row into hi and lo and writes them with 16-byte stores.  Each x
-//    plane has its own TMEM columns and its own full / free barriers, so the MMA of plane p for
-//    the next term starts as soon as plane p has been converted.  Operand tiles use the 32-byte
-//    swizzle: one sub-tile of `rows x 32 bytes` per MMA K-step, so K is padded only to the
-//    K-step.  Warp roles: 0-7 converters + epilogue, 8 TMA producer + TMEM owner, 9 MMA issuer.
+//    operand: it splits the row into hi and lo and writes them with 16-byte stores.  Operand
+//    tiles use the 32-byte swizzle: one sub-tile of `rows x 32 bytes` per MMA K-step, so K is
+//    padded only to the K-step.
 //  - k_consume_ts (single-pass precisions): stage 3 reads Y straight from TMEM; one CTA per
 //    (pair, slab) work item (described at its definition).
 //  - k_consume_tp: the same loop, persistent over the work items, with the epilogue of one item
@@ -91,12 +89,14 @@ struct ConsumeArgs {
     int yz, nzi;
     // converter kernel: the stage-3 B operand (mu_t A_t3) has a ring of its own after the
     // [A_t2][Z] stages, so that stage 2 releases its stage as soon as its MMAs have run
-    uint32_t loadB_bytes, b_off, stageB_tx;
+    uint32_t loadB_bytes, b_off, stageB_tx, stageZ_tx;   // stage_tx: A_t2 alone
+    uint32_t a3_rows;          // rows per K step of the converted stage-3 operand
     int nloadB;
 };
 
-constexpr int kThreads = 320;
+constexpr int kThreads = 384;       // converter kernel
 constexpr int kMaxLoadB = 2;       // converter kernel: stages of the stage-3 operand ring
+constexpr int kMaxYCv = 3;         // ... and Y buffers in TMEM
 constexpr int kThreadsTs = 352;   // single-pass kernel: one more producer warp (10)
 constexpr int kThreadsTp = 384;   // persistent single-pass kernel: a separate stage-3 warp (11)
 // epilogue shared memory (reuses the pipeline buffers): phi staging, 8 warps x 32 rows x 68
@@ -426,7 +426,98 @@ __device__ __forceinline__ void store_master(uint32_t tPhi, int q, int h, int ng
 // thread, i.e. nT3 * n3p <= 128 (the plan enforces it)
 constexpr int kMasterGroups = 4;
 
+// One accumulation over KS K steps: main += A_hi B_hi and, for the split precisions, cross += A_hi B_lo +
+// A_lo B_hi.  Descriptors advance by constants from a per-term base and the steps are unrolled: the
+// issuing warp, not the tensor pipe, bounds small tiles.
+template <bool TF32, bool SPLIT, int KS>
+__device__ __forceinline__ void cv_mmas_k(uint32_t d, uint32_t dc, uint64_t ad, uint64_t bd, uint32_t as, uint32_t bs,
+                                          uint32_t al, uint32_t bl, uint32_t id, uint32_t acc0) {
+#pragma unroll
+    for (int k = 0; k < KS; ++k) {
+        const uint32_t acc = k > 0 ? 1u : acc0;
+        const uint64_t a = ad + (uint32_t)k * as, b = bd + (uint32_t)k * bs;
+        mma_ss_w<TF32>(d, a, b, id, acc);
+        if constexpr (SPLIT) {
+            mma_ss_w<TF32>(dc, a, b + bl, id, acc);
+            mma_ss_w<TF32>(dc, a + al, b, id, 1u);
+        }
+    }
+}
 template <bool TF32, bool SPLIT>
+__device__ __forceinline__ void cv_mmas(int ks, uint32_t d, uint32_t dc, uint64_t ad, uint64_t bd, uint32_t as, uint32_t bs,
+                                        uint32_t al, uint32_t bl, uint32_t id, uint32_t acc0) {
+    switch (ks) {
+        case 2: cv_mmas_k<TF32, SPLIT, 2>(d, dc, ad, bd, as, bs, al, bl, id, acc0); break;
+        case 3: cv_mmas_k<TF32, SPLIT, 3>(d, dc, ad, bd, as, bs, al, bl, id, acc0); break;
+        case 4: cv_mmas_k<TF32, SPLIT, 4>(d, dc, ad, bd, as, bs, al, bl, id, acc0); break;
+        case 5: cv_mmas_k<TF32, SPLIT, 5>(d, dc, ad, bd, as, bs, al, bl, id, acc0); break;
+        case 6: cv_mmas_k<TF32, SPLIT, 6>(d, dc, ad, bd, as, bs, al, bl, id, acc0); break;
+        case 8: cv_mmas_k<TF32, SPLIT, 8>(d, dc, ad, bd, as, bs, al, bl, id, acc0); break;
+        default:
+            for (int k = 0; k < ks; ++k) {
+                const uint32_t acc = k > 0 ? 1u : acc0;
+                const uint64_t a = ad + (uint32_t)k * as, b = bd + (uint32_t)k * bs;
+                mma_ss_w<TF32>(d, a, b, id, acc);
+                if constexpr (SPLIT) {
+                    mma_ss_w<TF32>(dc, a, b + bl, id, acc);
+                    mma_ss_w<TF32>(dc, a + al, b, id, 1u);
+                }
+            }
+    }
+}
+
+// Stage 3 with A in TMEM: hi at column a, lo at column al (8 columns per K step)
+template <int KS>
+__device__ __forceinline__ void cv_mmas_ts_k(uint32_t d, uint32_t dc, uint32_t a, uint32_t al, uint64_t bd, uint32_t bs,
+                                             uint32_t bl, uint32_t id, uint32_t acc0) {
+#pragma unroll
+    for (int k = 0; k < KS; ++k) {
+        const uint32_t acc = k > 0 ? 1u : acc0;
+        const uint64_t b = bd + (uint32_t)k * bs;
+        mma_ts_tf32_w(d, a + 8u * k, b, id, acc);
+        mma_ts_tf32_w(dc, a + 8u * k, b + bl, id, acc);
+        mma_ts_tf32_w(dc, al + 8u * k, b, id, 1u);
+    }
+}
+__device__ __forceinline__ void cv_mmas_ts(int ks, uint32_t d, uint32_t dc, uint32_t a, uint32_t al, uint64_t bd, uint32_t bs,
+                                           uint32_t bl, uint32_t id, uint32_t acc0) {
+    switch (ks) {
+        case 2: cv_mmas_ts_k<2>(d, dc, a, al, bd, bs, bl, id, acc0); break;
+        case 3: cv_mmas_ts_k<3>(d, dc, a, al, bd, bs, bl, id, acc0); break;
+        case 4: cv_mmas_ts_k<4>(d, dc, a, al, bd, bs, bl, id, acc0); break;
+        case 5: cv_mmas_ts_k<5>(d, dc, a, al, bd, bs, bl, id, acc0); break;
+        case 6: cv_mmas_ts_k<6>(d, dc, a, al, bd, bs, bl, id, acc0); break;
+        case 8: cv_mmas_ts_k<8>(d, dc, a, al, bd, bs, bl, id, acc0); break;
+        default:
+            for (int k = 0; k < ks; ++k) {
+                const uint32_t acc = k > 0 ? 1u : acc0;
+                const uint64_t b = bd + (uint32_t)k * bs;
+                mma_ts_tf32_w(d, a + 8u * k, b, id, acc);
+                mma_ts_tf32_w(dc, a + 8u * k, b + bl, id, acc);
+                mma_ts_tf32_w(dc, al + 8u * k, b, id, 1u);
+            }
+    }
+}
+
+// The converter kernel (split precisions; single-pass shapes that no TMEM plan holds).  Every role is
+// a stage of one pipeline over the terms, each on warps of its own and one or two terms apart:
+//   8, 10  producers of A_t2 and mu_t A_t3, and of Z (tile copies are issued by one lane each)
+//   9      stage-2 MMAs into rotating Y buffers
+//   0-7    converters: Y -> hi + lo stage-3 operand, then the fold of the PREVIOUS term's phi
+//   11     stage-3 MMAs
+// A converter warp takes one TMEM lane quadrant and every other 16-column group.  The fold of term
+// t - 1 comes after the conversion of term t, so stage 3 of t - 1 runs under that conversion and the only
+// serial chain is stage 3 -> fold -> stage 3.  Operand sub-tiles keep just the rows they need (the MMA's
+// rows beyond them read the next sub-tile and land in lanes nobody reads), which is what lets every ring
+// hold two stages on a 96 x 96 plane.
+// TS3 (TF32x3, planes of more than 64 rows): hi and lo go back into the main and cross columns of Y
+// itself and stage 3 reads A from TMEM.  The converted operand's stores and the tensor core's reads of
+// it took over half of the shared-memory bandwidth, which bound the kernel: a clock64 trace showed 6,500
+// cycles per conversion under the MMAs' reads, 3,300 alone.  (Planes of up to 64 rows pack two planes
+// into one 128-row operand in shared memory, which TMEM lanes cannot do.)
+// Pt-shaped pair (14 terms): 27.2 us; 33.8 with the operand in shared memory, 44.6 with one
+// issuing lane for all MMAs, one for all copies and the fold before the next conversion.
+template <bool TF32, bool SPLIT, bool TS3>
 __global__ void __launch_bounds__(kThreads, 1)
     k_consume(const __grid_constant__ CUtensorMap mZ, const __grid_constant__ CUtensorMap mZlo,
               const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mA2lo,
@@ -434,10 +525,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int MK = TF32 ? 8 : 16;        // K per MMA instruction (32 bytes)
     constexpr int ES = TF32 ? 4 : 2;         // operand element bytes
     constexpr int CV = 16 / ES;              // values per 16-byte chunk
+    constexpr uint32_t M = SPLIT ? 2u : 1u;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[kMaxLoad], empty_bar[kMaxLoad], a3full[2], a3free[2], phidone;
+    __shared__ uint64_t fullA[kMaxLoad], fullZ[kMaxLoad], empty_bar[kMaxLoad], a3full[kMaxYCv], a3free[2], phidone, s2fin;
     __shared__ uint64_t fullB[kMaxLoadB], emptyB[kMaxLoadB];
-    __shared__ uint64_t yfull, yfree, chunkdone, phifree;
+    __shared__ uint64_t yfull[kMaxYCv], yfree[kMaxYCv], chunkdone, phifree;
     __shared__ uint32_t tmem_base;
     __shared__ double red[8];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -449,49 +541,49 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int y0 = a.yz ? (iyz / a.nzi) * 128 : 0, z0 = a.yz ? (iyz % a.nzi) * a.n3p : 0;
     const int x0 = slab * a.bx;
     const PairRec rec = a.recs[a.p0 + pl];
-    const int NL = a.nload, NA = a.na3, BX = a.bx;
+    const int NL = a.nload, NA = a.na3, NB = a.nloadB, NYB = a.nyb, BX = a.bx, NT = a.nt;
     // Split precisions: the tensor core rounds its float32 accumulator after every MMA, toward
     // zero, so the error of a long accumulation grows with its length.  The hi*hi products and
     // the cross products (hi*lo + lo*hi, 2^-11 smaller) go to separate accumulators, and phi is
     // accumulated on the tensor core over chunks of C terms only (default 1): after each chunk
     // the converter warps add both accumulators into a float32 register accumulator (round to
     // nearest) and the tensor core restarts.  Single-pass precisions accumulate every term.
-    const int C = SPLIT ? (a.chunk > 0 ? a.chunk : 1) : a.nt;
-    // Gaussian terms in the order of the exponential sum (theta ascending: wide terms first)
-    auto term_of = [&](int t) { return t; };
+    const int C = SPLIT ? (a.chunk > 0 ? a.chunk : 1) : NT;
 
     // load stage s: [A_t2 tile][Z tile], each hi then lo; stage-3 stage sb: [A_t3 tile] hi then lo;
     // then the NA converted stage-3 operands
-    const int NB = a.nloadB;
     auto YAs = [&](int s) { return smem + s * a.load_bytes; };
-    auto Zs = [&](int s) { return YAs(s) + (SPLIT ? 2 : 1) * a.ya_bytes; };
+    auto Zs = [&](int s) { return YAs(s) + M * a.ya_bytes; };
     auto B3s = [&](int sb) { return smem + a.b_off + sb * a.loadB_bytes; };
-    auto A3s = [&](int b) { return smem + a.a3_off + b * (SPLIT ? 2 : 1) * a.a3_bytes; };
+    auto A3s = [&](int b) { return smem + a.a3_off + b * M * a.a3_bytes; };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxLoad; ++s) {
-            mbar_init(&full_bar[s], 1);
+            mbar_init(&fullA[s], 1);
+            mbar_init(&fullZ[s], 1);
             mbar_init(&empty_bar[s], 1);
         }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&a3full[b], 8);
-            mbar_init(&a3free[b], 1);
+        // TS3: a3full is per Y buffer (its conversion), and stage 3 frees the buffer
+        for (int b = 0; b < kMaxYCv; ++b) {
+            mbar_init(&a3full[b], TS3 ? 2 * a.nq : 8);
+            mbar_init(&yfull[b], 1);
+            mbar_init(&yfree[b], TS3 ? 1 : 2 * a.nq);
         }
+        for (int b = 0; b < 2; ++b) mbar_init(&a3free[b], 1);
         for (int b = 0; b < kMaxLoadB; ++b) {
             mbar_init(&fullB[b], 1);
             mbar_init(&emptyB[b], 1);
         }
-        mbar_init(&yfull, 1);
-        mbar_init(&yfree, 2 * a.nq);
         mbar_init(&phidone, 1);
+        mbar_init(&s2fin, 1);
         mbar_init(&chunkdone, 1);
         mbar_init(&phifree, 8);
         fence_barrier_init();
     }
     // the stage-3 operand: rows past the slab's last (x, y) are never written and must be finite
-    {
+    if constexpr (!TS3) {
         uint4* p = (uint4*)A3s(0);
-        const int n16 = NA * (SPLIT ? 2 : 1) * a.a3_bytes / 16;
+        const int n16 = NA * (int)(M * a.a3_bytes) / 16;
         for (int i = threadIdx.x; i < n16; i += kThreads) p[i] = make_uint4(0, 0, 0, 0);
     }
     fence_async_smem();
@@ -503,180 +595,161 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base;
-    // TMEM: [Y][phi] for the single-pass precisions; [Y][Y cross][phi][phi cross] for the split ones
-    const uint32_t phi_cols = (uint32_t)(a.nT3 * a.n3p);
-    const uint32_t tY = tmem, tYc = tmem + a.y_cols;
-    const uint32_t tPhi = tmem + (SPLIT ? 2u : 1u) * a.y_cols, tPhiC = tPhi + phi_cols;
+    // TMEM: NYB x [Y][Y cross], then [phi][phi cross] (no cross accumulators in the single-pass precisions)
+    const uint32_t phi_cols = (uint32_t)(a.nT3 * a.n3p), y_stride = M * a.y_cols;
+    const uint32_t tPhi = tmem + (uint32_t)NYB * y_stride, tPhiC = tPhi + phi_cols;
     const uint32_t ya_sub = a.ya_rows * 32u;                  // one K-step sub-tile of each operand
     const uint32_t z_sub = a.z_rows * 32u;
-    const uint32_t a3_sub = (uint32_t)a.nT3 * 128u * 32u;
+    const uint32_t a3_sub = a.a3_rows * 32u;
 
     if (warp == 8) {
-        // ------------------------------ TMA producers ------------------------------
-        // lane 0: the [A_t2][Z] ring; lane 1: the [mu_t A_t3] ring (each waits on its own ring)
-        if (lane == 1) {
-            int issued = 0;
-            for (int t = 0; t < a.nt; ++t) {
-                const int sb = t % NB;
-                if (!mbar_wait(&emptyB[sb], ((t / NB) & 1) ^ 1, a.err, 39)) break;
-                issued = t + 1;
-                mbar_arrive_expect_tx(&fullB[sb], a.stageB_tx);
-                const int tt = term_of(t);
-                for (int k = 0; k < a.ks3; ++k) {
-                    tma_load_3d(B3s(sb) + k * a.n3p * 32u, &mA3, &fullB[sb], k * MK, z0, tt);
-                    if constexpr (SPLIT)
-                        tma_load_3d(B3s(sb) + a.b3_bytes + k * a.n3p * 32u, &mA3lo, &fullB[sb], k * MK, z0, tt);
-                }
-            }
-            if (issued < a.nt)
-                for (int t = (issued > NB ? issued - NB : 0); t < issued; ++t)
-                    mbar_drain(&fullB[t % NB], (t / NB) & 1, a.err);
-        }
+        // ------------------------------ producer: A_t2 and mu_t A_t3 ------------------------------
+        // (the wait for a stage-3 stage holds up the next A_t2 by at most the slack that the conversion and
+        // stage 3 of the term before give it)
         if (lane == 0) {
-            int issued = 0;
-            bool ok = true;
-            for (int t = 0; t < a.nt && ok; ++t) {
-                const int s = t % NL;
-                if (!mbar_wait(&empty_bar[s], ((t / NL) & 1) ^ 1, a.err, 31)) { ok = false; break; }
-                issued = t + 1;
-                // start the HBM reads of later Z tiles early (into L2 only)
-                for (int ahead = (t == 0 ? 1 : NL + 1); ahead <= NL + 1; ++ahead)
-                    if (t + ahead < a.nt)
-                        for (int p = 0; p < BX; ++p)
-                            for (int k = 0; k < a.ks2; ++k)
-                                tma_prefetch_l2_3d(&mZ, k * MK, (x0 + p) * a.r3, pl * a.nt + term_of(t + ahead));
-                mbar_arrive_expect_tx(&full_bar[s], a.stage_tx);
-                const int tt = term_of(t);
-                const int zdep = pl * a.nt + tt;
+            int ia = 0, ib = 0, s = 0, sb = 0;
+            uint32_t ph = 0, bph = 0;
+            for (int t = 0; t < NT; ++t) {
+                if (!mbar_wait(&empty_bar[s], ph ^ 1, a.err, 31)) break;
+                ia = t + 1;
+                mbar_arrive_expect_tx(&fullA[s], a.stage_tx);
                 for (int k = 0; k < a.ks2; ++k) {
-                    tma_load_3d(YAs(s) + k * ya_sub, &mA2, &full_bar[s], k * MK, y0, tt);
-                    if constexpr (SPLIT) tma_load_3d(YAs(s) + a.ya_bytes + k * ya_sub, &mA2lo, &full_bar[s], k * MK, y0, tt);
+                    tma_load_3d(YAs(s) + k * ya_sub, &mA2, &fullA[s], k * MK, y0, t);
+                    if constexpr (SPLIT) tma_load_3d(YAs(s) + a.ya_bytes + k * ya_sub, &mA2lo, &fullA[s], k * MK, y0, t);
+                }
+                if (++s == NL) { s = 0; ph ^= 1; }
+                if (!mbar_wait(&emptyB[sb], bph ^ 1, a.err, 39)) break;
+                ib = t + 1;
+                mbar_arrive_expect_tx(&fullB[sb], a.stageB_tx);
+                for (int k = 0; k < a.ks3; ++k) {
+                    tma_load_3d(B3s(sb) + k * a.n3p * 32u, &mA3, &fullB[sb], k * MK, z0, t);
+                    if constexpr (SPLIT)
+                        tma_load_3d(B3s(sb) + a.b3_bytes + k * a.n3p * 32u, &mA3lo, &fullB[sb], k * MK, z0, t);
+                }
+                if (++sb == NB) { sb = 0; bph ^= 1; }
+            }
+            if (ia < NT || ib < NT) {
+                for (int t = (ia > NL ? ia - NL : 0); t < ia; ++t) mbar_drain(&fullA[t % NL], (t / NL) & 1, a.err);
+                for (int t = (ib > NB ? ib - NB : 0); t < ib; ++t) mbar_drain(&fullB[t % NB], (t / NB) & 1, a.err);
+            }
+        }
+    } else if (warp == 10) {
+        // ------------------------------ producer: Z ------------------------------
+        if (lane == 0) {
+            int issued = 0, s = 0;
+            uint32_t ph = 0;
+            for (int t = 0; t < NT; ++t) {
+                if (!mbar_wait(&empty_bar[s], ph ^ 1, a.err, 40)) break;
+                issued = t + 1;
+                mbar_arrive_expect_tx(&fullZ[s], a.stageZ_tx);
+                const int zdep = pl * NT + t;
+                for (int k = 0; k < a.ks2; ++k)
                     // plane p's rows start at row p * Nz (a multiple of 16) of the Z tile
                     for (int p = 0; p < BX; ++p) {
                         const uint32_t off = k * z_sub + (uint32_t)(p * a.Nz) * 32u;
-                        tma_load_3d(Zs(s) + off, &mZ, &full_bar[s], k * MK, (x0 + p) * a.r3, zdep);
+                        tma_load_3d(Zs(s) + off, &mZ, &fullZ[s], k * MK, (x0 + p) * a.r3, zdep);
                         if constexpr (SPLIT)
-                            tma_load_3d(Zs(s) + a.z_bytes + off, &mZlo, &full_bar[s], k * MK, (x0 + p) * a.r3, zdep);
+                            tma_load_3d(Zs(s) + a.z_bytes + off, &mZlo, &fullZ[s], k * MK, (x0 + p) * a.r3, zdep);
                     }
-                }
+                // start the HBM reads of later Z tiles early (into L2 only)
+                for (int ahead = (t == 0 ? 1 : NL + 1); ahead <= NL + 1; ++ahead)
+                    if (t + ahead < NT)
+                        for (int p = 0; p < BX; ++p)
+                            for (int k = 0; k < a.ks2; ++k) {
+                                tma_prefetch_l2_3d(&mZ, k * MK, (x0 + p) * a.r3, zdep + ahead);
+                                if constexpr (SPLIT) tma_prefetch_l2_3d(&mZlo, k * MK, (x0 + p) * a.r3, zdep + ahead);
+                            }
+                if (++s == NL) { s = 0; ph ^= 1; }
             }
-            if (!ok)
-                for (int t = (issued > NL ? issued - NL : 0); t < issued; ++t)
-                    mbar_drain(&full_bar[t % NL], (t / NL) & 1, a.err);
+            if (issued < NT)
+                for (int t = (issued > NL ? issued - NL : 0); t < issued; ++t) mbar_drain(&fullZ[t % NL], (t / NL) & 1, a.err);
         }
     } else if (warp == 9) {
-        // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
-            const uint32_t id3 = TF32 ? idesc_tf32(128, a.n3p) : idesc_bf16(128, a.n3p);
-            // Event-driven issue: stage 2 of term t2 as soon as its load stage has landed and the
-            // converters have released Y; stage 3 of term t3 as soon as its operand is converted
-            // (and, at the start of an accumulation chunk, the previous chunk has been folded).
-            // All planes of a term go in one MMA per K step (N = planes x Nz, in chunks of <= 256).
-            // Descriptors are built once and advanced by adds.
-            const uint64_t d0 = sdesc_sw32(0);
-            const uint64_t ya_step = ya_sub >> 4, z_step = z_sub >> 4, b3_step = (uint32_t)a.n3p * 2u;
-            const uint64_t a3_step = a3_sub >> 4, ya_lo = a.ya_bytes >> 4, z_lo = a.z_bytes >> 4;
-            const uint64_t b3_lo = a.b3_bytes >> 4, a3_lo = a.a3_bytes >> 4;
-            auto stage2 = [&](int t) {
-                const int s = t % NL;
-                const uint64_t ya = d0 + (smem_u32(YAs(s)) >> 4), zb = d0 + (smem_u32(Zs(s)) >> 4);
-                for (int i = 0; i < a.nY; ++i)
-                    for (int p0 = 0; p0 < BX; p0 += a.npc) {
-                        const int N = min(a.npc, BX - p0) * a.Nz;
-                        const uint32_t id2 = TF32 ? idesc_tf32(128, N) : idesc_bf16(128, N);
-                        const uint32_t col = (uint32_t)((i * BX + p0) * a.Nz);
-                        uint64_t ad = ya + (uint32_t)i * 256u, bd = zb + (uint32_t)(p0 * a.Nz) * 2u;
-                        for (int k = 0; k < a.ks2; ++k) {
-                            mma_ss<TF32>(tY + col, ad, bd, id2, k > 0 ? 1u : 0u);
-                            if constexpr (SPLIT) {
-                                mma_ss<TF32>(tYc + col, ad, bd + z_lo, id2, k > 0 ? 1u : 0u);
-                                mma_ss<TF32>(tYc + col, ad + ya_lo, bd, id2, 1u);
-                            }
-                            ad += ya_step;
-                            bd += z_step;
-                        }
-                    }
-                mma_commit(&yfull);
-                mma_commit(&empty_bar[s]);          // the [A_t2][Z] stage is free once these have run
-            };
-            auto stage3 = [&](int t) {
-                const int sb = t % NB, b = t % NA;
-                const uint64_t a3 = d0 + (smem_u32(A3s(b)) >> 4), b3 = d0 + (smem_u32(B3s(sb)) >> 4);
-                const bool first = (t % C) == 0;
-                for (int j = 0; j < a.nT3; ++j) {
-                    uint64_t ad = a3 + (uint32_t)j * 256u, bd = b3;
-                    for (int k = 0; k < a.ks3; ++k) {
-                        const uint32_t acc = (!first || k > 0) ? 1u : 0u;
-                        mma_ss<TF32>(tPhi + j * a.n3p, ad, bd, id3, acc);
-                        if constexpr (SPLIT) {
-                            mma_ss<TF32>(tPhiC + j * a.n3p, ad, bd + b3_lo, id3, acc);
-                            mma_ss<TF32>(tPhiC + j * a.n3p, ad + a3_lo, bd, id3, 1u);
-                        }
-                        ad += a3_step;
-                        bd += b3_step;
-                    }
+        // ------------------------------ stage-2 MMAs ------------------------------
+        // all planes of a term go in one MMA per K step (N = planes x Nz, in chunks of <= 256)
+        const uint64_t d0 = sdesc_sw32(0);
+        int s = 0, yb = 0;
+        uint32_t ph = 0, yph = 0;
+        for (int t = 0; t < NT; ++t) {
+            bool w = mbar_wait(&fullA[s], ph, a.err, 32);
+            if (w) w = mbar_wait(&fullZ[s], ph, a.err, 33);
+            if (w && t >= NYB) w = mbar_wait(&yfree[yb], yph ^ 1, a.err, 34);     // conversion of term t - NYB
+            if (!__all_sync(0xffffffffu, w)) break;
+            tc_fence_after();
+            const uint64_t ya = d0 + (smem_u32(YAs(s)) >> 4), zb = d0 + (smem_u32(Zs(s)) >> 4);
+            const uint32_t tY = tmem + (uint32_t)yb * y_stride;
+            for (int i = 0; i < a.nY; ++i)
+                for (int p0 = 0; p0 < BX; p0 += a.npc) {
+                    const int N = min(a.npc, BX - p0) * a.Nz;
+                    const uint32_t id2 = TF32 ? idesc_tf32(128, N) : idesc_bf16(128, N);
+                    const uint32_t col = tY + (uint32_t)((i * BX + p0) * a.Nz);
+                    cv_mmas<TF32, SPLIT>(a.ks2, col, col + a.y_cols, ya + (uint32_t)i * 256u,
+                                         zb + (uint32_t)(p0 * a.Nz) * 2u, ya_sub >> 4, z_sub >> 4, a.ya_bytes >> 4,
+                                         a.z_bytes >> 4, id2, 0u);
                 }
-                mma_commit(&a3free[b]);
-                mma_commit(&emptyB[sb]);
-            };
-            bool ok = true, fresh = true;
-            int t2 = 0, t3 = 0;
-            uint32_t idle = 0;
-            uint64_t since = 0;
-            while (t3 < a.nt) {
-                bool prog = false;
-                if (t2 < a.nt && mbar_try_wait(&full_bar[t2 % NL], (t2 / NL) & 1) &&
-                    (t2 == 0 || mbar_try_wait(&yfree, (t2 - 1) & 1))) {
-                    tc_fence_after();
-                    stage2(t2);
-                    ++t2;
-                    prog = true;
-                }
-                // a new accumulation chunk starts once the previous one has been folded out of TMEM
-                if (t3 < t2 && mbar_try_wait(&a3full[t3 % NA], (t3 / NA) & 1) &&
-                    mbar_try_wait(&fullB[t3 % NB], (t3 / NB) & 1) &&
-                    (t3 % C != 0 || t3 == 0 || mbar_try_wait(&phifree, (t3 / C - 1) & 1))) {
-                    tc_fence_after();
-                    stage3(t3);
-                    if constexpr (SPLIT)
-                        if ((t3 + 1) % C == 0 || t3 + 1 == a.nt) mma_commit(&chunkdone);
-                    ++t3;
-                    prog = true;
-                }
-                if (prog) {
-                    fresh = true;
-                    idle = 0;
-                } else if ((++idle & 63) == 0) {
-                    if (*(volatile int*)a.err != 0) { ok = false; break; }
-                    const uint64_t now = globaltimer();
-                    if (fresh) {
-                        since = now;
-                        fresh = false;
-                    } else if (now - since > wait_limit_ns(a.err)) {
-                        if (atomicCAS(a.err, 0, 1) == 0) atomicExch(a.err + 1, 32);
-                        ok = false;
-                        break;
-                    }
-                }
-            }
-            mma_commit(&phidone);
-            // on the error path nobody else waits: keep the CTA (and its TMEM) until the MMAs
-            // already issued have finished
-            if (!ok) mbar_drain(&phidone, 0, a.err);
+            mma_commit_w(&yfull[yb]);
+            mma_commit_w(&empty_bar[s]);          // the [A_t2][Z] stage is free once these have run
+            if (++s == NL) { s = 0; ph ^= 1; }
+            if (++yb == NYB) { yb = 0; yph ^= 1; }
         }
+        // the CTA must not release TMEM while these MMAs run
+        mma_commit_w(&s2fin);
+        mbar_drain(&s2fin, 0, a.err);
+    } else if (warp == 11) {
+        // ------------------------------ stage-3 MMAs ------------------------------
+        const uint32_t id3 = TF32 ? idesc_tf32(128, a.n3p) : idesc_bf16(128, a.n3p);
+        const uint64_t d0 = sdesc_sw32(0);
+        int b = 0, sb = 0, in_chunk = 0;
+        uint32_t aph = 0, bph = 0, cph = 1;                  // cph: parity of the last folded chunk
+        bool ok = true;
+        for (int t = 0; t < NT; ++t) {
+            bool w = mbar_wait(&a3full[b], aph, a.err, 35);
+            if (w) w = mbar_wait(&fullB[sb], bph, a.err, 36);
+            // a new accumulation chunk starts once the previous one has been folded out of TMEM
+            if (SPLIT && w && in_chunk == 0 && t > 0) w = mbar_wait(&phifree, cph, a.err, 37);
+            if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
+            tc_fence_after();
+            const uint64_t b3 = d0 + (smem_u32(B3s(sb)) >> 4);
+            const uint32_t acc0 = in_chunk > 0 ? 1u : 0u;
+            if constexpr (TS3) {
+                const uint32_t tY = tmem + (uint32_t)b * y_stride;
+                for (int j = 0; j < a.nT3; ++j)          // one plane: tile j = y tile j
+                    cv_mmas_ts(a.ks3, tPhi + j * a.n3p, tPhiC + j * a.n3p, tY + (uint32_t)(j * a.Nz),
+                               tY + a.y_cols + (uint32_t)(j * a.Nz), b3, (uint32_t)a.n3p * 2u, a.b3_bytes >> 4, id3, acc0);
+            } else {
+                const uint64_t a3 = d0 + (smem_u32(A3s(b)) >> 4);
+                for (int j = 0; j < a.nT3; ++j)
+                    cv_mmas<TF32, SPLIT>(a.ks3, tPhi + j * a.n3p, tPhiC + j * a.n3p, a3 + (uint32_t)j * 256u, b3,
+                                         a3_sub >> 4, (uint32_t)a.n3p * 2u, a.a3_bytes >> 4, a.b3_bytes >> 4, id3, acc0);
+            }
+            if (++in_chunk == C || t + 1 == NT) {
+                if constexpr (SPLIT) mma_commit_w(&chunkdone);
+                in_chunk = 0;
+                cph ^= 1;
+            }
+            mma_commit_w(TS3 ? &yfree[b] : &a3free[b]);
+            mma_commit_w(&emptyB[sb]);
+            if (++b == (TS3 ? NYB : NA)) { b = 0; aph ^= 1; }
+            if (++sb == NB) { sb = 0; bph ^= 1; }
+        }
+        mma_commit_w(&phidone);
+        // on the error path nobody else waits: keep the CTA (and its TMEM) until the MMAs
+        // already issued have finished
+        if (!ok) mbar_drain(&phidone, 0, a.err);
     } else {
         // ------------------------------ converters (warps 0-7) ------------------------------
-        // warp (q, h) converts the TMEM lanes 32q..32q+31 (y) of the planes p = h, h + 2, ...
+        // warp (q, h) takes the TMEM lanes 32q .. 32q + 31 (y) of the 16-column groups h, h + 2, ... of Y
+        // (plane by plane) and of phi
         const int q = warp & 3, h = warp >> 2;
         const bool active = q < a.nq;
         bool ok = true;
         double e = 0.0;
         auto rows_of = [&](int jt, int r, int& x, int& y) {
             const int m3 = jt * 128 + r;
-            if (a.yz) {                      // one plane, rows y0 .. y0 + 127
+            if (a.yz || TS3) {               // one plane, rows from y0 on
                 y = y0 + m3;
                 x = x0;
-                return m3 < 128 && y < a.n2 && x < a.n1;
+                return (!a.yz || m3 < 128) && y < a.n2 && x < a.n1;
             }
             const int xl = m3 / a.n2;
             y = m3 - xl * a.n2;
@@ -687,83 +760,109 @@ __global__ void __launch_bounds__(kThreads, 1)
         float mst[kMasterGroups * 16];
 #pragma unroll
         for (int j = 0; j < kMasterGroups * 16; ++j) mst[j] = 0.f;
-        for (int t = 0; t < a.nt && ok; ++t) {
-            const int b = t % NA;
-            if (t >= NA && !mbar_wait(&a3free[b], ((t - NA) / NA) & 1, a.err, 36)) { ok = false; break; }
-            uint8_t* a3 = A3s(b);
+        uint32_t fph = 0;                    // parity of the next chunk to fold
+        auto fold = [&]() -> bool {
+            if (!mbar_wait(&chunkdone, fph, a.err, 38)) return false;
+            fph ^= 1;
+            tc_fence_after();
+            fold_chunk<kMasterGroups>(tPhi, tPhiC, q, h, ngroups, mst);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&phifree);
+            return true;
+        };
+        const int ngz = a.Nz / 16, nunits = BX * a.nY * ngz;
+        // 16 columns of Y (plane p, y tile i, first column g0) of this warp's lanes into the operand
+        auto put = [&](uint8_t* a3, int u, const uint32_t (&r)[16], const uint32_t (&rc)[16]) {
+            const int pi = u / ngz, g0 = 16 * (u - pi * ngz), i = pi / BX, p = pi - i * BX;
+            const int y = i * 128 + q * 32 + lane;
+            if (y0 + y >= a.n2) return;
+            const uint32_t m3 = (uint32_t)(a.yz ? y : p * a.n2 + y);
+#pragma unroll
+            for (int k = 0; k < 16 / CV; ++k) {
+                const int g = g0 + CV * k;                   // first column of the 16-byte chunk
+                if (g >= a.r3) continue;
+                float v[CV];
+#pragma unroll
+                for (int c = 0; c < CV; ++c) {
+                    float f = __uint_as_float(r[CV * k + c]);
+                    if constexpr (SPLIT) f += __uint_as_float(rc[CV * k + c]);      // Y = main + cross accumulator
+                    v[c] = g + c < a.r3 ? f : 0.f;
+                }
+                uint4 hi, lo;
+                convert_chunk<TF32, SPLIT>(v, hi, lo);
+                uint8_t* dst = a3 + (uint32_t)(g / MK) * a3_sub + sw32_offset(m3, (uint32_t)((g % MK) * ES));
+                *(uint4*)dst = hi;
+                if constexpr (SPLIT) *(uint4*)(dst + a.a3_bytes) = lo;
+            }
+        };
+        // the same in place: hi into the main columns, lo into the cross columns (zeros past r3)
+        auto put_tmem = [&](uint32_t col, int u, uint32_t (&r)[16], uint32_t (&rc)[16]) {
+            const int g0 = 16 * (u % ngz);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                const float v = g0 + c < a.r3 ? __uint_as_float(r[c]) + __uint_as_float(rc[c]) : 0.f;
+                const float hi = tf32_rna(v);
+                r[c] = __float_as_uint(hi);
+                rc[c] = __float_as_uint(tf32_rna(v - hi));
+            }
+            tmem_st16(col, r);
+            tmem_st16(col + a.y_cols, rc);
+        };
+        int b = 0, yb = 0, in_chunk = 0;
+        uint32_t aph = 0, yph = 0;
+        for (int t = 0; t < NT; ++t) {
+            if (!TS3 && t >= NA && !mbar_wait(&a3free[b], aph ^ 1, a.err, 41)) { ok = false; break; }
+            uint8_t* a3 = A3s(TS3 ? 0 : b);
             if (active) {
-                if (!mbar_wait(&yfull, t & 1, a.err, 35)) { ok = false; break; }
+                if (!mbar_wait(&yfull[yb], yph, a.err, 42)) { ok = false; break; }
                 tc_fence_after();
-                for (int p = h; p < BX; p += 2) {
-                    for (int i = 0; i < a.nY; ++i) {
-                        const int y = i * 128 + q * 32 + lane;
-                        const bool valid = y0 + y < a.n2;
-                        const uint32_t m3 = (uint32_t)(a.yz ? y : p * a.n2 + y);
-                        const uint32_t col = tY + ((uint32_t)(q * 32) << 16) + (uint32_t)((i * BX + p) * a.Nz);
-                        for (int g0 = 0; g0 < a.r3; g0 += 64) {
-                            const int nck = min(4, (min(a.Nz, g0 + 64) - g0) / 16);
-                            uint32_t r[4][16];
-#pragma unroll
-                            for (int c = 0; c < 4; ++c)
-                                if (c < nck) tmem_ld16(col + g0 + 16 * c, r[c]);
-                            tmem_ld_wait();
-                            if constexpr (SPLIT) {
-                                // Y = main + cross accumulator
-#pragma unroll
-                                for (int c = 0; c < 4; ++c)
-                                    if (c < nck) {
-                                        uint32_t rc[16];
-                                        tmem_ld16(col + a.y_cols + g0 + 16 * c, rc);
-                                        tmem_ld_wait();
-#pragma unroll
-                                        for (int j = 0; j < 16; ++j)
-                                            r[c][j] = __float_as_uint(__uint_as_float(r[c][j]) + __uint_as_float(rc[j]));
-                                    }
-                            }
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                if (c >= nck) break;
-#pragma unroll
-                                for (int u = 0; u < 16 / CV; ++u) {
-                                    const int g = g0 + 16 * c + CV * u;          // first column of the chunk
-                                    if (!valid || g >= a.r3) continue;
-                                    float v[CV];
-#pragma unroll
-                                    for (int e = 0; e < CV; ++e)
-                                        v[e] = (g + e < a.r3) ? __uint_as_float(r[c][CV * u + e]) : 0.f;
-                                    uint4 hi, lo;
-                                    convert_chunk<TF32, SPLIT>(v, hi, lo);
-                                    const uint32_t ks = (uint32_t)(g / MK), bin = (uint32_t)((g % MK) * ES);
-                                    uint8_t* dst = a3 + ks * a3_sub + sw32_offset(m3, bin);
-                                    *(uint4*)dst = hi;
-                                    if constexpr (SPLIT) *(uint4*)(dst + a.a3_bytes) = lo;
-                                }
-                            }
-                        }
+                const uint32_t tY = tmem + (uint32_t)yb * y_stride + ((uint32_t)(q * 32) << 16);
+                // two groups in flight per TMEM round trip
+                for (int u = h; u < nunits; u += 4) {
+                    uint32_t r0[16], c0[16], r1[16], c1[16];
+                    const bool two = u + 2 < nunits;
+                    const uint32_t col0 = tY + (uint32_t)(16 * u), col1 = col0 + 32u;   // (i BX + p) Nz + g0 = 16 u
+                    tmem_ld16(col0, r0);
+                    if constexpr (SPLIT) tmem_ld16(col0 + a.y_cols, c0);
+                    if (two) {
+                        tmem_ld16(col1, r1);
+                        if constexpr (SPLIT) tmem_ld16(col1 + a.y_cols, c1);
+                    }
+                    tmem_ld_wait();
+                    if constexpr (TS3) {
+                        put_tmem(col0, u, r0, c0);
+                        if (two) put_tmem(col1, u + 2, r1, c1);
+                    } else {
+                        put(a3, u, r0, c0);
+                        if (two) put(a3, u + 2, r1, c1);
                     }
                 }
+                if constexpr (TS3) tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&yfree);
+                if (lane == 0) mbar_arrive(TS3 ? &a3full[yb] : &yfree[yb]);
             }
-            fence_async_smem();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&a3full[b]);
+            if constexpr (!TS3) {
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&a3full[b]);
+            }
             if constexpr (SPLIT) {
-                // end of an accumulation chunk: fold phi into the register accumulator and let
-                // the tensor core restart
-                if ((t + 1) % C == 0 || t + 1 == a.nt) {
-                    if (!mbar_wait(&chunkdone, (t / C) & 1, a.err, 38)) { ok = false; break; }
-                    tc_fence_after();
-                    fold_chunk<kMasterGroups>(tPhi, tPhiC, q, h, ngroups, mst);
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&phifree);
+                // the previous chunk of phi, now that this term's operand is on its way
+                if (in_chunk == C) {
+                    if (!fold()) { ok = false; break; }
+                    in_chunk = 0;
                 }
+                ++in_chunk;
             }
+            if (++b == NA) { b = 0; aph ^= 1; }
+            if (++yb == NYB) { yb = 0; yph ^= 1; }
         }
+        if constexpr (SPLIT)
+            if (ok) ok = fold();
         // ------------------------------ epilogue ------------------------------
-        if (ok && mbar_wait_idle(&phidone, 0, a.err, 37) && *(volatile int*)a.err == 0) {
+        if (ok && mbar_wait_idle(&phidone, 0, a.err, 43) && *(volatile int*)a.err == 0) {
             tc_fence_after();
             if constexpr (SPLIT) {
                 // the register accumulator goes back into the main phi columns for the epilogue,
@@ -2197,7 +2296,7 @@ struct ConsumePlan {
     bool ysplit;             // single-pass, persistent only: one work item per 128-row y tile
     int nyi;                 // work items per slab (nY with ysplit, else 1)
     int bx, nY, Nz, npc, nT3, n2p, n3p, ks2, ks3, nq, nload, na3, nyb, gs, ycol_tile;
-    uint32_t ya_rows, z_rows, ya, zb, b3, a3, load, a3_off, tmem_cols, y_cols;
+    uint32_t ya_rows, z_rows, a3_rows, ya, zb, b3, a3, load, a3_off, tmem_cols, y_cols;
     int nload3;              // single-pass: stages of the stage-3 (mu_t A_t3) ring
     uint32_t load3;          // single-pass: stride of the stage-3 ring
     size_t smem;
@@ -2209,6 +2308,7 @@ struct ConsumePlan {
     bool dual;               // persistent form with two stage-2 and two stage-3 MMA warps (form 5)
     // split kernel, y/z items (one plane, one 128-row y tile of nyi and one z part of nzi per CTA)
     bool yz;
+    bool ts3;                // split kernel: stage 3 reads its converted operand from TMEM
     int nzi;
     uint32_t loadB;          // converter kernel: stride and stages of the stage-3 operand ring
     int nloadB;
@@ -2441,19 +2541,27 @@ static bool plan_cv(const tx_ctx* c, bool tf32, bool split, int bx, int nload, i
     p->ks3 = (r3 + MK - 1) / MK;
     p->y_cols = (uint32_t)(bx * p->nY * p->Nz);
     // split precisions keep the cross products in accumulators of their own (twice the columns)
-    const uint32_t cols = (split ? 2u : 1u) * (p->y_cols + (uint32_t)(p->nT3 * p->n3p));
+    // TF32x3 on planes too tall to pack: the converted operand stays in TMEM (one plane, a tile per y tile)
+    p->ts3 = tf32 && split && bx == 1 && n2 > 64;
+    if (p->ts3 && !p->yz) p->nT3 = p->nY;
+    // as many Y buffers as fit, up to two (three where a buffer also holds the converted operand)
+    const auto tmem = [&](int nyb) { return (split ? 2u : 1u) * (nyb * p->y_cols + (uint32_t)(p->nT3 * p->n3p)); };
+    for (p->nyb = p->ts3 ? tcc::kMaxYCv : 2; p->nyb > 1 && tmem(p->nyb) > 512;) --p->nyb;
+    const uint32_t cols = tmem(p->nyb);
     if (cols > 512) return false;
     // ... and fold phi into registers: kMasterGroups x 16 columns per converter thread
     if (split && p->nT3 * p->n3p > 2 * 16 * tcc::kMasterGroups) return false;
     p->tmem_cols = 32;
     while (p->tmem_cols < cols) p->tmem_cols <<= 1;
     const int m = split ? 2 : 1;
-    p->ya_rows = (uint32_t)(p->nY * 128);
+    // sub-tiles of one row tile keep only their own rows: the MMA's other rows read what follows
+    p->ya_rows = (uint32_t)(p->nY == 1 && !p->yz ? p->n2p : p->nY * 128);
+    p->a3_rows = (uint32_t)(p->nT3 == 1 && !p->yz ? pad16(bx * n2) : p->nT3 * 128);
     p->z_rows = (uint32_t)(bx * p->Nz);                   // plane p at rows p * Nz
     p->ya = (uint32_t)p->ks2 * p->ya_rows * 32u;
     p->zb = (uint32_t)p->ks2 * p->z_rows * 32u;
     p->b3 = (uint32_t)(p->ks3 * p->n3p * 32);
-    p->a3 = (uint32_t)(p->ks3 * p->nT3 * 128 * 32);
+    p->a3 = p->ts3 ? 0u : (uint32_t)p->ks3 * p->a3_rows * 32u;
     // two rings: nload stages of [A_t2][Z] (released by stage 2), then up to two stages of
     // [mu_t A_t3] (released by stage 3), then the na3 converted stage-3 A operands
     p->load = ((uint32_t)(m * (p->ya + p->zb)) + 1023) & ~1023u;
@@ -2462,7 +2570,7 @@ static bool plan_cv(const tx_ctx* c, bool tf32, bool split, int bx, int nload, i
     p->na3 = na3;
     for (p->nloadB = std::min(tcc::kMaxLoadB, nload + 1); p->nloadB >= 1; --p->nloadB) {
         p->a3_off = p->load * nload + p->loadB * p->nloadB;
-        const size_t total = (size_t)p->a3_off + (size_t)na3 * m * p->a3;
+        const size_t total = (size_t)p->a3_off + (size_t)na3 * m * p->a3 + 128 * 32;   // the last sub-tile's other rows
         p->smem = std::max(total, (size_t)tcc::kEpiBytes) + 1024;   // the epilogue reuses the front
         if (p->smem <= 226 * 1024) return true;
     }
@@ -2504,21 +2612,19 @@ static bool choose_plan(const tx_ctx* c, bool tf32, bool split, ConsumePlan* bes
             }
         return best_score > 0;
     }
-    // deepest load pipeline first, then the slab with the least padding per useful row.  With
-    // more than one load stage a single converted stage-3 operand buffer still lets the loads
-    // and stage 2 of the next term run under the conversion and stage 3 of this one (measured
-    // on the Pt-shaped block in TF32x3, one load stage runs load, stage 2, conversion and
-    // stage 3 of every term back to back), so two load stages with one operand buffer rank
-    // above one load stage.
+    // the slab with the least padding per useful row, then two of everything: a second converted
+    // operand and a second mu_t A_t3 stage let stage 3 of consecutive terms follow one another, a second
+    // [A_t2][Z] stage lets stage 2 run ahead; further [A_t2][Z] stages only cover the Z reads' jitter
+    // (they are prefetched into L2)
     for (int nl = tcc::kMaxLoad; nl >= 1; --nl)
         for (int bx = 1; bx <= tcc::kMaxPlanes; ++bx)
             for (int na3 = nl > 1 ? 2 : 1; na3 >= 1; --na3) {
                 ConsumePlan p;
                 if (!plan_for(c, tf32, split, bx, nl, na3, &p)) continue;
                 const double use3 = (double)(bx * c->n[1]) / (p.nT3 * 128.0);
-                const double depth = nl >= 4 ? 1.0 : (nl == 3 ? 0.95 : (nl == 2 ? 0.8 : 0.5));
-                const double score = depth * use3 * (1.0 + 0.03 * std::min(bx, 8)) * (na3 == 2 ? 1.0 : 0.97) *
-                                     (p.nloadB >= 2 ? 1.0 : 0.9);
+                const double depth = nl >= 3 ? 1.0 : (nl == 2 ? 0.97 : 0.7);
+                const double score = depth * use3 * (1.0 + 0.03 * std::min(bx, 8)) * (na3 == 2 ? 1.0 : 0.85) *
+                                     (p.nloadB >= 2 ? 1.0 : 0.85);
                 if (score > best_score) {
                     best_score = score;
                     *best = p;
@@ -2800,7 +2906,9 @@ int tc_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const void*
     a.load_bytes = p.load; a.a3_off = p.a3_off;
     // bytes the TMA delivers per stage (out-of-range rows and columns count: they are zero-filled):
     // converter kernel, [A_t2][Z] stages and the stage-3 operand ring after them
-    a.stage_tx = (uint32_t)(m * 32 * (p.ks2 * p.n2p + p.ks2 * p.bx * r3));
+    a.stage_tx = (uint32_t)(m * 32 * p.ks2 * p.n2p);
+    a.stageZ_tx = (uint32_t)(m * 32 * p.ks2 * p.bx * r3);
+    a.a3_rows = p.a3_rows;
     a.loadB_bytes = p.loadB; a.nloadB = p.nloadB; a.b_off = p.load * (uint32_t)p.nload;
     a.stageB_tx = (uint32_t)(m * 32 * p.ks3 * p.n3p);
     a.tmem_cols = p.tmem_cols; a.y_cols = p.y_cols;
@@ -2819,7 +2927,7 @@ int tc_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const void*
         a.nyi = p.nyi;
         a.nzi = p.nzi;
         grid.x *= (unsigned)(p.nyi * p.nzi);
-        a.stage_tx = (uint32_t)(m * 32 * (p.ks2 * 128 + p.ks2 * p.bx * r3));
+        a.stage_tx = (uint32_t)(m * 32 * p.ks2 * 128);
     }
     if (p.ts) {
         a.gs = p.gs; a.ycol_tile = p.ycol_tile; a.ns3 = std::min(p.bx, 8);
@@ -2978,17 +3086,17 @@ int tc_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const void*
         mA3lo = mA3;
     }
     const int ps = prof_begin("tc_consume", s);
-#define LAUNCH(TF, SP)                                                                                       \
+#define LAUNCH(TF, SP, TS)                                                                                   \
     do {                                                                                                     \
-        auto fn = tcc::k_consume<TF, SP>;                                                                    \
+        auto fn = tcc::k_consume<TF, SP, TS>;                                                                \
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);                  \
         fn<<<grid, tcc::kThreads, p.smem, s>>>(mZ, mZlo, mA2, mA2lo, mA3, mA3lo, a);                          \
     } while (0)
-    if (op->tf32) {
-        if (op->split) LAUNCH(true, true); else LAUNCH(true, false);
-    } else {
-        if (op->split) LAUNCH(false, true); else LAUNCH(false, false);
-    }
+    if (p.ts3) LAUNCH(true, true, true);
+    else if (op->tf32 && op->split) LAUNCH(true, true, false);
+    else if (op->tf32) LAUNCH(true, false, false);
+    else if (op->split) LAUNCH(false, true, false);
+    else LAUNCH(false, false, false);
 #undef LAUNCH
     prof_end(ps, s);
     TX_LAUNCHED();
