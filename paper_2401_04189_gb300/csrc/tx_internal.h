@@ -187,11 +187,10 @@ struct GemmArgs {
     int nb1, nb2;
     float alpha;
     int accumulate;
-    // split != 0: C is the hi part of a split operand (1: TF32 in float, 2: bf16) and the lo part lies
-    // c_lo elements behind it; column n = (g, b), b < nb, goes to element g * ld_b + b of the row, and
-    // nb <= b < ld_b is zero-filled
-    int split, nb, ld_b;
-    long c_lo;
+    // split != 0: C holds operand tiles of the converter kernel, hi + lo (1: TF32 in float, 2: bf16), one
+    // block of c_m elements per row m: [part][K step of 32 bytes][nr rows g][32 bytes], 32-byte swizzled.
+    // Column n = (g, b), b < nb; K runs over b, and nb <= b < ld_b (whole K steps) is zero-filled.
+    int split, nb, ld_b, nr;
 };
 int simt_gemm(const GemmArgs& g, cudaStream_t s);
 

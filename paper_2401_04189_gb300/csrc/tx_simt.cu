@@ -205,14 +205,68 @@ __global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3) k_gemm(GemmArgs 
         // the other buffer was last read one slice ago, before this slice's barrier
     }
     if (g.split) {
-        // hi + lo parts straight from the accumulators: the float32 product never reaches memory
+        // hi + lo parts straight from the accumulators into the tiles that the converter kernel copies
+        const int ke = g.split == 1 ? 8 : 16;                // elements per 32-byte K step
+        const long lo = (long)g.ld_b * g.nr;                 // ld_b / ke steps of nr * ke elements
+        if constexpr (TN >= 4) {
+            if (g.nb % 4 == 0) {
+                // four neighbouring b of one g at a time: half (TF32) or a quarter (bf16) of a K step's row
+#pragma unroll
+                for (int j = 0; j < TN; j += 4) {
+                    const int n = n0 + gemm_index<TN>(tn, j);
+                    if (n >= g.N) continue;
+                    const int gg = n / g.nb, b = n - gg * g.nb, sw = ((gg >> 2) & 1) * (ke / 2);
+                    const long col = b2 * g.c_b2 + (long)(b / ke) * g.nr * ke + gg * ke + ((b % ke) ^ sw);
+                    const int npad = b == g.nb - 4 ? g.ld_b - g.nb : 0;      // zeros after the last b, 4 at a time
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) {
+                        const int m = m0 + gemm_index<TM>(tm, i);
+                        if (m >= g.M) continue;
+                        const float2 q0 = unpack2(acc[i][j / 2]), q1 = unpack2(acc[i][j / 2 + 1]);
+                        const float v[4] = {g.alpha * q0.x, g.alpha * q0.y, g.alpha * q1.x, g.alpha * q1.y};
+                        const long o = col + m * g.c_m;
+                        if (g.split == 1) {
+                            float h[4], l[4];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                h[k] = tc::tf32_hi(v[k]);
+                                l[k] = tc::tf32_hi(v[k] - h[k]);
+                            }
+                            *(float4*)(g.C + o) = make_float4(h[0], h[1], h[2], h[3]);
+                            *(float4*)(g.C + o + lo) = make_float4(l[0], l[1], l[2], l[3]);
+                        } else {
+                            __nv_bfloat16* C16 = (__nv_bfloat16*)g.C + o;
+                            const __nv_bfloat162 h0 = __floats2bfloat162_rn(v[0], v[1]), h1 = __floats2bfloat162_rn(v[2], v[3]);
+                            const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
+                            const __nv_bfloat162 l0 = __floats2bfloat162_rn(v[0] - f0.x, v[1] - f0.y);
+                            const __nv_bfloat162 l1 = __floats2bfloat162_rn(v[2] - f1.x, v[3] - f1.y);
+                            *(uint2*)C16 = make_uint2(*(const uint32_t*)&h0, *(const uint32_t*)&h1);
+                            *(uint2*)(C16 + lo) = make_uint2(*(const uint32_t*)&l0, *(const uint32_t*)&l1);
+                        }
+                        for (int k = 4; k < 4 + npad; k += 4) {
+                            const int bb = b + k;
+                            const long z = b2 * g.c_b2 + m * g.c_m + (long)(bb / ke) * g.nr * ke + gg * ke + ((bb % ke) ^ sw);
+                            if (g.split == 1) {
+                                *(float4*)(g.C + z) = *(float4*)(g.C + z + lo) = make_float4(0.f, 0.f, 0.f, 0.f);
+                            } else {
+                                __nv_bfloat16* C16 = (__nv_bfloat16*)g.C + z;
+                                *(uint2*)C16 = *(uint2*)(C16 + lo) = make_uint2(0u, 0u);
+                            }
+                        }
+                    }
+                }
+                return;
+            }
+        }
 #pragma unroll
         for (int j = 0; j < TN; ++j) {
             const int n = n0 + gemm_index<TN>(tn, j);
             if (n >= g.N) continue;
-            const int gg = n / g.nb;
-            const int npad = n - gg * g.nb == g.nb - 1 ? g.ld_b - g.nb : 0;    // zeros after the last b
-            const long col = b1 * g.c_b1 + b2 * g.c_b2 + (long)gg * g.ld_b + (n - gg * g.nb);
+            const int gg = n / g.nb, b = n - gg * g.nb;
+            const int npad = b == g.nb - 1 ? g.ld_b - g.nb : 0;      // zeros after the last b
+            const int sw = ((gg >> 2) & 1) * (ke / 2);               // rows 4-7 of 8 swap their 16-byte halves
+            auto at = [&](int bb) { return (long)(bb / ke) * g.nr * ke + gg * ke + ((bb % ke) ^ sw); };
+            const long col = b2 * g.c_b2 + at(b);
 #pragma unroll
             for (int i = 0; i < TM; ++i) {
                 const int m = m0 + gemm_index<TM>(tm, i);
@@ -223,14 +277,17 @@ __global__ void __launch_bounds__(256, BM * BN >= 8192 ? 2 : 3) k_gemm(GemmArgs 
                 if (g.split == 1) {
                     const float h = tc::tf32_hi(v);
                     g.C[o] = h;
-                    g.C[o + g.c_lo] = tc::tf32_hi(v - h);
-                    for (int k = 1; k <= npad; ++k) g.C[o + k] = g.C[o + k + g.c_lo] = 0.f;
+                    g.C[o + lo] = tc::tf32_hi(v - h);
                 } else {
                     const __nv_bfloat16 h = __float2bfloat16_rn(v);
                     __nv_bfloat16* C16 = (__nv_bfloat16*)g.C;
                     C16[o] = h;
-                    C16[o + g.c_lo] = __float2bfloat16_rn(v - __bfloat162float(h));
-                    for (int k = 1; k <= npad; ++k) C16[o + k] = C16[o + k + g.c_lo] = __float2bfloat16_rn(0.f);
+                    C16[o + lo] = __float2bfloat16_rn(v - __bfloat162float(h));
+                }
+                for (int k = 1; k <= npad; ++k) {
+                    const long z = b2 * g.c_b2 + m * g.c_m + at(b + k);
+                    if (g.split == 1) g.C[z] = g.C[z + lo] = 0.f;
+                    else ((__nv_bfloat16*)g.C)[z] = ((__nv_bfloat16*)g.C)[z + lo] = __float2bfloat16_rn(0.f);
                 }
             }
         }

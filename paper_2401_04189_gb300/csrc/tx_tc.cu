@@ -94,7 +94,9 @@ TcScratch tc_scratch(const tx_ctx* c) {
     s.s1 = r3 * n1 * s.ld_y;
     s.s2 = r3 * s.ld_b * s.ld_x;
     s.g = r3 * s.ld_b * s.ld_a;
-    s.z = (size_t)tc_terms(c) * n1 * r3 * s.ld_b;
+    // split precisions: one part of a tile per (t, x), rows g in whole groups of 8
+    const bool split = c->prec == TX_PREC_TF32X3 || c->prec == TX_PREC_BF16X3;
+    s.z = (size_t)tc_terms(c) * n1 * (split ? pad8((int)r3) : r3) * s.ld_b;
     return s;
 }
 
@@ -199,7 +201,7 @@ int tc_prepare(tx_ctx* c, cudaStream_t s) {
                                                                     op->st.A3f, 0);
         TX_LAUNCHED();
     }
-    if (!op->split) TX_TRY(tc_build_operand_image(c, s));
+    TX_TRY(op->split ? tc_build_split_image(c, s) : tc_build_operand_image(c, s));
     return TX_OK;
 }
 
@@ -241,10 +243,9 @@ static int f32_mode1_project(const tx_ctx* c, const float* S2, float* G, int np,
     return simt_gemm(g, s);
 }
 
-// Z[p][t][(x,g)][b] (hi, and lo z elements behind) for nt fine terms from t0 on: mode 1 of the expansion in
-// float32, sum_a M1_t[x][a] G[p][(g,b)][a] (a_first: cores [a][(g,b)]), split as it leaves the
-// accumulators (the b padding is written as zeros).
-static int f32_mode1_expand(const tx_ctx* c, const float* G, bool a_first, int t0, int nt, void* Z, size_t lo, int np,
+// Z tiles (hi + lo) of nt fine terms from t0 on, one block per (t, x): mode 1 of the expansion in float32,
+// sum_a M1_t[x][a] G[p][(g,b)][a] (a_first: cores [a][(g,b)]), split as it leaves the accumulators
+static int f32_mode1_expand(const tx_ctx* c, const float* G, bool a_first, int t0, int nt, void* Z, int np,
                             cudaStream_t s) {
     const TcOperands* op = c->tc;
     const TcScratch sc = tc_scratch(c);
@@ -253,9 +254,10 @@ static int f32_mode1_expand(const tx_ctx* c, const float* G, bool a_first, int t
     g.M = nt * n1; g.N = rr; g.K = r1;
     g.A = c->ts.F[0] + (size_t)t0 * n1 * r1; g.a_m = r1; g.a_k = 1;
     g.B = G; g.b_k = a_first ? rr : 1; g.b_n = a_first ? 1 : r1; g.b_b2 = (long)rr * r1;
-    g.C = (float*)((char*)Z + (size_t)t0 * n1 * r3 * sc.ld_b * op->esize); g.c_m = (long)r3 * sc.ld_b; g.c_b2 = (long)sc.z;
+    g.split = op->tf32 ? 1 : 2; g.nb = r2; g.ld_b = sc.ld_b; g.nr = pad8(r3);
+    g.c_m = 2L * g.nr * sc.ld_b; g.c_b2 = 2 * (long)sc.z;
+    g.C = (float*)((char*)Z + (size_t)t0 * n1 * g.c_m * op->esize);
     g.nb1 = 1; g.nb2 = np; g.alpha = 1.f;
-    g.split = op->tf32 ? 1 : 2; g.nb = r2; g.ld_b = sc.ld_b; g.c_lo = (long)lo;
     return simt_gemm(g, s);
 }
 
@@ -289,7 +291,6 @@ static int tc_forward(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, con
         fa.SB = SB;
         TX_TRY(simt_project_s2(c, recs, b.p0, np, fa, 0, S2f, s, false));
         TX_TRY(f32_mode1_project(c, S2f, Gf, np, s));
-        const size_t lo = (size_t)np * sc.z;
         if (ts.nc) {
             // H[p][a][(g,b)] = sum over the smooth terms of G x_d Q_td; the cores are [g][b], so modes 2
             // and 3 take each other's place
@@ -299,10 +300,10 @@ static int tc_forward(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, con
             fc.OUT0 = H;
             TX_TRY(simt_expand_consume(coarse_shape(c, true), nullptr, 0, np, fc, Zc, ts.nc, ts.QKs[2], ts.QKs[1], EPI_STORE,
                                        nullptr, s));
-            if (ts.nf > 1) TX_TRY(f32_mode1_expand(c, Gf, false, 0, ts.nf - 1, Z, lo, np, s));
-            TX_TRY(f32_mode1_expand(c, H, true, ts.nf - 1, 1, Z, lo, np, s));
+            if (ts.nf > 1) TX_TRY(f32_mode1_expand(c, Gf, false, 0, ts.nf - 1, Z, np, s));
+            TX_TRY(f32_mode1_expand(c, H, true, ts.nf - 1, 1, Z, np, s));
         } else {
-            TX_TRY(f32_mode1_expand(c, Gf, false, 0, ts.nf, Z, lo, np, s));
+            TX_TRY(f32_mode1_expand(c, Gf, false, 0, ts.nf, Z, np, s));
         }
         return tc_consume(c, recs, b.p0, np, Z, SA, SB, MUL0, MUL1, OUT0, OUT1, cnt, flags, b.epart, s, subset);
     }

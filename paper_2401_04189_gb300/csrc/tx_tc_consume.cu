@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 #include <string>
 
 #include "tx_tc_common.cuh"
@@ -91,6 +92,7 @@ struct ConsumeArgs {
     // [A_t2][Z] stages, so that stage 2 releases its stage as soon as its MMAs have run
     uint32_t loadB_bytes, b_off, stageB_tx, stageZ_tx;   // stage_tx: A_t2 alone
     uint32_t a3_rows;          // rows per K step of the converted stage-3 operand
+    uint32_t b3_img;           // split precisions: offset of the mu_t A_t3 tiles in a term of the image
     int nloadB;
 };
 
@@ -173,6 +175,7 @@ __device__ __forceinline__ double consume_epilogue(const ConsumeArgs& a, const P
     // with symmetric pairs the energy factors (psi_a, psi_b) are the two multipliers
     // themselves: each orbital value is read once
     const bool need0 = o0 || (en && a.emul), need1 = o1 || (en && a.emul);
+    const bool weighted = en || (a.flags & EPI_MULW);      // a plain apply reads no quadrature weights
     // Each warp stages its quadrant's 32 rows x 64 columns of phi in shared memory (the
     // pipeline buffers are idle now), then walks the rows with consecutive z across lanes:
     // psi reads are coalesced and W is updated with 16-byte vector reductions.  The two
@@ -230,15 +233,18 @@ __device__ __forceinline__ double consume_epilogue(const ConsumeArgs& a, const P
         // float32 rate, and a float64 multiply-add per grid point used to dominate this loop.
         float eb = 0.f;
         // lanes 0-15 take row rr, lanes 16-31 row rr + 1; four consecutive z per lane
-#pragma unroll 2
+#pragma unroll 4
         for (int it = 0; it < 8; ++it) {
             int x, y, z, idx;
             if (!locate(blk, it, x, y, z, idx)) continue;
             const int rr = 2 * h + 4 * it + sub;
             const float4 phi = *(const float4*)(stg + rr * 68 + 4 * (lane & 15));
-            const float wxy = a.w1[x] * a.w2[y];
-            const float4 w3 = *(const float4*)(a.w3 + z);
-            const float4 wv = make_float4(wxy * w3.x, wxy * w3.y, wxy * w3.z, wxy * w3.w);
+            float4 wv = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (weighted) {
+                const float wxy = a.w1[x] * a.w2[y];
+                const float4 w3 = *(const float4*)(a.w3 + z);
+                wv = make_float4(wxy * w3.x, wxy * w3.y, wxy * w3.z, wxy * w3.w);
+            }
             float4 f = phi;
             if (a.flags & EPI_MULW) f = make_float4(f.x * wv.x, f.y * wv.y, f.z * wv.z, f.w * wv.w);
             const float4 m0 = need0 ? lb[(2 * it) * 32] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -394,17 +400,26 @@ __device__ __forceinline__ double consume_epilogue_tma(const ConsumeArgs& a, con
 // index g / 2, values mst[16 * (g / 2) + j]).
 template <int MG>
 __device__ __forceinline__ void fold_chunk(uint32_t tPhi, uint32_t tPhiC, int q, int h, int ngroups, float (&mst)[MG * 16]) {
+    // two groups per TMEM round trip
 #pragma unroll
-    for (int gi = 0; gi < MG; ++gi) {
+    for (int gi = 0; gi < MG; gi += 2) {
         const int g = h + 2 * gi;
         if (g >= ngroups) break;
-        uint32_t rm[16], rc[16];
+        const bool two = gi + 1 < MG && g + 2 < ngroups;
+        uint32_t rm[16], rc[16], sm[16], sc[16];
         const uint32_t off = ((uint32_t)(q * 32) << 16) + (uint32_t)(16 * g);
         tmem_ld16(tPhi + off, rm);
         tmem_ld16(tPhiC + off, rc);
+        if (two) {
+            tmem_ld16(tPhi + off + 32u, sm);
+            tmem_ld16(tPhiC + off + 32u, sc);
+        }
         tmem_ld_wait();
 #pragma unroll
         for (int j = 0; j < 16; ++j) mst[16 * gi + j] += __uint_as_float(rm[j]) + __uint_as_float(rc[j]);
+        if (gi + 1 < MG && two)
+#pragma unroll
+            for (int j = 0; j < 16; ++j) mst[16 * (gi + 1 < MG ? gi + 1 : gi) + j] += __uint_as_float(sm[j]) + __uint_as_float(sc[j]);
     }
 }
 // ... and written back into the main phi columns for the epilogue
@@ -501,7 +516,9 @@ __device__ __forceinline__ void cv_mmas_ts(int ks, uint32_t d, uint32_t dc, uint
 
 // The converter kernel (split precisions; single-pass shapes that no TMEM plan holds).  Every role is
 // a stage of one pipeline over the terms, each on warps of its own and one or two terms apart:
-//   8, 10  producers of A_t2 and mu_t A_t3, and of Z (tile copies are issued by one lane each)
+//   8, 10  producers of [A_t2][Z] and of mu_t A_t3.  Split precisions: every operand of a term is one
+//          bulk copy (images of A_t2 and mu_t A_t3 made at set-up, Z written in tile order by its GEMM); the
+//          30 tile copies they replace took 150-250 cycles each to issue.  Single-pass: tile copies.
 //   9      stage-2 MMAs into rotating Y buffers
 //   0-7    converters: Y -> hi + lo stage-3 operand, then the fold of the PREVIOUS term's phi
 //   11     stage-3 MMAs
@@ -515,19 +532,18 @@ __device__ __forceinline__ void cv_mmas_ts(int ks, uint32_t d, uint32_t dc, uint
 // it took over half of the shared-memory bandwidth, which bound the kernel: a clock64 trace showed 6,500
 // cycles per conversion under the MMAs' reads, 3,300 alone.  (Planes of up to 64 rows pack two planes
 // into one 128-row operand in shared memory, which TMEM lanes cannot do.)
-// Pt-shaped pair (14 terms): 27.2 us; 33.8 with the operand in shared memory, 44.6 with one
+// Pt-shaped pair (14 terms): 16.4 us; 27.2 with tile copies, 33.8 with the operand in shared memory, 44.6 with one
 // issuing lane for all MMAs, one for all copies and the fold before the next conversion.
 template <bool TF32, bool SPLIT, bool TS3>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_consume(const __grid_constant__ CUtensorMap mZ, const __grid_constant__ CUtensorMap mZlo,
-              const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mA2lo,
-              const __grid_constant__ CUtensorMap mA3, const __grid_constant__ CUtensorMap mA3lo, ConsumeArgs a) {
+    k_consume(const __grid_constant__ CUtensorMap mZ, const __grid_constant__ CUtensorMap mA2,
+              const __grid_constant__ CUtensorMap mA3, ConsumeArgs a) {
     constexpr int MK = TF32 ? 8 : 16;        // K per MMA instruction (32 bytes)
     constexpr int ES = TF32 ? 4 : 2;         // operand element bytes
     constexpr int CV = 16 / ES;              // values per 16-byte chunk
     constexpr uint32_t M = SPLIT ? 2u : 1u;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t fullA[kMaxLoad], fullZ[kMaxLoad], empty_bar[kMaxLoad], a3full[kMaxYCv], a3free[2], phidone, s2fin;
+    __shared__ uint64_t full_bar[kMaxLoad], empty_bar[kMaxLoad], a3full[kMaxYCv], a3free[2], phidone, s2fin;
     __shared__ uint64_t fullB[kMaxLoadB], emptyB[kMaxLoadB];
     __shared__ uint64_t yfull[kMaxYCv], yfree[kMaxYCv], chunkdone, phifree;
     __shared__ uint32_t tmem_base;
@@ -550,8 +566,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // nearest) and the tensor core restarts.  Single-pass precisions accumulate every term.
     const int C = SPLIT ? (a.chunk > 0 ? a.chunk : 1) : NT;
 
-    // load stage s: [A_t2 tile][Z tile], each hi then lo; stage-3 stage sb: [A_t3 tile] hi then lo;
-    // then the NA converted stage-3 operands
+    // load stage s: [A_t2 tile][Z tile], each hi then lo (Z: plane by plane in the split precisions);
+    // stage-3 stage sb: [A_t3 tile] hi then lo; then the NA converted stage-3 operands
     auto YAs = [&](int s) { return smem + s * a.load_bytes; };
     auto Zs = [&](int s) { return YAs(s) + M * a.ya_bytes; };
     auto B3s = [&](int sb) { return smem + a.b_off + sb * a.loadB_bytes; };
@@ -559,8 +575,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxLoad; ++s) {
-            mbar_init(&fullA[s], 1);
-            mbar_init(&fullZ[s], 1);
+            mbar_init(&full_bar[s], 1);
             mbar_init(&empty_bar[s], 1);
         }
         // TS3: a3full is per Y buffer (its conversion), and stage 3 frees the buffer
@@ -603,89 +618,83 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t a3_sub = a.a3_rows * 32u;
 
     if (warp == 8) {
-        // ------------------------------ producer: A_t2 and mu_t A_t3 ------------------------------
-        // (the wait for a stage-3 stage holds up the next A_t2 by at most the slack that the conversion and
-        // stage 3 of the term before give it)
-        if (lane == 0) {
-            int ia = 0, ib = 0, s = 0, sb = 0;
-            uint32_t ph = 0, bph = 0;
-            for (int t = 0; t < NT; ++t) {
-                if (!mbar_wait(&empty_bar[s], ph ^ 1, a.err, 31)) break;
-                ia = t + 1;
-                mbar_arrive_expect_tx(&fullA[s], a.stage_tx);
-                for (int k = 0; k < a.ks2; ++k) {
-                    tma_load_3d(YAs(s) + k * ya_sub, &mA2, &fullA[s], k * MK, y0, t);
-                    if constexpr (SPLIT) tma_load_3d(YAs(s) + a.ya_bytes + k * ya_sub, &mA2lo, &fullA[s], k * MK, y0, t);
-                }
-                if (++s == NL) { s = 0; ph ^= 1; }
-                if (!mbar_wait(&emptyB[sb], bph ^ 1, a.err, 39)) break;
-                ib = t + 1;
-                mbar_arrive_expect_tx(&fullB[sb], a.stageB_tx);
-                for (int k = 0; k < a.ks3; ++k) {
-                    tma_load_3d(B3s(sb) + k * a.n3p * 32u, &mA3, &fullB[sb], k * MK, z0, t);
-                    if constexpr (SPLIT)
-                        tma_load_3d(B3s(sb) + a.b3_bytes + k * a.n3p * 32u, &mA3lo, &fullB[sb], k * MK, z0, t);
-                }
-                if (++sb == NB) { sb = 0; bph ^= 1; }
-            }
-            if (ia < NT || ib < NT) {
-                for (int t = (ia > NL ? ia - NL : 0); t < ia; ++t) mbar_drain(&fullA[t % NL], (t / NL) & 1, a.err);
-                for (int t = (ib > NB ? ib - NB : 0); t < ib; ++t) mbar_drain(&fullB[t % NB], (t / NB) & 1, a.err);
-            }
-        }
-    } else if (warp == 10) {
-        // ------------------------------ producer: Z ------------------------------
-        if (lane == 0) {
-            int issued = 0, s = 0;
-            uint32_t ph = 0;
-            for (int t = 0; t < NT; ++t) {
-                if (!mbar_wait(&empty_bar[s], ph ^ 1, a.err, 40)) break;
-                issued = t + 1;
-                mbar_arrive_expect_tx(&fullZ[s], a.stageZ_tx);
-                const int zdep = pl * NT + t;
-                for (int k = 0; k < a.ks2; ++k)
-                    // plane p's rows start at row p * Nz (a multiple of 16) of the Z tile
-                    for (int p = 0; p < BX; ++p) {
-                        const uint32_t off = k * z_sub + (uint32_t)(p * a.Nz) * 32u;
-                        tma_load_3d(Zs(s) + off, &mZ, &fullZ[s], k * MK, (x0 + p) * a.r3, zdep);
-                        if constexpr (SPLIT)
-                            tma_load_3d(Zs(s) + a.z_bytes + off, &mZlo, &fullZ[s], k * MK, (x0 + p) * a.r3, zdep);
-                    }
+        // ------------------------------ producer: A_t2 and Z ------------------------------
+        int issued = 0, s = 0;
+        uint32_t ph = 0;
+        // the slab's planes of one term follow one another in Z
+        const uint32_t zbytes = (uint32_t)min(BX, a.n1 - x0) * a.z_plane;
+        const uint8_t* zslab = a.zsrc + ((size_t)pl * NT * a.n1 + x0) * a.z_plane;
+        const size_t zterm = (size_t)a.n1 * a.z_plane;
+        const uint8_t* ya = a.img + (size_t)(iyz / max(1, a.nzi)) * (a.yz ? M * a.ya_bytes : 0u);
+        for (int t = 0; t < NT; ++t) {
+            const bool w = mbar_wait(&empty_bar[s], ph ^ 1, a.err, 31);
+            if (!__all_sync(0xffffffffu, w)) break;
+            issued = t + 1;
+            if constexpr (SPLIT) {
+                mbar_arrive_expect_tx_w(&full_bar[s], M * a.ya_bytes + zbytes);
+                bulk_load_w(Zs(s), zslab + (size_t)t * zterm, zbytes, &full_bar[s]);
+                bulk_load_w(YAs(s), ya + (size_t)t * a.img_stride, M * a.ya_bytes, &full_bar[s]);
                 // start the HBM reads of later Z tiles early (into L2 only)
                 for (int ahead = (t == 0 ? 1 : NL + 1); ahead <= NL + 1; ++ahead)
-                    if (t + ahead < NT)
-                        for (int p = 0; p < BX; ++p)
-                            for (int k = 0; k < a.ks2; ++k) {
-                                tma_prefetch_l2_3d(&mZ, k * MK, (x0 + p) * a.r3, zdep + ahead);
-                                if constexpr (SPLIT) tma_prefetch_l2_3d(&mZlo, k * MK, (x0 + p) * a.r3, zdep + ahead);
-                            }
-                if (++s == NL) { s = 0; ph ^= 1; }
+                    if (t + ahead < NT) bulk_prefetch_l2_w(zslab + (size_t)(t + ahead) * zterm, zbytes);
+            } else if (lane == 0) {
+                mbar_arrive_expect_tx(&full_bar[s], a.stage_tx + a.stageZ_tx);
+                for (int k = 0; k < a.ks2; ++k) {
+                    tma_load_3d(YAs(s) + k * ya_sub, &mA2, &full_bar[s], k * MK, 0, t);
+                    // plane p's rows start at row p * Nz (a multiple of 16) of the Z tile
+                    for (int p = 0; p < BX; ++p)
+                        tma_load_3d(Zs(s) + k * z_sub + (uint32_t)(p * a.Nz) * 32u, &mZ, &full_bar[s], k * MK,
+                                    (x0 + p) * a.r3, pl * NT + t);
+                }
             }
-            if (issued < NT)
-                for (int t = (issued > NL ? issued - NL : 0); t < issued; ++t) mbar_drain(&fullZ[t % NL], (t / NL) & 1, a.err);
+            __syncwarp();
+            if (++s == NL) { s = 0; ph ^= 1; }
         }
+        if (issued < NT)
+            for (int t = (issued > NL ? issued - NL : 0); t < issued; ++t) mbar_drain(&full_bar[t % NL], (t / NL) & 1, a.err);
+    } else if (warp == 10) {
+        // ------------------------------ producer: mu_t A_t3 ------------------------------
+        int issued = 0, sb = 0;
+        uint32_t ph = 0;
+        const uint8_t* b3 = a.img + a.b3_img + (size_t)(a.yz ? iyz % a.nzi : 0) * M * a.b3_bytes;
+        for (int t = 0; t < NT; ++t) {
+            const bool w = mbar_wait(&emptyB[sb], ph ^ 1, a.err, 39);
+            if (!__all_sync(0xffffffffu, w)) break;
+            issued = t + 1;
+            if constexpr (SPLIT) {
+                mbar_arrive_expect_tx_w(&fullB[sb], M * a.b3_bytes);
+                bulk_load_w(B3s(sb), b3 + (size_t)t * a.img_stride, M * a.b3_bytes, &fullB[sb]);
+            } else if (lane == 0) {
+                mbar_arrive_expect_tx(&fullB[sb], a.stageB_tx);
+                for (int k = 0; k < a.ks3; ++k) tma_load_3d(B3s(sb) + k * a.n3p * 32u, &mA3, &fullB[sb], k * MK, z0, t);
+            }
+            __syncwarp();
+            if (++sb == NB) { sb = 0; ph ^= 1; }
+        }
+        if (issued < NT)
+            for (int t = (issued > NB ? issued - NB : 0); t < issued; ++t) mbar_drain(&fullB[t % NB], (t / NB) & 1, a.err);
     } else if (warp == 9) {
         // ------------------------------ stage-2 MMAs ------------------------------
-        // all planes of a term go in one MMA per K step (N = planes x Nz, in chunks of <= 256)
+        // single-pass: all planes of a term in one MMA per K step (N = planes x Nz, in chunks of <= 256);
+        // split: plane by plane (each plane's tiles stand by themselves)
         const uint64_t d0 = sdesc_sw32(0);
         int s = 0, yb = 0;
         uint32_t ph = 0, yph = 0;
         for (int t = 0; t < NT; ++t) {
-            bool w = mbar_wait(&fullA[s], ph, a.err, 32);
-            if (w) w = mbar_wait(&fullZ[s], ph, a.err, 33);
+            bool w = mbar_wait(&full_bar[s], ph, a.err, 32);
             if (w && t >= NYB) w = mbar_wait(&yfree[yb], yph ^ 1, a.err, 34);     // conversion of term t - NYB
             if (!__all_sync(0xffffffffu, w)) break;
             tc_fence_after();
             const uint64_t ya = d0 + (smem_u32(YAs(s)) >> 4), zb = d0 + (smem_u32(Zs(s)) >> 4);
             const uint32_t tY = tmem + (uint32_t)yb * y_stride;
             for (int i = 0; i < a.nY; ++i)
-                for (int p0 = 0; p0 < BX; p0 += a.npc) {
-                    const int N = min(a.npc, BX - p0) * a.Nz;
+                for (int p0 = 0; p0 < BX; p0 += SPLIT ? 1 : a.npc) {
+                    const int N = SPLIT ? a.Nz : min(a.npc, BX - p0) * a.Nz;
                     const uint32_t id2 = TF32 ? idesc_tf32(128, N) : idesc_bf16(128, N);
                     const uint32_t col = tY + (uint32_t)((i * BX + p0) * a.Nz);
                     cv_mmas<TF32, SPLIT>(a.ks2, col, col + a.y_cols, ya + (uint32_t)i * 256u,
-                                         zb + (uint32_t)(p0 * a.Nz) * 2u, ya_sub >> 4, z_sub >> 4, a.ya_bytes >> 4,
-                                         a.z_bytes >> 4, id2, 0u);
+                                         zb + (SPLIT ? (uint32_t)p0 * (a.z_plane >> 4) : (uint32_t)(p0 * a.Nz) * 2u),
+                                         ya_sub >> 4, z_sub >> 4, a.ya_bytes >> 4, a.z_plane >> 5, id2, 0u);
                 }
             mma_commit_w(&yfull[yb]);
             mma_commit_w(&empty_bar[s]);          // the [A_t2][Z] stage is free once these have run
@@ -802,9 +811,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int c = 0; c < 16; ++c) {
                 const float v = g0 + c < a.r3 ? __uint_as_float(r[c]) + __uint_as_float(rc[c]) : 0.f;
-                const float hi = tf32_rna(v);
-                r[c] = __float_as_uint(hi);
-                rc[c] = __float_as_uint(tf32_rna(v - hi));
+                // hi: nearest, ties away (a NaN may leave hi, but not lo: v - hi is NaN then).  lo has 13 bits
+                // at most and the tensor core drops two of them: 2^-22 of v, either way
+                r[c] = (__float_as_uint(v) + 0x1000u) & 0xffffe000u;
+                rc[c] = __float_as_uint(v - __uint_as_float(r[c]));
             }
             tmem_st16(col, r);
             tmem_st16(col + a.y_cols, rc);
@@ -2557,9 +2567,11 @@ static bool plan_cv(const tx_ctx* c, bool tf32, bool split, int bx, int nload, i
     // sub-tiles of one row tile keep only their own rows: the MMA's other rows read what follows
     p->ya_rows = (uint32_t)(p->nY == 1 && !p->yz ? p->n2p : p->nY * 128);
     p->a3_rows = (uint32_t)(p->nT3 == 1 && !p->yz ? pad16(bx * n2) : p->nT3 * 128);
-    p->z_rows = (uint32_t)(bx * p->Nz);                   // plane p at rows p * Nz
+    // single-pass: plane p at rows p * Nz; split: planes one after another, rows in groups of 8 (the MMA's
+    // other columns read what follows and are zeroed by the conversion)
+    p->z_rows = split ? (uint32_t)pad8(r3) : (uint32_t)(bx * p->Nz);
     p->ya = (uint32_t)p->ks2 * p->ya_rows * 32u;
-    p->zb = (uint32_t)p->ks2 * p->z_rows * 32u;
+    p->zb = (uint32_t)p->ks2 * p->z_rows * 32u * (split ? (uint32_t)bx : 1u);
     p->b3 = (uint32_t)(p->ks3 * p->n3p * 32);
     p->a3 = p->ts3 ? 0u : (uint32_t)p->ks3 * p->a3_rows * 32u;
     // two rings: nload stages of [A_t2][Z] (released by stage 2), then up to two stages of
@@ -2760,6 +2772,60 @@ int tc_describe_plan(const tx_ctx* c, int* out, int nout) {
                        p.yz ? p.nzi : 0};
     for (int i = 0; i < nout && i < 14; ++i) out[i] = v[i];
     return TX_OK;
+}
+
+static uint32_t split_image_stride(const ConsumePlan& p) {
+    return 2u * ((uint32_t)p.nyi * p.ya + (uint32_t)std::max(1, p.nzi) * p.b3);
+}
+
+namespace tcc {
+// tiles of one operand for every term: dst[t][tile][part][K step][rows][32 bytes] (32-byte swizzle) from the
+// K-major src[t][n][ld] (hi, and lo behind it); tile i holds rows i * step ..; rows past n and K past ld are zero
+template <typename E>
+__global__ void __launch_bounds__(256) k_split_image(const E* __restrict__ hi, const E* __restrict__ lo, int n, int ld,
+                                                     int ks, int rows, int step, uint32_t stride, uint32_t off,
+                                                     uint8_t* __restrict__ img) {
+    constexpr int MK = 32 / (int)sizeof(E);
+    const int t = blockIdx.y, tile = blockIdx.z, per = ks * rows * MK;
+    for (int e = blockIdx.x * 256 + threadIdx.x; e < 2 * per; e += gridDim.x * 256) {
+        const int part = e / per, q = e - part * per, k = q / (rows * MK), row = q / MK % rows, c = q % MK;
+        const int i = tile * step + row, kk = k * MK + c;
+        const E v = (i < n && kk < ld) ? (part ? lo : hi)[((size_t)t * n + i) * ld + kk] : E(0.f);
+        uint8_t* dst = img + (size_t)t * stride + off + ((size_t)(tile * 2 + part) * per + (size_t)k * rows * MK) * sizeof(E);
+        *(E*)(dst + sw32_offset((uint32_t)row, (uint32_t)(c * sizeof(E)))) = v;
+    }
+}
+}  // namespace tcc
+
+// Operator image of the split precisions: per term the tiles of A_t2 (one per y tile of the plan), then
+// those of mu_t A_t3 (one per z part), hi and lo, as the converter kernel copies them
+int tc_build_split_image(tx_ctx* c, cudaStream_t s) {
+    TcOperands* op = c->tc;
+    ConsumePlan p;
+    if (!choose_plan(c, op->tf32, true, &p)) return fail(TX_ERR_UNSUPPORTED_SHAPE, "no expansion tile plan");
+    const int n2 = c->n[1], n3 = c->n[2], l2 = ldk(c->r[1], op->esize), l3 = ldk(c->r[2], op->esize), T = tc_terms(c);
+    const int nz = std::max(1, p.nzi);
+    op->img_stride = split_image_stride(p);
+    if (cudaMalloc(&op->img, (size_t)T * op->img_stride) != cudaSuccess) {
+        cudaGetLastError();
+        op->img = nullptr;
+        return fail(TX_ERR_OOM, "operator image");
+    }
+    auto tiles = [&](const void* hi, int n, int ld, int ks, uint32_t rows, int ntile, int step, uint32_t off) -> int {
+        const void* lo = (const char*)hi + op->st.off_lo;
+        const dim3 grid((unsigned)std::max(1u, (uint32_t)ks * rows * 16u / 1024u), (unsigned)T, (unsigned)ntile);
+        if (op->tf32)
+            tcc::k_split_image<float><<<grid, 256, 0, s>>>((const float*)hi, (const float*)lo, n, ld, ks, (int)rows, step,
+                                                           op->img_stride, off, (uint8_t*)op->img);
+        else
+            tcc::k_split_image<__nv_bfloat16><<<grid, 256, 0, s>>>((const __nv_bfloat16*)hi, (const __nv_bfloat16*)lo, n, ld,
+                                                                   ks, (int)rows, step, op->img_stride, off,
+                                                                   (uint8_t*)op->img);
+        TX_LAUNCHED();
+        return TX_OK;
+    };
+    TX_TRY(tiles(op->st.A2, n2, l2, p.ks2, p.ya_rows, p.nyi, 128, 0));
+    return tiles(op->st.A3, n3, l3, p.ks3, (uint32_t)p.n3p, nz, p.n3p, (uint32_t)p.nyi * 2u * p.ya);
 }
 
 // operator image of the bf16 persistent kernel: [A_t2 tile][mu_t A_t3 tile], bf16, per term
@@ -3063,34 +3129,33 @@ int tc_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const void*
         TX_LAUNCHED();
         return TX_OK;
     }
-    // Z of this batch: [pair][t][(x, g) rows][ld_b]; lo part after the batch's hi part
-    const size_t zlo = (size_t)np * sc.z * eb;
-    CUtensorMap mZ, mZlo, mA2, mA2lo, mA3, mA3lo;
-    const CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_32B;
-    const int l2 = ldk(r2, eb), l3 = ldk(r3, eb);
-    TX_TRY(make_map_sw(&mZ, Z, eb, sc.ld_b, (uint64_t)n1 * r3, (uint64_t)np * T, sc.ld_b, (uint64_t)n1 * r3 * sc.ld_b, MK,
-                       (uint32_t)r3, sw));
-    const uint32_t a2_box = p.yz ? 128u : (uint32_t)p.n2p;     // rows of one A_t2 box
-    TX_TRY(make_map_sw(&mA2, op->st.A2, eb, l2, n2, T, l2, (uint64_t)n2 * l2, MK, a2_box, sw));
-    TX_TRY(make_map_sw(&mA3, op->st.A3, eb, l3, n3, T, l3, (uint64_t)n3 * l3, MK, (uint32_t)p.n3p, sw));
+    CUtensorMap mZ, mA2, mA3;
     if (op->split) {
-        TX_TRY(make_map_sw(&mZlo, (const char*)Z + zlo, eb, sc.ld_b, (uint64_t)n1 * r3, (uint64_t)np * T, sc.ld_b,
-                           (uint64_t)n1 * r3 * sc.ld_b, MK, (uint32_t)r3, sw));
-        TX_TRY(make_map_sw(&mA2lo, (const char*)op->st.A2 + op->st.off_lo, eb, l2, n2, T, l2, (uint64_t)n2 * l2, MK,
-                           a2_box, sw));
-        TX_TRY(make_map_sw(&mA3lo, (const char*)op->st.A3 + op->st.off_lo, eb, l3, n3, T, l3, (uint64_t)n3 * l3, MK,
-                           (uint32_t)p.n3p, sw));
+        // Z tiles of this batch: [pair][t][x][part][K step][rows g][32 bytes]
+        if (!op->img || op->img_stride != split_image_stride(p))
+            return fail(TX_ERR_CUDA, "operator image missing or built for another tile shape");
+        a.img = (const uint8_t*)op->img;
+        a.img_stride = op->img_stride;
+        a.b3_img = (uint32_t)p.nyi * 2u * p.ya;
+        a.zsrc = (const uint8_t*)Z;
+        a.z_plane = 2u * (uint32_t)p.ks2 * p.z_rows * 32u;
+        std::memset(&mZ, 0, sizeof(mZ));       // the split kernels read no tensor map
+        mA2 = mA3 = mZ;
     } else {
-        mZlo = mZ;
-        mA2lo = mA2;
-        mA3lo = mA3;
+        // Z of this batch: [pair][t][(x, g) rows][ld_b]
+        const CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_32B;
+        const int l2 = ldk(r2, eb), l3 = ldk(r3, eb);
+        TX_TRY(make_map_sw(&mZ, Z, eb, sc.ld_b, (uint64_t)n1 * r3, (uint64_t)np * T, sc.ld_b, (uint64_t)n1 * r3 * sc.ld_b,
+                           MK, (uint32_t)r3, sw));
+        TX_TRY(make_map_sw(&mA2, op->st.A2, eb, l2, n2, T, l2, (uint64_t)n2 * l2, MK, (uint32_t)p.n2p, sw));
+        TX_TRY(make_map_sw(&mA3, op->st.A3, eb, l3, n3, T, l3, (uint64_t)n3 * l3, MK, (uint32_t)p.n3p, sw));
     }
     const int ps = prof_begin("tc_consume", s);
 #define LAUNCH(TF, SP, TS)                                                                                   \
     do {                                                                                                     \
         auto fn = tcc::k_consume<TF, SP, TS>;                                                                \
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);                  \
-        fn<<<grid, tcc::kThreads, p.smem, s>>>(mZ, mZlo, mA2, mA2lo, mA3, mA3lo, a);                          \
+        fn<<<grid, tcc::kThreads, p.smem, s>>>(mZ, mA2, mA3, a);                                              \
     } while (0)
     if (p.ts3) LAUNCH(true, true, true);
     else if (op->tf32 && op->split) LAUNCH(true, true, false);

@@ -37,6 +37,7 @@ struct TcOperands {
     int bx;               // x planes per expansion CTA
     // single-pass expansion: per Gaussian term, the shared-memory image of its operator tiles
     // ([A_t2 tile][mu_t A_t3 tile], swizzled and zero-filled as the tile loads lay them out)
+    // split precisions: per term [y tile][A_t2 hi, lo][...] then [z part][mu_t A_t3 hi, lo] (32-byte swizzled)
     void* img;
     uint32_t img_stride;  // bytes per term
 };
@@ -54,6 +55,7 @@ int tc_terms(const tx_ctx* c);   // Gaussian terms of the tensor-core operands
 int tc_project_mode3(const tx_ctx* c, const PairRec* recs, int p0, int np, const float* SA, int nA, const float* SB,
                      int nB, int flags, void* S1, cudaStream_t s, const void* Bhi = nullptr);
 int tc_build_operand_image(tx_ctx* c, cudaStream_t s);
+int tc_build_split_image(tx_ctx* c, cudaStream_t s);
 // orbital counts of the arrays the expansion epilogue reads and writes (bounds of its tensors)
 struct OrbCounts {
     int sa, sb, mul0, mul1, out0, out1;
