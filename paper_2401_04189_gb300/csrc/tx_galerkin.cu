@@ -111,9 +111,7 @@ int galerkin_operators(const tx_ctx* c, float* ops, GalerkinOps* g, cudaStream_t
 // pairs): 845 us; 1456 as three GEMM passes over every term and a sum.
 int galerkin_core(const tx_ctx* c, const GalerkinOps& o, const float* G, float* X1, float* H, int np, cudaStream_t s) {
     TX_TRY(simt_expand_mode1_grid(c, G, o.B[0], c->r[0], c->T, X1, np, s));
-    FieldArgs f{};
-    f.OUT0 = H;
-    return simt_expand_consume(coarse_shape(c), nullptr, 0, np, f, X1, c->T, o.B[1], o.B[2], EPI_STORE, nullptr, s);
+    return simt_core_consume(coarse_shape(c), np, X1, c->T, o.B[1], o.B[2], H, s);
 }
 
 int galerkin_core_dot(const tx_ctx* c, const PairRec* recs, int p0, const float* G, const float* H, int np,

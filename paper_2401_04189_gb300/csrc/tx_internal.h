@@ -230,7 +230,10 @@ int simt_kmajor(const float* src, int nt, int n, int r, int ld, float* dst, cuda
 // With EPI_STORE phi itself goes to f.OUT0 [np][n1][n2][n3] instead.
 int simt_expand_consume(const Shape& sh, const PairRec* recs, int p0, int np, const FieldArgs& f,
                         const float* Z, int nterms, const float* M2, const float* M3, int flags,
-                        double* epart, cudaStream_t s, bool z_bg = true, long m2_ps = 0, long m3_ps = 0);
+                        double* epart, cudaStream_t s, bool z_bg = true, long m2_ps = 0, long m3_ps = 0, int group = 0);
+// H[p] = the expansion onto a grid of r_d points, stored (Z is overwritten where few pairs split the terms)
+int simt_core_consume(const Shape& sh, int np, float* Z, int nterms, const float* M2, const float* M3, float* H,
+                      cudaStream_t s);
 int simt_expand_consume_blocks(const Shape& sh);
 // adjoint stage: R[p][t][x][b][g] = sum_{y,z} A_t2[y][b] A_t3[z][g] (prod)[x][y][z]
 // for nt terms (M2 [nt][n2][r2], M3 [nt][n3][r3]); with PROD_PLAIN q_p is the field SA[p] itself

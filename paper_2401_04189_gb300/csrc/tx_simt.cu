@@ -674,6 +674,8 @@ struct ConsumeF32Args {
     double* epart;
     int ty, px, ny, gc, bc, rows, vec;
     int m2_flat, z_mode;       // M2 part / Z part as one contiguous run (z_mode 2), Z rows of g (1) or of b (0)
+    int tc;                    // terms per CTA: blockIdx.z takes terms z tc .. z tc + tc - 1 (EPI_STORE), nt otherwise
+    long out_ps, out_cs;       // EPI_STORE: floats between the results of two pairs, of two term groups
 };
 
 // Registers: 8 RN for phi, 8 per mode-2 column; the K part of mode 3 (gc) is at most CL * kMaxPart
@@ -753,8 +755,9 @@ __global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_co
         cp_async_commit();
     };
 
-    load2(0, 0, 0);
-    for (int t = 0; t < a.nt; ++t)
+    const int t0 = blockIdx.z * a.tc, t1 = min(a.nt, t0 + a.tc);
+    load2(t0, 0, 0);
+    for (int t = t0; t < t1; ++t)
         for (int gp = 0; gp < ng; ++gp) {
             const int gn = min(a.gc, d.r3 - gp * a.gc), rg = (gn + CL - 1) / CL;
             uint64_t y[MRG][4];
@@ -780,7 +783,7 @@ __global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_co
             cp_async_wait_all();
             __syncthreads();                   // Y and M3 are there, M2 and Z free
             if (gp + 1 < ng) load2(t, gp + 1, 0);
-            else if (t + 1 < a.nt) load2(t + 1, 0, 0);
+            else if (t + 1 < t1) load2(t + 1, 0, 0);
 #pragma unroll 2
             for (int g = 0; g < gn; ++g) {
                 const float4 ya = *(const float4*)(ys + g * ldy + row0), yb = *(const float4*)(ys + g * ldy + row0 + 4);
@@ -835,7 +838,7 @@ __global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_co
             else ph = unpack2(acc[i][c]);
             const float phi[2] = {ph.x, ph.y};
             if (a.flags & EPI_STORE) {
-                float* dst = a.f.OUT0 + pl * N3 + base + z;
+                float* dst = a.f.OUT0 + pl * a.out_ps + blockIdx.z * a.out_cs + base + z;
                 if (z < d.n3) dst[0] = phi[0];
                 if (z + 1 < d.n3) dst[1] = phi[1];
                 continue;
@@ -878,6 +881,17 @@ __global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_co
         const double s = block_sum(e * rec.ew, red);
         if (tid == 0) a.epart[(long)pl * gridDim.x + blockIdx.x] = s;
     }
+}
+
+// out[p][e] = sum_c part[p][c][e], the groups of terms in their order
+__global__ void __launch_bounds__(256) k_sum_groups(const float* __restrict__ part, long ps, long cs, int nc, long N,
+                                                    float* __restrict__ out) {
+    const long e = blockIdx.x * 256L + threadIdx.x;
+    if (e >= N) return;
+    const float* q = part + blockIdx.y * ps + e;
+    float v = q[0];
+    for (int c = 1; c < nc; ++c) v += q[c * cs];
+    out[blockIdx.y * N + e] = v;
 }
 
 // dst[t][k][i] (row stride ld, zero past n) = src[t][i][k]: operators with the grid index fastest
@@ -1101,10 +1115,30 @@ template <int CL, int RN4, int H>
 int launch_consume(const ConsumeF32Args& a, const SimtPlan& p, int np, cudaStream_t s) {
     TX_TRY(smem_attr((const void*)k_consume<CL, RN4, H>, p.smem));
     const int ps = prof_begin("consume", s);
-    k_consume<CL, RN4, H><<<dim3(p.nx * p.ny, np), p.threads, p.smem, s>>>(a);
+    k_consume<CL, RN4, H><<<dim3(p.nx * p.ny, np, (a.nt + a.tc - 1) / a.tc), p.threads, p.smem, s>>>(a);
     prof_end(ps, s);
     TX_LAUNCHED();
     return TX_OK;
+}
+
+int dispatch_consume(const ConsumeF32Args& a, const SimtPlan& p, int np, cudaStream_t s) {
+    if (p.cl == 8) {
+        switch (p.rn2) {
+            case 1: return launch_consume<8, 0, 1>(a, p, np, s);
+            case 2: return launch_consume<8, 1, 0>(a, p, np, s);
+            case 3: return launch_consume<8, 1, 1>(a, p, np, s);
+            case 4: return launch_consume<8, 2, 0>(a, p, np, s);
+            case 5: return launch_consume<8, 2, 1>(a, p, np, s);
+            default: return launch_consume<8, 3, 0>(a, p, np, s);
+        }
+    }
+    switch (p.rn2) {
+        case 4: return launch_consume<16, 2, 0>(a, p, np, s);
+        case 5: return launch_consume<16, 2, 1>(a, p, np, s);
+        case 6: return launch_consume<16, 3, 0>(a, p, np, s);
+        case 7: return launch_consume<16, 3, 1>(a, p, np, s);
+        default: return launch_consume<16, 4, 0>(a, p, np, s);
+    }
 }
 }  // namespace
 
@@ -1138,7 +1172,7 @@ int simt_kmajor(const float* src, int nt, int n, int r, int ld, float* dst, cuda
 
 int simt_expand_consume(const Shape& sh, const PairRec* recs, int p0, int np, const FieldArgs& f, const float* Z,
                         int nterms, const float* M2, const float* M3, int flags, double* epart, cudaStream_t s,
-                        bool z_bg, long m2_ps, long m3_ps) {
+                        bool z_bg, long m2_ps, long m3_ps, int group) {
     const Dims d = dims_of(sh);
     if (d.n3 > 256) return fail(TX_ERR_UNSUPPORTED_SHAPE, "float32 path supports n3 <= 256");
     SimtPlan p{};
@@ -1154,8 +1188,16 @@ int simt_expand_consume(const Shape& sh, const PairRec* recs, int p0, int np, co
     a.f = f;
     a.w1 = sh.w1; a.w2 = sh.w2; a.w3 = sh.w3;
     a.flags = flags; a.epart = epart;
+    a.tc = nterms;
+    a.out_ps = (long)d.n1 * d.n2 * d.n3;
     a.ty = p.ty; a.px = p.px; a.ny = p.ny; a.gc = p.gc; a.bc = p.bc; a.rows = p.rows;
     a.m2_flat = p.ny == 1;
+    if (group > 0 && group < nterms) {         // a group's sum goes where its first term was: see simt_core_consume
+        a.tc = group;
+        a.f.OUT0 = (float*)Z;
+        a.out_ps = nterms * ((long)d.n1 * d.n2 * d.n3);
+        a.out_cs = group * ((long)d.n1 * d.n2 * d.n3);
+    }
     // a part of Z is one 16-byte aligned run where g is its fastest index and the part holds every g
     const long rr = (long)d.r2 * d.r3;
     a.z_mode = !z_bg ? 0
@@ -1163,23 +1205,30 @@ int simt_expand_consume(const Shape& sh, const PairRec* recs, int p0, int np, co
                   ((uintptr_t)Z & 15u) == 0) ? 2 : 1;
     // pairs of z as one access: even rows, and arrays (callers' blocks and slices) that start on 8 bytes
     a.vec = d.n3 % 2 == 0 && (((uintptr_t)f.MUL0 | (uintptr_t)f.MUL1 | (uintptr_t)f.OUT0 | (uintptr_t)f.OUT1) & 7u) == 0;
-    if (p.cl == 8) {
-        switch (p.rn2) {
-            case 1: return launch_consume<8, 0, 1>(a, p, np, s);
-            case 2: return launch_consume<8, 1, 0>(a, p, np, s);
-            case 3: return launch_consume<8, 1, 1>(a, p, np, s);
-            case 4: return launch_consume<8, 2, 0>(a, p, np, s);
-            case 5: return launch_consume<8, 2, 1>(a, p, np, s);
-            default: return launch_consume<8, 3, 0>(a, p, np, s);
-        }
-    }
-    switch (p.rn2) {
-        case 4: return launch_consume<16, 2, 0>(a, p, np, s);
-        case 5: return launch_consume<16, 2, 1>(a, p, np, s);
-        case 6: return launch_consume<16, 3, 0>(a, p, np, s);
-        case 7: return launch_consume<16, 3, 1>(a, p, np, s);
-        default: return launch_consume<16, 4, 0>(a, p, np, s);
-    }
+    return dispatch_consume(a, p, np, s);
+}
+
+int simt_core_consume(const Shape& sh, int np, float* Z, int nterms, const float* M2, const float* M3, float* H,
+                      cudaStream_t s) {
+    const Dims d = dims_of(sh);
+    SimtPlan p{};
+    FieldArgs f{};
+    f.OUT0 = H;
+    if (d.n1 != d.r1 || d.n2 != d.r2 || d.n3 != d.r3 || d.n3 > 256 || !simt_plan(d, &p) || p.ny != 1)
+        return simt_expand_consume(sh, nullptr, 0, np, f, Z, nterms, M2, M3, EPI_STORE, nullptr, s);
+    // Fewer CTAs than SMs: groups of at least 4 terms go to CTAs of their own, towards two per SM, and a
+    // second kernel adds their sums, which lie where each group's first term of Z was (one y tile: no other
+    // CTA reads that slab).  A call of 6 pairs of rank (13, 18, 23), 22 terms: 144 us; 257 with every term
+    // in one CTA.  From one CTA per SM on the terms stay together and no second kernel is launched.
+    const long ctas = (long)p.nx * np;
+    const int groups = ctas >= 152 ? 1 : (int)std::min<long>((303 + ctas) / ctas, std::max(1, nterms / 4));
+    const int tc = (nterms + groups - 1) / groups, nc = (nterms + tc - 1) / tc;
+    if (nc == 1) return simt_expand_consume(sh, nullptr, 0, np, f, Z, nterms, M2, M3, EPI_STORE, nullptr, s);
+    TX_TRY(simt_expand_consume(sh, nullptr, 0, np, f, Z, nterms, M2, M3, EPI_STORE, nullptr, s, true, 0, 0, tc));
+    const long N = (long)d.n1 * d.n2 * d.n3;
+    k_sum_groups<<<dim3((unsigned)((N + 255) / 256), np), 256, 0, s>>>(Z, nterms * N, tc * N, nc, N, H);
+    TX_LAUNCHED();
+    return TX_OK;
 }
 
 int simt_adjoint_r(const Shape& sh, const PairRec* recs, int p0, int np, const FieldArgs& f, int nt, const float* M2,
