@@ -32,10 +32,10 @@ struct tx_transfer {
     int n[3];
     int n_nodes, n_cells, pu, ps;
     long n_map;                // structured nodes (every one is mapped to a cell)
-    int max_cell;              // most structured nodes in one cell
-    int* d_cell_start;         // [n_cells + 1] offsets into snode / N
+    int n_blocks;
+    void* d_blocks;            // [n_blocks] UBlock: each cell's mapped nodes in pieces
     int* d_snode;              // [n_map] flat structured index of each mapped node, grouped by cell
-    float* d_N;                // [n_map][(pu + 1)^3]
+    float* d_N;                // [(pu + 1)^3][n_map]
     int* d_conn;               // [n_cells][(pu + 1)^3]
     int* d_ebase;              // [n_nodes] flat structured index of local node 0 of b's element
     float* d_M;                // [n_nodes][(ps + 1)^3]
@@ -48,56 +48,94 @@ namespace {
 constexpr uint32_t kTransferMagic = 0x54555446u;
 constexpr int kChunk = 32;     // orbitals per pass
 
-// One CTA per (cell, block of kUNodes of its structured nodes): the cell's orbital rows
-// (kUChunk orbitals at a time) are staged in shared memory; each thread takes one structured
-// node, keeps its N row in registers and writes that node for every orbital of the chunk
-// (neighbouring threads on neighbouring nodes, so each orbital's writes are runs along z).
-// Splitting the large cells over several CTAs keeps all SMs busy when coarse and refined cells
-// hold very different numbers of nodes.
+// One CTA per block of one cell's structured nodes (UBlock; at most kUThreads * u_nodes of them, so that the
+// cells' different sizes fill all SMs).  The cell's orbital rows (kUChunk orbitals at a time) are staged in
+// shared memory; a thread holds the N rows of up to u_nodes structured nodes in registers and writes those
+// nodes for every orbital of the chunk (neighbouring threads on neighbouring nodes, so each orbital's writes
+// are runs along z).  N is stored [local node][mapped node], so a warp reads it in whole lines.
+// With one node per thread the shared-memory reads were the bound: a 16-byte broadcast occupies the port
+// for as long as 16 multiply-adds per lane take, and fed 4.  160^3 nodes, quadratic cells, 64 orbitals: 743
+// us with one node per thread and N rows read 108 bytes apart, 631 with two, 619 with four (the registers
+// allow two with 64 local nodes).  What is left is bound by the writes, runs as short as a cell is wide to
+// 64 orbitals 16 MB apart (1.7 TB/s).
 constexpr int kUChunk = 128;
-constexpr int kUNodes = 256;
+constexpr int kUThreads = 128;
+__host__ __device__ constexpr int u_nodes(int nb) { return nb > 27 ? 2 : 4; }
+
+struct UBlock {
+    int cell, k0, m;           // mapped nodes k0 .. k0 + m - 1, all of one cell
+};
+
+template <int NB, int NT>
+__device__ __forceinline__ void u_to_s_nodes(const float* v, const float* __restrict__ N, const int* __restrict__ snode,
+                                             long n_map, int k0, int m, int ni, long n3, float* __restrict__ dst) {
+    float w[NT][NB];
+    int at[NT], k[NT];
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+        k[j] = min((int)threadIdx.x + j * kUThreads, m - 1);
+        at[j] = snode[k0 + k[j]];
+    }
+    const float* Nb = N + k0;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        if (b % 8 == 7) asm volatile("" : "+l"(Nb));           // one running pointer, not one per local node
+#pragma unroll
+        for (int j = 0; j < NT; ++j) w[j][b] = __ldg(Nb + k[j]);
+        Nb += n_map;
+    }
+    // four orbitals per pass: one 16-byte broadcast feeds 4 NT FMAs (the staged chunk is zero up to the next
+    // multiple of four past ni; the stores are guarded)
+    for (int ii = 0; ii < ni; ii += 4, dst += 4 * n3) {
+        float s[NT][4];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) s[j][0] = s[j][1] = s[j][2] = s[j][3] = 0.f;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            if (b % 4 == 0) asm volatile("" ::: "memory");     // at most four reads in flight: the registers hold N
+            const float4 q = *reinterpret_cast<const float4*>(v + b * kUChunk + ii);
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                s[j][0] = fmaf(w[j][b], q.x, s[j][0]);
+                s[j][1] = fmaf(w[j][b], q.y, s[j][1]);
+                s[j][2] = fmaf(w[j][b], q.z, s[j][2]);
+                s[j][3] = fmaf(w[j][b], q.w, s[j][3]);
+            }
+        }
+        float* row = dst;
+#pragma unroll
+        for (int o = 0; o < 4; ++o, row += n3)
+            if (ii + o < ni)
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+                    if (threadIdx.x + j * kUThreads < m) row[at[j]] = s[j][o];
+    }
+}
 
 template <int NB>
-__global__ void __launch_bounds__(256) k_u_to_s(const int* __restrict__ cell_start, const int* __restrict__ snode,
-                                                const float* __restrict__ N, const int* __restrict__ conn,
-                                                const float* __restrict__ psi_u, int n_orb, long n3,
-                                                float* __restrict__ psi_s) {
+__global__ void __launch_bounds__(kUThreads, NB == 8 ? 6 : 3)
+    k_u_to_s(const UBlock* __restrict__ blocks, const int* __restrict__ snode, const float* __restrict__ N, long n_map,
+             const int* __restrict__ conn, const float* __restrict__ psi_u, int n_orb, long n3, float* __restrict__ psi_s) {
     extern __shared__ __align__(16) float v[];   // [NB][kUChunk]
-    const int c = blockIdx.x;
-    const int kc = cell_start[c], kb = blockIdx.y * kUNodes;
-    const int k0 = kc + kb, m = min(kUNodes, cell_start[c + 1] - k0);
-    if (m <= 0) return;
+    const UBlock blk = blocks[blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i0 = 0; i0 < n_orb; i0 += kUChunk) {
         const int ni = min(kUChunk, n_orb - i0);
         __syncthreads();
-        for (int e = threadIdx.x; e < NB * kUChunk; e += blockDim.x) {
-            const int b = e / kUChunk, ii = e % kUChunk;
-            v[e] = ii < ni ? psi_u[(long)conn[(long)c * NB + b] * n_orb + i0 + ii] : 0.f;
+        for (int b = warp; b < NB; b += kUThreads / 32) {
+            const float* src = psi_u + (long)conn[(long)blk.cell * NB + b] * n_orb + i0;
+            for (int ii = lane; ii < ((ni + 3) & ~3); ii += 32) v[b * kUChunk + ii] = ii < ni ? src[ii] : 0.f;
         }
         __syncthreads();
-        for (int k = threadIdx.x; k < m; k += blockDim.x) {
-            float w[NB];
-            const float* Nk = N + (long)(k0 + k) * NB;
-#pragma unroll
-            for (int b = 0; b < NB; ++b) w[b] = __ldg(Nk + b);
-            float* dst = psi_s + (long)i0 * n3 + snode[k0 + k];
-            // four orbitals per pass: one 16-byte shared-memory broadcast feeds four FMAs (the
-            // staged chunk is zero beyond ni, so the reads stay inside it; the stores are guarded)
-            for (int ii = 0; ii < ni; ii += 4) {
-                float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    const float4 q = *reinterpret_cast<const float4*>(v + b * kUChunk + ii);
-                    s0 = fmaf(w[b], q.x, s0);
-                    s1 = fmaf(w[b], q.y, s1);
-                    s2 = fmaf(w[b], q.z, s2);
-                    s3 = fmaf(w[b], q.w, s3);
+        float* dst = psi_s + (long)i0 * n3;
+        switch ((blk.m + kUThreads - 1) / kUThreads) {
+            case 1: u_to_s_nodes<NB, 1>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst); break;
+            case 2: u_to_s_nodes<NB, 2>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst); break;
+            default:
+                if constexpr (u_nodes(NB) > 2) {
+                    if (blk.m <= 3 * kUThreads) u_to_s_nodes<NB, 3>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst);
+                    else u_to_s_nodes<NB, 4>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst);
                 }
-                dst[(long)ii * n3] = s0;
-                if (ii + 1 < ni) dst[(long)(ii + 1) * n3] = s1;
-                if (ii + 2 < ni) dst[(long)(ii + 2) * n3] = s2;
-                if (ii + 3 < ni) dst[(long)(ii + 3) * n3] = s3;
-            }
         }
     }
 }
@@ -152,7 +190,7 @@ void lagrange(const double* nd, int p, double x, double* out) {
 
 void transfer_free(tx_transfer* t) {
     if (!t) return;
-    cudaFree(t->d_cell_start);
+    cudaFree(t->d_blocks);
     cudaFree(t->d_snode);
     cudaFree(t->d_N);
     cudaFree(t->d_conn);
@@ -211,7 +249,7 @@ extern "C" int tx_transfer_create(tx_transfer** out, tx_ctx* c, int order_s, con
     // ---- unstructured -> structured: structured nodes of each cell, first cell wins ----
     std::vector<char> done(N3, 0);
     std::vector<int> cell_start(n_cells + 1, 0), snode;
-    std::vector<float> Nv;
+    std::vector<float> Nv((size_t)nb * N3);        // [local node][mapped node]
     std::vector<double> ax[3];
     for (int d = 0; d < 3; ++d) ax[d].resize(pu + 1);
     double L[3][4];
@@ -240,13 +278,14 @@ extern "C" int tx_transfer_create(tx_transfer** out, tx_ctx* c, int order_s, con
                     const long a = ((long)i * n2 + j) * n3 + k;
                     if (done[a]) continue;
                     done[a] = 1;
+                    float* Nk = Nv.data() + snode.size();
                     snode.push_back((int)a);
                     lagrange(ax[0].data(), pu, xs[0][i], L[0]);
                     lagrange(ax[1].data(), pu, xs[1][j], L[1]);
                     lagrange(ax[2].data(), pu, xs[2][k], L[2]);
                     for (int lx = 0; lx <= pu; ++lx)
                         for (int ly = 0; ly <= pu; ++ly)
-                            for (int lz = 0; lz <= pu; ++lz) Nv.push_back((float)(L[0][lx] * L[1][ly] * L[2][lz]));
+                            for (int lz = 0; lz <= pu; ++lz, Nk += N3) *Nk = (float)(L[0][lx] * L[1][ly] * L[2][lz]);
                 }
     }
     cell_start[n_cells] = (int)snode.size();
@@ -278,10 +317,18 @@ extern "C" int tx_transfer_create(tx_transfer** out, tx_ctx* c, int order_s, con
     t->pu = pu;
     t->ps = ps;
     t->n_map = (long)snode.size();
-    t->max_cell = 0;
-    for (int cc = 0; cc < n_cells; ++cc) t->max_cell = std::max(t->max_cell, cell_start[cc + 1] - cell_start[cc]);
+    std::vector<UBlock> blocks;
+    const int most = kUThreads * u_nodes(nb);
+    for (int cc = 0; cc < n_cells; ++cc) {
+        const int k0 = cell_start[cc], cnt = cell_start[cc + 1] - k0, pieces = (cnt + most - 1) / most;
+        for (int q = 0; q < pieces; ++q) {
+            const int a = (int)((long)cnt * q / pieces), b = (int)((long)cnt * (q + 1) / pieces);
+            blocks.push_back(UBlock{cc, k0 + a, b - a});
+        }
+    }
+    t->n_blocks = (int)blocks.size();
     std::vector<int> connv(conn, conn + (long)n_cells * nb);
-    int st = upload(&t->d_cell_start, cell_start, "cell offsets");
+    int st = upload((UBlock**)&t->d_blocks, blocks, "cell blocks");
     if (st == TX_OK) st = upload(&t->d_snode, snode, "structured nodes");
     if (st == TX_OK) st = upload(&t->d_N, Nv, "shape values");
     if (st == TX_OK) st = upload(&t->d_conn, connv, "cells");
@@ -305,11 +352,12 @@ extern "C" int tx_transfer_u_to_s(tx_transfer* t, const float* psi_u, int n_orb,
     cudaStream_t s = (cudaStream_t)stream;
     const long N3 = (long)t->n[0] * t->n[1] * t->n[2];
     const size_t sm1 = sizeof(float) * 8 * kUChunk, sm2 = sizeof(float) * 27 * kUChunk, sm3 = sizeof(float) * 64 * kUChunk;
-    const dim3 grid((unsigned)t->n_cells, (unsigned)std::max(1, (t->max_cell + kUNodes - 1) / kUNodes));
+    const UBlock* blk = (const UBlock*)t->d_blocks;
+    const unsigned grid = (unsigned)t->n_blocks;
     switch (t->pu) {
-        case 1: k_u_to_s<8><<<grid, 256, sm1, s>>>(t->d_cell_start, t->d_snode, t->d_N, t->d_conn, psi_u, n_orb, N3, psi_s); break;
-        case 2: k_u_to_s<27><<<grid, 256, sm2, s>>>(t->d_cell_start, t->d_snode, t->d_N, t->d_conn, psi_u, n_orb, N3, psi_s); break;
-        default: k_u_to_s<64><<<grid, 256, sm3, s>>>(t->d_cell_start, t->d_snode, t->d_N, t->d_conn, psi_u, n_orb, N3, psi_s); break;
+        case 1: k_u_to_s<8><<<grid, kUThreads, sm1, s>>>(blk, t->d_snode, t->d_N, t->n_map, t->d_conn, psi_u, n_orb, N3, psi_s); break;
+        case 2: k_u_to_s<27><<<grid, kUThreads, sm2, s>>>(blk, t->d_snode, t->d_N, t->n_map, t->d_conn, psi_u, n_orb, N3, psi_s); break;
+        default: k_u_to_s<64><<<grid, kUThreads, sm3, s>>>(blk, t->d_snode, t->d_N, t->n_map, t->d_conn, psi_u, n_orb, N3, psi_s); break;
     }
     TX_LAUNCHED();
     return TX_OK;
@@ -337,7 +385,7 @@ extern "C" int tx_transfer_s_to_u(tx_transfer* t, const float* psi_s, int n_orb,
 extern "C" long tx_transfer_map_bytes(const tx_transfer* t) {
     if (!t || t->magic != kTransferMagic) return 0;
     const long nb = (long)(t->pu + 1) * (t->pu + 1) * (t->pu + 1), ns = (long)(t->ps + 1) * (t->ps + 1) * (t->ps + 1);
-    return 4L * (t->n_cells + 1) + 4L * t->n_map * (1 + nb) + 4L * t->n_cells * nb + 4L * t->n_nodes * (1 + ns);
+    return (long)sizeof(UBlock) * t->n_blocks + 4L * t->n_map * (1 + nb) + 4L * t->n_cells * nb + 4L * t->n_nodes * (1 + ns);
 }
 
 extern "C" void tx_transfer_destroy(tx_transfer* t) {
