@@ -292,6 +292,7 @@ int tx_set_tile_plan(tx_ctx* ctx, int bx, int nstage);
 
 /* Split precisions (TF32x3, BF16x3): phi = sum_t mu_t G x_d A_td (the final contraction of the
  * expansion, Eq. final) is accumulated on the tensor core for `terms` Gaussian terms at a time
+ * (of those that run there: smooth terms are summed in float32 on a coarse grid)
  * and then added into a float32 accumulator held in registers (round to nearest).  The tensor
  * core rounds its float32 accumulator toward zero after every MMA, so the error grows with the
  * length of each tensor-core chunk; the hi*hi and the cross products (hi*lo + lo*hi) are
