@@ -55,12 +55,13 @@ constexpr int kChunk = 32;     // orbitals per pass
 // are runs along z).  N is stored [local node][mapped node], so a warp reads it in whole lines.
 // With one node per thread the shared-memory reads were the bound: a 16-byte broadcast occupies the port
 // for as long as 16 multiply-adds per lane take, and fed 4.  160^3 nodes, quadratic cells, 64 orbitals: 743
-// us with one node per thread and N rows read 108 bytes apart, 631 with two, 619 with four (the registers
-// allow two with 64 local nodes).  What is left is bound by the writes, runs as short as a cell is wide to
+// us with one node per thread and N rows read 108 bytes apart; 605 with two and six CTAs per SM, 619 with four
+// and three, 611 with three and four, which is 3 to 8% ahead of four on smaller quadratic meshes.  Linear cells
+// take four nodes, cubic ones the two that the registers allow.  What is left is bound by the writes, runs as short as a cell is wide to
 // 64 orbitals 16 MB apart (1.7 TB/s).
 constexpr int kUChunk = 128;
 constexpr int kUThreads = 128;
-__host__ __device__ constexpr int u_nodes(int nb) { return nb > 27 ? 2 : 4; }
+__host__ __device__ constexpr int u_nodes(int nb) { return nb > 27 ? 2 : nb > 8 ? 3 : 4; }
 
 struct UBlock {
     int cell, k0, m;           // mapped nodes k0 .. k0 + m - 1, all of one cell
@@ -113,7 +114,7 @@ __device__ __forceinline__ void u_to_s_nodes(const float* v, const float* __rest
 }
 
 template <int NB>
-__global__ void __launch_bounds__(kUThreads, NB == 8 ? 6 : 3)
+__global__ void __launch_bounds__(kUThreads, NB == 8 ? 6 : NB == 27 ? 4 : 3)
     k_u_to_s(const UBlock* __restrict__ blocks, const int* __restrict__ snode, const float* __restrict__ N, long n_map,
              const int* __restrict__ conn, const float* __restrict__ psi_u, int n_orb, long n3, float* __restrict__ psi_s) {
     extern __shared__ __align__(16) float v[];   // [NB][kUChunk]
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(kUThreads, NB == 8 ? 6 : 3)
             default:
                 if constexpr (u_nodes(NB) > 2) {
                     if (blk.m <= 3 * kUThreads) u_to_s_nodes<NB, 3>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst);
-                    else u_to_s_nodes<NB, 4>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst);
+                    else u_to_s_nodes<NB, u_nodes(NB)>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst);
                 }
         }
     }
