@@ -202,7 +202,7 @@ struct Shape {
     const float* w3;
 };
 Shape fine_shape(const tx_ctx* c);
-// the coarse grid of the smooth terms: r_d nodes, ranks r_d (weights unused); swapped: modes 2 and 3 exchanged
+// the coarse grid of the smooth terms: r_d nodes, ranks r_d, no weights; swapped: modes 2 and 3 exchanged
 Shape coarse_shape(const tx_ctx* c, bool swapped = false);
 
 struct FieldArgs {          // orbital-space arrays of one call

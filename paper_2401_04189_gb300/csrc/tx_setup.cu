@@ -300,9 +300,10 @@ Shape fine_shape(const tx_ctx* c) {
     return Shape{c->n[0], c->n[1], c->n[2], c->r[0], c->r[1], c->r[2], c->f_w[0], c->f_w[1], c->f_w[2]};
 }
 Shape coarse_shape(const tx_ctx* c, bool swapped) {
-    if (swapped)
-        return Shape{c->r[0], c->r[2], c->r[1], c->r[0], c->r[2], c->r[1], c->f_w[0], c->f_w[1], c->f_w[2]};
-    return Shape{c->r[0], c->r[1], c->r[2], c->r[0], c->r[1], c->r[2], c->f_w[0], c->f_w[1], c->f_w[2]};
+    // the grid's own weights are not the coarse nodes', and with modes 2 and 3 exchanged n_2 of them may be
+    // fewer than the r_3 rows
+    const int r2 = swapped ? c->r[2] : c->r[1], r3 = swapped ? c->r[1] : c->r[2];
+    return Shape{c->r[0], r2, r3, c->r[0], r2, r3, nullptr, nullptr, nullptr};
 }
 
 }  // namespace tx

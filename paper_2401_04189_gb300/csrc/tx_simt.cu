@@ -823,12 +823,14 @@ __global__ void __launch_bounds__(consume_max_threads(CL, 4 * RN4 + 2 * H)) k_co
     const float* mul1 = a.f.MUL1 + rec.m1 * N3;
     float* out0 = a.f.OUT0 + rec.o0 * N3;
     float* out1 = a.f.OUT1 + rec.o1 * N3;
-    const float wx = x < d.n1 ? a.w1[x] : 0.f;
+    // a coarse grid has no weights (they are null)
+    const bool weighted = (a.flags & (EPI_MULW | EPI_ENERGY)) != 0;
+    const float wx = weighted && x < d.n1 ? a.w1[x] : 0.f;
 #pragma unroll
     for (int i = 0; i < kRows; ++i) {
         const int y = y0 + yr + i;
         if (!rows_ok || y >= d.n2) continue;
-        const float wxy = wx * a.w2[y];
+        const float wxy = weighted ? wx * a.w2[y] : 0.f;
         const long base = ((long)x * d.n2 + y) * d.n3;
 #pragma unroll
         for (int c = 0; c < NP; ++c) {
