@@ -2580,9 +2580,17 @@ static bool plan_cv(const tx_ctx* c, bool tf32, bool split, int bx, int nload, i
     p->loadB = ((uint32_t)(m * p->b3) + 1023) & ~1023u;
     p->nload = nload;
     p->na3 = na3;
+    // rows that the MMAs of a last sub-tile read behind it (see above): of A_t2 and Z inside the rings where
+    // those are long enough, of the converted operand behind everything.  Charged as read and no more: a flat
+    // 4 KB here refused shapes within 4 KB of the limit, (40, 192, 84) with ranks (20, 89, 71) in TF32 among them.
+    const size_t ya_over = (size_t)(p->nY * 128 - (int)p->ya_rows) * 32;
+    const size_t z_over = split ? (size_t)(p->Nz - (int)p->z_rows) * 32 : 0;
+    const size_t a3_over = p->ts3 ? 0 : (size_t)(p->nT3 * 128 - (int)p->a3_rows) * 32;
+    const size_t last = (size_t)p->load * (nload - 1) + (size_t)m * p->ya;       // the last stage's Z
     for (p->nloadB = std::min(tcc::kMaxLoadB, nload + 1); p->nloadB >= 1; --p->nloadB) {
         p->a3_off = p->load * nload + p->loadB * p->nloadB;
-        const size_t total = (size_t)p->a3_off + (size_t)na3 * m * p->a3 + 128 * 32;   // the last sub-tile's other rows
+        const size_t total = std::max({last + ya_over, last + (size_t)m * p->zb + z_over,
+                                       (size_t)p->a3_off + (size_t)na3 * m * p->a3 + a3_over});
         p->smem = std::max(total, (size_t)tcc::kEpiBytes) + 1024;   // the epilogue reuses the front
         if (p->smem <= 226 * 1024) return true;
     }
