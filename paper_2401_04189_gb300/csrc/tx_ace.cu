@@ -1,7 +1,7 @@
 // Adaptively compressed exchange (the paper's "ACE implementation" section, Eqs. eta and ace1),
 // built on top of the exchange potentials W_i = K psi_i of the hot path:
 //
-//   M_ij = <psi_i, W_j>_w                 weighted Gram matrix (float32 products, float64 sums)
+//   M_ij = <psi_i, W_j>_w                 weighted Gram matrix (float32 sums of 32, float64 beyond)
 //   M_s  = (M + M^T) / 2                  (the paper is silent on the asymmetry a truncated Tucker
 //                                          rank leaves; the symmetric part is factorised)
 //   -M_s = L L^T                          Cholesky, float64 (M_s is negative definite)
@@ -9,8 +9,8 @@
 //   V_ACE f = - sum_k xi_k <xi_k, f>_w    the ACE operator applied to a block
 //
 // The Gram matrices and the two small-by-large products cost O(N^2 n^3) flops, about 0.1% of the
-// N^2 / 2 pair potentials behind W, so they run on the CUDA cores: float32 products summed in
-// float64 across the grid (the factorisation needs M to about the accuracy of W).
+// N^2 / 2 pair potentials behind W, so they run on the CUDA cores: float32 sums of 32
+// products, summed in float64 across the grid (the factorisation needs M to about the accuracy of W).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -25,6 +25,7 @@ namespace {
 
 constexpr int kGramChunk = 64;    // grid points per shared-memory chunk
 constexpr int kGramLd = kGramChunk + 4;
+constexpr int kGramFold = 64;     // chunks per float64 addition
 
 __device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
@@ -34,6 +35,27 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+    uint64_t r;       // a - 1 b: the product is exact
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
+    return r;
+}
+// the rounded sum, and its exact error in e (Knuth's TwoSum; no condition on the magnitudes)
+__device__ __forceinline__ uint64_t two_sum(uint64_t a, uint64_t b, uint64_t& e) {
+    const uint64_t t = add2(a, b), c = sub2(t, a);
+    e = add2(sub2(a, sub2(t, c)), sub2(b, c));
+    return t;
+}
+__device__ __forceinline__ float lo2(uint64_t v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    return (uint64_t)__float_as_uint(a) | (uint64_t)__float_as_uint(b) << 32;
+}
 __device__ __forceinline__ void cp_async16(float* dst, const float* src, bool ok) {
     const int bytes = ok ? 16 : 0;       // 0: the 16 bytes are zero-filled and src is not read
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
@@ -41,14 +63,18 @@ __device__ __forceinline__ void cp_async16(float* dst, const float* src, bool ok
                  : "memory");
 }
 
-// partial[s][i][j] = sum over slice s of the grid of w(x) A_i(x) B_j(x): float32 within a chunk of 64
-// points (two sums of 32), and across chunks a compensated float32 sum (Kahan; a pair of floats
-// carries 48 bits), as this GPU adds float64 at 1/64 of the float32 rate.  BI x BJ outputs per CTA
+// partial[s][i][j] = sum over slice s of the grid of w(x) A_i(x) B_j(x): float32 sums of 32 products (the even and
+// the odd points of a chunk of 64), added in float64 in effect.  This GPU adds float64 at 1/64 of the float32 rate,
+// so the sums of up to 64 chunks are added in float32 with every rounding error caught exactly (Knuth's TwoSum) and
+// summed beside, and the pair is then added to the float64 partial in memory, which only this thread touches.
+// What a group loses is the rounding of its error sum, at most 2^-34 of the sum of its terms' magnitudes; the
+// terms' own rounding is 2^-24 and more.  (With a Kahan sum in place of this, chunk sums of 1, 1e8, 1, -1e8 came out
+// as 0.)  BI x BJ outputs per CTA
 // of 128 threads (8 x 16), (BI / 8) x (BJ / 16) each.  The orbitals keep their own layout in shared
 // memory (rows along the grid, stride 68: the 16-byte reads of 16 rows hit different banks) and the
 // packed multiply-adds run along the grid, so nothing is transposed or duplicated; two buffers, filled
-// by cp.async.  64 x 64 orbitals of 96^3: 245 us; 317 with 4 x 4 outputs per thread and chunks of
-// 32, 1554 with one output per thread and a float64 add per chunk (the orbitals take 67 us of HBM time).
+// by cp.async.  The whole apply of 64 x 64 orbitals of 96^3: 439 us; 448 with a Kahan sum, 2,024 with one output
+// per thread and a float64 add per 32 points (the orbitals take 67 us of HBM time).
 template <int BI, int BJ>
 __global__ void __launch_bounds__(128) k_wgram(const float* __restrict__ A, int na, const float* __restrict__ B, int nb,
                                                const float* __restrict__ w1, const float* __restrict__ w2,
@@ -96,62 +122,72 @@ __global__ void __launch_bounds__(128) k_wgram(const float* __restrict__ A, int 
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float sum[TI][TJ], comp[TI][TJ];
-#pragma unroll
-    for (int i = 0; i < TI; ++i)
-#pragma unroll
-        for (int j = 0; j < TJ; ++j) sum[i][j] = comp[i][j] = 0.f;
+    uint64_t sum[TI / 2][TJ], err[TI / 2][TJ];             // rows i and i + 1 in one register pair
     if (x0 < x1) load(x0, 0);
     int buf = 0;
-    for (long xc = x0; xc < x1; xc += kGramChunk, buf ^= 1) {
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();                 // this chunk has landed; the other buffer has been read
-        if (xc + kGramChunk < x1) load(xc + kGramChunk, buf ^ 1);
-        const float* As = sm + buf * kBuf;
-        const float* Bs = As + BI * kGramLd;
-        const float* ws = Bs + BJ * kGramLd;
-        uint64_t acc[TI][TJ];
+    bool first = true;
+    for (long xc = x0; first || xc < x1; first = false) {
 #pragma unroll
-        for (int i = 0; i < TI; ++i)
+        for (int i = 0; i < TI / 2; ++i)
 #pragma unroll
-            for (int j = 0; j < TJ; ++j) acc[i][j] = 0ull;
-#pragma unroll 4
-        for (int k = 0; k < kGramChunk; k += 4) {
-            const ulonglong2 w = *(const ulonglong2*)(ws + k);
-            ulonglong2 a[TI], b[TJ];
-#pragma unroll
-            for (int j = 0; j < TJ; ++j) {
-                const ulonglong2 v = *(const ulonglong2*)(Bs + (tj + 16 * j) * kGramLd + k);
-                b[j] = make_ulonglong2(mul2(v.x, w.x), mul2(v.y, w.y));
-            }
-#pragma unroll
-            for (int i = 0; i < TI; ++i) a[i] = *(const ulonglong2*)(As + (ti + 8 * i) * kGramLd + k);
+            for (int j = 0; j < TJ; ++j) sum[i][j] = err[i][j] = 0ull;
+        for (int n = 0; n < kGramFold && xc < x1; ++n, xc += kGramChunk, buf ^= 1) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();             // this chunk has landed; the other buffer has been read
+            if (xc + kGramChunk < x1) load(xc + kGramChunk, buf ^ 1);
+            const float* As = sm + buf * kBuf;
+            const float* Bs = As + BI * kGramLd;
+            const float* ws = Bs + BJ * kGramLd;
+            uint64_t acc[TI][TJ];
 #pragma unroll
             for (int i = 0; i < TI; ++i)
 #pragma unroll
+                for (int j = 0; j < TJ; ++j) acc[i][j] = 0ull;
+#pragma unroll 4
+            for (int k = 0; k < kGramChunk; k += 4) {
+                const ulonglong2 w = *(const ulonglong2*)(ws + k);
+                ulonglong2 a[TI], b[TJ];
+#pragma unroll
                 for (int j = 0; j < TJ; ++j) {
-                    fma2(acc[i][j], a[i].x, b[j].x);
-                    fma2(acc[i][j], a[i].y, b[j].y);
+                    const ulonglong2 v = *(const ulonglong2*)(Bs + (tj + 16 * j) * kGramLd + k);
+                    b[j] = make_ulonglong2(mul2(v.x, w.x), mul2(v.y, w.y));
+                }
+#pragma unroll
+                for (int i = 0; i < TI; ++i) a[i] = *(const ulonglong2*)(As + (ti + 8 * i) * kGramLd + k);
+#pragma unroll
+                for (int i = 0; i < TI; ++i)
+#pragma unroll
+                    for (int j = 0; j < TJ; ++j) {
+                        fma2(acc[i][j], a[i].x, b[j].x);
+                        fma2(acc[i][j], a[i].y, b[j].y);
+                    }
+            }
+#pragma unroll
+            for (int i = 0; i < TI / 2; ++i)
+#pragma unroll
+                for (int j = 0; j < TJ; ++j) {
+                    const uint64_t x = pack2(lo2(acc[2 * i][j]), lo2(acc[2 * i + 1][j]));
+                    const uint64_t y = pack2(hi2(acc[2 * i][j]), hi2(acc[2 * i + 1][j]));
+                    uint64_t ef, et;
+                    const uint64_t f = two_sum(x, y, ef), t = two_sum(sum[i][j], f, et);
+                    err[i][j] = add2(err[i][j], add2(et, ef));
+                    sum[i][j] = t;
                 }
         }
 #pragma unroll
         for (int i = 0; i < TI; ++i)
 #pragma unroll
             for (int j = 0; j < TJ; ++j) {
-                const float f = __uint_as_float((uint32_t)acc[i][j]) + __uint_as_float((uint32_t)(acc[i][j] >> 32));
-                const float y = f - comp[i][j], t = sum[i][j] + y;
-                const float r = (t - sum[i][j]) - y;
-                comp[i][j] = fabsf(r) < INFINITY ? r : 0.f;      // an infinite sum stays infinite
-                sum[i][j] = t;
+                const int r = i0 + ti + 8 * i, c = j0 + tj + 16 * j;
+                if (r >= na || c >= nb) continue;
+                const uint64_t t = sum[i / 2][j], e = err[i / 2][j];
+                const float ef = i & 1 ? hi2(e) : lo2(e);
+                double v = (double)(i & 1 ? hi2(t) : lo2(t));
+                if (fabsf(ef) < INFINITY) v += (double)ef;       // an infinite sum stays infinite
+                double* p = partial + ((long)blockIdx.z * na + r) * nb + c;
+                *p = first ? v : *p + v;
             }
     }
-#pragma unroll
-    for (int i = 0; i < TI; ++i)
-#pragma unroll
-        for (int j = 0; j < TJ; ++j) {
-            const int r = i0 + ti + 8 * i, c = j0 + tj + 16 * j;
-            if (r < na && c < nb) partial[((long)blockIdx.z * na + r) * nb + c] = (double)sum[i][j] - (double)comp[i][j];
-        }
 }
 
 // G[i][j] = sum_s partial[s][i][j] (fixed order: 8 interleaved sums, then their sum), and
