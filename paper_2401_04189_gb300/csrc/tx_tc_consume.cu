@@ -2785,6 +2785,10 @@ int tc_describe_plan(const tx_ctx* c, int* out, int nout) {
 static uint32_t split_image_stride(const ConsumePlan& p) {
     return 2u * ((uint32_t)p.nyi * p.ya + (uint32_t)std::max(1, p.nzi) * p.b3);
 }
+// what the layout of the split image depends on beside the shape: different tiles can share a stride
+static void split_image_tiles(const ConsumePlan& p, int (&t)[4]) {
+    t[0] = (int)p.ya_rows; t[1] = p.nyi; t[2] = p.n3p; t[3] = std::max(1, p.nzi);
+}
 
 namespace tcc {
 // tiles of one operand for every term: dst[t][tile][part][K step][rows][32 bytes] (32-byte swizzle) from the
@@ -2814,6 +2818,7 @@ int tc_build_split_image(tx_ctx* c, cudaStream_t s) {
     const int n2 = c->n[1], n3 = c->n[2], l2 = ldk(c->r[1], op->esize), l3 = ldk(c->r[2], op->esize), T = tc_terms(c);
     const int nz = std::max(1, p.nzi);
     op->img_stride = split_image_stride(p);
+    split_image_tiles(p, op->img_tiles);
     if (cudaMalloc(&op->img, (size_t)T * op->img_stride) != cudaSuccess) {
         cudaGetLastError();
         op->img = nullptr;
@@ -3140,7 +3145,9 @@ int tc_consume(const tx_ctx* c, const PairRec* recs, int p0, int np, const void*
     CUtensorMap mZ, mA2, mA3;
     if (op->split) {
         // Z tiles of this batch: [pair][t][x][part][K step][rows g][32 bytes]
-        if (!op->img || op->img_stride != split_image_stride(p))
+        int tiles[4];
+        split_image_tiles(p, tiles);
+        if (!op->img || op->img_stride != split_image_stride(p) || std::memcmp(tiles, op->img_tiles, sizeof(tiles)) != 0)
             return fail(TX_ERR_CUDA, "operator image missing or built for another tile shape");
         a.img = (const uint8_t*)op->img;
         a.img_stride = op->img_stride;

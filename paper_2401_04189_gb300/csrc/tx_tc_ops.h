@@ -40,6 +40,7 @@ struct TcOperands {
     // split precisions: per term [y tile][A_t2 hi, lo][...] then [z part][mu_t A_t3 hi, lo] (32-byte swizzled)
     void* img;
     uint32_t img_stride;  // bytes per term
+    int img_tiles[4];     // split precisions, the tiles it was built for: rows per K step and count of A_t2, then of mu_t A_t3
 };
 
 // per-pair scratch (elements of the operand type; doubled for split precisions)
