@@ -74,8 +74,10 @@ __global__ void __launch_bounds__(256) k_core_dot(const PairRec* __restrict__ re
 
 int ldb_of(const tx_ctx* c, int d) { return d == 0 ? 0 : d == 1 ? simt_ld2(c->r[1]) : simt_ld3(c->r[2]); }
 int ldu_of(const tx_ctx* c, int d) { return d == 0 ? 0 : d == 1 ? simt_ld2(c->n[1]) : simt_ld3(c->n[2]); }
-size_t b_floats(const tx_ctx* c, int d) { return (size_t)pad4(c->T * c->r[d] * (d ? ldb_of(c, d) : c->r[d])); }
-size_t ut_floats(const tx_ctx* c, int d) { return (size_t)pad4(c->r[d] * (d ? ldu_of(c, d) : c->n[d])); }
+// (sizes in 64 bits: T r_d^2 passes 2^31 for modes of many thousand points)
+size_t up4(size_t v) { return (v + 3) & ~(size_t)3; }
+size_t b_floats(const tx_ctx* c, int d) { return up4((size_t)c->T * c->r[d] * (d ? ldb_of(c, d) : c->r[d])); }
+size_t ut_floats(const tx_ctx* c, int d) { return up4((size_t)c->r[d] * (d ? ldu_of(c, d) : c->n[d])); }
 
 }  // namespace
 
