@@ -352,6 +352,16 @@ int tx_set_expansion_form(tx_ctx* ctx, int form);
  * where tx_set_precision would refuse the shape. */
 int tx_describe_expansion_plan(const int n[3], const int r[3], int T, int precision, int form, int* out, int nout);
 
+/* Host-only: which Gaussian terms the float32 and split precisions sum on a coarse grid of r_d Chebyshev
+ * nodes per mode (the terms whose kernel exp(-theta (x - c)^2) those nodes interpolate to 1e-9 of its
+ * maximum over a grid of length extent[d] in every mode), for a context of these sizes.  Needs no device
+ * and no context.  smooth[T] receives 1 for each term that qualifies, *n_coarse how many run on the coarse
+ * grid: all that qualify, or 0 where that would take more operations than the grid itself.
+ * Returns TX_OK; TX_ERR_INVALID_ARG for NULL arguments, T < 1, exponents that are not finite and > 0 or
+ * extents that are not finite and >= 0; TX_ERR_SHAPE as above. */
+int tx_describe_term_split(const int n[3], const int r[3], const double extent[3], int T,
+                           const double* gauss_exponents, int* smooth, int* n_coarse);
+
 /*
  * tx_exchange_apply_static -- out = K psi_occ (targets = the occupied block), like
  * tx_exchange_apply with psi_tgt NULL, for callers that cannot let a library allocate device

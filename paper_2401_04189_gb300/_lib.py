@@ -26,7 +26,7 @@ EXPORTED = [
     "tx_reset_launch_count", "tx_exchange_apply_energy", "tx_profile_enable", "tx_profile_reset",
     "tx_profile_read", "tx_selftest_gemm", "tx_batch_plan", "tx_batch_launch", "tx_batch_capture",
     "tx_batch_replay", "tx_batch_item_plan", "tx_plan_destroy", "tx_set_tile_plan", "tx_set_accumulation_chunk", "tx_set_expansion_form",
-    "tx_exchange_apply_static", "tx_describe_expansion_plan", "tx_set_wait_limit", "tx_selftest_wait",
+    "tx_exchange_apply_static", "tx_describe_expansion_plan", "tx_describe_term_split", "tx_set_wait_limit", "tx_selftest_wait",
     "tx_exchange_energy_from_w", "tx_ace_projectors", "tx_ace_apply", "tx_set_quadrature",
     "tx_exchange_apply_galerkin", "tx_exchange_energy_galerkin", "tx_transfer_create", "tx_transfer_u_to_s",
     "tx_transfer_s_to_u", "tx_transfer_map_bytes", "tx_transfer_destroy", "tx_exchange_apply_sthosvd",
@@ -122,6 +122,9 @@ def lib():
     L.tx_set_accumulation_chunk.restype = _I
     L.tx_describe_expansion_plan.argtypes = [ctypes.POINTER(_I), ctypes.POINTER(_I), _I, _I, _I, ctypes.POINTER(_I), _I]
     L.tx_describe_expansion_plan.restype = _I
+    L.tx_describe_term_split.argtypes = [ctypes.POINTER(_I), ctypes.POINTER(_I), ctypes.POINTER(ctypes.c_double), _I, _P,
+                                         ctypes.POINTER(_I), ctypes.POINTER(_I)]
+    L.tx_describe_term_split.restype = _I
     L.tx_set_expansion_form.argtypes = [_P, _I]
     L.tx_set_expansion_form.restype = _I
     L.tx_selftest_gemm.argtypes = [_I, _I, _I, _I, _I, _P, _P, _P, _P]
@@ -523,6 +526,18 @@ def tx_describe_expansion_plan(n, r, T, precision, form=0):
     d = dict(zip(PLAN_FIELDS, (int(v) for v in out)))
     d["kernel"] = PLAN_KERNELS[d["kernel"]]
     return d
+
+
+def tx_describe_term_split(n, r, extent, exponents):
+    """(smooth, n_coarse): for each Gaussian exponent whether the float32 and split precisions may sum
+    its term on the coarse grid (host only), and how many terms of such a context run there."""
+    th = np.ascontiguousarray(exponents, dtype=np.float64)
+    smooth, nc = (_I * len(th))(), _I()
+    st = lib().tx_describe_term_split((_I * 3)(*[int(v) for v in n]), (_I * 3)(*[int(v) for v in r]),
+                                      (ctypes.c_double * 3)(*[float(v) for v in extent]), len(th),
+                                      th.ctypes.data_as(_P), smooth, ctypes.byref(nc))
+    _check(st, "tx_describe_term_split")
+    return [bool(v) for v in smooth], int(nc.value)
 
 
 def tx_launch_count() -> int:

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <fstream>
@@ -155,6 +156,23 @@ extern "C" int tx_describe_expansion_plan(const int n[3], const int r[3], int T,
     std::string why;
     if (!tc_supported(&c, &why)) return fail(TX_ERR_UNSUPPORTED_SHAPE, why);
     return tc_describe_plan(&c, out, nout);
+}
+
+extern "C" int tx_describe_term_split(const int n[3], const int r[3], const double extent[3], int T,
+                                      const double* gauss_exponents, int* smooth, int* n_coarse) {
+    if (!n || !r || !extent || !gauss_exponents || !smooth || !n_coarse)
+        return fail(TX_ERR_INVALID_ARG, "arguments must not be NULL");
+    if (T < 1) return fail(TX_ERR_INVALID_ARG, "T must be >= 1");
+    for (int t = 0; t < T; ++t)
+        if (!std::isfinite(gauss_exponents[t]) || gauss_exponents[t] <= 0)
+            return fail(TX_ERR_INVALID_ARG, "gauss_exponents must be finite and > 0");
+    for (int d = 0; d < 3; ++d) {
+        if (n[d] < 2 || n[d] > 4096) return fail(TX_ERR_SHAPE, "grid sizes must be in [2, 4096]");
+        if (r[d] < 1 || r[d] > n[d]) return fail(TX_ERR_SHAPE, "ranks must satisfy 1 <= r_d <= n_d");
+        if (!std::isfinite(extent[d]) || extent[d] < 0) return fail(TX_ERR_INVALID_ARG, "extents must be finite and >= 0");
+    }
+    *n_coarse = smooth_terms(n, r, extent, T, gauss_exponents, smooth);
+    return TX_OK;
 }
 
 extern "C" int tx_set_tile_plan(tx_ctx* c, int bx, int nstage) {

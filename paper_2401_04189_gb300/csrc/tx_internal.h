@@ -247,6 +247,9 @@ int finalize_energy(const double* batches, int nb, double scale, double* e_dev, 
 int weighted_dot(const tx_ctx* c, const float* A, const float* B, int count, double* partial, int nblocks, double scale,
                  double* e_dev, cudaStream_t s);
 
+// the rule of the term split: smooth[t] = 1 for the terms that a coarse grid of r_d Chebyshev nodes over `extent`
+// takes to the tolerance; returns how many of them run there (all, or 0 where that costs more)
+int smooth_terms(const int n[3], const int r[3], const double extent[3], int T, const double* theta, int* smooth);
 // decides the term split of a new context and allocates its operators (host float64 inputs)
 int plan_terms(tx_ctx* c, const double* const x[3], const double* theta, const double* mu);
 void free_terms(tx_ctx* c);

@@ -194,32 +194,42 @@ static double chebyshev_bound(double theta, double h, int N) {
 // 60 times below the float32 rounding of the operators, so the split changes results by rounding only.
 constexpr double kSmoothTol = 1e-9;
 
-int plan_terms(tx_ctx* c, const double* const x[3], const double* theta, const double* mu) {
-    TermSplit& ts = c->ts;
-    std::memset(&ts, 0, sizeof(ts));
-    double lo[3], hi[3];
-    for (int d = 0; d < 3; ++d) {
-        lo[d] = *std::min_element(x[d], x[d] + c->n[d]);
-        hi[d] = *std::max_element(x[d], x[d] + c->n[d]);
-    }
-    std::vector<double> th, m, th_c, m_c;
-    for (int t = 0; t < c->T; ++t) {
-        bool smooth = true;
-        for (int d = 0; d < 3 && smooth; ++d)
-            smooth = chebyshev_bound(theta[t], 0.5 * (hi[d] - lo[d]), c->r[d] - 1) <= kSmoothTol;
-        (smooth ? th_c : th).push_back(theta[t]);
-        (smooth ? m_c : m).push_back(mu[t]);
+int smooth_terms(const int n[3], const int r[3], const double extent[3], int T, const double* theta, int* smooth) {
+    int count = 0;
+    for (int t = 0; t < T; ++t) {
+        smooth[t] = 1;
+        for (int d = 0; d < 3 && smooth[t]; ++d)
+            smooth[t] = chebyshev_bound(theta[t], 0.5 * extent[d], r[d] - 1) <= kSmoothTol;
+        count += smooth[t];
     }
     // worth it where the smooth terms' fine-grid work is more than their coarse work plus the
     // interpolation (one fine term); a tenth of a fine term stands for the extra launches
-    auto mode_flops = [&](const int n[3]) {
-        const double r1 = c->r[0], r2 = c->r[1], r3 = c->r[2];
-        return n[0] * r1 * r2 * r3 + (double)n[0] * n[1] * r2 * r3 + (double)n[0] * n[1] * n[2] * r3;
+    auto mode_flops = [&](const int m[3]) {
+        const double r1 = r[0], r2 = r[1], r3 = r[2];
+        return m[0] * r1 * r2 * r3 + (double)m[0] * m[1] * r2 * r3 + (double)m[0] * m[1] * m[2] * r3;
     };
-    const double fine = mode_flops(c->n), coarse = mode_flops(c->r), nc = (double)th_c.size();
+    const double fine = mode_flops(n), coarse = mode_flops(r), nc = (double)count;
     // (coarse grids up to 160 nodes per mode: every float32 kernel takes them)
-    const bool on = nc * fine > 1.1 * fine + nc * coarse && std::max(c->r[1], c->r[2]) <= 160;
-    ts.nc = on ? (int)th_c.size() : 0;
+    return nc * fine > 1.1 * fine + nc * coarse && std::max(r[1], r[2]) <= 160 ? count : 0;
+}
+
+int plan_terms(tx_ctx* c, const double* const x[3], const double* theta, const double* mu) {
+    TermSplit& ts = c->ts;
+    std::memset(&ts, 0, sizeof(ts));
+    double lo[3], hi[3], extent[3];
+    for (int d = 0; d < 3; ++d) {
+        lo[d] = *std::min_element(x[d], x[d] + c->n[d]);
+        hi[d] = *std::max_element(x[d], x[d] + c->n[d]);
+        extent[d] = hi[d] - lo[d];
+    }
+    std::vector<int> smooth(c->T);
+    std::vector<double> th, m, th_c, m_c;
+    ts.nc = smooth_terms(c->n, c->r, extent, c->T, theta, smooth.data());
+    for (int t = 0; t < c->T; ++t) {
+        (smooth[t] ? th_c : th).push_back(theta[t]);
+        (smooth[t] ? m_c : m).push_back(mu[t]);
+    }
+    const bool on = ts.nc > 0;
     ts.nf = on ? (int)th.size() + 1 : c->T;
     auto dalloc = [&](auto** p, size_t count) -> int {
         if (cudaMalloc((void**)p, sizeof(**p) * std::max<size_t>(count, 1)) == cudaSuccess) return TX_OK;
