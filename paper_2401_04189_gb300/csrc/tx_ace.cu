@@ -18,6 +18,7 @@
 #include <string>
 
 #include "tx_internal.h"
+#include "tx_packed.cuh"
 #include "tx_paths.h"
 
 namespace tx {
@@ -26,42 +27,6 @@ namespace {
 constexpr int kGramChunk = 64;    // grid points per shared-memory chunk
 constexpr int kGramLd = kGramChunk + 4;
 constexpr int kGramFold = 64;     // chunks per float64 addition
-
-__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
-    uint64_t r;       // a - 1 b: the product is exact
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
-    return r;
-}
-// the rounded sum, and its exact error in e (Knuth's TwoSum; no condition on the magnitudes)
-__device__ __forceinline__ uint64_t two_sum(uint64_t a, uint64_t b, uint64_t& e) {
-    const uint64_t t = add2(a, b), c = sub2(t, a);
-    e = add2(sub2(a, sub2(t, c)), sub2(b, c));
-    return t;
-}
-__device__ __forceinline__ float lo2(uint64_t v) { return __uint_as_float((uint32_t)v); }
-__device__ __forceinline__ float hi2(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-    return (uint64_t)__float_as_uint(a) | (uint64_t)__float_as_uint(b) << 32;
-}
-__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool ok) {
-    const int bytes = ok ? 16 : 0;       // 0: the 16 bytes are zero-filled and src is not read
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
-                 "r"(bytes)
-                 : "memory");
-}
 
 // partial[s][i][j] = sum over slice s of the grid of w(x) A_i(x) B_j(x): float32 sums of 32 products (the even and
 // the odd points of a chunk of 64), added in float64 in effect.  This GPU adds float64 at 1/64 of the float32 rate,
@@ -120,7 +85,7 @@ __global__ void __launch_bounds__(128) k_wgram(const float* __restrict__ A, int 
             }
             Bs[BJ * kGramLd + tid] = wv;
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        cp_async_commit();
     };
     uint64_t sum[TI / 2][TJ], err[TI / 2][TJ];             // rows i and i + 1 in one register pair
     if (x0 < x1) load(x0, 0);
@@ -132,7 +97,7 @@ __global__ void __launch_bounds__(128) k_wgram(const float* __restrict__ A, int 
 #pragma unroll
             for (int j = 0; j < TJ; ++j) sum[i][j] = err[i][j] = 0ull;
         for (int n = 0; n < kGramFold && xc < x1; ++n, xc += kGramChunk, buf ^= 1) {
-            asm volatile("cp.async.wait_all;" ::: "memory");
+            cp_async_wait_all();
             __syncthreads();             // this chunk has landed; the other buffer has been read
             if (xc + kGramChunk < x1) load(xc + kGramChunk, buf ^ 1);
             const float* As = sm + buf * kBuf;

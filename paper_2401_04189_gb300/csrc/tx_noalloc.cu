@@ -46,18 +46,6 @@ int static_scratch(int dev, void** out) {
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// G[p][(b,g)][a] = sum_x S2[p][x][(b,g)] U1[x][a]  (mode 1 of the projection)
-int simt_mode1_project(const tx_ctx* c, const float* S2, float* G, int np, cudaStream_t s) {
-    const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
-    GemmArgs q{};
-    q.M = rr; q.N = r1; q.K = n1;
-    q.A = S2; q.a_m = 1; q.a_k = rr; q.a_b2 = (long)n1 * rr;
-    q.B = c->f_U[0]; q.b_k = r1; q.b_n = 1;
-    q.C = G; q.c_m = r1; q.c_n = 1; q.c_b2 = (long)rr * r1;
-    q.nb1 = 1; q.nb2 = np; q.alpha = 1.f;
-    return simt_gemm(q, s);
-}
-
 }  // namespace
 }  // namespace tx
 
@@ -112,7 +100,7 @@ extern "C" int tx_exchange_apply_static(tx_ctx* c, const float* psi_occ, int n_o
     for (long p0 = 0; p0 < P; p0 += Pb) {
         const int np = (int)std::min<long>(Pb, P - p0);
         TX_TRY(simt_project_s2(c, recs, (int)p0, np, f, 0, S2, s));
-        TX_TRY(simt_mode1_project(c, S2, G, np, s));
+        TX_TRY(simt_project_mode1(c, S2, G, np, s));
         TX_TRY(simt_expand_all(c, G, S2, Z, np, s));
         TX_TRY(simt_expand_consume(fine_shape(c), recs, (int)p0, np, f, Z, c->ts.nf, c->ts.FK[1], c->ts.FK[2], EPI_OUT,
                                    nullptr, s));

@@ -27,18 +27,6 @@ SimtLayout simt_layout(const tx_ctx* c) {
     return L;
 }
 
-// G[p][(b,g)][a] = sum_x S2[p][x][(b,g)] M1[x][a]   (mode 1 of the projection; M1 = U1)
-int gemm_mode1_project(const tx_ctx* c, const float* S2, const float* M1, float* G, int np, cudaStream_t s) {
-    const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
-    GemmArgs g{};
-    g.M = rr; g.N = r1; g.K = n1;
-    g.A = S2; g.a_m = 1; g.a_k = rr; g.a_b1 = 0; g.a_b2 = (long)n1 * rr;
-    g.B = M1; g.b_k = r1; g.b_n = 1; g.b_b1 = 0; g.b_b2 = 0;
-    g.C = G; g.c_m = r1; g.c_n = 1; g.c_b1 = 0; g.c_b2 = (long)rr * r1;
-    g.nb1 = 1; g.nb2 = np; g.alpha = 1.f; g.accumulate = 0;
-    return simt_gemm(g, s);
-}
-
 // H[p][(b,g)][a] (+)= sum_{t,x} R[p][t][x][(b,g)] M1_t[x][a] over the first nt of R's nr terms on a grid
 // of n1 nodes (mode 1 of the adjoint, summed over t)
 int gemm_mode1_adjoint(const tx_ctx* c, const float* R, const float* M1, int n1, int nt, int nr, float* H, bool add,
@@ -70,6 +58,17 @@ int gemm_mode1_expand(const tx_ctx* c, const float* G, const float* M1, int n1, 
 
 }  // namespace
 
+int simt_project_mode1(const tx_ctx* c, const float* S2, float* G, int np, cudaStream_t s) {
+    const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
+    GemmArgs g{};
+    g.M = rr; g.N = r1; g.K = n1;
+    g.A = S2; g.a_m = 1; g.a_k = rr; g.a_b2 = (long)n1 * rr;
+    g.B = c->f_U[0]; g.b_k = r1; g.b_n = 1;
+    g.C = G; g.c_m = r1; g.c_n = 1; g.c_b2 = (long)rr * r1;
+    g.nb1 = 1; g.nb2 = np; g.alpha = 1.f;
+    return simt_gemm(g, s);
+}
+
 int simt_expand_all(const tx_ctx* c, const float* G, float* H, float* Z, int np, cudaStream_t s) {
     const TermSplit& ts = c->ts;
     const int n1 = c->n[0];
@@ -83,10 +82,6 @@ int simt_expand_all(const tx_ctx* c, const float* G, float* H, float* Z, int np,
     if (ts.nf > 1) TX_TRY(gemm_mode1_expand(c, G, ts.F[0], n1, ts.nf - 1, 0, ts.nf, Z, np, s));
     return gemm_mode1_expand(c, H, ts.F[0] + (size_t)(ts.nf - 1) * n1 * c->r[0], n1, 1, ts.nf - 1, ts.nf, Z, np, s, 0, true);
 }
-
-namespace {
-
-}  // namespace
 
 int simt_adjoint_core(const tx_ctx* c, const PairRec* recs, int p0, int np, const FieldArgs& f, int flags, float* Y,
                       float* R, float* H, cudaStream_t s) {
@@ -138,7 +133,7 @@ int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec
             f.OUT1 = cs.out0;
             if (cs.kind == CALL_GRAD) TX_TRY(simt_adjoint_limit(sh));
             TX_TRY(simt_project_s2(c, recs, p0, np, f, 0, S2, s));
-            TX_TRY(gemm_mode1_project(c, S2, c->f_U[0], G, np, s));
+            TX_TRY(simt_project_mode1(c, S2, G, np, s));
             TX_TRY(simt_expand_all(c, G, S2, Z, np, s));
             int flags = 0;
             if (cs.kind == CALL_APPLY) flags = EPI_OUT | (cs.e_dev ? EPI_ENERGY : 0);
@@ -161,7 +156,7 @@ int simt_batch(tx_ctx* c, const CallSpec& cs, const PairRec* recs, const PairRec
                 f.MUL0 = cs.cot; f.OUT0 = cs.out0;
                 f.MUL1 = nullptr; f.OUT1 = nullptr;
                 TX_TRY(simt_project_s2(c, recs, p0, np, f, 0, S2, s));
-                TX_TRY(gemm_mode1_project(c, S2, c->f_U[0], G, np, s));
+                TX_TRY(simt_project_mode1(c, S2, G, np, s));
                 TX_TRY(simt_expand_all(c, G, S2, Z, np, s));
                 TX_TRY(simt_expand_consume(sh, recs, p0, np, f, Z, c->ts.nf, c->ts.FK[1], c->ts.FK[2], EPI_OUT, epart, s));
             }
@@ -193,7 +188,7 @@ int galerkin_batch(tx_ctx* c, const CallSpec& cs, const GalerkinOps& o, const Pa
     f.OUT0 = cs.out0;
     f.OUT1 = cs.out0;
     TX_TRY(simt_project_s2(c, recs, p0, np, f, 0, S2, s));
-    TX_TRY(gemm_mode1_project(c, S2, c->f_U[0], G, np, s));
+    TX_TRY(simt_project_mode1(c, S2, G, np, s));
     TX_TRY(galerkin_core(c, o, G, X1, H, np, s));
     if (cs.kind == CALL_ENERGY) return galerkin_core_dot(c, recs, p0, G, H, np, epart, s);
     float* Z = S2;   // [np][1][n1][r2 r3]: the size of S2

@@ -14,44 +14,12 @@
 #include <string>
 
 #include "tx_internal.h"
+#include "tx_packed.cuh"
 #include "tx_tc_common.cuh"
 
 namespace tx {
 
-// ====================================================================================
-// packed float32 arithmetic: two fused multiply-adds per instruction (fma.rn.f32x2 rounds each
-// half as fmaf does), which halves the issue slots of the inner loops and leaves the rest of
-// them to the shared-memory reads
-// ====================================================================================
 namespace {
-__device__ __forceinline__ uint64_t dup2(float v) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
-    return r;
-}
-__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(uint64_t v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // ====================================================================================
 // strided batched GEMM: C[b1,b2][m][n] = alpha * sum_k A[m][k] B[k][n] (+ C)
 // BM x BN tiles of 256 threads, each (BM / 16) x (BN / 16) outputs; 16-deep K slices, two
@@ -678,7 +646,7 @@ struct ConsumeF32Args {
     long out_ps, out_cs;       // EPI_STORE: floats between the results of two pairs, of two term groups
 };
 
-// Registers: 8 RN for phi, 8 per mode-2 column; the K part of mode 3 (gc) is at most CL * kMaxPart
+// Registers: 8 RN for phi, 8 per mode-2 column; the K part of mode 3 (gc) is at most CL * consume_max_rg
 // columns so that both fit the 168 registers that leave 12 warps per SM (255 above 12 columns).
 __host__ __device__ constexpr int consume_max_rg(int cl, int rn) { return cl == 16 ? 4 : (rn > 8 ? 5 : (rn == 6 ? 6 : 8)); }
 __host__ __device__ constexpr int consume_max_threads(int cl, int rn) { return rn <= 12 ? 384 : 256; }

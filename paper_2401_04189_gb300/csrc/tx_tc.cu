@@ -139,11 +139,12 @@ int tc_prepare(tx_ctx* c, cudaStream_t s) {
     double* const* A64 = op->split && c->ts.nc ? c->ts.F64 : c->d_A64;
     // every static operand row is K padded with zeros to a whole number of 32-byte sectors
     const int eb = op->esize;
-    const size_t e_u3 = (size_t)r3 * ldk(n3, eb), e_u2 = (size_t)r2 * ldk(n2, eb), e_u1 = (size_t)r1 * ldk(n1, eb);
-    // (the split forms run mode 1 of the expansion and the adjoint in float32)
-    const size_t e_a1 = op->split ? 0 : (size_t)T * n1 * ldk(r1, eb), e_a2 = (size_t)T * n2 * ldk(r2, eb);
+    // (the split forms run the projection, mode 1 of the expansion and the adjoint in float32)
+    const size_t single = op->split ? 0 : 1;
+    const size_t e_u3 = single * r3 * ldk(n3, eb), e_u2 = single * r2 * ldk(n2, eb), e_u1 = single * r1 * ldk(n1, eb);
+    const size_t e_a1 = single * T * n1 * ldk(r1, eb), e_a2 = (size_t)T * n2 * ldk(r2, eb);
     const size_t e_a3 = (size_t)T * n3 * ldk(r3, eb), e_a3f = (size_t)T * n3 * pad8(r3);
-    const size_t e_a3t = op->split ? 0 : (size_t)T * r3 * ldk(n3, eb), e_a2t = op->split ? 0 : (size_t)T * r2 * ldk(n2, eb);
+    const size_t e_a3t = single * T * r3 * ldk(n3, eb), e_a2t = single * T * r2 * ldk(n2, eb);
     auto al = [](size_t e) { return (e + 127) & ~(size_t)127; };   // 256-byte aligned pieces
     const size_t tot = al(e_u3) + al(e_u2) + al(e_u1) + al(e_a1) + al(e_a2) + al(e_a3) + al(e_a3t) + al(e_a2t);
     // bf16 single pass: the stage-3 B operand also in float32 (TF32), after everything else
@@ -180,12 +181,14 @@ int tc_prepare(tx_ctx* c, cudaStream_t s) {
         TX_LAUNCHED();
         return TX_OK;
     };
-    // U_d^T: rows r_d, K = n_d  (U_d is [n_d][r_d])
-    TX_TRY(conv(c->d_U[2], r3, n3, 1, r3, ldk(n3, eb), op->st.U3T));
-    TX_TRY(conv(c->d_U[1], r2, n2, 1, r2, ldk(n2, eb), op->st.U2T));
-    TX_TRY(conv(c->d_U[0], r1, n1, 1, r1, ldk(n1, eb), op->st.U1T));
+    if (!op->split) {
+        // U_d^T: rows r_d, K = n_d  (U_d is [n_d][r_d])
+        TX_TRY(conv(c->d_U[2], r3, n3, 1, r3, ldk(n3, eb), op->st.U3T));
+        TX_TRY(conv(c->d_U[1], r2, n2, 1, r2, ldk(n2, eb), op->st.U2T));
+        TX_TRY(conv(c->d_U[0], r1, n1, 1, r1, ldk(n1, eb), op->st.U1T));
+        TX_TRY(conv(A64[0], (long)T * n1, r1, r1, 1, ldk(r1, eb), op->st.A1s));
+    }
     // A_td: [T][n_d][r_d] -> rows (t, x), K = r_d
-    if (!op->split) TX_TRY(conv(A64[0], (long)T * n1, r1, r1, 1, ldk(r1, eb), op->st.A1s));
     TX_TRY(conv(A64[1], (long)T * n2, r2, r2, 1, ldk(r2, eb), op->st.A2));
     TX_TRY(conv(A64[2], (long)T * n3, r3, r3, 1, ldk(r3, eb), op->st.A3));
     // the adjoint's transposed operators, one term at a time: rows gamma (beta), K = z (y)
@@ -229,18 +232,6 @@ size_t tc_batch_bytes_per_pair(const tx_ctx* c, int kind) {
     }
     if (kind == CALL_GRAD || kind == CALL_VJP) return std::max(fwd, tc_adjoint_bytes_per_pair(c));
     return fwd;
-}
-
-// G[p][(g,b)][a] = sum_x S2[p][x][(g,b)] U1[x][a]  (float32, mode 1 of the projection)
-static int f32_mode1_project(const tx_ctx* c, const float* S2, float* G, int np, cudaStream_t s) {
-    const int n1 = c->n[0], r1 = c->r[0], rr = c->r[1] * c->r[2];
-    GemmArgs g{};
-    g.M = rr; g.N = r1; g.K = n1;
-    g.A = S2; g.a_m = 1; g.a_k = rr; g.a_b2 = (long)n1 * rr;
-    g.B = c->f_U[0]; g.b_k = r1; g.b_n = 1;
-    g.C = G; g.c_m = r1; g.c_n = 1; g.c_b2 = (long)rr * r1;
-    g.nb1 = 1; g.nb2 = np; g.alpha = 1.f;
-    return simt_gemm(g, s);
 }
 
 // Z tiles (hi + lo) of nt fine terms from t0 on, one block per (t, x): mode 1 of the expansion in float32,
@@ -290,7 +281,7 @@ static int tc_forward(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, con
         fa.SA = SA;
         fa.SB = SB;
         TX_TRY(simt_project_s2(c, recs, b.p0, np, fa, 0, S2f, s, false));
-        TX_TRY(f32_mode1_project(c, S2f, Gf, np, s));
+        TX_TRY(simt_project_mode1(c, S2f, Gf, np, s));
         if (ts.nc) {
             // H[p][a][(g,b)] = sum over the smooth terms of G x_d Q_td; the cores are [g][b], so modes 2
             // and 3 take each other's place

@@ -9,7 +9,7 @@
 
 namespace tx {
 
-enum TcOutType { TC_OUT_F32 = 0, TC_OUT_BF16 = 1, TC_OUT_F32_SPLIT = 2, TC_OUT_BF16_SPLIT = 3 };
+enum TcOutType { TC_OUT_F32 = 0, TC_OUT_BF16 = 1 };
 
 // A K-major operand in global memory: element (z, row, k) at base + z*depth_stride + row*row_stride + k
 // (strides in elements, 16-byte multiples); `lo` is the low part for the 3-pass precisions.
@@ -21,13 +21,13 @@ struct TcOperand {
 
 // One batched GEMM launch.  Batch b = (b1, b2) with b1 = b % nb1; operand rows are offset by
 // b1*x_row1 + b2*x_row2 and the depth coordinate is b1*x_z1 + b2*x_z2.  Output element (m, n)
-// of batch b goes to C + b1*c_b1 + b2*c_b2 + m*c_m + n*c_n (+ c_lo for the low part).
+// of batch b goes to C + b1*c_b1 + b2*c_b2 + m*c_m + n*c_n.
 struct TcGemmArgs {
     int M, N, K, BN, nb1, nb2;
     int a_row1, a_row2, a_z1, a_z2;
     int b_row1, b_row2, b_z1, b_z2;
     void* C;
-    long c_m, c_n, c_b1, c_b2, c_lo;
+    long c_m, c_n, c_b1, c_b2;
     int rdiv, cdiv;          // row / column index splits (0 = none)
     long c_mh, c_nh;         // strides of m / rdiv and n / cdiv
     int c_type;

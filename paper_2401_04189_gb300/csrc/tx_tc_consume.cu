@@ -811,8 +811,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int c = 0; c < 16; ++c) {
                 const float v = g0 + c < a.r3 ? __uint_as_float(r[c]) + __uint_as_float(rc[c]) : 0.f;
-                // hi: nearest, ties away (a NaN may leave hi, but not lo: v - hi is NaN then).  lo has 13 bits
-                // at most and the tensor core drops two of them: 2^-22 of v, either way
+                // hi: nearest, ties away (a NaN may leave hi, but not lo: v - hi is NaN then).  lo has 12 bits
+                // at most and the tensor core drops the last: rounding it would be a tie, off by as much, 2^-23 of v
                 r[c] = (__float_as_uint(v) + 0x1000u) & 0xffffe000u;
                 rc[c] = __float_as_uint(v - __uint_as_float(r[c]));
             }

@@ -1,8 +1,7 @@
 // Generic batched tensor-core GEMM on tcgen05: D[b][m][n] = alpha * sum_k A[b][m][k] B[b][n][k]
 // with A and B K-major in global memory, loaded by TMA (128-byte swizzle) through a multi-
 // stage mbarrier pipeline, accumulated in TMEM by one issuing thread, and written back by
-// four epilogue warps with arbitrary output strides (float32 or bf16, optionally split into
-// hi + lo parts for the 3-pass precisions).
+// four epilogue warps with arbitrary output strides (float32 or bf16).
 //
 // Used for the small mode products of the hot path: the second and third modes of the
 // projection onto the Tucker core, the first mode of the expansion for every Gaussian term
@@ -27,45 +26,24 @@ using namespace tx::tc;
 constexpr int kMaxStages = 4;
 constexpr int kBM = 128;
 
-// 16-byte store of VE consecutive outputs (8 bf16 or 4 float), hi and, for split types, lo
+// 16-byte store of VE consecutive outputs (8 bf16 or 4 float)
 __device__ __forceinline__ void store_vec(const TcGemmArgs& g, long o, const float* v) {
-    if (g.c_type == TC_OUT_F32 || g.c_type == TC_OUT_F32_SPLIT) {
-        float h[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) h[e] = g.c_type == TC_OUT_F32 ? v[e] : tf32_hi(v[e]);
-        *(float4*)((float*)g.C + o) = make_float4(h[0], h[1], h[2], h[3]);
-        if (g.c_type == TC_OUT_F32_SPLIT)
-            *(float4*)((float*)g.C + o + g.c_lo) = make_float4(tf32_hi(v[0] - h[0]), tf32_hi(v[1] - h[1]),
-                                                               tf32_hi(v[2] - h[2]), tf32_hi(v[3] - h[3]));
+    if (g.c_type == TC_OUT_F32) {
+        *(float4*)((float*)g.C + o) = make_float4(v[0], v[1], v[2], v[3]);
     } else {
-        uint32_t w[4], l[4];
+        uint32_t w[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const __nv_bfloat162 hv = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
             w[e] = *(const uint32_t*)&hv;
-            const float2 hf = __bfloat1622float2(hv);
-            const __nv_bfloat162 lv = __floats2bfloat162_rn(v[2 * e] - hf.x, v[2 * e + 1] - hf.y);
-            l[e] = *(const uint32_t*)&lv;
         }
         *(uint4*)((__nv_bfloat16*)g.C + o) = make_uint4(w[0], w[1], w[2], w[3]);
-        if (g.c_type == TC_OUT_BF16_SPLIT) *(uint4*)((__nv_bfloat16*)g.C + o + g.c_lo) = make_uint4(l[0], l[1], l[2], l[3]);
     }
 }
 
 __device__ __forceinline__ void store_out(const TcGemmArgs& g, long o, float v) {
-    if (g.c_type == TC_OUT_F32) {
-        ((float*)g.C)[o] = v;
-    } else if (g.c_type == TC_OUT_BF16) {
-        ((__nv_bfloat16*)g.C)[o] = __float2bfloat16_rn(v);
-    } else if (g.c_type == TC_OUT_F32_SPLIT) {
-        const float hi = tf32_hi(v);
-        ((float*)g.C)[o] = hi;
-        ((float*)g.C)[o + g.c_lo] = tf32_hi(v - hi);
-    } else {   // TC_OUT_BF16_SPLIT
-        const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-        ((__nv_bfloat16*)g.C)[o] = hi;
-        ((__nv_bfloat16*)g.C)[o + g.c_lo] = __float2bfloat16_rn(v - __bfloat162float(hi));
-    }
+    if (g.c_type == TC_OUT_F32) ((float*)g.C)[o] = v;
+    else ((__nv_bfloat16*)g.C)[o] = __float2bfloat16_rn(v);
 }
 
 template <bool TF32, bool SPLIT>
@@ -233,7 +211,7 @@ __global__ void __launch_bounds__(128, 1)
             __syncwarp();
             if (g.vec) {
                 // contiguous 16-byte aligned rows: each lane stores one vector of one row
-                const int VE = (g.c_type == TC_OUT_F32 || g.c_type == TC_OUT_F32_SPLIT) ? 4 : 8;
+                const int VE = g.c_type == TC_OUT_F32 ? 4 : 8;
                 const int lpr = 64 / VE, rpp = 32 / lpr;            // lanes per row, rows per pass
                 const int sub = lane / lpr, cv = (lane % lpr) * VE;
                 for (int rr0 = 0; rr0 < 32; rr0 += rpp) {
@@ -367,11 +345,10 @@ int tc_gemm_launch(const TcOperand& A, const TcOperand& B, TcGemmArgs g, bool tf
     g.nacc = split ? std::max(1, std::min({nk_atoms, 4, 512 / g.BN})) : 1;
     g.tmem_cols = tmem_cols_for(g.nacc * g.BN);
     {
-        // vector stores: contiguous columns, no column split, every row start and the lo copy
-        // 16-byte aligned, whole vectors
-        const long ve = (g.c_type == TC_OUT_F32 || g.c_type == TC_OUT_F32_SPLIT) ? 4 : 8;
+        // vector stores: contiguous columns, no column split, every row start 16-byte aligned, whole vectors
+        const long ve = g.c_type == TC_OUT_F32 ? 4 : 8;
         g.vec = g.c_n == 1 && g.cdiv >= g.N && g.c_m != 1 && ((uintptr_t)g.C % 16) == 0 && g.c_m % ve == 0 &&
-                g.c_mh % ve == 0 && g.c_b1 % ve == 0 && g.c_b2 % ve == 0 && g.c_lo % ve == 0 && g.N % ve == 0;
+                g.c_mh % ve == 0 && g.c_b1 % ve == 0 && g.c_b2 % ve == 0 && g.N % ve == 0;
     }
     g.stages = (int)std::min<size_t>({(size_t)tcg::kMaxStages, (budget - 1024) / stage, (size_t)nk_atoms});
     // the epilogue stages 4 warps x 32 rows x 65 floats in the (then idle) pipeline buffers

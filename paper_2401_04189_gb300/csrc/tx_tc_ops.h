@@ -14,7 +14,8 @@ inline int pad16(int v) { return (v + 15) & ~15; }
 inline int ldk(int k, int elem_bytes) { return elem_bytes == 2 ? pad16(k) : pad8(k); }
 
 // Static operands, K-major with 16-byte row strides, in the operand type of the precision
-// (bf16, or float32 holding TF32 values).  For the 3-pass precisions `lo` holds x - hi.
+// (bf16, or float32 holding TF32 values).  For the 3-pass precisions only A2 and A3 are made,
+// and `lo` holds x - hi.
 struct TcStatic {
     void* U3T;   // [r3][ld(n3)]     rows gamma, K = z        (projection, mode 3)
     void* U2T;   // [r2][ld(n2)]     rows beta,  K = y        (projection, mode 2)
