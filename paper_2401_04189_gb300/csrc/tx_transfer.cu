@@ -48,43 +48,79 @@ namespace {
 constexpr uint32_t kTransferMagic = 0x54555446u;
 constexpr int kChunk = 32;     // orbitals per pass
 
-// One CTA per block of one cell's structured nodes (UBlock; at most kUThreads * u_nodes of them, so that the
-// cells' different sizes fill all SMs).  The cell's orbital rows (kUChunk orbitals at a time) are staged in
-// shared memory; a thread holds the N rows of up to u_nodes structured nodes in registers and writes those
-// nodes for every orbital of the chunk (neighbouring threads on neighbouring nodes, so each orbital's writes
-// are runs along z).  N is stored [local node][mapped node], so a warp reads it in whole lines.
-// With one node per thread the shared-memory reads were the bound: a 16-byte broadcast occupies the port
-// for as long as 16 multiply-adds per lane take, and fed 4.  160^3 nodes, quadratic cells, 64 orbitals: 743
-// us with one node per thread and N rows read 108 bytes apart; 605 with two and six CTAs per SM, 619 with four
-// and three, 611 with three and four, which is 3 to 8% ahead of four on smaller quadratic meshes.  Linear cells
-// take four nodes, cubic ones the two that the registers allow.  What is left is bound by the writes, runs as short as a cell is wide to
-// 64 orbitals 16 MB apart (1.7 TB/s).
-constexpr int kUChunk = 128;
+// One CTA per (block of one cell's structured nodes, chunk of orbitals).  A block (UBlock) holds at most
+// kUThreads * kUNodes nodes, so that the cells' different sizes fill all SMs.  A thread holds the N rows of up to
+// kUNodes structured nodes in registers, the cell's values of the chunk's orbitals lie in shared memory, and the
+// thread writes its nodes for every orbital of the chunk (neighbouring threads on neighbouring nodes, so each
+// orbital's writes are runs along z).  N is stored [local node][mapped node], so a warp reads it in whole lines.
+// Two nodes per thread: with one the shared-memory reads are the bound (a 16-byte broadcast occupies the port for
+// as long as 16 multiply-adds per lane take, and feeds 4), with three or four fewer CTAs fit an SM.
+// What is left is bound by the writes, runs as short as a cell is wide to orbitals N3 values apart.  The pieces of a
+// line that other cells write have to come while it is in L2, so the chunks are the outer order of the grid and few
+// orbitals are written at a time (u_to_s_chunk).  160^3 nodes, quadratic cells, 64 and 256 orbitals: 677 and
+// 2,658 us; 733 and 2,819 with one node per thread and rows of N 108 bytes apart, 690 and 3,070 with three nodes and
+// the chunks inside a CTA.  97^3, linear cells: 104 and 398 us; 147 and 717, 163 and 841.
 constexpr int kUThreads = 128;
-__host__ __device__ constexpr int u_nodes(int nb) { return nb > 27 ? 2 : nb > 8 ? 3 : 4; }
+constexpr int kUNodes = 2;
+__host__ __device__ constexpr int u_chunk_max(int nb) { return nb == 8 ? 256 : 128; }    // orbitals staged at most
 
 struct UBlock {
     int cell, k0, m;           // mapped nodes k0 .. k0 + m - 1, all of one cell
 };
 
+// Orbitals per chunk.  A chunk reads the shape values again, (order + 1)^3 floats a node, so the chunk grows with the
+// order: 128 in cubic cells, about 64 in quadratic ones.  Linear cells take 8 at a time where they write more than
+// L2 holds (129 MB), more on small grids, whose chunks would otherwise be shorter than a CTA's own latency.
+// Linear cells, 256 orbitals, by 8 / 24 / 256 at a time: 130^3 1,455 / 1,737 / 1,936 us, 50^3 122 / 77 / 88; and
+// 200 orbitals of 50^3 in one chunk 50, by 32 57.  Quadratic, 160^3, 384 orbitals by 32 / 64 / 128: 4,185 / 4,015 /
+// 4,132; cubic, 97^3, 256 by 64 / 128: 971 / 833.
+int u_to_s_chunk(int nb, int n_orb, long n3) {
+    if (nb == 64) return u_chunk_max(64);
+    int chunks;
+    if (nb == 8) {
+        const double bytes = 4.0 * (double)n3;
+        int ch = bytes * n_orb <= 100e6 ? n_orb : std::max(8, (int)std::ceil(12e6 / bytes));
+        ch = std::min(ch, u_chunk_max(8));
+        chunks = (n_orb + ch - 1) / ch;
+    } else {
+        // where 64 orbitals fill half of L2, rather a longer chunk (up to 127) than one more
+        chunks = n3 > 262144 ? std::max(1, n_orb / 64) : (n_orb + 63) / 64;
+    }
+    return ((n_orb + chunks - 1) / chunks + 3) & ~3;           // of equal length, in whole groups of four
+}
+
 template <int NB, int NT>
-__device__ __forceinline__ void u_to_s_nodes(const float* v, const float* __restrict__ N, const int* __restrict__ snode,
-                                             long n_map, int k0, int m, int ni, long n3, float* __restrict__ dst) {
+__device__ __forceinline__ void u_to_s_nodes(float* v, const UBlock blk, const float* __restrict__ N,
+                                             const int* __restrict__ snode, long n_map, const int* __restrict__ conn,
+                                             const float* __restrict__ psi_u, int n_orb, int i0, int ni, long n3,
+                                             float* __restrict__ dst) {
+    constexpr int LD = u_chunk_max(NB);
     float w[NT][NB];
     int at[NT], k[NT];
+    auto load = [&]() {
 #pragma unroll
-    for (int j = 0; j < NT; ++j) {
-        k[j] = min((int)threadIdx.x + j * kUThreads, m - 1);
-        at[j] = snode[k0 + k[j]];
+        for (int j = 0; j < NT; ++j) {
+            k[j] = min((int)threadIdx.x + j * kUThreads, blk.m - 1);
+            at[j] = snode[blk.k0 + k[j]];
+        }
+        const float* Nb = N + blk.k0;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            if (b % 8 == 7) asm volatile("" : "+l"(Nb));       // one running pointer, not one per local node
+#pragma unroll
+            for (int j = 0; j < NT; ++j) w[j][b] = __ldg(Nb + k[j]);
+            Nb += n_map;
+        }
+    };
+    // (linear cells: the shape values are on their way while the cell's values come; 3 to 6% on grids of 50^3)
+    if constexpr (NB == 8) load();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int b = warp; b < NB; b += kUThreads / 32) {
+        const float* src = psi_u + (long)conn[(long)blk.cell * NB + b] * n_orb + i0;
+        for (int ii = lane; ii < ((ni + 3) & ~3); ii += 32) v[b * LD + ii] = ii < ni ? src[ii] : 0.f;
     }
-    const float* Nb = N + k0;
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        if (b % 8 == 7) asm volatile("" : "+l"(Nb));           // one running pointer, not one per local node
-#pragma unroll
-        for (int j = 0; j < NT; ++j) w[j][b] = __ldg(Nb + k[j]);
-        Nb += n_map;
-    }
+    __syncthreads();
+    if constexpr (NB != 8) load();
     // four orbitals per pass: one 16-byte broadcast feeds 4 NT FMAs (the staged chunk is zero up to the next
     // multiple of four past ni; the stores are guarded)
     for (int ii = 0; ii < ni; ii += 4, dst += 4 * n3) {
@@ -94,7 +130,7 @@ __device__ __forceinline__ void u_to_s_nodes(const float* v, const float* __rest
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
             if (b % 4 == 0) asm volatile("" ::: "memory");     // at most four reads in flight: the registers hold N
-            const float4 q = *reinterpret_cast<const float4*>(v + b * kUChunk + ii);
+            const float4 q = *reinterpret_cast<const float4*>(v + b * LD + ii);
 #pragma unroll
             for (int j = 0; j < NT; ++j) {
                 s[j][0] = fmaf(w[j][b], q.x, s[j][0]);
@@ -109,34 +145,31 @@ __device__ __forceinline__ void u_to_s_nodes(const float* v, const float* __rest
             if (ii + o < ni)
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
-                    if (threadIdx.x + j * kUThreads < m) row[at[j]] = s[j][o];
+                    if (threadIdx.x + j * kUThreads < blk.m) row[at[j]] = s[j][o];
     }
 }
 
 template <int NB>
-__global__ void __launch_bounds__(kUThreads, NB == 8 ? 6 : NB == 27 ? 4 : 3)
-    k_u_to_s(const UBlock* __restrict__ blocks, const int* __restrict__ snode, const float* __restrict__ N, long n_map,
-             const int* __restrict__ conn, const float* __restrict__ psi_u, int n_orb, long n3, float* __restrict__ psi_s) {
-    extern __shared__ __align__(16) float v[];   // [NB][kUChunk]
-    const UBlock blk = blocks[blockIdx.x];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i0 = 0; i0 < n_orb; i0 += kUChunk) {
-        const int ni = min(kUChunk, n_orb - i0);
-        __syncthreads();
-        for (int b = warp; b < NB; b += kUThreads / 32) {
-            const float* src = psi_u + (long)conn[(long)blk.cell * NB + b] * n_orb + i0;
-            for (int ii = lane; ii < ((ni + 3) & ~3); ii += 32) v[b * kUChunk + ii] = ii < ni ? src[ii] : 0.f;
-        }
-        __syncthreads();
+__global__ void __launch_bounds__(kUThreads, NB == 8 ? 10 : NB == 27 ? 6 : 3)
+    k_u_to_s(const UBlock* __restrict__ blocks, int n_blocks, const int* __restrict__ snode, const float* __restrict__ N,
+             long n_map, const int* __restrict__ conn, const float* __restrict__ psi_u, int n_orb, int chunk, long n3,
+             float* __restrict__ psi_s) {
+    extern __shared__ __align__(16) float v[];   // [NB][u_chunk_max(NB)]
+    const int part = blockIdx.x / n_blocks;
+    const UBlock blk = blocks[blockIdx.x - part * n_blocks];
+    auto pass = [&](int i0) {
+        const int ni = min(chunk, n_orb - i0);
         float* dst = psi_s + (long)i0 * n3;
-        switch ((blk.m + kUThreads - 1) / kUThreads) {
-            case 1: u_to_s_nodes<NB, 1>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst); break;
-            case 2: u_to_s_nodes<NB, 2>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst); break;
-            default:
-                if constexpr (u_nodes(NB) > 2) {
-                    if (blk.m <= 3 * kUThreads) u_to_s_nodes<NB, 3>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst);
-                    else u_to_s_nodes<NB, u_nodes(NB)>(v, N, snode, n_map, blk.k0, blk.m, ni, n3, dst);
-                }
+        if (blk.m <= kUThreads) u_to_s_nodes<NB, 1>(v, blk, N, snode, n_map, conn, psi_u, n_orb, i0, ni, n3, dst);
+        else u_to_s_nodes<NB, kUNodes>(v, blk, N, snode, n_map, conn, psi_u, n_orb, i0, ni, n3, dst);
+    };
+    if constexpr (NB == 8) {
+        pass(part * chunk);
+    } else {
+        // one pass as well: as a loop the compiler keeps the shape values' loads behind the barrier, without spills
+        for (int i0 = part * chunk; i0 < min(n_orb, (part + 1) * chunk); i0 += chunk) {
+            __syncthreads();
+            pass(i0);
         }
     }
 }
@@ -319,7 +352,7 @@ extern "C" int tx_transfer_create(tx_transfer** out, tx_ctx* c, int order_s, con
     t->ps = ps;
     t->n_map = (long)snode.size();
     std::vector<UBlock> blocks;
-    const int most = kUThreads * u_nodes(nb);
+    const int most = kUThreads * kUNodes;
     for (int cc = 0; cc < n_cells; ++cc) {
         const int k0 = cell_start[cc], cnt = cell_start[cc + 1] - k0, pieces = (cnt + most - 1) / most;
         for (int q = 0; q < pieces; ++q) {
@@ -352,14 +385,19 @@ extern "C" int tx_transfer_u_to_s(tx_transfer* t, const float* psi_u, int n_orb,
     TX_TRY(dg.use(t->device));
     cudaStream_t s = (cudaStream_t)stream;
     const long N3 = (long)t->n[0] * t->n[1] * t->n[2];
-    const size_t sm1 = sizeof(float) * 8 * kUChunk, sm2 = sizeof(float) * 27 * kUChunk, sm3 = sizeof(float) * 64 * kUChunk;
     const UBlock* blk = (const UBlock*)t->d_blocks;
-    const unsigned grid = (unsigned)t->n_blocks;
+    const int nb = (t->pu + 1) * (t->pu + 1) * (t->pu + 1), chunk = u_to_s_chunk(nb, n_orb, N3);
+    const size_t smem = sizeof(float) * nb * u_chunk_max(nb);
+    const unsigned grid = (unsigned)t->n_blocks * (unsigned)((n_orb + chunk - 1) / chunk);
+#define TX_U_TO_S(NB_) \
+    k_u_to_s<NB_><<<grid, kUThreads, smem, s>>>(blk, t->n_blocks, t->d_snode, t->d_N, t->n_map, t->d_conn, psi_u, n_orb, chunk, \
+                                            N3, psi_s)
     switch (t->pu) {
-        case 1: k_u_to_s<8><<<grid, kUThreads, sm1, s>>>(blk, t->d_snode, t->d_N, t->n_map, t->d_conn, psi_u, n_orb, N3, psi_s); break;
-        case 2: k_u_to_s<27><<<grid, kUThreads, sm2, s>>>(blk, t->d_snode, t->d_N, t->n_map, t->d_conn, psi_u, n_orb, N3, psi_s); break;
-        default: k_u_to_s<64><<<grid, kUThreads, sm3, s>>>(blk, t->d_snode, t->d_N, t->n_map, t->d_conn, psi_u, n_orb, N3, psi_s); break;
+        case 1: TX_U_TO_S(8); break;
+        case 2: TX_U_TO_S(27); break;
+        default: TX_U_TO_S(64); break;
     }
+#undef TX_U_TO_S
     TX_LAUNCHED();
     return TX_OK;
 }
