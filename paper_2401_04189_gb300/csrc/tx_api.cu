@@ -170,14 +170,13 @@ static void free_ctx(tx_ctx* c) {
         cudaFree(c->d_x[d]);
         cudaFree(c->d_w[d]);
         cudaFree(c->d_U[d]);
-        cudaFree(c->d_UW[d]);
         cudaFree(c->d_A64[d]);
         cudaFree(c->f_U[d]);
         cudaFree(c->f_A[d]);
-        cudaFree(c->f_UK[d]);
         cudaFree(c->f_w[d]);
         cudaFree(c->f_C[d]);
     }
+    cudaFree(c->d_UW[0]);
     free_terms(c);
     cudaFree(c->d_theta);
     cudaFree(c->d_mu);
@@ -241,26 +240,17 @@ extern "C" int tx_tucker_setup(tx_ctx** out, const int n[3], const double* x1, c
         SETUP_TRY(dalloc(&c->d_x[d], nd));
         SETUP_TRY(dalloc(&c->d_w[d], nd));
         SETUP_TRY(dalloc(&c->d_U[d], nd * rd));
-        SETUP_TRY(dalloc(&c->d_UW[d], nd * rd));
         SETUP_TRY(dalloc(&c->d_A64[d], (size_t)T * nd * rd));
         SETUP_TRY(dalloc(&c->f_U[d], nd * rd));
         SETUP_TRY(dalloc(&c->f_A[d], (size_t)T * nd * rd));
-        if (d > 0) {
-            SETUP_TRY(dalloc(&c->f_UK[d], rd * (d == 1 ? simt_ld2((int)nd) : simt_ld3((int)nd))));
-        }
         SETUP_TRY(dalloc(&c->f_w[d], nd));
         // host float32 copies are made synchronously (the host arrays may be freed on return)
         std::vector<float> fu(nd * rd), fw(nd);
-        std::vector<double> uw(nd * rd);
-        for (size_t i = 0; i < nd * rd; ++i) {
-            fu[i] = (float)Us[d][i];
-            uw[i] = Us[d][i] * ws[d][i / rd];
-        }
+        for (size_t i = 0; i < nd * rd; ++i) fu[i] = (float)Us[d][i];
         for (size_t i = 0; i < nd; ++i) fw[i] = (float)ws[d][i];
         if (cudaMemcpy(c->d_x[d], xs[d], sizeof(double) * nd, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(c->d_w[d], ws[d], sizeof(double) * nd, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(c->d_U[d], Us[d], sizeof(double) * nd * rd, cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(c->d_UW[d], uw.data(), sizeof(double) * nd * rd, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(c->f_U[d], fu.data(), sizeof(float) * nd * rd, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(c->f_w[d], fw.data(), sizeof(float) * nd, cudaMemcpyHostToDevice) != cudaSuccess)
             SETUP_TRY(fail(TX_ERR_CUDA, "set-up copy failed"));
@@ -272,7 +262,18 @@ extern "C" int tx_tucker_setup(tx_ctx** out, const int n[3], const double* x1, c
         cudaMemcpy(c->d_mu, gauss_weights, sizeof(double) * T, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(c->d_err, 0, sizeof(int) * kErrWords) != cudaSuccess)
         SETUP_TRY(fail(TX_ERR_CUDA, "set-up copy failed"));
-    for (int d = 1; d < 3; ++d) SETUP_TRY(simt_kmajor(c->f_U[d], 1, n[d], r[d], d == 1 ? simt_ld2(n[d]) : simt_ld3(n[d]), c->f_UK[d], s));
+    {
+        // the basis in the forms that the float32 kernels read, in one allocation
+        const size_t m[3] = {(size_t)n[0] * r[0], (size_t)n[1] * r[1], (size_t)n[2] * r[2]};
+        const size_t k2 = (size_t)r[1] * simt_ld2(n[1]), k3 = (size_t)r[2] * simt_ld3(n[2]);
+        const size_t doubles = (m[0] + m[1] + m[2] + 31) & ~(size_t)31;           // (256 bytes)
+        SETUP_TRY(dalloc(&c->d_UW[0], doubles + (((k2 + 63) & ~(size_t)63) + k3 + 1) / 2));
+        c->d_UW[1] = c->d_UW[0] + m[0];
+        c->d_UW[2] = c->d_UW[1] + m[1];
+        c->f_UK[1] = (float*)(c->d_UW[0] + doubles);
+        c->f_UK[2] = c->f_UK[1] + ((k2 + 63) & ~(size_t)63);
+    }
+    SETUP_TRY(setup_basis_forms(c, s));
     SETUP_TRY(plan_terms(c, xs, gauss_exponents, gauss_weights));
     SETUP_TRY(setup_factor_matrices(c, s));
     SETUP_TRY(tx_set_precision(c, precision, stream));

@@ -90,7 +90,9 @@ struct TcOperands;   // tensor-core operand copies (tx_tc.cu)
 // nf = T and F is the context's f_A.
 struct TermSplit {
     int nf, nc;
-    double* d_theta;     // exponents, sharp then smooth
+    void* pool;          // the allocation that holds everything below (but F without a split)
+    int* d_idx;          // [nf - 1] the sharp terms among the context's
+    double* d_theta;     // [nc] exponents and weights of the smooth terms
     double* d_mu;
     double* d_xi[3];     // [r_d] coarse nodes
     double* F64[3];      // [nf][n_d][r_d] fine operators (mu_t folded into mode 3); null without a split
@@ -253,6 +255,8 @@ int smooth_terms(const int n[3], const int r[3], const double extent[3], int T, 
 // decides the term split of a new context and allocates its operators (host float64 inputs)
 int plan_terms(tx_ctx* c, const double* const x[3], const double* theta, const double* mu);
 void free_terms(tx_ctx* c);
+// U_d w_d, and modes 2 and 3 of U with the grid index fastest (a new context's d_UW, f_UK)
+int setup_basis_forms(tx_ctx* c, cudaStream_t s);
 // setup -- tx_setup.cu (with_c: also write the float32 convolution matrices f_C)
 int setup_factor_matrices(tx_ctx* c, cudaStream_t s, bool with_c = false);
 // the same with finite-element quadrature (Lagrange elements of `order`, `points` Gauss points)

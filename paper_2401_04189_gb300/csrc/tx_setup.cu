@@ -131,7 +131,53 @@ static int conv_factors(const tx_ctx* c, int d, const double* xt, int na, const 
     return TX_OK;
 }
 
+// the sharp terms' fine operators are some of the context's own (terms idx[0 .. ns - 1]), and the term after them
+// (the interpolation, already there in float64) gets its float32 form
+__global__ void __launch_bounds__(256) k_gather_terms(const double* __restrict__ A64, const float* __restrict__ A32,
+                                                      const int* __restrict__ idx, int ns, long per,
+                                                      double* __restrict__ F64, float* __restrict__ F32) {
+    const long e = blockIdx.x * 256L + threadIdx.x, o = blockIdx.y * per + e;
+    if (e >= per) return;
+    if ((int)blockIdx.y < ns) {
+        const long q = idx[blockIdx.y] * per + e;
+        F64[o] = A64[q];
+        F32[o] = A32[q];
+    } else {
+        F32[o] = (float)F64[o];
+    }
+}
+
 static int ld_of(int d, int n) { return d == 1 ? simt_ld2(n) : simt_ld3(n); }
+
+struct BasisArgs {
+    const double* U[3];
+    const double* w[3];
+    double* UW[3];
+    int r[3];
+    long m[3];
+};
+__global__ void __launch_bounds__(256) k_weighted_basis(const BasisArgs a) {
+    const int d = blockIdx.y;
+    const long e = blockIdx.x * 256L + threadIdx.x;
+    if (e < a.m[d]) a.UW[d][e] = a.U[d][e] * a.w[d][e / a.r[d]];
+}
+
+int setup_basis_forms(tx_ctx* c, cudaStream_t s) {
+    BasisArgs a{};
+    long most = 0;
+    for (int d = 0; d < 3; ++d) {
+        a.U[d] = c->d_U[d];
+        a.w[d] = c->d_w[d];
+        a.UW[d] = c->d_UW[d];
+        a.r[d] = c->r[d];
+        a.m[d] = (long)c->n[d] * c->r[d];
+        most = std::max(most, a.m[d]);
+    }
+    k_weighted_basis<<<dim3((unsigned)((most + 255) / 256), 3), 256, 0, s>>>(a);
+    TX_LAUNCHED();
+    for (int d = 1; d < 3; ++d) TX_TRY(simt_kmajor(c->f_U[d], 1, c->n[d], c->r[d], ld_of(d, c->n[d]), c->f_UK[d], s));
+    return TX_OK;
+}
 
 // every operator of the context for one quadrature rule
 static int all_factors(tx_ctx* c, int order, int points, const double* gx, cudaStream_t s, bool with_c) {
@@ -142,9 +188,11 @@ static int all_factors(tx_ctx* c, int order, int points, const double* gx, cudaS
                             with_c ? c->f_C[d] : nullptr, s));
         if (ts.nc) {
             const int ns = ts.nf - 1;
-            if (ns) TX_TRY(conv_factors(c, d, c->d_x[d], n, ts.d_theta, ts.d_mu, ns, order, points, gx, ts.F64[d], ts.F[d],
-                                        nullptr, s));
-            TX_TRY(conv_factors(c, d, ts.d_xi[d], r, ts.d_theta + ns, ts.d_mu + ns, ts.nc, order, points, gx, ts.Q64[d],
+            const long per = (long)n * r;
+            k_gather_terms<<<dim3((unsigned)((per + 255) / 256), (unsigned)ts.nf), 256, 0, s>>>(c->d_A64[d], c->f_A[d],
+                                                                                                ts.d_idx, ns, per, ts.F64[d], ts.F[d]);
+            TX_LAUNCHED();
+            TX_TRY(conv_factors(c, d, ts.d_xi[d], r, ts.d_theta, ts.d_mu, ts.nc, order, points, gx, ts.Q64[d],
                                 ts.Q[d], nullptr, s));
             if (d > 0) {
                 TX_TRY(simt_kmajor(ts.Q[d], ts.nc, r, r, ld_of(d, r), ts.QK[d], s));
@@ -223,38 +271,63 @@ int plan_terms(tx_ctx* c, const double* const x[3], const double* theta, const d
         extent[d] = hi[d] - lo[d];
     }
     std::vector<int> smooth(c->T);
-    std::vector<double> th, m, th_c, m_c;
+    std::vector<double> host;          // smooth exponents, weights, then the coarse nodes
+    std::vector<int> idx;              // sharp terms
     ts.nc = smooth_terms(c->n, c->r, extent, c->T, theta, smooth.data());
-    for (int t = 0; t < c->T; ++t) {
-        (smooth[t] ? th_c : th).push_back(theta[t]);
-        (smooth[t] ? m_c : m).push_back(mu[t]);
-    }
+    for (int t = 0; t < c->T; ++t)
+        if (!smooth[t]) idx.push_back(t);
     const bool on = ts.nc > 0;
-    ts.nf = on ? (int)th.size() + 1 : c->T;
-    auto dalloc = [&](auto** p, size_t count) -> int {
-        if (cudaMalloc((void**)p, sizeof(**p) * std::max<size_t>(count, 1)) == cudaSuccess) return TX_OK;
-        cudaGetLastError();
-        *p = nullptr;
-        return fail(TX_ERR_OOM, "operators of the term split");
+    ts.nf = on ? (int)idx.size() + 1 : c->T;
+    // one allocation for every operator of the split
+    struct Piece {
+        void** p;
+        size_t bytes;
     };
+    std::vector<Piece> pieces;
+    auto want = [&](auto** p, size_t count) { pieces.push_back(Piece{(void**)p, (sizeof(**p) * count + 255) & ~(size_t)255}); };
     for (int d = 0; d < 3; ++d) {
         const size_t n = c->n[d], r = c->r[d];
-        if (d > 0) TX_TRY(dalloc(&ts.FK[d], (size_t)ts.nf * r * ld_of(d, (int)n)));
+        if (d > 0) want(&ts.FK[d], (size_t)ts.nf * r * ld_of(d, (int)n));
         if (!on) {
             ts.F[d] = c->f_A[d];
             continue;
         }
-        TX_TRY(dalloc(&ts.F64[d], (size_t)ts.nf * n * r));
-        TX_TRY(dalloc(&ts.F[d], (size_t)ts.nf * n * r));
-        TX_TRY(dalloc(&ts.Q64[d], (size_t)ts.nc * r * r));
-        TX_TRY(dalloc(&ts.Q[d], (size_t)ts.nc * r * r));
-        if (d > 0) TX_TRY(dalloc(&ts.QK[d], (size_t)ts.nc * r * ld_of(d, (int)r)));
-        if (d > 0) TX_TRY(dalloc(&ts.QKs[d], (size_t)ts.nc * r * ld_of(3 - d, (int)r)));
-        TX_TRY(dalloc(&ts.d_xi[d], r));
+        want(&ts.F64[d], (size_t)ts.nf * n * r);
+        want(&ts.F[d], (size_t)ts.nf * n * r);
+        want(&ts.Q64[d], (size_t)ts.nc * r * r);
+        want(&ts.Q[d], (size_t)ts.nc * r * r);
+        if (d > 0) want(&ts.QK[d], (size_t)ts.nc * r * ld_of(d, (int)r));
+        if (d > 0) want(&ts.QKs[d], (size_t)ts.nc * r * ld_of(3 - d, (int)r));
+    }
+    // ... and one copy for the smooth terms' exponents and weights, the coarse nodes and the sharp terms' indices
+    const size_t nodes = (size_t)c->r[0] + c->r[1] + c->r[2], small = sizeof(double) * (2 * ts.nc + nodes) + sizeof(int) * idx.size();
+    if (on) want(&ts.d_theta, (small + 7) / 8);
+    size_t total = 0;
+    for (const Piece& q : pieces) total += q.bytes;
+    if (cudaMalloc(&ts.pool, total) != cudaSuccess) {
+        cudaGetLastError();
+        ts.pool = nullptr;
+        return fail(TX_ERR_OOM, "operators of the term split");
+    }
+    char* at = (char*)ts.pool;
+    for (const Piece& q : pieces) {
+        *q.p = at;
+        at += q.bytes;
+    }
+    if (!on) return TX_OK;
+    ts.d_mu = ts.d_theta + ts.nc;
+    ts.d_xi[0] = ts.d_mu + ts.nc;
+    ts.d_xi[1] = ts.d_xi[0] + c->r[0];
+    ts.d_xi[2] = ts.d_xi[1] + c->r[1];
+    ts.d_idx = (int*)(ts.d_xi[2] + c->r[2]);
+    for (const double* v : {theta, mu})
+        for (int t = 0; t < c->T; ++t)
+            if (smooth[t]) host.push_back(v[t]);
+    for (int d = 0; d < 3; ++d) {
         // Chebyshev nodes and the barycentric Lagrange values at the grid nodes
+        const size_t n = c->n[d], r = c->r[d];
         const double pi = 3.14159265358979323846;
         std::vector<double> xi(r), bw(r), I(n * r);
-        std::vector<float> If(n * r);
         for (size_t k = 0; k < r; ++k) {
             xi[k] = 0.5 * (lo[d] + hi[d]) - 0.5 * (hi[d] - lo[d]) * std::cos(pi * (k + 0.5) / r);
             bw[k] = (k % 2 ? -1.0 : 1.0) * std::sin(pi * (k + 0.5) / r);
@@ -266,44 +339,24 @@ int plan_terms(tx_ctx* c, const double* const x[3], const double* theta, const d
                 if (x[d][a] == xi[k]) hit = k;
                 else den += bw[k] / (x[d][a] - xi[k]);
             }
-            for (size_t k = 0; k < r; ++k) {
+            for (size_t k = 0; k < r; ++k)
                 I[a * r + k] = hit < r ? (k == hit ? 1.0 : 0.0) : bw[k] / (x[d][a] - xi[k]) / den;
-                If[a * r + k] = (float)I[a * r + k];
-            }
         }
-        const size_t o = (size_t)(ts.nf - 1) * n * r;
-        if (cudaMemcpy(ts.d_xi[d], xi.data(), sizeof(double) * r, cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(ts.F64[d] + o, I.data(), sizeof(double) * n * r, cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(ts.F[d] + o, If.data(), sizeof(float) * n * r, cudaMemcpyHostToDevice) != cudaSuccess)
+        host.insert(host.end(), xi.begin(), xi.end());
+        if (cudaMemcpy(ts.F64[d] + (size_t)(ts.nf - 1) * n * r, I.data(), sizeof(double) * n * r, cudaMemcpyHostToDevice) != cudaSuccess)
             return fail(TX_ERR_CUDA, "term split copy");
     }
-    if (on) {
-        th.insert(th.end(), th_c.begin(), th_c.end());
-        m.insert(m.end(), m_c.begin(), m_c.end());
-        TX_TRY(dalloc(&ts.d_theta, th.size()));
-        TX_TRY(dalloc(&ts.d_mu, m.size()));
-        if (cudaMemcpy(ts.d_theta, th.data(), sizeof(double) * th.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(ts.d_mu, m.data(), sizeof(double) * m.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-            return fail(TX_ERR_CUDA, "term split copy");
-    }
+    const size_t words = host.size();
+    host.resize(words + (idx.size() + 1) / 2);
+    std::memcpy(host.data() + words, idx.data(), sizeof(int) * idx.size());
+    if (cudaMemcpy(ts.d_theta, host.data(), sizeof(double) * host.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+        return fail(TX_ERR_CUDA, "term split copy");
     return TX_OK;
 }
 
 void free_terms(tx_ctx* c) {
-    TermSplit& ts = c->ts;
-    for (int d = 0; d < 3; ++d) {
-        cudaFree(ts.d_xi[d]);
-        cudaFree(ts.F64[d]);
-        if (ts.F[d] != c->f_A[d]) cudaFree(ts.F[d]);
-        cudaFree(ts.FK[d]);
-        cudaFree(ts.Q64[d]);
-        cudaFree(ts.Q[d]);
-        cudaFree(ts.QK[d]);
-        cudaFree(ts.QKs[d]);
-    }
-    cudaFree(ts.d_theta);
-    cudaFree(ts.d_mu);
-    std::memset(&ts, 0, sizeof(ts));
+    cudaFree(c->ts.pool);
+    std::memset(&c->ts, 0, sizeof(c->ts));
 }
 
 Shape fine_shape(const tx_ctx* c) {
