@@ -350,7 +350,8 @@ __device__ __forceinline__ void panel8(const float* __restrict__ A, int lda, con
         }
     }
 }
-// the same for rg column groups, rg <= NA (a runtime value: every warp takes the same branch)
+// the same for rg column groups, rg <= NA (a runtime value: every warp takes the same branch); seven groups run as
+// eight, the last on values that lie behind the row and are not stored
 template <int CL, int NA>
 __device__ __forceinline__ void panel8_any(int rg, const float* A, int lda, const float* B, int ldb, int K,
                                            uint64_t (&acc)[NA][4]) {

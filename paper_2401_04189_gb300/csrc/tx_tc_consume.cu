@@ -443,7 +443,8 @@ constexpr int kMasterGroups = 4;
 
 // One accumulation over KS K steps: main += A_hi B_hi and, for the split precisions, cross += A_hi B_lo +
 // A_lo B_hi.  Descriptors advance by constants from a per-term base and the steps are unrolled: the
-// issuing warp, not the tensor pipe, bounds small tiles.
+// issuing warp, not the tensor pipe, bounds small tiles.  Instances: 2 to 6 and 8 steps, the ranks from 9 to 48
+// and 57 to 64 in TF32 (twice that in bf16); other step counts are right but loop.
 template <bool TF32, bool SPLIT, int KS>
 __device__ __forceinline__ void cv_mmas_k(uint32_t d, uint32_t dc, uint64_t ad, uint64_t bd, uint32_t as, uint32_t bs,
                                           uint32_t al, uint32_t bl, uint32_t id, uint32_t acc0) {
