@@ -273,8 +273,9 @@ extern "C" int tx_tucker_setup(tx_ctx** out, const int n[3], const double* x1, c
         c->f_UK[1] = (float*)(c->d_UW[0] + doubles);
         c->f_UK[2] = c->f_UK[1] + ((k2 + 63) & ~(size_t)63);
     }
-    SETUP_TRY(setup_basis_forms(c, s));
     SETUP_TRY(plan_terms(c, xs, gauss_exponents, gauss_weights));
+    SETUP_TRY(copies_done());
+    SETUP_TRY(setup_basis_forms(c, s));
     SETUP_TRY(setup_factor_matrices(c, s));
     SETUP_TRY(tx_set_precision(c, precision, stream));
 #undef SETUP_TRY

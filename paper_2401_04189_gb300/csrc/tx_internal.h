@@ -34,6 +34,13 @@ void prof_end(int slot, cudaStream_t s);
         if (s_ != TX_OK) return s_;       \
     } while (0)
 
+// A copy from pageable memory may return before it has reached the device, and other streams do not wait for the
+// default one: before the first kernel on a caller's stream reads what was copied.
+inline int copies_done() {
+    TX_TRY_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+    return TX_OK;
+}
+
 // launch bookkeeping: every kernel launch goes through this so a failed launch is caught
 #define TX_LAUNCHED()                                                                  \
     do {                                                                               \

@@ -216,6 +216,7 @@ int setup_factor_matrices_fe(tx_ctx* c, int order, int points, cudaStream_t s, b
     if (cudaMemcpy(d, hx, sizeof(double) * points, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d + points, hw, sizeof(double) * points, cudaMemcpyHostToDevice) != cudaSuccess)
         st = fail(TX_ERR_CUDA, "quadrature points copy");
+    if (st == TX_OK) st = copies_done();
     if (st == TX_OK) st = all_factors(c, order, points, d, s, with_c);
     cudaStreamSynchronize(s);
     cudaFree(d);

@@ -368,6 +368,7 @@ extern "C" int tx_transfer_create(tx_transfer** out, tx_ctx* c, int order_s, con
     if (st == TX_OK) st = upload(&t->d_conn, connv, "cells");
     if (st == TX_OK) st = upload(&t->d_ebase, ebase, "elements");
     if (st == TX_OK) st = upload(&t->d_M, Mv, "structured shape values");
+    if (st == TX_OK) st = copies_done();
     if (st != TX_OK) {
         transfer_free(t);
         return st;
