@@ -244,6 +244,8 @@ int simt_expand_consume(const Shape& sh, const PairRec* recs, int p0, int np, co
 int simt_core_consume(const Shape& sh, int np, float* Z, int nterms, const float* M2, const float* M3, float* H,
                       cudaStream_t s);
 int simt_expand_consume_blocks(const Shape& sh);
+// whether the expansion consumer takes a grid and core of these sizes (not for EPI_STORE)
+bool simt_expand_fits(const Shape& sh);
 // adjoint stage: R[p][t][x][b][g] = sum_{y,z} A_t2[y][b] A_t3[z][g] (prod)[x][y][z]
 // for nt terms (M2 [nt][n2][r2], M3 [nt][n3][r3]); with PROD_PLAIN q_p is the field SA[p] itself
 int simt_adjoint_r(const Shape& sh, const PairRec* recs, int p0, int np, const FieldArgs& f, int nt, const float* M2,

@@ -69,6 +69,11 @@ int simt_project_mode1(const tx_ctx* c, const float* S2, float* G, int np, cudaS
     return simt_gemm(g, s);
 }
 
+int simt_expand_mode1_carried(const tx_ctx* c, const float* H, float* Z, int np, cudaStream_t s) {
+    const int n1 = c->n[0];
+    return gemm_mode1_expand(c, H, c->ts.F[0] + (size_t)(c->ts.nf - 1) * n1 * c->r[0], n1, 1, 0, 1, Z, np, s, 0, true);
+}
+
 int simt_expand_all(const tx_ctx* c, const float* G, float* H, float* Z, int np, cudaStream_t s) {
     const TermSplit& ts = c->ts;
     const int n1 = c->n[0];

@@ -47,6 +47,8 @@ int galerkin_core_dot(const tx_ctx* c, const PairRec* recs, int p0, const float*
 
 // G[p][(b,g)][a] = sum_x S2[p][x][(b,g)] U1[x][a]: mode 1 of the projection (either order of b and g)
 int simt_project_mode1(const tx_ctx* c, const float* S2, float* G, int np, cudaStream_t s);
+// Z[p][x][..] of the interpolation alone from the smooth terms' sum H[p][a][..] (either order of b and g)
+int simt_expand_mode1_carried(const tx_ctx* c, const float* H, float* Z, int np, cudaStream_t s);
 // Z[p][t][x][(b,g)] for every fine term of the split (nf of them) from the cores G[p][(b,g)][a]; H holds
 // r1 r2 r3 floats per pair of scratch (untouched without a split)
 int simt_expand_all(const tx_ctx* c, const float* G, float* H, float* Z, int np, cudaStream_t s);

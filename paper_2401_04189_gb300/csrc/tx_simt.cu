@@ -1127,6 +1127,13 @@ int simt_expand_consume_blocks(const Shape& sh) {
     return simt_plan(dims_of(sh), &p) ? p.nx * p.ny : 1;
 }
 
+bool simt_expand_fits(const Shape& sh) {
+    const Dims d = dims_of(sh);
+    SimtPlan p{};
+    return d.n3 <= 256 && simt_plan(d, &p) &&
+           sizeof(float) * ((size_t)d.r3 * (d.r2 + 1) + 32 * (size_t)(d.r3 + 1) + (size_t)d.n3 * (d.r3 | 1)) <= kSmemLimit;
+}
+
 int simt_ld2(int n2) { return (n2 + 7) & ~7; }
 int simt_ld3(int n3) {
     if (n3 > 256) return pad4(n3);             // no float32 consumer: never read
@@ -1147,8 +1154,7 @@ int simt_expand_consume(const Shape& sh, const PairRec* recs, int p0, int np, co
     const Dims d = dims_of(sh);
     if (d.n3 > 256) return fail(TX_ERR_UNSUPPORTED_SHAPE, "float32 path supports n3 <= 256");
     SimtPlan p{};
-    if (!simt_plan(d, &p) || (!(flags & EPI_STORE) && sizeof(float) * ((size_t)d.r3 * (d.r2 + 1) + 32 * (size_t)(d.r3 + 1) +
-                                              (size_t)d.n3 * (d.r3 | 1)) > kSmemLimit))
+    if (!simt_plan(d, &p) || (!(flags & EPI_STORE) && !simt_expand_fits(sh)))
         return fail(TX_ERR_CUDA, "float32 expansion: (r2 + n3) * r3 too large");
     ConsumeF32Args a{};
     a.d = d;

@@ -76,11 +76,22 @@ int tc_wait_selftest(tx_ctx* c, int hold_tmem, cudaStream_t s) {
     return TX_OK;
 }
 
+static bool smooth_in_f32(const tx_ctx* c);
+
 // Gaussian terms the tensor-core operands hold: the split precisions sum the smooth terms on the
 // coarse grid in float32 and run only the sharp ones and the interpolation on the tensor cores.  The
 // single-pass precisions keep every term: their results are fixed by the rounding of each term's operands.
 int tc_terms(const tx_ctx* c) {
-    return (c->prec == TX_PREC_TF32X3 || c->prec == TX_PREC_BF16X3) ? c->ts.nf : c->T;
+    if (c->prec != TX_PREC_TF32X3 && c->prec != TX_PREC_BF16X3) return c->T;
+    return c->ts.nf - (smooth_in_f32(c) ? 1 : 0);
+}
+
+// BF16x3: the smooth terms' sum is expanded in float32 as well.  As one term on the tensor core it would carry the
+// rounding of one pair of 16-bit operands, where the terms one by one carry many that average out: over nine shapes
+// the error of W rose by 15% on average (46% at most).  (In TF32x3 the operands carry 22 bits and the errors are those of
+// float32 either way.)
+static bool smooth_in_f32(const tx_ctx* c) {
+    return c->prec == TX_PREC_BF16X3 && c->ts.nc > 0 && c->ts.nf > 1 && simt_expand_fits(fine_shape(c));
 }
 
 TcScratch tc_scratch(const tx_ctx* c) {
@@ -209,13 +220,13 @@ int tc_prepare(tx_ctx* c, cudaStream_t s) {
 }
 
 // float32 scratch of the split precisions (elements per pair): the projection's modes and the coarse
-// grid's first expansion mode
+// grid's first expansion mode (or, after it, that of the smooth terms' sum)
 struct SplitF32 {
     size_t s2, g, z;
 };
 static SplitF32 split_f32(const tx_ctx* c) {
     const size_t n1 = c->n[0], r1 = c->r[0], r2 = c->r[1], r3 = c->r[2];
-    return SplitF32{n1 * r3 * r2, r3 * r2 * r1, (size_t)c->ts.nc * r1 * r3 * r2};
+    return SplitF32{n1 * r3 * r2, r3 * r2 * r1, std::max((size_t)c->ts.nc * r1, smooth_in_f32(c) ? n1 : 0) * r3 * r2};
 }
 
 size_t tc_adjoint_bytes_per_pair(const tx_ctx* c);
@@ -252,7 +263,9 @@ static int f32_mode1_expand(const tx_ctx* c, const float* G, bool a_first, int t
     return simt_gemm(g, s);
 }
 
-long tc_epart_per_pair(const tx_ctx* c) { return tc_consume_blocks(c); }
+long tc_epart_per_pair(const tx_ctx* c) {
+    return tc_consume_blocks(c) + (smooth_in_f32(c) ? simt_expand_consume_blocks(fine_shape(c)) : 0);
+}
 
 // The forward hot path of one pair batch (Eq. final, Eq. hadam): pair densities SA[ia] * SB[ib]
 // projected onto the core, expanded over every Gaussian term, and out0[o0] -= mul0[m0] * phi,
@@ -292,7 +305,17 @@ static int tc_forward(tx_ctx* c, const BatchBuffers& b, const PairRec* recs, con
             TX_TRY(simt_expand_consume(coarse_shape(c, true), nullptr, 0, np, fc, Zc, ts.nc, ts.QKs[2], ts.QKs[1], EPI_STORE,
                                        nullptr, s));
             if (ts.nf > 1) TX_TRY(f32_mode1_expand(c, Gf, false, 0, ts.nf - 1, Z, np, s));
-            TX_TRY(f32_mode1_expand(c, H, true, ts.nf - 1, 1, Z, np, s));
+            if (smooth_in_f32(c)) {
+                // its own share of W and, behind the tensor-core kernel's, of the energy sums
+                const size_t last = (size_t)(ts.nf - 1);
+                fa.MUL0 = MUL0; fa.MUL1 = MUL1; fa.OUT0 = OUT0; fa.OUT1 = OUT1;
+                TX_TRY(simt_expand_mode1_carried(c, H, Zc, np, s));
+                TX_TRY(simt_expand_consume(fine_shape(c), recs, b.p0, np, fa, Zc, 1,
+                                           ts.FK[1] + last * r2 * simt_ld2(n2), ts.FK[2] + last * r3 * simt_ld3(c->n[2]), flags,
+                                           b.epart + (size_t)np * tc_consume_blocks(c), s, false));
+            } else {
+                TX_TRY(f32_mode1_expand(c, H, true, ts.nf - 1, 1, Z, np, s));
+            }
         } else {
             TX_TRY(f32_mode1_expand(c, Gf, false, 0, ts.nf, Z, np, s));
         }
@@ -354,7 +377,7 @@ struct AdjF32 {
 static AdjF32 adj_f32(const tx_ctx* c) {
     const size_t n1 = c->n[0], r1 = c->r[0], rr = (size_t)c->r[1] * c->r[2];
     const size_t coarse = c->tc->split ? (size_t)c->ts.nc * r1 * rr : 0;
-    return AdjF32{std::max((size_t)tc_terms(c) * n1 * rr, coarse), rr * r1, n1 * rr};
+    return AdjF32{std::max((size_t)(c->tc->split ? c->ts.nf : c->T) * n1 * rr, coarse), rr * r1, n1 * rr};
 }
 
 // S1 of the tensor-core adjoint (single-pass precisions)
